@@ -78,8 +78,10 @@ int64_t adanns_launch_count(void);
  * feature off) and ADANNS_SCRATCH_GB (GiB); nothing reads the environment
  * after that.  A change applies to calls issued after it; a search plan keeps
  * what it captured.
- *   ADANNS_OPT_FP32_STREAM    1 (default): streaming FP32 scan where few
- *                             queries share a probed list; 0: tiled scan always
+ *   ADANNS_OPT_FP32_STREAM    1 (default): FP32 search by the streaming scan
+ *                             where few queries share a probed list, through
+ *                             the certified tensor-core filter where several
+ *                             do; 0: tiled scan always
  *   ADANNS_OPT_ADC_SELECT     1 (default): IVF-OPQ distance-then-select stage
  *                             for nprobe <= 256; 0: running top-k per list
  *   ADANNS_OPT_COARSE_TC      1 (default): tensor-core cluster mapping where it
@@ -297,8 +299,14 @@ int adanns_kmeans_update(const float *points, int64_t n, int ld, int dim, int me
  *            With few queries per probed list (B * nprobe / nlist <= 16,
  *            nprobe <= 256) the lists are streamed once per 16-query tile
  *            and the distances selected per query afterwards (4 bytes per
- *            probed member of scratch); ADANNS_FP32_STREAM=0 keeps the
- *            shared-memory tiled scan.  Both give the same result.
+ *            probed member of scratch).  Where more share one (prefix-
+ *            normalised metric, k <= 256, nprobe <= 128, and a batch large
+ *            enough to pay for it), FP16 tensor-core products of the probed
+ *            lists first shortlist every member within a rounding-error bound
+ *            of the query's k-th nearest (scratch: 2 d_s bytes per database
+ *            row, at most half of ADANNS_OPT_SCRATCH_BYTES), and the scan's own
+ *            FP32 arithmetic re-scores those.  ADANNS_FP32_STREAM=0 keeps the
+ *            shared-memory tiled scan.  All give the same result, bit for bit.
  *            ADANNS_STORE_BF16 / ADANNS_STORE_FP8E4M3 (tier built into the
  *            index, metric ADANNS_METRIC_L2_PREFIXNORM, nprobe <= 128): the
  *            probed lists are scanned on the tensor cores with FP32
@@ -501,7 +509,8 @@ int adanns_search_ivfopq_budgets(const adanns_index *idx, const float *queries, 
  * (1 warm-up, 3 timed runs; synchronises) and records the fastest for the
  * bucket (device, k rounded up to a power of two, d_s,
  * floor(log2(1 + B * nprobe / nlist))).  Later FP32 searches in the same
- * bucket use it.  All variants give the same results.  *chosen gets the winner
+ * bucket use it (batches that take the certified tensor-core filter, see
+ * adanns_search_ivf, do so tuned or not).  All variants give the same results.  *chosen gets the winner
  * (4 or 1: the tiled scan's queries per thread; 16: the streaming scan),
  * *best_ms its time per call; both may be NULL.  out_ids / out_dist receive
  * the batch's results.  adanns_tune_save / adanns_tune_load write / merge the

@@ -69,6 +69,7 @@ void free_index(adanns_index *x) {
     cudaFree(x->lowp_cx[i]);
   }
   for (int i = 0; i < 4; ++i) cudaFree(x->rr_cmap[i]);
+  cudaFree(x->rr_rank);
   delete[] x->h_list_off;
   delete x;
 }
@@ -306,6 +307,11 @@ int build_rerank_order(adanns_index *x, cudaStream_t st) {
     }
   }
   int rc;
+  std::vector<int32_t> rank((size_t)nl);
+  for (int i = 0; i < nl; ++i) rank[(size_t)ord[(size_t)i]] = i;
+  if ((rc = dmalloc(&x->rr_rank, (size_t)nl))) return rc;
+  ADN_CUDA(cudaMemcpyAsync(x->rr_rank, rank.data(), sizeof(int32_t) * nl, cudaMemcpyHostToDevice,
+                           st));
   std::vector<int4> cm[4];
   for (int ci = 0; ci < 4; ++ci) {
     const int mc = 64 >> ci;
@@ -499,35 +505,89 @@ int adanns_index_status(const adanns_index *idx, void *cuda_stream) {
 }  // extern "C"
 
 namespace adn {
+void tiled_scan_shape(const adanns_index *idx, int64_t B, int d_s, int nprobe, int k,
+                      TiledScan *t) {
+  fp32_scan_shape(idx, B, d_s, nprobe, k, &t->tq, &t->qt, &t->nsplit);
+}
+
+int tiled_scan_scratch(Scratch &s, const adanns_index *idx, int64_t Bc, int nprobe, int k,
+                       TiledScan *t) {
+  const int nlist = idx->nlist;
+  const int64_t max_tiles = (Bc * nprobe + t->qt - 1) / t->qt + nlist;
+  int rc;
+  if ((rc = s.get(&t->pkeys, (size_t)Bc * nprobe * t->nsplit * k)) ||
+      (rc = s.get(&t->lcnt, nlist)) || (rc = s.get(&t->lbeg, nlist)) ||
+      (rc = s.get(&t->lfill, nlist)) || (rc = s.get(&t->tbeg, nlist)) ||
+      (rc = s.get(&t->pair_q, (size_t)Bc * nprobe)) ||
+      (rc = s.get(&t->pair_out, (size_t)Bc * nprobe)) || (rc = s.get(&t->tl, max_tiles)) ||
+      (rc = s.get(&t->tb, max_tiles)) || (rc = s.get(&t->tc, max_tiles)) ||
+      (rc = s.get(&t->ntiles, 1)))
+    return rc;
+  return ADANNS_OK;
+}
+
+int run_tiled_scan(const adanns_index *idx, const TiledScan &t, const float *qs, int ldq,
+                   int64_t nb, int d_s, int nprobe, int k, const uint64_t *ckeys, int *counter,
+                   int32_t *probes_out, int64_t *out_ids, float *out_dist, const MergeMask &mm,
+                   cudaStream_t st) {
+  int rc;
+  {
+    StageTimer tm(ST_INVERT, st);
+    if ((rc = launch_invert_probes(ckeys, nb, nprobe, idx->nlist, t.qt, t.lcnt, t.lbeg, t.lfill,
+                                   t.tbeg, t.pair_q, t.pair_out, t.tl, t.tb, t.tc, t.ntiles,
+                                   probes_out, st)))
+      return rc;
+  }
+  // linear scan of the probed lists at d_s
+  ScanArgs l{};
+  l.xpm = idx->xpm;
+  l.d_pad = idx->d_pad;
+  l.dims = d_s;
+  l.list_off = idx->list_off;
+  l.list_ids = idx->list_ids;
+  l.mscale = idx->metric == ADANNS_METRIC_L2_PREFIXNORM
+                 ? idx->invn + (int64_t)gran_index(d_s) * idx->N
+                 : nullptr;
+  l.qn = qs;
+  l.ldq = ldq;
+  l.tile_list = t.tl;
+  l.tile_beg = t.tb;
+  l.tile_cnt = t.tc;
+  l.ntiles_dev = t.ntiles;
+  l.counter = counter;
+  l.pair_q = t.pair_q;
+  l.pair_out = t.pair_out;
+  l.k = k;
+  l.out_keys = t.pkeys;
+  l.tq = t.tq;
+  l.nsplit = t.nsplit;
+  {
+    StageTimer tm(ST_SCAN, st);
+    if ((rc = launch_scan_f32(l, st))) return rc;
+  }
+  StageTimer tm(ST_MERGE, st);
+  return launch_merge(t.pkeys, nb, nprobe * t.nsplit, k, out_ids, out_dist, st, mm);
+}
+
 int search_f32_tiled(const adanns_index *idx, const float *queries, int64_t B, int d_c, int d_s,
                      int nprobe, int k, int64_t *out_ids, float *out_dist, int32_t *out_probes,
                      cudaStream_t st, const QueryBudgets *qb, const int32_t *rows) {
   int rc;
-  const int nlist = idx->nlist;
   const int dcp = pad16(d_c), dsp = pad16(d_s);
-  int tq, qt, nsplit;
-  fp32_scan_shape(idx, B, d_s, nprobe, k, &tq, &qt, &nsplit);
+  TiledScan ts{};
+  tiled_scan_shape(idx, B, d_s, nprobe, k, &ts);
   // slice the batch so that the per-(query, probe) partial results stay ~2 GiB
   const int64_t per_q =
-      (int64_t)nprobe * nsplit * k * 8 + (int64_t)(dcp + dsp) * 4 + nprobe * 24;
+      (int64_t)nprobe * ts.nsplit * k * 8 + (int64_t)(dcp + dsp) * 4 + nprobe * 24;
   const int64_t Bc = std::max<int64_t>(1, std::min<int64_t>(B, (2ll << 30) / per_q));
-  const int64_t max_tiles = (Bc * nprobe + qt - 1) / qt + nlist;
   Scratch s(st);
   float *qc, *qs;
-  uint64_t *ckeys, *pkeys;
-  int32_t *lcnt, *lbeg, *lfill, *tbeg, *pair_q, *pair_out, *tl, *tb, *tc;
-  int *ntiles, *counter;
+  uint64_t *ckeys;
+  int *counter;
   if ((rc = s.get(&qc, (size_t)Bc * dcp)) || (rc = s.get(&qs, (size_t)Bc * dsp)) ||
-      (rc = s.get(&ckeys, (size_t)Bc * nprobe)) || (rc = s.get(&pkeys, (size_t)Bc * nprobe * nsplit * k)) ||
-      (rc = s.get(&lcnt, nlist)) || (rc = s.get(&lbeg, nlist)) || (rc = s.get(&lfill, nlist)) ||
-      (rc = s.get(&tbeg, nlist)) || (rc = s.get(&pair_q, (size_t)Bc * nprobe)) ||
-      (rc = s.get(&pair_out, (size_t)Bc * nprobe)) || (rc = s.get(&tl, max_tiles)) ||
-      (rc = s.get(&tb, max_tiles)) || (rc = s.get(&tc, max_tiles)) || (rc = s.get(&ntiles, 1)) ||
-      (rc = s.get(&counter, 2)))
+      (rc = s.get(&ckeys, (size_t)Bc * nprobe)) ||
+      (rc = tiled_scan_scratch(s, idx, Bc, nprobe, k, &ts)) || (rc = s.get(&counter, 2)))
     return rc;
-  const float *mscale = idx->metric == ADANNS_METRIC_L2_PREFIXNORM
-                            ? idx->invn + (int64_t)gran_index(d_s) * idx->N
-                            : nullptr;
   for (int64_t b0 = 0; b0 < B; b0 += Bc) {
     const int64_t nb = std::min(Bc, B - b0);
     const QueryBudgets bq = qb ? qb->at(b0) : QueryBudgets{};
@@ -545,51 +605,18 @@ int search_f32_tiled(const adanns_index *idx, const float *queries, int64_t B, i
       if ((rc = run_coarse(idx, qc, dcp, nb, d_c, nprobe, ckeys, counter, st))) return rc;
       if ((rc = launch_mask_probes(ckeys, nb, nprobe, bq.np, st))) return rc;
     }
-    {
-      StageTimer t(ST_INVERT, st);
-      if ((rc = launch_invert_probes(ckeys, nb, nprobe, nlist, qt, lcnt, lbeg, lfill, tbeg, pair_q,
-                                     pair_out, tl, tb, tc, ntiles,
-                                     out_probes ? out_probes + b0 * nprobe : nullptr, st)))
-        return rc;
+    MergeMask mm;
+    if (bq.np) {
+      mm.ckeys = ckeys;
+      mm.nsplit = ts.nsplit;
     }
-    // linear scan of the probed lists at d_s
-    ScanArgs l{};
-    l.xpm = idx->xpm;
-    l.d_pad = idx->d_pad;
-    l.dims = d_s;
-    l.list_off = idx->list_off;
-    l.list_ids = idx->list_ids;
-    l.mscale = mscale;
-    l.qn = qs;
-    l.ldq = dsp;
-    l.tile_list = tl;
-    l.tile_beg = tb;
-    l.tile_cnt = tc;
-    l.ntiles_dev = ntiles;
-    l.counter = counter + 1;
-    l.pair_q = pair_q;
-    l.pair_out = pair_out;
-    l.k = k;
-    l.out_keys = pkeys;
-    l.tq = tq;
-    l.nsplit = nsplit;
-    {
-      StageTimer t(ST_SCAN, st);
-      if ((rc = launch_scan_f32(l, st))) return rc;
-    }
-    {
-      StageTimer t(ST_MERGE, st);
-      MergeMask mm;
-      if (bq.np) {
-        mm.ckeys = ckeys;
-        mm.nsplit = nsplit;
-      }
-      mm.kq = bq.k;
-      mm.orow = rws;
-      if ((rc = launch_merge(pkeys, nb, nprobe * nsplit, k, rws ? out_ids : out_ids + b0 * k,
-                             rws ? out_dist : out_dist + b0 * k, st, mm)))
-        return rc;
-    }
+    mm.kq = bq.k;
+    mm.orow = rws;
+    if ((rc = run_tiled_scan(idx, ts, qs, dsp, nb, d_s, nprobe, k, ckeys, counter + 1,
+                             out_probes ? out_probes + b0 * nprobe : nullptr,
+                             rws ? out_ids : out_ids + b0 * k, rws ? out_dist : out_dist + b0 * k,
+                             mm, st)))
+      return rc;
   }
   return ADANNS_OK;
 }
@@ -618,6 +645,8 @@ int64_t adanns_search_scratch_bytes(const adanns_index *idx, int64_t B, int d_c,
     const int64_t Bc = std::max<int64_t>(1, std::min<int64_t>(B, scratch_budget() / per_q));
     return Bc * per_q + (int64_t)idx->nlist * 64 + (64ll << 20);
   }
+  if (f32_certified(idx, B, d_s, nprobe, k))
+    return certified_scratch_bytes(idx, B, d_c, d_s, nprobe, k);
   if (fp32_stream_enabled((double)B * nprobe / idx->nlist, nprobe, k, d_s))
     return stream_scratch_bytes(idx, B, d_c, d_s, nprobe, k);
   int tq, qt, nsplit;
@@ -710,6 +739,9 @@ int adanns_search_ivf(const adanns_index *idx, const float *queries, int64_t B, 
   if (rerank_k != 0) return fail(ADANNS_ERR_ARG, "rerank_k must be 0 for the FP32 scan");
   if (B == 0) return ADANNS_OK;
   cudaStream_t st = S(cuda_stream);
+  if (f32_certified(idx, B, d_s, nprobe, k))
+    return search_f32_certified(idx, queries, B, d_c, d_s, nprobe, k, out_ids, out_dist,
+                                out_probes, st);
   if (fp32_stream_enabled((double)B * nprobe / idx->nlist, nprobe, k, d_s))
     return search_f32_stream(idx, queries, B, d_c, d_s, nprobe, k, out_ids, out_dist, out_probes,
                              st);

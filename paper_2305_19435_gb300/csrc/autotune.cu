@@ -81,6 +81,8 @@ int tuned_lowp_qt(int which, int d_s, double queries_per_list) {
   return it == g_table.end() ? 0 : it->second;
 }
 
+bool scan_choice_forced() { return g_force_tq != 0; }
+
 int tuned_scan_tq(int k, int d_s, double queries_per_list) {
   if (g_force_tq) return g_force_tq;
   std::lock_guard<std::mutex> g(g_tmu);

@@ -198,4 +198,39 @@ __device__ __forceinline__ void warp_sort(uint64_t *a, int n) {
   }
 }
 
+// Ascending bitonic sort of 256 keys held 8 per lane (lane l holds positions
+// 8l .. 8l + 7): strides below 8 compare within a lane, larger ones across
+// lanes by shuffles; the direction of each compare-exchange is that of the
+// block of `size` positions holding it (ascending for even blocks).
+__device__ __forceinline__ void warp_sort256(uint64_t (&v)[8]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int size = 2; size <= 256; size <<= 1) {
+#pragma unroll
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      if (stride >= 8) {
+        const int ls = stride >> 3;
+        const bool lower = (lane & ls) == 0;
+        const bool asc = ((lane * 8) & size) == 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint64_t o = __shfl_xor_sync(0xffffffffu, v[j], ls);
+          const uint64_t lo = o < v[j] ? o : v[j], hi = o < v[j] ? v[j] : o;
+          v[j] = lower == asc ? lo : hi;
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          if (j & stride) continue;
+          const bool asc = ((lane * 8 + j) & size) == 0;
+          const uint64_t a = v[j], b = v[j | stride];
+          const uint64_t lo = a < b ? a : b, hi = a < b ? b : a;
+          v[j] = asc ? lo : hi;
+          v[j | stride] = asc ? hi : lo;
+        }
+      }
+    }
+  }
+}
+
 }  // namespace adn

@@ -210,10 +210,11 @@ int launch_invert_probe_slots(const uint64_t *ckeys, int64_t B, int nprobe, int 
                               int *ntiles, int32_t *probes_out, cudaStream_t st);
 // Per-query budgets in the merge (all null: none): ckeys / nsplit mark the runs
 // of masked probe slots, kq the per-query k, orow each query's output row.
+// only: merge (and write) just the queries with only[q] < 0.
 struct MergeMask {
   const uint64_t *ckeys = nullptr;
   int nsplit = 1;
-  const int32_t *kq = nullptr, *orow = nullptr;
+  const int32_t *kq = nullptr, *orow = nullptr, *only = nullptr;
 };
 int launch_merge(const uint64_t *pkeys, int64_t B, int nprobe, int k, int64_t *out_ids,
                  float *out_dist, cudaStream_t st, const MergeMask &mm = MergeMask{});
@@ -256,8 +257,9 @@ struct MmaScanArgs {
   int64_t pstride;           // > 0: key segment of pair p at (p / nprobe) * pstride instead
                              // (one segment per query: a scan of the nearest list only)
   const float *cx;           // per member (list order): s_x * nu_x(d_s), 0 for a zero prefix
+                             // (NULL: 1, operands that already are the normalised prefixes)
   const float *qn2;          // per query: |P_ds(q)|^2
-  const float *qsc;          // per query: operand scale s_q
+  const float *qsc;          // per query: operand scale s_q (NULL: 1)
   int nprobe;
   int nkb;                   // K-blocks of the d_s prefix
   int d_blocks;              // storage blocks per vector
@@ -267,6 +269,7 @@ struct MmaScanArgs {
   int *err;
   int *tile_counter;         // zeroed before the launch: next tile to take
   int fp8;
+  int f16;                   // 16-bit operands are FP16 instead of BF16
   int few;                   // few queries per probed list (memory-bound): FP8 takes the
                              // four-stage ring with narrow key staging, as BF16 does
   // filtered mode (rec != NULL, tau != NULL): instead of every key, each
@@ -339,10 +342,53 @@ int search_f32_tiled(const adanns_index *idx, const float *queries, int64_t B, i
 int search_f32_stream(const adanns_index *idx, const float *queries, int64_t B, int d_c, int d_s,
                       int nprobe, int k, int64_t *out_ids, float *out_dist, int32_t *out_probes,
                       cudaStream_t st, const QueryBudgets *qb = nullptr);
+// The tiled scan of a batch's probe keys: its work shape and scratch, then the
+// probe inversion, the scan and the merge.
+struct TiledScan {
+  int tq, qt, nsplit;  // queries per thread, queries per tile, member ranges per tile
+  uint64_t *pkeys;
+  int32_t *lcnt, *lbeg, *lfill, *tbeg, *pair_q, *pair_out, *tl, *tb, *tc;
+  int *ntiles;
+};
+void tiled_scan_shape(const adanns_index *idx, int64_t B, int d_s, int nprobe, int k, TiledScan *t);
+// scratch for Bc queries of the shape set before
+int tiled_scan_scratch(Scratch &s, const adanns_index *idx, int64_t Bc, int nprobe, int k,
+                       TiledScan *t);
+// nb prepared queries qs (rows of ldq) with their probe keys; counter: zeroed
+int run_tiled_scan(const adanns_index *idx, const TiledScan &t, const float *qs, int ldq,
+                   int64_t nb, int d_s, int nprobe, int k, const uint64_t *ckeys, int *counter,
+                   int32_t *probes_out, int64_t *out_ids, float *out_dist, const MergeMask &mm,
+                   cudaStream_t st);
+// The FP32 search through a certified tensor-core filter (certified.cu): same
+// results as the tiled and streaming scans, bit for bit.  The first says
+// whether a batch of this shape takes it.
+bool f32_certified(const adanns_index *idx, int64_t B, int d_s, int nprobe, int k);
+int64_t certified_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,
+                                int k);
+int search_f32_certified(const adanns_index *idx, const float *queries, int64_t B, int d_c,
+                         int d_s, int nprobe, int k, int64_t *out_ids, float *out_dist,
+                         int32_t *out_probes, cudaStream_t st);
+bool scan_choice_forced();  // an FFMA scan variant is being timed by the autotuner
+int launch_mma_scan(const void *qtiles, int64_t qrows, const void *xlow, int64_t xrows,
+                    const MmaScanArgs &a, cudaStream_t st);
+int launch_mma_narrow(const void *qtiles, int64_t qrows, const void *xlow, int64_t xrows,
+                      const MmaScanArgs &a, cudaStream_t st);
+int launch_gather_qtiles(const unsigned char *qlow, int nkb, int64_t max_tiles,
+                         const int32_t *tile_beg, const int32_t *tile_cnt, const int *ntiles,
+                         const int32_t *pair_q, int rows_per_tile, unsigned char *qt,
+                         cudaStream_t st);
 int launch_select16(const uint16_t *cand, const uint64_t *ckeys, int nprobe, const int64_t *qbase,
                     const int64_t *list_off, int kk, int k, const float *qrho, float rmax,
                     float e_rest, int prune, int64_t B, int64_t *out, unsigned long long *stats,
                     cudaStream_t st);
+// Certified shortlist: every candidate whose key is within the query's error
+// bound of its k-th smallest key, at most kk of them, as (list << 32 | member);
+// cnt[q] = how many, or -1 when they exceed kk (out row q is then undefined).
+// stats (NULL, or 2 zeroed device counters): candidates listed, queries with -1.
+int launch_certify16(const uint16_t *cand, const uint64_t *ckeys, int nprobe, const int64_t *qbase,
+                     const int64_t *list_off, int kk, int k, const float *qrho, float rmax,
+                     float e_rest, int64_t B, int64_t *out, int32_t *cnt,
+                     unsigned long long *stats, cudaStream_t st);
 // Filtered tensor-core scan: from the keys of each query's nearest list
 // (cand0 + q * stride0, the list of probe slot 0), tau = their kk-th smallest
 // (0xFFFF with fewer than kk members) and slot 0's records with key <= tau;
@@ -451,6 +497,7 @@ struct adanns_index {
   // chunk count
   int4 *rr_cmap[4] = {nullptr, nullptr, nullptr, nullptr};
   int rr_chunks[4] = {0, 0, 0, 0};
+  int32_t *rr_rank = nullptr;     // each list's place in that order
   int64_t *h_list_off = nullptr;  // host copy of list offsets
   int *dev_err = nullptr;         // sticky device status word (tensor-core pipeline timeouts)
 };

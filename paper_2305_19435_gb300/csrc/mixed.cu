@@ -227,6 +227,17 @@ __global__ void gather_qtiles_kernel(const unsigned char *__restrict__ qlow, int
   }
 }
 
+int launch_gather_qtiles(const unsigned char *qlow, int nkb, int64_t max_tiles,
+                         const int32_t *tile_beg, const int32_t *tile_cnt, const int *ntiles,
+                         const int32_t *pair_q, int rows_per_tile, unsigned char *qt,
+                         cudaStream_t st) {
+  if (max_tiles <= 0) return ADANNS_OK;
+  gather_qtiles_kernel<<<(unsigned)max_tiles, 256, 0, st>>>(qlow, nkb, tile_beg, tile_cnt, ntiles,
+                                                            pair_q, rows_per_tile, qt);
+  ADN_LAUNCH("gather_qtiles_kernel");
+  return ADANNS_OK;
+}
+
 // ---------------------------------------------------------------- candidate segments
 // qtot[q] = sum over slots of the list size rounded up to 8
 __global__ void cand_count_kernel(const uint64_t *__restrict__ ckeys, int64_t B, int nprobe,
@@ -367,13 +378,6 @@ int launch_cand_segments(const uint64_t *ckeys, int64_t B, int nprobe, const int
   ADN_LAUNCH("cand_base_kernel");
   return ADANNS_OK;
 }
-
-// ---------------------------------------------------------------- tensor-core scan launcher
-int launch_mma_scan(const void *qtiles, int64_t qrows, const void *xlow, int64_t xrows,
-                    const MmaScanArgs &a, cudaStream_t st);
-// tiles of 128 members x MMA_NARROW_QT queries (few queries per probed list)
-int launch_mma_narrow(const void *qtiles, int64_t qrows, const void *xlow, int64_t xrows,
-                      const MmaScanArgs &a, cudaStream_t st);
 
 // Certified shortlist pruning (exact: the result equals the unpruned rerank).
 // A shortlisted candidate c is dropped before the exact rerank when its key
@@ -538,9 +542,8 @@ int search_mixed(const adanns_index *idx, const float *queries, int64_t B, int d
       if ((rc = launch_invert_probe_slots(ckeys, nb, nprobe, 0, ns0, nlist, qt, lcnt, lbeg, lfill,
                                           tbeg, pair_q, pair_out, tl, tb, tc, ntiles, probes, st)))
         return rc;
-      gather_qtiles_kernel<<<(unsigned)tiles_a, 256, 0, st>>>(qlow, nkb, tb, tc, ntiles, pair_q, qt,
-                                                              qtile);
-      ADN_LAUNCH("gather_qtiles_kernel");
+      if ((rc = launch_gather_qtiles(qlow, nkb, tiles_a, tb, tc, ntiles, pair_q, qt, qtile, st)))
+        return rc;
       if (tiles_b > 0) {
         const int64_t o1 = nb;  // pairs of set 0
         if ((rc = launch_invert_probe_slots(ckeys, nb, nprobe, 1, nprobe - 1, nlist, qt, lcnt,
@@ -548,10 +551,9 @@ int search_mixed(const adanns_index *idx, const float *queries, int64_t B, int d
                                             tl + tiles_a, tb + tiles_a, tc + tiles_a, ntiles + 1,
                                             probes, st)))
           return rc;
-        gather_qtiles_kernel<<<(unsigned)tiles_b, 256, 0, st>>>(
-            qlow, nkb, tb + tiles_a, tc + tiles_a, ntiles + 1, pair_q + o1, qt,
-            qtile + tiles_a * nkb * qt * 128);
-        ADN_LAUNCH("gather_qtiles_kernel");
+        if ((rc = launch_gather_qtiles(qlow, nkb, tiles_b, tb + tiles_a, tc + tiles_a, ntiles + 1,
+                                       pair_q + o1, qt, qtile + tiles_a * nkb * qt * 128, st)))
+          return rc;
       }
       if ((rc = launch_cand_segments(ckeys, nb, nprobe, idx->list_off, qtot, qbase, pbase, st)))
         return rc;

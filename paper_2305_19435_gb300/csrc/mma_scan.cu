@@ -155,6 +155,13 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// instruction descriptor of an m x n tile: FP32 accumulators; A and B E4M3
+// (kind::f8f6f4) or FP16 (kind::f16), format 0 in both, or BF16 (format 1)
+__device__ __forceinline__ uint32_t mma_idesc(const MmaScanArgs &a, int m, int n) {
+  const uint32_t fmt = a.fp8 || a.f16 ? 0u : (1u << 7) | (1u << 10);
+  return (1u << 4) | fmt | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+}
+
 __device__ __forceinline__ int ld_abort(const int *flag) { return *(const volatile int *)flag; }
 
 // bit e set for each of the 8 16-bit keys of v (key e in half e & 1 of word
@@ -237,9 +244,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = tmem_base_s;
   const int ntiles = *a.ntiles_dev;
-  const uint32_t idesc = a.fp8 ? ((1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24))
-                               : ((1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                                  ((uint32_t)(BM >> 4) << 24));
+  const uint32_t idesc = mma_idesc(a, BM, BN);
 
   // filtered mode: the last work item with member tiles whose survivor counts
   // this epilogue thread still has to write (see the epilogue)
@@ -390,7 +395,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         const int q = p / a.nprobe;
         base = a.pstride ? (int64_t)(p / a.nprobe) * a.pstride : a.pbase[p];
         q2 = a.qn2[q];
-        qs = a.qsc[q];
+        qs = a.qsc ? a.qsc[q] : 1.f;
         pidx = p;
         if (a.tau) tau = a.tau[q];
       }
@@ -406,7 +411,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         float2 v = make_float2(0.f, 0.f);
         if (et < BN) {
           const int m = mt * BN + et;
-          const float c = m < nl ? __ldg(a.cx + off + m) : 0.f;
+          const float c = m < nl ? (a.cx ? __ldg(a.cx + off + m) : 1.f) : 0.f;
           v.x = -2.f * c;
           // |x|^2 in key units (x 2^14, exact); members past the list end: huge
           v.y = m < nl ? 16384.f * (a.x2 ? __ldg(a.x2 + off + m) : (c > 0.f ? 1.f : 0.f)) : 3.0e38f;
@@ -615,9 +620,7 @@ __global__ void __launch_bounds__(N_THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = tmem_base_s;
   const int ntiles = *a.ntiles_dev;
-  const uint32_t idesc = a.fp8 ? ((1u << 4) | ((uint32_t)(NQ >> 3) << 17) | ((uint32_t)(NMT >> 4) << 24))
-                               : ((1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NQ >> 3) << 17) |
-                                  ((uint32_t)(NMT >> 4) << 24));
+  const uint32_t idesc = mma_idesc(a, NMT, NQ);
   auto give_up = [&](int code) {
     atomicExch(&abort_s, 1);
     atomicCAS(a.err, 0, code);
@@ -736,7 +739,7 @@ __global__ void __launch_bounds__(N_THREADS, 1)
         const int p = a.pair_out[a.tile_beg[t] + lane];
         const int q = p / a.nprobe;
         base = a.pbase[p];
-        qsk = 16384.f * a.qsc[q];
+        qsk = 16384.f * (a.qsc ? a.qsc[q] : 1.f);
         q2k = 16384.f * a.qn2[q];
       }
       bool stop = false;
@@ -744,7 +747,7 @@ __global__ void __launch_bounds__(N_THREADS, 1)
         const int m = mt * NMT + quarter * 32 + lane;
         float cb = 0.f, cak = 3.0e38f;  // members past the list end: the largest key
         if (m < nl) {
-          const float c = __ldg(a.cx + off + m);
+          const float c = a.cx ? __ldg(a.cx + off + m) : 1.f;
           cb = -2.f * c;
           cak = 16384.f * (a.x2 ? __ldg(a.x2 + off + m) : (c > 0.f ? 1.f : 0.f));
         }

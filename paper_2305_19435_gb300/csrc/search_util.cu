@@ -567,7 +567,7 @@ __global__ void merge_kernel(const uint64_t *__restrict__ pkeys, int64_t B, int 
   extern __shared__ uint64_t msmem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t qi = (int64_t)blockIdx.x * MERGE_WPB + warp;
-  if (qi >= B) return;
+  if (qi >= B || (m.only && m.only[qi] >= 0)) return;
   uint64_t *buf = msmem + (size_t)warp * cap;
   const uint64_t *src = pkeys + qi * (int64_t)nprobe * k;
   const int nslot = m.ckeys ? nprobe / m.nsplit : 0;

@@ -29,6 +29,9 @@ constexpr int SW_BUF = 1024;
 constexpr int SW_TIE = 128;
 constexpr int SW_MAXP = 128;
 constexpr int SW_PF = 12;
+// survivors aimed at by the certified shortlist: the k nearest (k <= 256) and
+// those within the error bound of the k-th, well inside the buffer
+constexpr int SW_CERT_AIM = 680;
 
 // Per-warp state with a buffer of BUF keys (8.6 KB for the 1,024 of
 // select16_kernel, so that six CTAs of four warps fit on an SM).  The
@@ -36,7 +39,6 @@ constexpr int SW_PF = 12;
 // dead when the compaction fills the buffer, so each pair shares its space.
 template <int BUF>
 struct SwStateT {
-  static constexpr int kBuf = BUF;
   union {
     int hist[256];
     uint64_t ties[SW_TIE];  // (candidate position << 32 | index) of the keys at the cut
@@ -153,11 +155,41 @@ __device__ __forceinline__ bool warp_select16(int n, int kk, int kq, int prune_d
   return true;
 }
 
+// The keys up to (k-th smallest + delta) of n keys, written to o in any order
+// when they number at most kk: their count, else -1 (also when the bound
+// reaches key_limit: only keys below it are known to be among the n).
+template <class KeyF, class IdF, class St>
+__device__ __forceinline__ int warp_certify16(int n, int kk, int k, int delta, KeyF key, IdF id,
+                                              int64_t *o, St &s, uint32_t key_limit) {
+  const int lane = threadIdx.x & 31;
+  int b2, n2;
+  const uint32_t keep_max = warp_kth16(n, k, key, s, b2, n2) + (uint32_t)delta;
+  if (keep_max >= key_limit && key_limit <= 0xFFFFu) return -1;
+  int c = 0;
+  for (int i = lane; i < n; i += 32) c += key(i) <= keep_max ? 1 : 0;
+#pragma unroll
+  for (int o2 = 16; o2 > 0; o2 >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o2);
+  if (c > kk) return -1;
+  int base = 0;
+  for (int i0 = 0; i0 < n; i0 += 32) {
+    const int i = i0 + lane;
+    const bool in = i < n && key(i) <= keep_max;
+    const unsigned b = __ballot_sync(0xffffffffu, in);
+    if (in) o[base + __popc(b & lanemask_lt())] = id(i);
+    base += __popc(b);
+  }
+  return c;
+}
+
+// CERT (launch_certify16): the row gets every candidate that can be among the
+// k nearest, cnt[q] of them, or cnt[q] = -1 when they exceed kk.
+template <bool CERT>
 __global__ void __launch_bounds__(SW_WARPS * 32, 6) select16_kernel(
     const uint16_t *__restrict__ cand, const uint64_t *__restrict__ ckeys, int nprobe,
     const int64_t *__restrict__ qbase, const int64_t *__restrict__ list_off, int kk, int k,
     const float *__restrict__ qrho, float rmax, float e_rest, int prune, int64_t B,
-    int64_t *__restrict__ out, unsigned long long *__restrict__ stats) {
+    int64_t *__restrict__ out, int32_t *__restrict__ cnt,
+    unsigned long long *__restrict__ stats) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   SwState &s = ((SwState *)smem)[warp];
@@ -223,7 +255,11 @@ __global__ void __launch_bounds__(SW_WARPS * 32, 6) select16_kernel(
       for (int m = lane; m < nl; m += 32) o[p0 + m] = ((int64_t)s.lid[sl] << 32) | (int64_t)m;
       p0 += nl;
     }
-    for (int r = total + lane; r < kk; r += 32) o[r] = -1;
+    if (CERT) {
+      if (lane == 0) cnt[q] = total;
+    } else {
+      for (int r = total + lane; r < kk; r += 32) o[r] = -1;
+    }
     return;
   }
   const int kq = prune ? k : 0;
@@ -241,7 +277,9 @@ __global__ void __launch_bounds__(SW_WARPS * 32, 6) select16_kernel(
       for (int e = 0; e < 8; ++e) s.u.samp[8 * j + e] = (uint16_t)((w[e >> 1] >> ((e & 1) * 16)) & 0xFFFFu);
     }
     __syncwarp();
-    int r = (int)((0.5 * (kk + SW_BUF) * ns) / ptotal);
+    // the buffer must hold the keys up to the pruning bound (certified), or kk
+    const int want = CERT ? SW_CERT_AIM : (kk + SW_BUF) / 2;
+    int r = (int)(((double)want * ns) / ptotal);
     r = max(0, min(r, ns - 1));
     int b_, n_;
     const uint32_t kv =
@@ -305,16 +343,35 @@ __global__ void __launch_bounds__(SW_WARPS * 32, 6) select16_kernel(
       }
       __syncwarp();
       const int n = s.n;
-      if (stats && lane == 0) atomicAdd(stats, (unsigned long long)n);
+      if (!CERT && stats && lane == 0) atomicAdd(stats, (unsigned long long)n);
       // 3. exact select on the buffer
-      if (n >= kk && n <= SW_BUF &&
+      if (CERT) {
+        if (n >= k && n <= SW_BUF) {
+          const int c = warp_certify16(n, kk, k, prune_delta,
+                                       [&](int i) -> uint32_t { return s.u.b.key[i]; },
+                                       [&](int i) -> int64_t { return id_at((int)s.u.b.idx[i]); },
+                                       o, s, T);
+          if (c >= 0) {
+            if (lane == 0) cnt[q] = c;
+            if (stats && lane == 0) atomicAdd(stats, (unsigned long long)c);
+            return;
+          }
+        }
+      } else if (n >= kk && n <= SW_BUF &&
           warp_select16<false>(n, kk, kq, prune_delta,
                                [&](int i) -> uint32_t { return s.u.b.key[i]; },
                                [&](int i) -> int64_t { return id_at((int)s.u.b.idx[i]); },
                                [&](int i) -> int { return (int)s.u.b.idx[i]; }, o, s, T))
         return;
     }
-    if (stats && lane == 0) atomicAdd(stats + 1, 1ull);  // the buffer path failed
+    if (!CERT && stats && lane == 0) atomicAdd(stats + 1, 1ull);  // the buffer path failed
+  }
+  if (CERT) {
+    const int c = warp_certify16(ptotal, kk, k, prune_delta,
+                                 [&](int i) -> uint32_t { return src[i]; }, id_at, o, s, 0x10000u);
+    if (lane == 0) cnt[q] = c;
+    if (stats && lane == 0) atomicAdd(stats + (c < 0 ? 1 : 0), (unsigned long long)(c < 0 ? 1 : c));
+    return;
   }
   // exact select over the whole region (index = candidate position)
   warp_select16<true>(ptotal, kk, kq, prune_delta, [&](int i) -> uint32_t { return src[i]; }, id_at,
@@ -541,9 +598,24 @@ int launch_select16(const uint16_t *cand, const uint64_t *ckeys, int nprobe, con
   if (nprobe > SW_MAXP) return fail(ADANNS_ERR_ARG, "select16: nprobe above 128");
   if (B <= 0) return ADANNS_OK;
   const size_t sm = sizeof(SwState) * SW_WARPS;
-  ADN_CUDA(ensure_smem((const void *)select16_kernel, sm));
-  select16_kernel<<<(unsigned)((B + SW_WARPS - 1) / SW_WARPS), SW_WARPS * 32, sm, st>>>(
-      cand, ckeys, nprobe, qbase, list_off, kk, k, qrho, rmax, e_rest, prune, B, out, stats);
+  ADN_CUDA(ensure_smem((const void *)select16_kernel<false>, sm));
+  select16_kernel<false><<<(unsigned)((B + SW_WARPS - 1) / SW_WARPS), SW_WARPS * 32, sm, st>>>(
+      cand, ckeys, nprobe, qbase, list_off, kk, k, qrho, rmax, e_rest, prune, B, out, nullptr,
+      stats);
+  ADN_LAUNCH("select16_kernel");
+  return ADANNS_OK;
+}
+
+int launch_certify16(const uint16_t *cand, const uint64_t *ckeys, int nprobe, const int64_t *qbase,
+                     const int64_t *list_off, int kk, int k, const float *qrho, float rmax,
+                     float e_rest, int64_t B, int64_t *out, int32_t *cnt,
+                     unsigned long long *stats, cudaStream_t st) {
+  if (nprobe > SW_MAXP) return fail(ADANNS_ERR_ARG, "certify16: nprobe above 128");
+  if (B <= 0) return ADANNS_OK;
+  const size_t sm = sizeof(SwState) * SW_WARPS;
+  ADN_CUDA(ensure_smem((const void *)select16_kernel<true>, sm));
+  select16_kernel<true><<<(unsigned)((B + SW_WARPS - 1) / SW_WARPS), SW_WARPS * 32, sm, st>>>(
+      cand, ckeys, nprobe, qbase, list_off, kk, k, qrho, rmax, e_rest, 1, B, out, cnt, stats);
   ADN_LAUNCH("select16_kernel");
   return ADANNS_OK;
 }
