@@ -478,7 +478,12 @@ int adanns_index_get_opq(const adanns_index *idx, float *R, float *codebooks,
  * scratch (4 bytes per member of the probed lists; the batch is sliced so
  * that this stays within the scratch budget) and the best are selected
  * afterwards; ADANNS_ADC_SELECT=0, or nprobe > 256, keeps a running top-k per
- * (query, list) instead.  Both give the same result.
+ * (query, list) instead.  Where many queries share a probed list (plain codes,
+ * prefix-normalised metric, nprobe <= 128, shortlist up to 512, decoded rows of
+ * norm up to 2) the lists are decoded to FP16 rows (2 d_s bytes per database
+ * row of scratch, at most half of the budget), tensor-core products shortlist
+ * every member within a rounding-error bound, and only those are scored by the
+ * lookup tables.  All give the same result.
  */
 int adanns_search_ivfopq(const adanns_index *idx, const float *queries, int64_t B, int d_c,
                          int nprobe, int k, int rerank_k, int64_t *out_ids, float *out_dist,

@@ -63,6 +63,7 @@ void free_index(adanns_index *x) {
   cudaFree(x->opq_R);
   cudaFree(x->opq_C);
   cudaFree(x->codes);
+  cudaFree(x->opq_y2);
   for (int i = 0; i < 2; ++i) {
     cudaFree(x->lowp[i]);
     cudaFree(x->lowp_sx[i]);

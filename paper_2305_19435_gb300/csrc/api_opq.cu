@@ -15,7 +15,7 @@ int launch_pq_update(const float *z, int64_t n, int ldz, int M, int dsub, const 
 int launch_pq_decode(const uint8_t *codes, int64_t n, int M, int dsub, const float *C, float *out,
                      int ldo, cudaStream_t st);
 int launch_pq_lut(const float *z, int64_t B, int ldz, int M, int dsub, const float *C, float *lut,
-                  cudaStream_t st);
+                  cudaStream_t st, const int32_t *only = nullptr);
 int launch_sum_f32(const float *v, int64_t n, double *out, cudaStream_t st);
 int launch_sum_sq(const float *v, int64_t n, double *out, cudaStream_t st);
 int launch_permute_codes(const uint8_t *by_id, const int32_t *list_ids, int64_t N, int M,
@@ -136,6 +136,9 @@ void free_opq(adanns_index *x) {
   cudaFree(x->opq_R);
   cudaFree(x->opq_C);
   cudaFree(x->codes);
+  cudaFree(x->opq_y2);
+  x->opq_y2 = nullptr;
+  x->opq_y2max = INFINITY;
   x->opq_R = x->opq_C = nullptr;
   x->codes = nullptr;
   x->opq_ds = x->opq_M = 0;
@@ -163,6 +166,17 @@ int finish_residual(adanns_index *x, cudaStream_t st) {
                             x->opq_w, d_s, st)))
     return rc;
   return launch_residual_tables(x->opq_w, x->nlist, d_s, M, x->opq_C, x->opq_S, x->opq_w2, st);
+}
+
+// squared norms of the decoded rows, for the tensor-core filter (plain codes
+// of the prefix-normalised metric); synchronises
+int finish_code_norms(adanns_index *x, cudaStream_t st) {
+  if (x->metric != ADANNS_METRIC_L2_PREFIXNORM) return ADANNS_OK;
+  if (cudaMalloc(&x->opq_y2, sizeof(float) * x->N) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(ADANNS_ERR_OOM, "OPQ allocation failed");
+  }
+  return launch_code_norms(x, x->opq_y2, &x->opq_y2max, st);
 }
 
 int alloc_opq(adanns_index *x, int d_s, int M) {
@@ -223,84 +237,185 @@ int search_ivfopq_select(const adanns_index *idx, const float *queries, int64_t 
   const int dcp = pad16(d_c), dsp = pad16(d_s);
   const int qa = adc_dist_query_tile(M);
   const int64_t seg_q = max_probe_members(idx, nprobe);
-  const int64_t per_q = seg_q * 4 + (int64_t)(dcp + dsp + d_s) * 4 + (int64_t)M * 1024 +
-                        (int64_t)kr * 16 + (int64_t)nprobe * 40 + 16;
-  const int64_t Bc = std::max<int64_t>(1, std::min<int64_t>(B, scratch_budget() / per_q));
+  // many queries per probed list: 16-bit keys from the tensor cores, the exact
+  // scores for the certified shortlist only, the lookup scan (in `parts` parts
+  // of the batch, in the keys' space) for the queries left over
+  const bool cert = adc_certified(idx, B, nprobe, kr);
+  const int nkb = (d_s + 63) / 64, QT = 128, kk = CERT_MAX_KK;
+  const int64_t budget = scratch_budget() - (cert ? idx->N * nkb * 128ll : 0);
+  auto per_q_of = [&](int cand_bytes) -> int64_t {
+    return seg_q * cand_bytes + (int64_t)(dcp + dsp + d_s) * 4 + (int64_t)M * 1024 +
+           (int64_t)kr * 16 + (int64_t)nprobe * 40 + 16 +
+           (cert ? (int64_t)nprobe * nkb * 128 + nkb * 128 + kk * 8 + 12 : 0);
+  };
+  const int parts = cert && budget / per_q_of(4) < B ? 2 : 1;
+  const int64_t Bc =
+      std::max<int64_t>(1, std::min<int64_t>(B, budget / per_q_of(parts == 2 ? 2 : 4)));
+  const int64_t Bp = (Bc + parts - 1) / parts;  // queries per lookup scan
   const int64_t max_tiles = (Bc * nprobe + qa - 1) / qa + nlist;
+  const int64_t mma_tiles = (Bc * nprobe + QT - 1) / QT + nlist;
   Scratch s(st);
-  float *qc, *qs, *z, *lut;
+  float *qc, *qs, *z, *lut, *qn2 = nullptr, *qerr = nullptr;
   uint64_t *ckeys, *keys;
   uint32_t *cand;
-  int64_t *qtot, *qbase, *pbase, *cids;
-  int32_t *lcnt, *lbeg, *lfill, *tbeg, *pair_q, *pair_out, *tl, *tb, *tc;
+  int64_t *qtot, *qbase, *pbase, *cids, *list = nullptr;
+  int32_t *lcnt, *lbeg, *lfill, *tbeg, *pair_q, *pair_out, *tl, *tb, *tc, *cnt = nullptr;
   int *ntiles, *counter;
+  unsigned char *rows = nullptr, *qlow = nullptr, *qtile = nullptr;
+  unsigned long long *stats = nullptr;
   int rc;
   if ((rc = s.get(&qc, (size_t)Bc * dcp)) || (rc = s.get(&qs, (size_t)Bc * dsp)) ||
-      (rc = s.get(&z, (size_t)Bc * d_s)) || (rc = s.get(&lut, (size_t)Bc * M * 256)) ||
-      (rc = s.get(&ckeys, (size_t)Bc * nprobe)) || (rc = s.get(&cand, (size_t)(Bc * seg_q))) ||
+      (rc = s.get(&z, (size_t)Bc * d_s)) || (rc = s.get(&lut, (size_t)Bp * M * 256)) ||
+      (rc = s.get(&ckeys, (size_t)Bc * nprobe)) || (rc = s.get(&cand, (size_t)(Bp * seg_q))) ||
       (rc = s.get(&keys, (size_t)Bc * kr)) || (rc = s.get(&cids, (size_t)Bc * kr)) ||
       (rc = s.get(&qtot, (size_t)Bc)) || (rc = s.get(&qbase, (size_t)Bc)) ||
       (rc = s.get(&pbase, (size_t)Bc * nprobe)) || (rc = s.get(&lcnt, nlist)) ||
       (rc = s.get(&lbeg, nlist)) || (rc = s.get(&lfill, nlist)) || (rc = s.get(&tbeg, nlist)) ||
       (rc = s.get(&pair_q, (size_t)Bc * nprobe)) || (rc = s.get(&pair_out, (size_t)Bc * nprobe)) ||
       (rc = s.get(&tl, max_tiles)) || (rc = s.get(&tb, max_tiles)) ||
-      (rc = s.get(&tc, max_tiles)) || (rc = s.get(&ntiles, 1)) || (rc = s.get(&counter, 2)))
+      (rc = s.get(&tc, max_tiles)) || (rc = s.get(&ntiles, 1)) || (rc = s.get(&counter, 4)))
+    return rc;
+  if (cert && ((rc = s.get(&rows, (size_t)idx->N * nkb * 128)) ||
+               (rc = s.get(&qlow, (size_t)Bc * nkb * 128)) ||
+               (rc = s.get(&qtile, (size_t)mma_tiles * nkb * QT * 128)) ||
+               (rc = s.get(&qn2, Bc)) || (rc = s.get(&qerr, Bc)) || (rc = s.get(&cnt, Bc)) ||
+               (rc = s.get(&list, (size_t)Bc * kk)) || (profiling() && (rc = s.get(&stats, 2)))))
     return rc;
   const float *mscale = idx->metric == ADANNS_METRIC_L2_PREFIXNORM
                             ? idx->invn + (int64_t)gran_index(d_s) * idx->N
                             : nullptr;
+  // the lookup scan and the selection of queries [p0, p0 + np) of the slice
+  // (with cert, those of them with cnt < 0: the others' probe slots are masked)
+  auto lookup_scan = [&](int64_t p0, int64_t np, int *work, int32_t *probes) -> int {
+    const uint64_t *ck = ckeys + p0 * nprobe;
+    const int32_t *only = cert ? cnt + p0 : nullptr;
+    {
+      StageTimer t(ST_INVERT, st);
+      if ((rc = launch_invert_probes(ck, np, nprobe, nlist, qa, lcnt, lbeg, lfill, tbeg, pair_q,
+                                     pair_out, tl, tb, tc, ntiles, probes, st)))
+        return rc;
+      if ((rc = launch_cand_segments(ck, np, nprobe, idx->list_off, qtot, qbase, pbase, st)))
+        return rc;
+    }
+    {
+      StageTimer t(ST_LUT, st);
+      if ((rc = launch_pq_lut(z + p0 * d_s, np, d_s, M, dsub, idx->opq_C, lut, st, only)))
+        return rc;
+    }
+    {
+      StageTimer t(ST_ADC, st);
+      // few work items (few queries, or one long list as in the exhaustive
+      // search): split each list into member ranges so every SM has work
+      const int64_t tiles_est = (np * nprobe + qa - 1) / qa;
+      const int64_t target = (int64_t)num_sms() * 4;
+      const int nsplit = tiles_est >= target
+                             ? 1
+                             : (int)std::min<int64_t>((target + tiles_est - 1) / tiles_est,
+                                                      ((int64_t)idx->max_list + 255) / 256);
+      if ((rc = launch_adc_dist(idx->codes, idx->list_off, M, lut, tl, tb, tc, ntiles, work, pair_q,
+                                pair_out, pbase, cand, qa, nsplit, st, idx->opq_S, idx->opq_w,
+                                idx->opq_w2, z + p0 * d_s, d_s)))
+        return rc;
+    }
+    StageTimer t(ST_MERGE, st);
+    return launch_select32(cand, ck, nprobe, qbase, idx->list_off, idx->list_ids, np, kr,
+                           keys + p0 * kr, st, only);
+  };
   for (int64_t b0 = 0; b0 < B; b0 += Bc) {
     const int64_t nb = std::min(Bc, B - b0);
+    int32_t *probes = out_probes ? out_probes + b0 * nprobe : nullptr;
     {
       StageTimer t(ST_PREP, st);
       if ((rc = launch_prep_queries(queries + b0 * idx->d, nb, idx->d, d_c, d_s, idx->metric, qc,
                                     dcp, qs, dsp, st)))
         return rc;
     }
-    ADN_CUDA(cudaMemsetAsync(counter, 0, 2 * sizeof(int), st));
+    // work counters: cluster mapping, tensor-core scan, lookup scans
+    ADN_CUDA(cudaMemsetAsync(counter, 0, 4 * sizeof(int), st));
     {
       StageTimer t(ST_COARSE, st);
       if ((rc = run_coarse(idx, qc, dcp, nb, d_c, nprobe, ckeys, counter, st))) return rc;
       if (qb && (rc = launch_mask_probes(ckeys, nb, nprobe, qb->at(b0).np, st))) return rc;
     }
     {
-      StageTimer t(ST_INVERT, st);
-      if ((rc = launch_invert_probes(ckeys, nb, nprobe, nlist, qa, lcnt, lbeg, lfill, tbeg, pair_q,
-                                     pair_out, tl, tb, tc, ntiles,
-                                     out_probes ? out_probes + b0 * nprobe : nullptr, st)))
-        return rc;
-      if ((rc = launch_cand_segments(ckeys, nb, nprobe, idx->list_off, qtot, qbase, pbase, st)))
-        return rc;
-    }
-    {
       StageTimer t(ST_LUT, st);
       if ((rc = launch_gemm_f32(false, (int)nb, d_s, d_s, 1.f, qs, dsp, idx->opq_R, d_s, 0.f, z,
                                 d_s, st)))
         return rc;
-      if ((rc = launch_pq_lut(z, nb, d_s, M, dsub, idx->opq_C, lut, st))) return rc;
     }
-    {
-      StageTimer t(ST_ADC, st);
-      // few work items (few queries, or one long list as in the exhaustive
-      // search): split each list into member ranges so every SM has work
-      const int64_t tiles_est = (nb * nprobe + qa - 1) / qa;
-      const int64_t target = (int64_t)num_sms() * 4;
-      const int nsplit = tiles_est >= target
-                             ? 1
-                             : (int)std::min<int64_t>((target + tiles_est - 1) / tiles_est,
-                                                      ((int64_t)idx->max_list + 255) / 256);
-      if ((rc = launch_adc_dist(idx->codes, idx->list_off, M, lut, tl, tb, tc, ntiles, counter + 1,
-                                pair_q, pair_out, pbase, cand, qa, nsplit, st, idx->opq_S,
-                                idx->opq_w, idx->opq_w2, z, d_s)))
-        return rc;
+    if (!cert) {
+      if ((rc = lookup_scan(0, nb, counter + 2, probes))) return rc;
+    } else {
+      {
+        StageTimer t(ST_INVERT, st);
+        if ((rc = launch_invert_probes(ckeys, nb, nprobe, nlist, QT, lcnt, lbeg, lfill, tbeg,
+                                       pair_q, pair_out, tl, tb, tc, ntiles, probes, st)))
+          return rc;
+        if ((rc = launch_cand_segments(ckeys, nb, nprobe, idx->list_off, qtot, qbase, pbase, st)))
+          return rc;
+      }
+      {
+        StageTimer t(ST_PREP, st);
+        // every list when the batch is sliced, else the probed ones
+        if (b0 == 0 && (rc = launch_decode_f16(idx, Bc < B ? nullptr : lcnt, nkb, rows, st)))
+          return rc;
+        const float yn = sqrtf(idx->opq_y2max) * 1.0001f;
+        const float yr = (float)(yn * std::ldexp(1.0, -11) + d_s * std::ldexp(1.0, -25));
+        if ((rc = launch_f16_queries(z, d_s, nb, d_s, nkb, nullptr, yn, yr, 4.f, qlow, qn2, qerr,
+                                     st)))
+          return rc;
+        if ((rc = launch_gather_qtiles(qlow, nkb, mma_tiles, tb, tc, ntiles, pair_q, QT, qtile,
+                                       st)))
+          return rc;
+      }
+      {
+        StageTimer t(ST_MMA, st);
+        MmaScanArgs m{};
+        m.tile_list = tl;
+        m.tile_beg = tb;
+        m.tile_cnt = tc;
+        m.ntiles_dev = ntiles;
+        m.list_off = idx->list_off;
+        m.pair_out = pair_out;
+        m.pbase = pbase;
+        m.qn2 = qn2;
+        m.x2 = idx->opq_y2;
+        m.nprobe = nprobe;
+        m.nkb = nkb;
+        m.d_blocks = nkb;
+        m.cand = (uint16_t *)cand;
+        m.err = idx->dev_err;
+        m.tile_counter = counter + 1;
+        m.f16 = 1;
+        m.nsplit = mma_scan_nsplit(idx, nb * nprobe);
+        if ((rc = launch_mma_scan(qtile, mma_tiles * nkb * QT, rows, idx->N * (int64_t)nkb, m,
+                                  st)))
+          return rc;
+      }
+      {
+        StageTimer t(ST_SELECT, st);
+        if (stats) ADN_CUDA(cudaMemsetAsync(stats, 0, 2 * sizeof(unsigned long long), st));
+        if ((rc = launch_certify16((const uint16_t *)cand, ckeys, nprobe, qbase, idx->list_off, kk,
+                                   kr, qerr, nb, list, cnt, stats, st)))
+          return rc;
+        if (stats) {
+          profile_count(PC_SURVIVORS, (const int64_t *)stats, st);
+          profile_count(PC_SELECT_SLOW, (const int64_t *)stats + 1, st);
+        }
+      }
+      {
+        StageTimer t(ST_MERGE, st);
+        if ((rc = launch_adc_rescore(idx, list, cnt, kk, z, nb, kr, keys, st))) return rc;
+        if ((rc = launch_mask_answered(ckeys, nb, nprobe, cnt, st))) return rc;
+      }
+      for (int h = 0; h < parts; ++h) {
+        const int64_t p0 = h * Bp, np = std::min(Bp, nb - p0);
+        if (np > 0 && (rc = lookup_scan(p0, np, counter + 2 + h, nullptr))) return rc;
+      }
     }
-    {
+    if (!rerank) {
       StageTimer t(ST_MERGE, st);
-      if ((rc = launch_select32(cand, ckeys, nprobe, qbase, idx->list_off, idx->list_ids, nb, kr,
-                                keys, st)))
-        return rc;
-      if (!rerank &&
-          (rc = launch_final_topk(keys, kr, nb, k, out_ids + b0 * k, out_dist + b0 * k, st)))
+      if ((rc = launch_final_topk(keys, kr, nb, k, out_ids + b0 * k, out_dist + b0 * k, st)))
         return rc;
     }
     if (rerank) {
@@ -496,7 +611,7 @@ static int build_opq_impl(adanns_index *idx, const float *db, int d_s, int M, in
     return rc;
   put(dist);
   if ((rc = encode_lists(idx, db, st))) return rc;
-  if (residual && (rc = finish_residual(idx, st))) return rc;
+  if ((rc = residual ? finish_residual(idx, st) : finish_code_norms(idx, st))) return rc;
   ADN_CUDA(cudaStreamSynchronize(st));
   return ADANNS_OK;
 }
@@ -511,7 +626,9 @@ int adanns_index_set_opq(adanns_index *idx, int d_s, int M, const float *R,
   ADN_CUDA(cudaMemcpyAsync(idx->opq_R, R, sizeof(float) * d_s * d_s, cudaMemcpyDeviceToDevice, st));
   ADN_CUDA(cudaMemcpyAsync(idx->opq_C, codebooks, sizeof(float) * M * 256 * (d_s / M),
                            cudaMemcpyDeviceToDevice, st));
-  if ((rc = launch_permute_codes(codes_by_id, idx->list_ids, idx->N, M, idx->codes, st))) return rc;
+  if ((rc = launch_permute_codes(codes_by_id, idx->list_ids, idx->N, M, idx->codes, st)) ||
+      (rc = finish_code_norms(idx, st)))
+    return rc;
   ADN_CUDA(cudaStreamSynchronize(st));
   return ADANNS_OK;
 }

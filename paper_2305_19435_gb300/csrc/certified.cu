@@ -27,7 +27,7 @@
 // The bound.  With u = 2^-11 (FP16 rounding; entries of a unit vector below
 // 2^-14 lose at most 2^-25 each), p = P(q), y = P(x) of norm at most 1.005:
 // |p.y - p~.y~| <= |p||r_y| + |r_p||y| + |r_p||r_y|, |r_y| <= 1.005 u + d 2^-25
-// (member side, a constant), |r_p| measured per query; the FP32 accumulation
+// (member side, a constant), |p| and |r_p| measured per query; the FP32 accumulation
 // and re-score terms are those of the mixed-precision pruning (e_rest).
 // Prefixes whose computed norm is off (sums of squares in the denormal range)
 // make the whole call take the tiled scan through the same mechanism.
@@ -44,7 +44,7 @@ namespace {
 
 constexpr int CE_MAX_K = 256;       // the shortlist buffer holds k and the bound's margin
 constexpr float CE_NORM2 = 1.01f;   // largest |P(v)|^2 the bound covers
-constexpr float CE_UNSURE = 1e3f;   // residual that makes a query's bound useless
+constexpr float CE_UNSURE = 1e3f;   // the bound of a query that has none: it keeps every member
 
 __device__ __forceinline__ uint2 half4(float a, float b, float c, float d) {
   const __half2 lo = __floats2half2_rn(a, b), hi = __floats2half2_rn(c, d);
@@ -107,12 +107,13 @@ __global__ void __launch_bounds__(256) f16_rows_kernel(
   }
 }
 
-// Per query (one warp): |P(q)|^2, the FP16 row (nkb blocks of 64, zero beyond
-// d_s) and the residual norm |P(q) - q~|.
+// Per query (one warp) of rows v: |v|^2, the FP16 row (nkb blocks of 64, zero
+// beyond d_s) and a bound of |approximate - exact distance| to any member of
+// norm at most yn whose FP16 residual is at most yr (see the file's header).
 __global__ void f16_queries_kernel(const float *__restrict__ qs, int ldq, int64_t B, int d_s,
-                                   int nkb, const int *__restrict__ unsure,
-                                   uint2 *__restrict__ out, float *__restrict__ qn2,
-                                   float *__restrict__ qrho) {
+                                   int nkb, const int *__restrict__ unsure, float yn, float yr,
+                                   float zmax2, float e_rest, uint2 *__restrict__ out,
+                                   float *__restrict__ qn2, float *__restrict__ qerr) {
   const int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (q >= B) return;
@@ -138,8 +139,11 @@ __global__ void f16_queries_kernel(const float *__restrict__ qs, int ldq, int64_
     r2 += __shfl_xor_sync(0xffffffffu, r2, o);
   }
   if (lane == 0) {
+    const float zn = sqrtf(s2), rho = sqrtf(r2), h = 0.5f * (zn + yn);
     qn2[q] = s2;
-    qrho[q] = *unsure || !(s2 <= CE_NORM2) ? CE_UNSURE : sqrtf(r2);
+    qerr[q] = (unsure && *unsure) || !(s2 <= zmax2)
+                  ? CE_UNSURE
+                  : 2.f * (zn * yr + rho * yn + rho * yr) * 1.001f + e_rest * fmaxf(1.f, h * h);
   }
 }
 
@@ -272,8 +276,35 @@ __global__ void __launch_bounds__(RS_W * 32) rescore_kernel(
   }
 }
 
+}  // namespace
+
+int launch_f16_queries(const float *v, int ldv, int64_t B, int d_s, int nkb, const int *unsure,
+                       float yn, float yr, float zmax2, void *out, float *qn2, float *qerr,
+                       cudaStream_t st) {
+  if (B <= 0) return ADANNS_OK;
+  // FP32 accumulation on the tensor cores, the FP32 norms and the re-score's rounding
+  const float e_rest = (float)(2.0 * nkb * 64 * std::ldexp(1.0, -22) +
+                               8.0 * (d_s + 2) * std::ldexp(1.0, -24) + 1e-4);
+  f16_queries_kernel<<<(unsigned)((B + 7) / 8), 256, 0, st>>>(v, ldv, B, d_s, nkb, unsure, yn, yr,
+                                                              zmax2, e_rest, (uint2 *)out, qn2,
+                                                              qerr);
+  ADN_LAUNCH("f16_queries_kernel");
+  return ADANNS_OK;
+}
+
+int launch_mask_answered(uint64_t *ckeys, int64_t B, int nprobe, const int32_t *cnt,
+                         cudaStream_t st) {
+  const int64_t n = B * nprobe;
+  if (n <= 0) return ADANNS_OK;
+  mask_answered_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(ckeys, n, nprobe, cnt);
+  ADN_LAUNCH("mask_answered_kernel");
+  return ADANNS_OK;
+}
+
+namespace {
+
 // shortlist slots: room for the k nearest and as many more near the k-th
-int shortlist_cap(int k) { return std::min(1024, std::max(4 * k, 256)); }
+int shortlist_cap(int k) { return std::min(CERT_MAX_KK, std::max(4 * k, 256)); }
 
 struct Shape {
   int nkb, kk;
@@ -343,7 +374,7 @@ int search_f32_certified(const adanns_index *idx, const float *queries, int64_t 
   const int64_t max_tiles = (Bc * nprobe + QT - 1) / QT + nlist;
   const bool ordered = Bc >= 4096 && nlist > 1;  // fewer queries: their rows fit in L2 anyway
   Scratch s(st);
-  float *qc, *qs, *qn2, *qrho, *x2;
+  float *qc, *qs, *qn2, *qerr, *x2;
   uint64_t *ckeys;
   int32_t *lcnt, *lbeg, *lfill, *tbeg, *pair_q, *pair_out, *tl, *tb, *tc, *cnt, *ocur = nullptr,
       *order = nullptr;
@@ -355,7 +386,7 @@ int search_f32_certified(const adanns_index *idx, const float *queries, int64_t 
   int rc;
   if ((rc = s.get(&rows, (size_t)idx->N * nkb * 128 + 256)) || (rc = s.get(&x2, idx->N)) ||
       (rc = s.get(&qc, (size_t)Bc * dcp)) || (rc = s.get(&qs, (size_t)Bc * dsp)) ||
-      (rc = s.get(&qn2, Bc)) || (rc = s.get(&qrho, Bc)) ||
+      (rc = s.get(&qn2, Bc)) || (rc = s.get(&qerr, Bc)) ||
       (rc = s.get(&ckeys, (size_t)Bc * nprobe)) || (rc = s.get(&lcnt, nlist)) ||
       (rc = s.get(&lbeg, nlist)) || (rc = s.get(&lfill, nlist)) || (rc = s.get(&tbeg, nlist)) ||
       (rc = s.get(&pair_q, (size_t)Bc * nprobe)) || (rc = s.get(&pair_out, (size_t)Bc * nprobe)) ||
@@ -371,9 +402,8 @@ int search_f32_certified(const adanns_index *idx, const float *queries, int64_t 
   if (ordered && ((rc = s.get(&ocur, nlist)) || (rc = s.get(&order, Bc)))) return rc;
   if (profiling() && (rc = s.get(&stats, 2))) return rc;
   const float *nu = idx->invn + (int64_t)gran_index(d_s) * idx->N;
-  const float rmax = (float)(1.005 * std::ldexp(1.0, -11) + d_s * std::ldexp(1.0, -25));
-  const float e_rest = (float)(2.0 * nkb * 64 * std::ldexp(1.0, -22) +
-                               8.0 * (d_s + 2) * std::ldexp(1.0, -24) + 1e-4);
+  const float yn = sqrtf(CE_NORM2);
+  const float yr = (float)(yn * std::ldexp(1.0, -11) + d_s * std::ldexp(1.0, -25));
   const size_t rsm = (size_t)pad16(d_s) * 4 + (size_t)RS_W * RS_ST * 32 * RS_ROW * 4 + (size_t)kk * 8;
   ADN_CUDA(ensure_smem((const void *)rescore_kernel, rsm));
   for (int64_t b0 = 0; b0 < B; b0 += Bc) {
@@ -410,9 +440,9 @@ int search_f32_certified(const adanns_index *idx, const float *queries, int64_t 
             (uint2 *)rows, x2, flags + 3);
         ADN_LAUNCH("f16_rows_kernel");
       }
-      f16_queries_kernel<<<(unsigned)((nb + 7) / 8), 256, 0, st>>>(qs, dsp, nb, d_s, nkb, flags + 3,
-                                                                   (uint2 *)qlow, qn2, qrho);
-      ADN_LAUNCH("f16_queries_kernel");
+      if ((rc = launch_f16_queries(qs, dsp, nb, d_s, nkb, flags + 3, yn, yr, CE_NORM2, qlow, qn2,
+                                   qerr, st)))
+        return rc;
       if ((rc = launch_gather_qtiles(qlow, nkb, max_tiles, tb, tc, ntiles, pair_q, QT, qtile, st)))
         return rc;
     }
@@ -435,14 +465,15 @@ int search_f32_certified(const adanns_index *idx, const float *queries, int64_t 
       m.err = idx->dev_err;
       m.tile_counter = flags + 1;
       m.f16 = 1;
+      m.nsplit = mma_scan_nsplit(idx, nb * nprobe);
       if ((rc = launch_mma_scan(qtile, max_tiles * nkb * QT, rows, idx->N * (int64_t)nkb, m, st)))
         return rc;
     }
     {
       StageTimer t(ST_SELECT, st);
       if (stats) ADN_CUDA(cudaMemsetAsync(stats, 0, 2 * sizeof(unsigned long long), st));
-      if ((rc = launch_certify16(cand, ckeys, nprobe, qbase, idx->list_off, kk, k, qrho, rmax,
-                                 e_rest, nb, cids, cnt, stats, st)))
+      if ((rc = launch_certify16(cand, ckeys, nprobe, qbase, idx->list_off, kk, k, qerr, nb,
+                                 cids, cnt, stats, st)))
         return rc;
       if (stats) {
         profile_count(PC_RERANK_PAIRS, (const int64_t *)stats, st);
@@ -465,9 +496,7 @@ int search_f32_certified(const adanns_index *idx, const float *queries, int64_t 
       ADN_LAUNCH("rescore_kernel");
     }
     // the queries left over (usually none): the tiled scan on them alone
-    const int64_t np = nb * nprobe;
-    mask_answered_kernel<<<(unsigned)((np + 255) / 256), 256, 0, st>>>(ckeys, np, nprobe, cnt);
-    ADN_LAUNCH("mask_answered_kernel");
+    if ((rc = launch_mask_answered(ckeys, nb, nprobe, cnt, st))) return rc;
     MergeMask mm;
     mm.ckeys = ckeys;
     mm.nsplit = h.ts.nsplit;

@@ -233,4 +233,27 @@ __device__ __forceinline__ void warp_sort256(uint64_t (&v)[8]) {
   }
 }
 
+// Ascending sort of a[0:n) in shared memory by the NT threads of a block (the
+// flip form of the bitonic network, as warp_sort); ends synchronised.
+template <int NT>
+__device__ __forceinline__ void block_sort(uint64_t *a, int n) {
+  int P = 1;
+  while (P < n) P <<= 1;
+  for (int size = 2; size <= P; size <<= 1) {
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      const bool flip = stride == size >> 1;
+      const int ls = __ffs(stride) - 1;
+      for (int p = threadIdx.x; p < P >> 1; p += NT) {
+        const int off = p & (stride - 1), base = (p >> ls) << (ls + 1);
+        const int i = base + off, j = flip ? base + 2 * stride - 1 - off : i + stride;
+        if (j < n) {
+          const uint64_t x = a[i], y = a[j];
+          if (y < x) { a[i] = y; a[j] = x; }
+        }
+      }
+      __syncthreads();
+    }
+  }
+}
+
 }  // namespace adn

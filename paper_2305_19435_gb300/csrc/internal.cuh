@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <cmath>
 #include <string>
 
 #include "../../include/adanns.h"
@@ -270,6 +271,7 @@ struct MmaScanArgs {
   int *tile_counter;         // zeroed before the launch: next tile to take
   int fp8;
   int f16;                   // 16-bit operands are FP16 instead of BF16
+  int nsplit;                // > 1: work items are (tile, member range r of nsplit) (wide tiles)
   int few;                   // few queries per probed list (memory-bound): FP8 takes the
                              // four-stage ring with narrow key staging, as BF16 does
   // filtered mode (rec != NULL, tau != NULL): instead of every key, each
@@ -368,11 +370,22 @@ int64_t certified_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int
 int search_f32_certified(const adanns_index *idx, const float *queries, int64_t B, int d_c,
                          int d_s, int nprobe, int k, int64_t *out_ids, float *out_dist,
                          int32_t *out_probes, cudaStream_t st);
+// FP16 rows (nkb blocks of 64) of the B x d_s rows v, their squared norms and a
+// bound qerr of the approximate distances' error to members of norm at most yn
+// with FP16 residuals up to yr; rows of squared norm above zmax2, or any row
+// while *unsure (or null) is set, get a bound that keeps every member.
+int launch_f16_queries(const float *v, int ldv, int64_t B, int d_s, int nkb, const int *unsure,
+                       float yn, float yr, float zmax2, void *out, float *qn2, float *qerr,
+                       cudaStream_t st);
+// probe slots of queries with cnt[q] >= 0 -> PROBE_NONE
+int launch_mask_answered(uint64_t *ckeys, int64_t B, int nprobe, const int32_t *cnt,
+                         cudaStream_t st);
 bool scan_choice_forced();  // an FFMA scan variant is being timed by the autotuner
 int launch_mma_scan(const void *qtiles, int64_t qrows, const void *xlow, int64_t xrows,
                     const MmaScanArgs &a, cudaStream_t st);
 int launch_mma_narrow(const void *qtiles, int64_t qrows, const void *xlow, int64_t xrows,
                       const MmaScanArgs &a, cudaStream_t st);
+int mma_scan_nsplit(const adanns_index *idx, int64_t pairs);  // for launch_mma_scan
 int launch_gather_qtiles(const unsigned char *qlow, int nkb, int64_t max_tiles,
                          const int32_t *tile_beg, const int32_t *tile_cnt, const int *ntiles,
                          const int32_t *pair_q, int rows_per_tile, unsigned char *qt,
@@ -384,11 +397,13 @@ int launch_select16(const uint16_t *cand, const uint64_t *ckeys, int nprobe, con
 // Certified shortlist: every candidate whose key is within the query's error
 // bound of its k-th smallest key, at most kk of them, as (list << 32 | member);
 // cnt[q] = how many, or -1 when they exceed kk (out row q is then undefined).
-// stats (NULL, or 2 zeroed device counters): candidates listed, queries with -1.
+// qerr[q]: a bound of |approximate - exact distance|; k <= CERT_MAX_K, kk <=
+// CERT_MAX_KK.  stats (NULL, or 2 zeroed device counters): candidates listed,
+// queries with -1.
+constexpr int CERT_MAX_K = 512, CERT_MAX_KK = 1024;
 int launch_certify16(const uint16_t *cand, const uint64_t *ckeys, int nprobe, const int64_t *qbase,
-                     const int64_t *list_off, int kk, int k, const float *qrho, float rmax,
-                     float e_rest, int64_t B, int64_t *out, int32_t *cnt,
-                     unsigned long long *stats, cudaStream_t st);
+                     const int64_t *list_off, int kk, int k, const float *qerr, int64_t B,
+                     int64_t *out, int32_t *cnt, unsigned long long *stats, cudaStream_t st);
 // Filtered tensor-core scan: from the keys of each query's nearest list
 // (cand0 + q * stride0, the list of probe slot 0), tau = their kk-th smallest
 // (0xFFFF with fewer than kk members) and slot 0's records with key <= tau;
@@ -416,9 +431,21 @@ int launch_adc_dist(const uint8_t *codes, const int64_t *list_off, int M, const 
                     const int64_t *pbase, uint32_t *cand, int qa, int nsplit, cudaStream_t st,
                     const float *res_S = nullptr, const float *res_w = nullptr,
                     const float *res_w2 = nullptr, const float *z = nullptr, int d_s = 0);
+// only (or null): just the queries with only[q] < 0
 int launch_select32(const uint32_t *cand, const uint64_t *ckeys, int nprobe, const int64_t *qbase,
                     const int64_t *list_off, const int32_t *list_ids, int64_t B, int kk,
-                    uint64_t *out, cudaStream_t st);
+                    uint64_t *out, cudaStream_t st, const int32_t *only = nullptr);
+// IVF-OPQ through the certified tensor-core filter (certified_adc.cu): rows of
+// decoded codes for the scan, and the exact ADC scores of the shortlist.
+// Squared norms of every decoded code row y2 [N] and their maximum.
+int launch_code_norms(const adanns_index *x, float *y2, float *y2max_host, cudaStream_t st);
+bool adc_certified(const adanns_index *idx, int64_t B, int nprobe, int kr);
+int launch_decode_f16(const adanns_index *idx, const int32_t *lcnt, int nkb, void *rows,
+                      cudaStream_t st);
+// per query with cnt[q] >= 0: the kr smallest (ADC score, id) keys of its cnt[q]
+// shortlisted (list << 32 | member) entries, ascending, KEY_MAX padding
+int launch_adc_rescore(const adanns_index *idx, const int64_t *cids, const int32_t *cnt, int kk,
+                       const float *z, int64_t B, int kr, uint64_t *keys, cudaStream_t st);
 
 // Records an event pair around its scope on `st` when profiling is enabled.
 class StageTimer {
@@ -482,6 +509,10 @@ struct adanns_index {
   // list), w = lcent R [nlist][d_s], w2 = |w_l|^2 [nlist], S[l][m][c] =
   // 2 <w_l,m, C_m[c]> [nlist][M][256]; NULL for plain codes
   float *opq_lcent = nullptr, *opq_w = nullptr, *opq_w2 = nullptr, *opq_S = nullptr;
+  // squared norms of the decoded code rows [N] (list order) and their maximum
+  // (infinity: not known; the tensor-core filter is then not used)
+  float *opq_y2 = nullptr;
+  float opq_y2max = INFINITY;
   // low-precision tiers [0] BF16 (64-dim blocks), [1] FP8-E4M3 (128-dim blocks)
   void *lowp[2] = {nullptr, nullptr};
   int lowp_blocks[2] = {0, 0};

@@ -28,6 +28,7 @@
 #include <cuda.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "devutil.cuh"
@@ -162,6 +163,12 @@ __device__ __forceinline__ uint32_t mma_idesc(const MmaScanArgs &a, int m, int n
   return (1u << 4) | fmt | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
+// member tiles [first, end) of range r of nsplit of a list of nl members
+__device__ __forceinline__ int2 member_tiles(int nl, int r, int nsplit) {
+  const int nmt = (nl + BN - 1) / BN, per = (nmt + nsplit - 1) / nsplit;
+  return make_int2(min(nmt, r * per), min(nmt, (r + 1) * per));
+}
+
 __device__ __forceinline__ int ld_abort(const int *flag) { return *(const volatile int *)flag; }
 
 // bit e set for each of the 8 16-bit keys of v (key e in half e & 1 of word
@@ -243,7 +250,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base_s;
-  const int ntiles = *a.ntiles_dev;
+  const int nsplit = a.nsplit > 1 ? a.nsplit : 1;
+  const int nitems = *a.ntiles_dev * nsplit;
   const uint32_t idesc = mma_idesc(a, BM, BN);
 
   // filtered mode: the last work item with member tiles whose survivor counts
@@ -262,7 +270,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       uint32_t qph = 0;
       for (;;) {
         int t = atomicAdd(a.tile_counter, 1);
-        if (t >= ntiles || ld_abort(&abort_s)) t = -1;
+        if (t >= nitems || ld_abort(&abort_s)) t = -1;
         if (!mbar_wait(&qempty[qs], qph ^ 1, a.wait_ns)) {
           atomicExch(&abort_s, 1);
           atomicCAS(a.err, 0, 6);
@@ -272,11 +280,11 @@ __global__ void __launch_bounds__(THREADS, 1)
         mbar_arrive(&qfull[qs]);
         if (++qs == TQD) { qs = 0; qph ^= 1; }
         if (t < 0) break;
-        const int list = a.tile_list[t];
+        const int tile = t / nsplit, list = a.tile_list[tile];
         const int64_t off = a.list_off[list];
         const int nl = (int)(a.list_off[list + 1] - off);
-        const int nmt = (nl + BN - 1) / BN;
-        for (int mt = 0; mt < nmt && !ld_abort(&abort_s); ++mt)
+        const int2 mr = member_tiles(nl, t - tile * nsplit, nsplit);
+        for (int mt = mr.x; mt < mr.y && !ld_abort(&abort_s); ++mt)
           for (int kb = 0; kb < a.nkb; ++kb) {
             if (!mbar_wait(&empty[stage], phase ^ 1, a.wait_ns)) {
               atomicExch(&abort_s, 1);
@@ -290,7 +298,7 @@ __global__ void __launch_bounds__(THREADS, 1)
               continue;
             }
             mbar_expect_tx(&full[stage], STAGE_BYTES);
-            tma_load_2d(sA + stage * A_BYTES, &tmA, &full[stage], 0, (t * a.nkb + kb) * BM);
+            tma_load_2d(sA + stage * A_BYTES, &tmA, &full[stage], 0, (tile * a.nkb + kb) * BM);
             tma_load_2d(sB + stage * B_BYTES, &tmB, &full[stage], 0,
                         (int)(off * a.d_blocks) + kb * nl + mt * BN);
             if (++stage == NS) { stage = 0; phase ^= 1; }
@@ -316,10 +324,10 @@ __global__ void __launch_bounds__(THREADS, 1)
         mbar_arrive(&qempty[qs]);
         if (++qs == TQD) { qs = 0; qph ^= 1; }
         if (t < 0) break;
-        const int list = a.tile_list[t];
+        const int tile = t / nsplit, list = a.tile_list[tile];
         const int nl = (int)(a.list_off[list + 1] - a.list_off[list]);
-        const int nmt = (nl + BN - 1) / BN;
-        for (int mt = 0; mt < nmt && !ld_abort(&abort_s); ++mt) {
+        const int2 mr = member_tiles(nl, t - tile * nsplit, nsplit);
+        for (int mt = mr.x; mt < mr.y && !ld_abort(&abort_s); ++mt) {
           if (!mbar_wait(&tempty[acc], aphase ^ 1, a.wait_ns)) {
             atomicExch(&abort_s, 1);
             atomicCAS(a.err, 0, 2);
@@ -379,19 +387,19 @@ __global__ void __launch_bounds__(THREADS, 1)
       mbar_arrive(&qempty[qs]);
       if (++qs == TQD) { qs = 0; qph ^= 1; }
       if (t < 0) break;
-      const int list = a.tile_list[t];
+      const int tile = t / nsplit, list = a.tile_list[tile];
       const int64_t off = a.list_off[list];
       const int nl = (int)(a.list_off[list + 1] - off);
       const int npad = (nl + 7) & ~7;
-      const int nmt = (nl + BN - 1) / BN;
-      const int cnt = a.tile_cnt[t];
+      const int2 mr = member_tiles(nl, t - tile * nsplit, nsplit);
+      const int cnt = a.tile_cnt[tile];
       const bool valid = row < cnt;
       int64_t base = 0;
       float q2 = 0.f, qs = 0.f;
       uint32_t tau = 0xFFFFu;  // filtered mode: members with key <= tau survive
       int pidx = 0;
       if (valid) {
-        const int p = a.pair_out[a.tile_beg[t] + row];
+        const int p = a.pair_out[a.tile_beg[tile] + row];
         const int q = p / a.nprobe;
         base = a.pstride ? (int64_t)(p / a.nprobe) * a.pstride : a.pbase[p];
         q2 = a.qn2[q];
@@ -418,8 +426,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         return v;
       };
-      float2 terms = load_terms(0);
-      for (int mt = 0; mt < nmt; ++mt) {
+      float2 terms = load_terms(mr.x);
+      for (int mt = mr.x; mt < mr.y; ++mt) {
         if (!mbar_wait(&tfull[acc], aphase, a.wait_ns)) {
           atomicExch(&abort_s, 1);
           atomicCAS(a.err, 0, 4);
@@ -442,11 +450,11 @@ __global__ void __launch_bounds__(THREADS, 1)
             break;
           }
         }
-        if (filt && mt == 0 && ib > 0 && c_lo == 0) {
+        if (filt && mt == mr.x && ib > 0 && c_lo == 0) {
           if (fl_pv) a.rcnt[fl_pp] = s_rc[fl_buf][row];
           s_rc[fl_buf][row] = 0;
         }
-        if (mt + 1 < nmt) terms = load_terms(mt + 1);
+        if (mt + 1 < mr.y) terms = load_terms(mt + 1);
         // a lane quadrant with no valid query row (a tile with few queries)
         // has nothing to drain: its warps skip the TMEM loads and the stores
         if (quarter * 32 < cnt) {
@@ -537,7 +545,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (++acc == 2) { acc = 0; aphase ^= 1; }
       }
       if (stop) break;
-      if (nmt > 0) {
+      if (mr.x < mr.y) {
         fl_pv = valid;
         fl_pp = pidx;
         fl_buf = cbuf;
@@ -854,6 +862,18 @@ int launch_mma_narrow(const void *qtiles, int64_t qrows, const void *xlow, int64
   return ADANNS_OK;
 }
 
+// Member ranges per query tile for the wide kernel: with fewer tiles than a few
+// per SM (a small batch, or one long list as in the exhaustive search) each
+// list is cut into ranges of whole 256-member tiles so that every SM has work.
+int mma_scan_nsplit(const adanns_index *idx, int64_t pairs) {
+  const int64_t tiles = std::max<int64_t>(1, std::max<int64_t>((pairs + BM - 1) / BM,
+                                                               std::min<int64_t>(idx->nlist, pairs)));
+  const int64_t want = (int64_t)num_sms() * 4;
+  if (tiles >= want) return 1;
+  return (int)std::max<int64_t>(1, std::min<int64_t>((want + tiles - 1) / tiles,
+                                                     ((int64_t)idx->max_list + BN - 1) / BN));
+}
+
 // stage count and staging width per element type (see the kernel's notes)
 constexpr int NS_BF16 = 4, SC_BF16 = 16, NS_FP8 = 3, SC_FP8 = 64;
 size_t mma_scan_smem(int ns, int sc) {
@@ -866,6 +886,7 @@ int launch_mma_scan(const void *qtiles, int64_t qrows, const void *xlow, int64_t
   int rc;
   if ((rc = make_map(&tA, qtiles, qrows, BM, a.fp8 != 0))) return rc;
   if ((rc = make_map(&tB, xlow, xrows, BN, a.fp8 != 0))) return rc;
+  if (a.nsplit > 1 && a.rec) return fail(ADANNS_ERR_ARG, "filtered scan: whole lists only");
   MmaScanArgs b = a;
   b.wait_ns = (uint64_t)option(ADANNS_OPT_WAIT_LIMIT_NS);
   b.skip_fill = (int)take_option(ADANNS_OPT_TEST_SKIP_LOAD, -1);

@@ -126,21 +126,28 @@ __global__ void sum_f32_kernel(const float *__restrict__ v, int64_t n, double *o
 }
 
 // ---------------------------------------------------------------- query LUT
-// lut[q][m][c] = sum_t (z[q][m*dsub + t] - C[m][c][t])^2; grid (B, M), c = thread.
+// lut[q][m][c] = sum_t (z[q][m*dsub + t] - C[m][c][t])^2; grid (B, M or 1), c = thread.
+// only (or null): just the queries with only[q] < 0 (usually none: one CTA per
+// query then loops over the sub-vectors, so that few CTAs start for nothing).
 __global__ void pq_lut_kernel(const float *__restrict__ z, int ldz, int M, int dsub,
-                              const float *__restrict__ C, float *__restrict__ lut) {
+                              const float *__restrict__ C, float *__restrict__ lut,
+                              const int32_t *__restrict__ only) {
   const int64_t q = blockIdx.x;
-  const int m = blockIdx.y, c = threadIdx.x;
+  if (only && only[q] >= 0) return;
+  const int c = threadIdx.x;
   extern __shared__ float zq[];
-  for (int t = threadIdx.x; t < dsub; t += 256) zq[t] = z[q * ldz + (int64_t)m * dsub + t];
-  __syncthreads();
-  const float *cw = C + ((int64_t)m * 256 + c) * dsub;
-  float acc = 0.f;
-  for (int t = 0; t < dsub; ++t) {
-    const float df = zq[t] - cw[t];
-    acc = fmaf(df, df, acc);
+  for (int m = blockIdx.y; m < M; m += gridDim.y) {
+    __syncthreads();  // the previous sub-vector is no longer read
+    for (int t = threadIdx.x; t < dsub; t += 256) zq[t] = z[q * ldz + (int64_t)m * dsub + t];
+    __syncthreads();
+    const float *cw = C + ((int64_t)m * 256 + c) * dsub;
+    float acc = 0.f;
+    for (int t = 0; t < dsub; ++t) {
+      const float df = zq[t] - cw[t];
+      acc = fmaf(df, df, acc);
+    }
+    lut[(q * M + m) * 256 + c] = acc;
   }
-  lut[(q * M + m) * 256 + c] = acc;
 }
 
 // ---------------------------------------------------------------- ADC list scan
@@ -510,10 +517,10 @@ int polar_factor(const float *Mx, int d, float *R, cudaStream_t st) {
 }
 
 int launch_pq_lut(const float *z, int64_t B, int ldz, int M, int dsub, const float *C, float *lut,
-                  cudaStream_t st) {
+                  cudaStream_t st, const int32_t *only) {
   if (B <= 0) return ADANNS_OK;
-  dim3 grid((unsigned)B, M);
-  pq_lut_kernel<<<grid, 256, dsub * 4, st>>>(z, ldz, M, dsub, C, lut);
+  dim3 grid((unsigned)B, only ? 1 : M);
+  pq_lut_kernel<<<grid, 256, dsub * 4, st>>>(z, ldz, M, dsub, C, lut, only);
   ADN_LAUNCH("pq_lut_kernel");
   return ADANNS_OK;
 }

@@ -29,9 +29,6 @@ constexpr int SW_BUF = 1024;
 constexpr int SW_TIE = 128;
 constexpr int SW_MAXP = 128;
 constexpr int SW_PF = 12;
-// survivors aimed at by the certified shortlist: the k nearest (k <= 256) and
-// those within the error bound of the k-th, well inside the buffer
-constexpr int SW_CERT_AIM = 680;
 
 // Per-warp state with a buffer of BUF keys (8.6 KB for the 1,024 of
 // select16_kernel, so that six CTAs of four warps fit on an SM).  The
@@ -45,7 +42,7 @@ struct SwStateT {
   } h;
   int sh[2], n, cnt, ecnt;
   int lid[SW_MAXP], nl[SW_MAXP], pst[SW_MAXP + 1];
-  union {
+  union alignas(16) {
     uint16_t samp[SW_SAMPLE];
     struct {
       uint16_t key[BUF];
@@ -155,61 +152,19 @@ __device__ __forceinline__ bool warp_select16(int n, int kk, int kq, int prune_d
   return true;
 }
 
-// The keys up to (k-th smallest + delta) of n keys, written to o in any order
-// when they number at most kk: their count, else -1 (also when the bound
-// reaches key_limit: only keys below it are known to be among the n).
-template <class KeyF, class IdF, class St>
-__device__ __forceinline__ int warp_certify16(int n, int kk, int k, int delta, KeyF key, IdF id,
-                                              int64_t *o, St &s, uint32_t key_limit) {
+// probed lists of a query: ids, sizes and padded starts into the warp's state
+// (a warp scan over 4 entries per lane), members and padded members in all
+template <class St>
+__device__ __forceinline__ void warp_lists(St &s, const uint64_t *ck, int nprobe,
+                                           const int64_t *list_off, int &total, int &ptotal) {
   const int lane = threadIdx.x & 31;
-  int b2, n2;
-  const uint32_t keep_max = warp_kth16(n, k, key, s, b2, n2) + (uint32_t)delta;
-  if (keep_max >= key_limit && key_limit <= 0xFFFFu) return -1;
-  int c = 0;
-  for (int i = lane; i < n; i += 32) c += key(i) <= keep_max ? 1 : 0;
-#pragma unroll
-  for (int o2 = 16; o2 > 0; o2 >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o2);
-  if (c > kk) return -1;
-  int base = 0;
-  for (int i0 = 0; i0 < n; i0 += 32) {
-    const int i = i0 + lane;
-    const bool in = i < n && key(i) <= keep_max;
-    const unsigned b = __ballot_sync(0xffffffffu, in);
-    if (in) o[base + __popc(b & lanemask_lt())] = id(i);
-    base += __popc(b);
-  }
-  return c;
-}
-
-// CERT (launch_certify16): the row gets every candidate that can be among the
-// k nearest, cnt[q] of them, or cnt[q] = -1 when they exceed kk.
-template <bool CERT>
-__global__ void __launch_bounds__(SW_WARPS * 32, 6) select16_kernel(
-    const uint16_t *__restrict__ cand, const uint64_t *__restrict__ ckeys, int nprobe,
-    const int64_t *__restrict__ qbase, const int64_t *__restrict__ list_off, int kk, int k,
-    const float *__restrict__ qrho, float rmax, float e_rest, int prune, int64_t B,
-    int64_t *__restrict__ out, int32_t *__restrict__ cnt,
-    unsigned long long *__restrict__ stats) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  SwState &s = ((SwState *)smem)[warp];
-  const int64_t q = (int64_t)blockIdx.x * SW_WARPS + warp;
-  if (q >= B) return;
-  int prune_delta = 0;
-  if (prune) {
-    const double rq = (double)qrho[q];
-    const double E = 2.0 * (rmax + rq + rmax * rq) * (1.0 + 1e-3) + e_rest;
-    prune_delta = (int)ceil(2.0 * 16384.0 * (ldexp(1.0, -15) + E)) + 1;
-    if (prune_delta > (1 << 20)) prune_delta = 1 << 20;
-  }
-  // probed lists: ids, sizes, padded starts (warp scan over 4 entries per lane)
   int ln[4], pl[4], tot = 0, ptot = 0;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const int sl = lane * 4 + j;
     ln[j] = 0;
     if (sl < nprobe) {
-      const int l = probe_list(ckeys[q * nprobe + sl]);
+      const int l = probe_list(ck[sl]);
       s.lid[sl] = l;
       ln[j] = l >= 0 ? (int)(list_off[l + 1] - list_off[l]) : 0;
       s.nl[sl] = ln[j];
@@ -235,9 +190,30 @@ __global__ void __launch_bounds__(SW_WARPS * 32, 6) select16_kernel(
   }
 #pragma unroll
   for (int o2 = 16; o2 > 0; o2 >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o2);
-  const int ptotal = __shfl_sync(0xffffffffu, inc, 31);
-  const int total = tot;
+  ptotal = __shfl_sync(0xffffffffu, inc, 31);
+  total = tot;
   __syncwarp();
+}
+
+__global__ void __launch_bounds__(SW_WARPS * 32, 6) select16_kernel(
+    const uint16_t *__restrict__ cand, const uint64_t *__restrict__ ckeys, int nprobe,
+    const int64_t *__restrict__ qbase, const int64_t *__restrict__ list_off, int kk, int k,
+    const float *__restrict__ qrho, float rmax, float e_rest, int prune, int64_t B,
+    int64_t *__restrict__ out, unsigned long long *__restrict__ stats) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  SwState &s = ((SwState *)smem)[warp];
+  const int64_t q = (int64_t)blockIdx.x * SW_WARPS + warp;
+  if (q >= B) return;
+  int prune_delta = 0;
+  if (prune) {
+    const double rq = (double)qrho[q];
+    const double E = 2.0 * (rmax + rq + rmax * rq) * (1.0 + 1e-3) + e_rest;
+    prune_delta = (int)ceil(2.0 * 16384.0 * (ldexp(1.0, -15) + E)) + 1;
+    if (prune_delta > (1 << 20)) prune_delta = 1 << 20;
+  }
+  int total, ptotal;
+  warp_lists(s, ckeys + q * nprobe, nprobe, list_off, total, ptotal);
   int64_t *o = out + q * kk;
   auto id_at = [&](int i) -> int64_t {
     int lo = 0, hi = nprobe - 1;
@@ -255,11 +231,7 @@ __global__ void __launch_bounds__(SW_WARPS * 32, 6) select16_kernel(
       for (int m = lane; m < nl; m += 32) o[p0 + m] = ((int64_t)s.lid[sl] << 32) | (int64_t)m;
       p0 += nl;
     }
-    if (CERT) {
-      if (lane == 0) cnt[q] = total;
-    } else {
-      for (int r = total + lane; r < kk; r += 32) o[r] = -1;
-    }
+    for (int r = total + lane; r < kk; r += 32) o[r] = -1;
     return;
   }
   const int kq = prune ? k : 0;
@@ -277,9 +249,7 @@ __global__ void __launch_bounds__(SW_WARPS * 32, 6) select16_kernel(
       for (int e = 0; e < 8; ++e) s.u.samp[8 * j + e] = (uint16_t)((w[e >> 1] >> ((e & 1) * 16)) & 0xFFFFu);
     }
     __syncwarp();
-    // the buffer must hold the keys up to the pruning bound (certified), or kk
-    const int want = CERT ? SW_CERT_AIM : (kk + SW_BUF) / 2;
-    int r = (int)(((double)want * ns) / ptotal);
+    int r = (int)((0.5 * (kk + SW_BUF) * ns) / ptotal);
     r = max(0, min(r, ns - 1));
     int b_, n_;
     const uint32_t kv =
@@ -343,39 +313,210 @@ __global__ void __launch_bounds__(SW_WARPS * 32, 6) select16_kernel(
       }
       __syncwarp();
       const int n = s.n;
-      if (!CERT && stats && lane == 0) atomicAdd(stats, (unsigned long long)n);
+      if (stats && lane == 0) atomicAdd(stats, (unsigned long long)n);
       // 3. exact select on the buffer
-      if (CERT) {
-        if (n >= k && n <= SW_BUF) {
-          const int c = warp_certify16(n, kk, k, prune_delta,
-                                       [&](int i) -> uint32_t { return s.u.b.key[i]; },
-                                       [&](int i) -> int64_t { return id_at((int)s.u.b.idx[i]); },
-                                       o, s, T);
-          if (c >= 0) {
-            if (lane == 0) cnt[q] = c;
-            if (stats && lane == 0) atomicAdd(stats, (unsigned long long)c);
-            return;
-          }
-        }
-      } else if (n >= kk && n <= SW_BUF &&
+      if (n >= kk && n <= SW_BUF &&
           warp_select16<false>(n, kk, kq, prune_delta,
                                [&](int i) -> uint32_t { return s.u.b.key[i]; },
                                [&](int i) -> int64_t { return id_at((int)s.u.b.idx[i]); },
                                [&](int i) -> int { return (int)s.u.b.idx[i]; }, o, s, T))
         return;
     }
-    if (!CERT && stats && lane == 0) atomicAdd(stats + 1, 1ull);  // the buffer path failed
-  }
-  if (CERT) {
-    const int c = warp_certify16(ptotal, kk, k, prune_delta,
-                                 [&](int i) -> uint32_t { return src[i]; }, id_at, o, s, 0x10000u);
-    if (lane == 0) cnt[q] = c;
-    if (stats && lane == 0) atomicAdd(stats + (c < 0 ? 1 : 0), (unsigned long long)(c < 0 ? 1 : c));
-    return;
+    if (stats && lane == 0) atomicAdd(stats + 1, 1ull);  // the buffer path failed
   }
   // exact select over the whole region (index = candidate position)
   warp_select16<true>(ptotal, kk, kq, prune_delta, [&](int i) -> uint32_t { return src[i]; }, id_at,
                       [&](int i) -> int { return i; }, o, s, 0x10000u);
+}
+
+// ---------------------------------------------------------------- certified shortlist
+// Every candidate that can be among a query's k nearest: with |approximate -
+// exact| <= E, those whose key is at most the k-th smallest key plus
+// 2 * 16384 * (2^-15 + E).  One warp per query.  A sampled threshold T, as
+// above, lets one pass collect the small keys in the buffer; when the buffer
+// fills, T is lowered to the bound that the keys seen so far already give (the
+// k-th smallest of a part is at least that of the whole), so the pass never
+// needs a second one unless the sampled T was too low.  More than kk
+// candidates, or more than the buffer holds within the bound: cnt[q] = -1.
+__global__ void __launch_bounds__(SW_WARPS * 32, 6) certify16_kernel(
+    const uint16_t *__restrict__ cand, const uint64_t *__restrict__ ckeys, int nprobe,
+    const int64_t *__restrict__ qbase, const int64_t *__restrict__ list_off, int kk, int k,
+    const float *__restrict__ qerr, int64_t B, int64_t *__restrict__ out,
+    int32_t *__restrict__ cnt, unsigned long long *__restrict__ stats) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  SwState &s = ((SwState *)smem)[warp];
+  const int64_t q = (int64_t)blockIdx.x * SW_WARPS + warp;
+  if (q >= B) return;
+  const int delta =
+      (int)fmin(ceil(2.0 * 16384.0 * (ldexp(1.0, -15) + (double)qerr[q])) + 1.0, 1048576.0);
+  int total, ptotal;
+  warp_lists(s, ckeys + q * nprobe, nprobe, list_off, total, ptotal);
+  int64_t *o = out + q * kk;
+  if (total <= kk) {
+    int p0 = 0;
+    for (int sl = 0; sl < nprobe; ++sl) {
+      const int nl = s.nl[sl];
+      for (int m = lane; m < nl; m += 32) o[p0 + m] = ((int64_t)s.lid[sl] << 32) | (int64_t)m;
+      p0 += nl;
+    }
+    if (lane == 0) cnt[q] = total;
+    return;
+  }
+  auto id_at = [&](int i) -> int64_t {
+    int lo = 0, hi = nprobe - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (s.pst[mid] <= i) lo = mid; else hi = mid - 1;
+    }
+    const int m = i - s.pst[lo];
+    return m < s.nl[lo] ? (((int64_t)s.lid[lo] << 32) | (int64_t)m) : -1;
+  };
+  auto key = [&](int i) -> uint32_t { return s.u.b.key[i]; };
+  const uint16_t *src = cand + qbase[q];
+  const uint4 *g = (const uint4 *)src;
+  const int nvec = ptotal >> 3;
+  uint32_t T = 0xFFFFu;  // keys strictly below T are collected (every key is)
+  if (ptotal > 2 * SW_BUF) {
+    const int nrun = min(SW_SAMPLE / 8, nvec), ns = 8 * nrun;
+    const uint64_t step = ((uint64_t)nvec << 20) / (uint64_t)nrun;  // 2^-20 units
+    for (int j = lane; j < nrun; j += 32)
+      *(uint4 *)&s.u.samp[8 * j] = g[(int)(((uint64_t)j * step) >> 20)];
+    __syncwarp();
+    // room for the k nearest and those near the k-th; a standard deviation of
+    // the sample's rank on top, since a T too low costs a second pass and one
+    // too high only a few tightenings
+    const float rf = (float)(max(680, k + 300)) * ns / ptotal;
+    const int r = max(0, min((int)(rf + sqrtf(rf)), ns - 1));
+    int b_, n_;
+    T = min(0xFFFFu,
+            warp_kth16(ns, r + 1, [&](int i) -> uint32_t { return s.u.samp[i]; }, s, b_, n_) + 1u);
+    __syncwarp();  // the sample's space becomes the buffer
+  }
+  constexpr int HB = SW_PF / 2;
+  auto load = [&](uint4(&v)[HB], int cb) {
+#pragma unroll
+    for (int f = 0; f < HB; ++f) {
+      const int c = cb + f * 32 + lane;
+      v[f] = c < nvec ? g[c] : make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+    }
+  };
+  auto collect = [&](const uint4 &v, int c) {  // the keys below T of one 8-key run per lane
+    const uint32_t TT = T | (T << 16), TL = TT & 0x7FFF7FFFu;
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    uint32_t lt[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t x = w[i], d = (x | 0x80008000u) - TL;
+      lt[i] = ((~x & TT) | (~(x ^ TT) & ~d)) & 0x80008000u;
+    }
+    uint64_t M = ((uint64_t)__byte_perm(lt[2], lt[3], 0x7531) << 32) |
+                 (uint64_t)__byte_perm(lt[0], lt[1], 0x7531);
+    if (M) {
+      int p = atomicAdd(&s.n, __popcll(M));
+      const uint64_t k01 = ((uint64_t)w[1] << 32) | w[0], k23 = ((uint64_t)w[3] << 32) | w[2];
+      while (M) {
+        const int e = (__ffsll((long long)M) - 1) >> 3;
+        M &= M - 1;
+        if (p < SW_BUF) {
+          s.u.b.key[p] = (uint16_t)(((e < 4 ? k01 : k23) >> (16 * (e & 3))) & 0xFFFFu);
+          s.u.b.idx[p] = (uint32_t)(c * 8 + e);
+        }
+        ++p;
+      }
+    }
+  };
+  // lower T to the bound given by the n >= k keys collected so far and drop
+  // those at or above it; the count left
+  auto tighten = [&](int n) -> int {
+    int b_, n_;
+    const uint32_t t = warp_kth16(n, k, key, s, b_, n_) + (uint32_t)delta + 1u;
+    if (t < T) T = t;
+    int w = 0;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+      const int i = i0 + lane;
+      const uint32_t kv = i < n ? s.u.b.key[i] : 0xFFFFFFFFu;
+      const uint32_t ix = i < n ? s.u.b.idx[i] : 0u;
+      const unsigned b = __ballot_sync(0xffffffffu, kv < T);
+      if (kv < T) {
+        const int d = w + __popc(b & lanemask_lt());
+        s.u.b.key[d] = (uint16_t)kv;
+        s.u.b.idx[d] = ix;
+      }
+      w += __popc(b);
+      __syncwarp();
+    }
+    if (lane == 0) s.n = w;
+    __syncwarp();
+    return w;
+  };
+  int c = -1;
+  for (int attempt = 0; attempt < 2 && c < 0; ++attempt) {
+    if (attempt > 0) {
+      if (T >= 0xFFFFu) break;
+      T = 0xFFFFu;  // the sampled threshold was below the bound: collect every key
+    }
+    const uint32_t T0 = T;
+    if (lane == 0) s.n = 0;
+    __syncwarp();
+    int n = 0;
+    bool full = false;
+    auto batch = [&](const uint4(&v)[HB], int cb) {
+#pragma unroll
+      for (int f = 0; f < HB; ++f) collect(v[f], cb + f * 32 + lane);
+      __syncwarp();
+      int m = s.n;
+      if (m > SW_BUF) {  // again, 64 keys at a time, tightening in between
+        __syncwarp();
+        if (lane == 0) s.n = n;
+        __syncwarp();
+        m = n;
+#pragma unroll
+        for (int f = 0; f < HB; ++f)
+#pragma unroll 1
+          for (int h = 0; h < 4; ++h) {
+            if (m > SW_BUF - 64) m = tighten(m);
+            if (m > SW_BUF - 64) full = true;
+            if (full) break;
+            if (lane >> 3 == h) collect(v[f], cb + f * 32 + lane);
+            __syncwarp();
+            m = s.n;
+            __syncwarp();
+          }
+      }
+      n = m;
+    };
+    uint4 va[HB], vb[HB];
+    load(va, 0);
+    for (int c0 = 0; c0 < nvec && !full; c0 += 2 * 32 * HB) {
+      load(vb, c0 + 32 * HB);
+      batch(va, c0);
+      load(va, c0 + 2 * 32 * HB);
+      if (!full) batch(vb, c0 + 32 * HB);
+    }
+    __syncwarp();
+    if (full) break;
+    if (n < k) continue;
+    int b_, n_;
+    const uint32_t keep_max = warp_kth16(n, k, key, s, b_, n_) + (uint32_t)delta;
+    if (keep_max >= T0 && T0 < 0xFFFFu) continue;
+    int w = 0;
+    for (int i = lane; i < n; i += 32) w += key(i) <= keep_max ? 1 : 0;
+#pragma unroll
+    for (int o2 = 16; o2 > 0; o2 >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o2);
+    if (w > kk) break;
+    c = w;
+    w = 0;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+      const int i = i0 + lane;
+      const bool in = i < n && key(i) <= keep_max;
+      const unsigned b = __ballot_sync(0xffffffffu, in);
+      if (in) o[w + __popc(b & lanemask_lt())] = id_at((int)s.u.b.idx[i]);
+      w += __popc(b);
+    }
+  }
+  if (lane == 0) cnt[q] = c;
+  if (stats && lane == 0) atomicAdd(stats + (c < 0 ? 1 : 0), (unsigned long long)(c < 0 ? 1 : c));
 }
 
 // ---------------------------------------------------------------- filtered scan
@@ -598,25 +739,24 @@ int launch_select16(const uint16_t *cand, const uint64_t *ckeys, int nprobe, con
   if (nprobe > SW_MAXP) return fail(ADANNS_ERR_ARG, "select16: nprobe above 128");
   if (B <= 0) return ADANNS_OK;
   const size_t sm = sizeof(SwState) * SW_WARPS;
-  ADN_CUDA(ensure_smem((const void *)select16_kernel<false>, sm));
-  select16_kernel<false><<<(unsigned)((B + SW_WARPS - 1) / SW_WARPS), SW_WARPS * 32, sm, st>>>(
-      cand, ckeys, nprobe, qbase, list_off, kk, k, qrho, rmax, e_rest, prune, B, out, nullptr,
-      stats);
+  ADN_CUDA(ensure_smem((const void *)select16_kernel, sm));
+  select16_kernel<<<(unsigned)((B + SW_WARPS - 1) / SW_WARPS), SW_WARPS * 32, sm, st>>>(
+      cand, ckeys, nprobe, qbase, list_off, kk, k, qrho, rmax, e_rest, prune, B, out, stats);
   ADN_LAUNCH("select16_kernel");
   return ADANNS_OK;
 }
 
 int launch_certify16(const uint16_t *cand, const uint64_t *ckeys, int nprobe, const int64_t *qbase,
-                     const int64_t *list_off, int kk, int k, const float *qrho, float rmax,
-                     float e_rest, int64_t B, int64_t *out, int32_t *cnt,
-                     unsigned long long *stats, cudaStream_t st) {
-  if (nprobe > SW_MAXP) return fail(ADANNS_ERR_ARG, "certify16: nprobe above 128");
+                     const int64_t *list_off, int kk, int k, const float *qerr, int64_t B,
+                     int64_t *out, int32_t *cnt, unsigned long long *stats, cudaStream_t st) {
+  if (nprobe > SW_MAXP || k > CERT_MAX_K || kk > CERT_MAX_KK || kk < k)
+    return fail(ADANNS_ERR_ARG, "certify16: shape outside its buffers");
   if (B <= 0) return ADANNS_OK;
   const size_t sm = sizeof(SwState) * SW_WARPS;
-  ADN_CUDA(ensure_smem((const void *)select16_kernel<true>, sm));
-  select16_kernel<true><<<(unsigned)((B + SW_WARPS - 1) / SW_WARPS), SW_WARPS * 32, sm, st>>>(
-      cand, ckeys, nprobe, qbase, list_off, kk, k, qrho, rmax, e_rest, 1, B, out, cnt, stats);
-  ADN_LAUNCH("select16_kernel");
+  ADN_CUDA(ensure_smem((const void *)certify16_kernel, sm));
+  certify16_kernel<<<(unsigned)((B + SW_WARPS - 1) / SW_WARPS), SW_WARPS * 32, sm, st>>>(
+      cand, ckeys, nprobe, qbase, list_off, kk, k, qerr, B, out, cnt, stats);
+  ADN_LAUNCH("certify16_kernel");
   return ADANNS_OK;
 }
 

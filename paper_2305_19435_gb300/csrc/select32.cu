@@ -83,7 +83,9 @@ __device__ void select_into(int n, int kk, KeyF key, IdF id, ValF val, uint64_t 
 __global__ void __launch_bounds__(S32_THREADS) select32_kernel(
     const uint32_t *__restrict__ cand, const uint64_t *__restrict__ ckeys, int nprobe,
     const int64_t *__restrict__ qbase, const int64_t *__restrict__ list_off,
-    const int32_t *__restrict__ list_ids, int kk, uint64_t *__restrict__ out) {
+    const int32_t *__restrict__ list_ids, int kk, uint64_t *__restrict__ out,
+    const int32_t *__restrict__ only) {
+  if (only && only[blockIdx.x] >= 0) return;
   __shared__ S32State st;
   // the sample, then (once the threshold is known) the compacted keys and positions
   __shared__ __align__(16) uint32_t space[S32_SAMPLE];
@@ -222,11 +224,11 @@ int launch_keys_to_ids(const uint64_t *keys, int64_t n, int64_t *ids, cudaStream
 
 int launch_select32(const uint32_t *cand, const uint64_t *ckeys, int nprobe, const int64_t *qbase,
                     const int64_t *list_off, const int32_t *list_ids, int64_t B, int kk,
-                    uint64_t *out, cudaStream_t st) {
+                    uint64_t *out, cudaStream_t st, const int32_t *only) {
   if (nprobe > S32_MAXP) return fail(ADANNS_ERR_ARG, "select32: nprobe above 256");
   if (B <= 0) return ADANNS_OK;
   select32_kernel<<<(unsigned)B, S32_THREADS, 0, st>>>(cand, ckeys, nprobe, qbase, list_off,
-                                                       list_ids, kk, out);
+                                                       list_ids, kk, out, only);
   ADN_LAUNCH("select32_kernel");
   return ADANNS_OK;
 }

@@ -1,7 +1,7 @@
-"""The FP32 search through the certified tensor-core filter (many queries per
-probed list) gives the tiled FP32 scan's ids and distance bits: the re-score
-uses the scan's arithmetic, and the filter keeps every member that can be
-among the k nearest, so no tolerance applies."""
+"""Searches through the certified tensor-core filter (many queries per probed
+list) give the direct scans' ids and distance bits: the re-score uses the
+scan's arithmetic, and the filter keeps every member that can be among the k
+nearest, so no tolerance applies."""
 import numpy as np
 import pytest
 
@@ -103,4 +103,68 @@ def test_slices(P):
         a, b = both(P, g, q, 16, 128, 4, 40)
     same(a, b)
     same(a, both(P, g, q, 16, 128, 4, 40)[0])
+    g.free()
+
+
+# ------------------------------------------------------------------ IVF-OPQ
+def opq_index(P, n, d, d_s, M, nlist, seed, db=None):
+    """An index with a random orthonormal rotation and codebooks of sampled rows."""
+    data = synthdata.small(n, 8, d, 24, seed)
+    x = torch.from_numpy(data["db"] if db is None else db).cuda()
+    g = P.build_ivf(x, 16, nlist, 3, n, seed) if nlist > 1 else P.flat_index(x)
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    R = torch.linalg.qr(torch.randn(d_s, d_s, device="cuda", generator=gen))[0].contiguous()
+    z = torch.nn.functional.normalize(x[:256, :d_s], dim=1) @ R
+    C = z.view(256, M, d_s // M).transpose(0, 1).contiguous()
+    P.set_opq(g, d_s, M, R, C, P.opq_encode(x, d_s, M, R, C))
+    return data["means"], g
+
+
+def opq_both(P, g, q, *args, filtered=True, **kw):
+    """(filtered, lookups): the option that turns distance-then-select off keeps
+    the running top-k over table lookups."""
+    P.profile_enable(True)
+    a = [t.cpu().numpy() for t in P.search_ivfopq(g, q, *args, return_probes=True, **kw)]
+    # the cluster mapping has no stage of that name
+    assert ("mma" in P.profile_read()) == filtered
+    P.profile_enable(False)
+    with P.option(P.OPT_ADC_SELECT, 0):
+        b = [t.cpu().numpy() for t in P.search_ivfopq(g, q, *args, return_probes=True, **kw)]
+    g.status()
+    return a, b
+
+
+# sub-vectors of 1 to 16 coordinates (whole and crossing groups of four),
+# sums of words and of bytes, one list and several, shortlists up to the
+# largest filtered one and one above
+@pytest.mark.parametrize("d,d_s,M,nlist,nprobe,k,rerank,B", [
+    (64, 64, 8, 4, 4, 10, 0, 3601), (64, 64, 64, 4, 3, 100, 400, 700),
+    (96, 96, 32, 4, 4, 5, 0, 1000), (96, 96, 6, 1, 1, 10, 0, 8001),
+    (128, 128, 16, 1, 1, 10, 40, 2047), (256, 192, 16, 6, 5, 100, 0, 2500),
+    (384, 384, 32, 6, 6, 128, 512, 800), (384, 384, 32, 6, 6, 128, 513, 800)])
+def test_opq_equals_lookups(P, d, d_s, M, nlist, nprobe, k, rerank, B):
+    means, g = opq_index(P, 20000, d, d_s, M, nlist, d_s + M)
+    q = torch.from_numpy(synthdata.sample_points(B, d, means, 99, threads=1)[0]).cuda()
+    same(*opq_both(P, g, q, 8 if nlist == 1 else 16, nprobe, k, rerank_k=rerank,
+                   filtered=rerank <= 512))
+    g.free()
+
+
+def test_opq_left_over_queries(P):
+    """Thousands of rows with one code: certified sets that overflow, and a
+    batch cut into slices by the scratch budget."""
+    data = synthdata.small(20000, 8, 64, 16, 31)
+    db = data["db"].copy()
+    db[2000:6000] = db[5]
+    means, g = opq_index(P, 20000, 64, 64, 16, 3, 31, db=db)
+    q = synthdata.sample_points(3000, 64, means, 7, threads=1)[0]
+    q[::9] = db[5]
+    q[4::50] = 0
+    q = torch.from_numpy(q).cuda()
+    a, b = opq_both(P, g, q, 16, 3, 20, rerank_k=80)
+    same(a, b)
+    with P.option(P.OPT_SCRATCH_BYTES, 160 << 20):
+        c = [t.cpu().numpy() for t in P.search_ivfopq(g, q, 16, 3, 20, rerank_k=80,
+                                                      return_probes=True)]
+    same(c, b)
     g.free()
