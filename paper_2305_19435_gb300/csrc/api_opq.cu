@@ -30,9 +30,9 @@ int launch_sub_list_centre(float *rows, int64_t n, int ldr, int d_s, const int64
 int launch_residual_tables(const float *w, int nlist, int d_s, int M, const float *C, float *S,
                            float *w2, cudaStream_t st);
 struct AdcArgs;
-int launch_rerank(const int64_t *cand, int kr, int64_t B, const float *qs, int ldq, int d_s,
-                  const adanns_index *idx, const float *mscale, int k, int64_t *out_ids,
-                  float *out_dist, cudaStream_t st);
+int launch_rerank(const int64_t *cand, int kr, int64_t B, const int32_t *order, const float *qs,
+                  int ldq, int d_s, const adanns_index *idx, const float *mscale, int k,
+                  int64_t *out_ids, float *out_dist, cudaStream_t st);
 int launch_adc(const uint8_t *codes, const int64_t *list_off, const int32_t *list_ids, int M,
                const float *lut, const int32_t *tl, const int32_t *tb, const int32_t *tc,
                const int *ntiles, int *counter, const int32_t *pair_q, const int32_t *pair_out,
@@ -281,6 +281,8 @@ int search_ivfopq_select(const adanns_index *idx, const float *queries, int64_t 
                (rc = s.get(&qn2, Bc)) || (rc = s.get(&qerr, Bc)) || (rc = s.get(&cnt, Bc)) ||
                (rc = s.get(&list, (size_t)Bc * kk)) || (profiling() && (rc = s.get(&stats, 2)))))
     return rc;
+  int32_t *order = nullptr;
+  if (rerank && rerank_order_pays(idx, Bc * kr, d_s) && (rc = s.get(&order, Bc))) return rc;
   const float *mscale = idx->metric == ADANNS_METRIC_L2_PREFIXNORM
                             ? idx->invn + (int64_t)gran_index(d_s) * idx->N
                             : nullptr;
@@ -337,6 +339,8 @@ int search_ivfopq_select(const adanns_index *idx, const float *queries, int64_t 
       if ((rc = run_coarse(idx, qc, dcp, nb, d_c, nprobe, ckeys, counter, st))) return rc;
       if (qb && (rc = launch_mask_probes(ckeys, nb, nprobe, qb->at(b0).np, st))) return rc;
     }
+    // (before the answered queries' probe slots are masked)
+    if (order && (rc = launch_query_order(idx, ckeys, nb, nprobe, order, st))) return rc;
     {
       StageTimer t(ST_LUT, st);
       if ((rc = launch_gemm_f32(false, (int)nb, d_s, d_s, 1.f, qs, dsp, idx->opq_R, d_s, 0.f, z,
@@ -421,7 +425,7 @@ int search_ivfopq_select(const adanns_index *idx, const float *queries, int64_t 
     if (rerank) {
       StageTimer t(ST_RERANK, st);
       if ((rc = launch_keys_to_ids(keys, nb * kr, cids, st))) return rc;
-      if ((rc = launch_rerank(cids, kr, nb, qs, dsp, d_s, idx, mscale, k, out_ids + b0 * k,
+      if ((rc = launch_rerank(cids, kr, nb, order, qs, dsp, d_s, idx, mscale, k, out_ids + b0 * k,
                               out_dist + b0 * k, st)))
         return rc;
     }
@@ -769,7 +773,7 @@ int adanns_search_ivfopq(const adanns_index *idx, const float *queries, int64_t 
         if ((rc = launch_merge(pkeys, nb, nprobe, kr, cids, cdist, st))) return rc;
       }
       StageTimer t(ST_RERANK, st);
-      if ((rc = launch_rerank(cids, kr, nb, qs, dsp, d_s, idx, mscale, k, out_ids + b0 * k,
+      if ((rc = launch_rerank(cids, kr, nb, nullptr, qs, dsp, d_s, idx, mscale, k, out_ids + b0 * k,
                               out_dist + b0 * k, st)))
         return rc;
     } else {

@@ -255,19 +255,9 @@ __global__ void __launch_bounds__(RS_W * 32) rescore_kernel(
   }
   __syncthreads();
   if (warp != 0) return;
-  if (n <= 256) {
-    uint64_t v[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = lane * 8 + j < n ? keys[lane * 8 + j] : KEY_MAX;
-    __syncwarp();
-    warp_sort256(v);
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (lane * 8 + j < n) keys[lane * 8 + j] = v[j];
-    __syncwarp();
-  } else {
-    warp_sort(keys, n);
-  }
+  if (n <= 256) warp_sort_regs<8>(keys, n, k);
+  else if (n <= 512) warp_sort_regs<16>(keys, n, k);
+  else warp_sort(keys, n);
   for (int r = lane; r < k; r += 32) {
     const uint64_t key = r < n ? keys[r] : KEY_MAX;
     out_ids[q * k + r] = key == KEY_MAX ? -1 : (int64_t)(uint32_t)(key & 0xffffffffu);
@@ -289,6 +279,23 @@ int launch_f16_queries(const float *v, int ldv, int64_t B, int d_s, int nkb, con
                                                               zmax2, e_rest, (uint2 *)out, qn2,
                                                               qerr);
   ADN_LAUNCH("f16_queries_kernel");
+  return ADANNS_OK;
+}
+
+int launch_query_order(const adanns_index *idx, const uint64_t *ckeys, int64_t B, int nprobe,
+                       int32_t *order, cudaStream_t st) {
+  if (B <= 0) return ADANNS_OK;
+  Scratch s(st);
+  int32_t *cur;
+  int rc;
+  if ((rc = s.get(&cur, idx->nlist))) return rc;
+  const unsigned g = (unsigned)((B + 255) / 256);
+  ADN_CUDA(cudaMemsetAsync(cur, 0, sizeof(int32_t) * idx->nlist, st));
+  order_count_kernel<<<g, 256, 0, st>>>(ckeys, B, nprobe, idx->rr_rank, cur);
+  ADN_LAUNCH("order_count_kernel");
+  if ((rc = launch_scan_i32(cur, idx->nlist, cur, st))) return rc;
+  order_fill_kernel<<<g, 256, 0, st>>>(ckeys, B, nprobe, idx->rr_rank, cur, order);
+  ADN_LAUNCH("order_fill_kernel");
   return ADANNS_OK;
 }
 
@@ -376,8 +383,7 @@ int search_f32_certified(const adanns_index *idx, const float *queries, int64_t 
   Scratch s(st);
   float *qc, *qs, *qn2, *qerr, *x2;
   uint64_t *ckeys;
-  int32_t *lcnt, *lbeg, *lfill, *tbeg, *pair_q, *pair_out, *tl, *tb, *tc, *cnt, *ocur = nullptr,
-      *order = nullptr;
+  int32_t *lcnt, *lbeg, *lfill, *tbeg, *pair_q, *pair_out, *tl, *tb, *tc, *cnt, *order = nullptr;
   int *ntiles, *flags;  // flags: [0] cluster mapping, [1] scan, [2] tiled scan counters, [3] unsure
   int64_t *qtot, *qbase, *pbase, *cids;
   unsigned char *qlow, *qtile, *rows;
@@ -399,7 +405,7 @@ int search_f32_certified(const adanns_index *idx, const float *queries, int64_t 
       (rc = s.get(&cand, (size_t)(Bc * h.seg))) ||
       (rc = tiled_scan_scratch(s, idx, Bc, nprobe, k, &h.ts)))
     return rc;
-  if (ordered && ((rc = s.get(&ocur, nlist)) || (rc = s.get(&order, Bc)))) return rc;
+  if (ordered && (rc = s.get(&order, Bc))) return rc;
   if (profiling() && (rc = s.get(&stats, 2))) return rc;
   const float *nu = idx->invn + (int64_t)gran_index(d_s) * idx->N;
   const float yn = sqrtf(CE_NORM2);
@@ -482,14 +488,7 @@ int search_f32_certified(const adanns_index *idx, const float *queries, int64_t 
     }
     {
       StageTimer t(ST_RERANK, st);
-      if (ordered) {
-        ADN_CUDA(cudaMemsetAsync(ocur, 0, sizeof(int32_t) * nlist, st));
-        order_count_kernel<<<gq, 256, 0, st>>>(ckeys, nb, nprobe, idx->rr_rank, ocur);
-        ADN_LAUNCH("order_count_kernel");
-        if ((rc = launch_scan_i32(ocur, nlist, ocur, st))) return rc;
-        order_fill_kernel<<<gq, 256, 0, st>>>(ckeys, nb, nprobe, idx->rr_rank, ocur, order);
-        ADN_LAUNCH("order_fill_kernel");
-      }
+      if (ordered && (rc = launch_query_order(idx, ckeys, nb, nprobe, order, st))) return rc;
       rescore_kernel<<<(unsigned)nb, RS_W * 32, rsm, st>>>(
           cids, cnt, kk, order, qs, dsp, d_s, idx->xpm, idx->d_pad, idx->list_off, idx->list_ids,
           nu, k, oi, od);

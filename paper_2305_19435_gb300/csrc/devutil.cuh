@@ -198,31 +198,32 @@ __device__ __forceinline__ void warp_sort(uint64_t *a, int n) {
   }
 }
 
-// Ascending bitonic sort of 256 keys held 8 per lane (lane l holds positions
-// 8l .. 8l + 7): strides below 8 compare within a lane, larger ones across
+// Ascending bitonic sort of 32 J keys held J per lane (lane l holds positions
+// J l .. J l + J - 1): strides below J compare within a lane, larger ones across
 // lanes by shuffles; the direction of each compare-exchange is that of the
 // block of `size` positions holding it (ascending for even blocks).
-__device__ __forceinline__ void warp_sort256(uint64_t (&v)[8]) {
+template <int J>
+__device__ __forceinline__ void warp_sort_lanes(uint64_t (&v)[J]) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int size = 2; size <= 256; size <<= 1) {
+  for (int size = 2; size <= 32 * J; size <<= 1) {
 #pragma unroll
     for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      if (stride >= 8) {
-        const int ls = stride >> 3;
+      if (stride >= J) {
+        const int ls = stride / J;
         const bool lower = (lane & ls) == 0;
-        const bool asc = ((lane * 8) & size) == 0;
+        const bool asc = ((lane * J) & size) == 0;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < J; ++j) {
           const uint64_t o = __shfl_xor_sync(0xffffffffu, v[j], ls);
           const uint64_t lo = o < v[j] ? o : v[j], hi = o < v[j] ? v[j] : o;
           v[j] = lower == asc ? lo : hi;
         }
       } else {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < J; ++j) {
           if (j & stride) continue;
-          const bool asc = ((lane * 8 + j) & size) == 0;
+          const bool asc = ((lane * J + j) & size) == 0;
           const uint64_t a = v[j], b = v[j | stride];
           const uint64_t lo = a < b ? a : b, hi = a < b ? b : a;
           v[j] = asc ? lo : hi;
@@ -231,6 +232,22 @@ __device__ __forceinline__ void warp_sort256(uint64_t (&v)[8]) {
       }
     }
   }
+}
+
+// One warp: ascending sort of a[0:n), n <= 32 J, in shared memory through
+// registers; only the first `keep` are put back.
+template <int J>
+__device__ __forceinline__ void warp_sort_regs(uint64_t *a, int n, int keep) {
+  const int lane = threadIdx.x & 31;
+  uint64_t v[J];
+#pragma unroll
+  for (int j = 0; j < J; ++j) v[j] = lane * J + j < n ? a[lane * J + j] : ~0ull;
+  __syncwarp();
+  warp_sort_lanes<J>(v);
+#pragma unroll
+  for (int j = 0; j < J; ++j)
+    if (lane * J + j < min(n, keep)) a[lane * J + j] = v[j];
+  __syncwarp();
 }
 
 // Ascending sort of a[0:n) in shared memory by the NT threads of a block (the

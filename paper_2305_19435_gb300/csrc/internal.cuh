@@ -377,6 +377,9 @@ int search_f32_certified(const adanns_index *idx, const float *queries, int64_t 
 int launch_f16_queries(const float *v, int ldv, int64_t B, int d_s, int nkb, const int *unsure,
                        float yn, float yr, float zmax2, void *out, float *qn2, float *qerr,
                        cudaStream_t st);
+// the queries in the order of their nearest list along the index's chain of lists
+int launch_query_order(const adanns_index *idx, const uint64_t *ckeys, int64_t B, int nprobe,
+                       int32_t *order, cudaStream_t st);
 // probe slots of queries with cnt[q] >= 0 -> PROBE_NONE
 int launch_mask_answered(uint64_t *ckeys, int64_t B, int nprobe, const int32_t *cnt,
                          cudaStream_t st);
@@ -419,8 +422,17 @@ int launch_select_surv(const uint32_t *rec, const int *rcnt, const int64_t *pbas
                        const float *qrho, float rmax, float e_rest, int prune, int64_t B,
                        int64_t *out, unsigned long long *stats, cudaStream_t st);
 int launch_keys_to_ids(const uint64_t *keys, int64_t n, int64_t *ids, cudaStream_t st);
+// dense: most slots hold a key
 int launch_final_topk(const uint64_t *keys, int kr, int64_t B, int k, int64_t *out_ids,
-                      float *out_dist, cudaStream_t st);
+                      float *out_dist, cudaStream_t st, bool dense = false);
+bool rerank_order_pays(const adanns_index *idx, int64_t slots, int d_s);
+// exact re-score of each query's kr shortlisted candidates, query by query
+// (rerank_query.cu): keys [B][kr], KEY_MAX for empty slots; order (or null):
+// the order in which the queries are taken
+int launch_rerank_query(const int64_t *cand, int kr, int64_t B, const int32_t *order,
+                        const float *qs, int ldq, int d_s, const adanns_index *idx,
+                        const float *mscale, int lanes, uint64_t *keys, cudaStream_t st,
+                        int64_t *npairs = nullptr);  // zeroed counter of re-scored pairs
 int adc_dist_query_tile(int M);
 // res_S / res_w / res_w2 / z (NULL for plain codes): residual terms and the
 // queries' rotated vectors [B][d_s]; the score of a member of list l is then

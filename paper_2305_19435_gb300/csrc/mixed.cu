@@ -15,12 +15,11 @@
 
 namespace adn {
 
-int launch_rerank(const int64_t *cand, int kr, int64_t B, const float *qs, int ldq, int d_s,
-                  const adanns_index *idx, const float *mscale, int k, int64_t *out_ids,
-                  float *out_dist, cudaStream_t st);
-// cand: B x kr shortlisted candidates as (list << 32 | member position), -1 padding
-int launch_rerank_lists(const int64_t *cand, int kr, int64_t B, const float *qs, int ldq, int d_s,
-                        const adanns_index *idx, const float *mscale, int k, int64_t *out_ids,
+// cand: B x kr shortlisted candidates as (list << 32 | member position), -1 padding;
+// ckeys: the queries' probe keys; dense: little of it was pruned
+int launch_rerank_lists(const int64_t *cand, int kr, int64_t B, const uint64_t *ckeys, int nprobe,
+                        const float *qs, int ldq, int d_s, const adanns_index *idx,
+                        const float *mscale, int k, bool dense, int64_t *out_ids,
                         float *out_dist, cudaStream_t st);
 
 // ---------------------------------------------------------------- storage
@@ -588,8 +587,8 @@ int search_mixed(const adanns_index *idx, const float *queries, int64_t B, int d
     }
     {
       StageTimer t(ST_RERANK, st);
-      if ((rc = launch_rerank_lists(cids, kk, nb, qs, dsp, d_s, idx, mscale, k, out_ids + b0 * k,
-                                    out_dist + b0 * k, st)))
+      if ((rc = launch_rerank_lists(cids, kk, nb, ckeys, nprobe, qs, dsp, d_s, idx, mscale, k,
+                                    fp8 || !prune, out_ids + b0 * k, out_dist + b0 * k, st)))
         return rc;
       if (qb && (rc = launch_pad_rows(out_ids + b0 * k, out_dist + b0 * k, nb, k, qb->at(b0).k,
                                       st)))

@@ -343,77 +343,19 @@ int launch_adc_scan(const AdcArgs &a, int qa, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------- exact rerank
-// One warp per query: the kr candidate ids are re-scored with the exact FP32
-// difference-form distance on the d_s prefix (read from the prefix-major
-// storage, 8 lanes per candidate), then the k best by (distance, id) are kept.
-constexpr int RR_WARPS = 4;
-
-__global__ void rerank_kernel(const int64_t *__restrict__ cand, int kr, int64_t B,
-                              const float *__restrict__ qs, int ldq, int d_s,
-                              const float *__restrict__ xpm, int d_pad,
-                              const int64_t *__restrict__ list_off,
-                              const int32_t *__restrict__ assign, const int32_t *__restrict__ pos,
-                              const float *__restrict__ mscale, int k, int cap,
-                              int64_t *__restrict__ out_ids, float *__restrict__ out_dist) {
-  extern __shared__ __align__(16) unsigned char rsm[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t q = (int64_t)blockIdx.x * RR_WARPS + warp;
-  float *sq = (float *)rsm + (size_t)warp * ldq;
-  uint64_t *buf = (uint64_t *)((float *)rsm + (size_t)RR_WARPS * ldq) + (size_t)warp * cap;
-  if (q >= B) return;
-  for (int j = lane; j < ldq; j += 32) sq[j] = qs[q * ldq + j];
-  __syncwarp();
-  const int g = lane >> 3, s = lane & 7;
-  const int nseg = d_s >> 2;  // float4 segments (d_s is a multiple of 8)
-  for (int r0 = 0; r0 < kr; r0 += 4) {
-    const int r = r0 + g;
-    const int64_t id = r < kr ? cand[q * kr + r] : -1;
-    float acc = 0.f;
-    if (id >= 0) {
-      const int l = assign[id];
-      const int64_t p = pos[id];
-      const int64_t off = list_off[l];
-      const int64_t nl = list_off[l + 1] - off;
-      const float *base = xpm + off * d_pad + (p - off) * 16;
-      const float nu = mscale ? mscale[p] : 1.f;
-      for (int e = s; e < nseg; e += 8) {
-        const int b = e >> 2, part = e & 3;
-        const float4 x = *(const float4 *)(base + (int64_t)b * 16 * nl + part * 4);
-        const float4 qv = *(const float4 *)(sq + e * 4);
-        float t;
-        t = fmaf(-nu, x.x, qv.x); acc = fmaf(t, t, acc);
-        t = fmaf(-nu, x.y, qv.y); acc = fmaf(t, t, acc);
-        t = fmaf(-nu, x.z, qv.z); acc = fmaf(t, t, acc);
-        t = fmaf(-nu, x.w, qv.w); acc = fmaf(t, t, acc);
-      }
-    }
-    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-    acc += __shfl_xor_sync(0xffffffffu, acc, 4);
-    if (s == 0 && r < kr) buf[r] = id >= 0 ? pack_key(acc, (uint32_t)id) : KEY_MAX;
-  }
-  __syncwarp();
-  warp_sort(buf, kr);
-  for (int r = lane; r < k; r += 32) {
-    const uint64_t key = r < kr ? buf[r] : KEY_MAX;
-    out_ids[q * k + r] = key == KEY_MAX ? -1 : (int64_t)(uint32_t)(key & 0xffffffffu);
-    out_dist[q * k + r] = key == KEY_MAX ? __int_as_float(0x7f800000)
-                                         : __uint_as_float((uint32_t)(key >> 32));
-  }
-}
-
-int launch_rerank(const int64_t *cand, int kr, int64_t B, const float *qs, int ldq, int d_s,
-                  const adanns_index *idx, const float *mscale, int k, int64_t *out_ids,
-                  float *out_dist, cudaStream_t st) {
+// The kr candidate ids of each query re-scored exactly, the k best kept; order
+// (or null): the order in which the queries are taken.
+int launch_rerank(const int64_t *cand, int kr, int64_t B, const int32_t *order, const float *qs,
+                  int ldq, int d_s, const adanns_index *idx, const float *mscale, int k,
+                  int64_t *out_ids, float *out_dist, cudaStream_t st) {
   if (B <= 0) return ADANNS_OK;
-  const int cap = kr;
-  const size_t smem = (size_t)RR_WARPS * ldq * 4 + (size_t)RR_WARPS * cap * 8;
-  ADN_CUDA(ensure_smem((const void *)rerank_kernel, (size_t)(smem)));
-  rerank_kernel<<<(unsigned)((B + RR_WARPS - 1) / RR_WARPS), RR_WARPS * 32, smem, st>>>(
-      cand, kr, B, qs, ldq, d_s, idx->xpm, idx->d_pad, idx->list_off, idx->assign, idx->pos_of_id,
-      mscale, k, cap, out_ids, out_dist);
-  ADN_LAUNCH("rerank_kernel");
-  return ADANNS_OK;
+  Scratch s(st);
+  uint64_t *keys;
+  int rc;
+  if ((rc = s.get(&keys, (size_t)B * kr)) ||
+      (rc = launch_rerank_query(cand, kr, B, order, qs, ldq, d_s, idx, mscale, 8, keys, st)))
+    return rc;
+  return launch_final_topk(keys, kr, B, k, out_ids, out_dist, st, true);
 }
 
 // ---------------------------------------------------------------- misc

@@ -210,7 +210,11 @@ __global__ void __launch_bounds__(NT, MINB) rerank_chunks_kernel(
   }
 }
 
-// per query (one warp): sort its kr keys, write the k best
+// per query (one warp): sort its kr keys, write the k best.  Up to 256 keys (a
+// pruned shortlist) are sorted in registers, with DENSE up to 512: the wider
+// sort's registers cost a third of the warps in flight, so it is a kernel of
+// its own for shortlists that are known to be full.
+template <bool DENSE>
 __global__ void final_topk_kernel(const uint64_t *__restrict__ keys, int kr, int64_t B, int k,
                                   int64_t *__restrict__ out_ids, float *__restrict__ out_dist) {
   extern __shared__ uint64_t kb[];
@@ -235,31 +239,11 @@ __global__ void final_topk_kernel(const uint64_t *__restrict__ keys, int kr, int
     }
   }
   __syncwarp();
-  if (n <= 256) {
-    // the common case (pruned shortlists): sorted in registers
-    uint64_t v[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int r = lane * 8 + j;
-      v[j] = r < n ? buf[r] : KEY_MAX;
-    }
-    warp_sort256(v);
-    // back through shared memory (the first min(k, 256) positions, k <= kr), so
-    // that the results leave as whole rows: lanes write consecutive entries
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (lane * 8 + j < k) buf[lane * 8 + j] = v[j];
-    __syncwarp();
-    for (int r = lane; r < k; r += 32) {
-      const uint64_t key = r < 256 ? buf[r] : KEY_MAX;  // k above 256: padding
-      out_ids[q * k + r] = key == KEY_MAX ? -1 : (int64_t)(uint32_t)(key & 0xffffffffu);
-      out_dist[q * k + r] = key == KEY_MAX ? __int_as_float(0x7f800000)
-                                           : __uint_as_float((uint32_t)(key >> 32));
-    }
-    return;
-  }
-  warp_sort(buf, n);
+  // put back in shared memory, so that the results leave as whole rows (lanes
+  // write consecutive entries)
+  if (n <= 256) warp_sort_regs<8>(buf, n, k);
+  else if (DENSE && n <= 512) warp_sort_regs<16>(buf, n, k);
+  else warp_sort(buf, n);
   for (int r = lane; r < k; r += 32) {
     const uint64_t key = r < n ? buf[r] : KEY_MAX;
     out_ids[q * k + r] = key == KEY_MAX ? -1 : (int64_t)(uint32_t)(key & 0xffffffffu);
@@ -270,23 +254,59 @@ __global__ void final_topk_kernel(const uint64_t *__restrict__ keys, int kr, int
 
 // per query: the k best of kr packed keys, as (ids, distances)
 int launch_final_topk(const uint64_t *keys, int kr, int64_t B, int k, int64_t *out_ids,
-                      float *out_dist, cudaStream_t st) {
+                      float *out_dist, cudaStream_t st, bool dense) {
   if (B <= 0) return ADANNS_OK;
   const size_t fs = (size_t)4 * kr * 8;
-  ADN_CUDA(ensure_smem((const void *)final_topk_kernel, fs));
-  final_topk_kernel<<<(unsigned)((B + 3) / 4), 128, fs, st>>>(keys, kr, B, k, out_ids, out_dist);
+  auto kern = dense && kr > 256 ? final_topk_kernel<true> : final_topk_kernel<false>;
+  ADN_CUDA(ensure_smem((const void *)kern, fs));
+  kern<<<(unsigned)((B + 3) / 4), 128, fs, st>>>(keys, kr, B, k, out_ids, out_dist);
   ADN_LAUNCH("final_topk_kernel");
   return ADANNS_OK;
 }
 
-int launch_rerank_lists(const int64_t *cand, int kr, int64_t B, const float *qs, int ldq, int d_s,
-                        const adanns_index *idx, const float *mscale, int k, int64_t *out_ids,
+// The query-major rerank (rerank_query.cu) unless the shortlists hold many slots
+// per database row: then a row read once for all its pairs, by the member-major
+// kernels here, costs less than the sort that brings them together.  Measured
+// (1.28 M rows, BF16 / FP8 shortlists of 40 and 400, ms by query / by member):
+// d_s 512, 0.6 slots per row 0.27 / 0.55, 2.6: 0.57 / 0.77 and 0.87 / 1.04, 6.2:
+// 0.95 / 1.10 and 1.75 / 1.87, 15.6: 2.05 / 2.02 and 4.15 / 4.04; d_s 2048, 0.6:
+// 0.94 / 1.95, 6.2: 3.4 / 3.9 and 5.5 / 5.5, 15.6: 7.5 / 7.0; d_s 128, 2.6:
+// 0.31 / 0.34 and 0.60 / 0.54, 6.2: 0.60 / 0.55.
+static bool rerank_by_query(int64_t slots, int64_t N, int d_s) {
+  return slots <= (d_s >= 512 ? 7 : 2) * N;
+}
+
+int launch_rerank_lists(const int64_t *cand, int kr, int64_t B, const uint64_t *ckeys, int nprobe,
+                        const float *qs, int ldq, int d_s, const adanns_index *idx,
+                        const float *mscale, int k, bool dense, int64_t *out_ids,
                         float *out_dist, cudaStream_t st) {
   if (B <= 0) return ADANNS_OK;
   const int64_t n = B * kr;
   if (n > INT32_MAX) return fail(ADANNS_ERR_ARG, "rerank slice too large");
   const int64_t N = idx->N;
   Scratch s(st);
+  if (rerank_by_query(n, N, d_s)) {
+    uint64_t *qk;
+    int64_t *np = nullptr;
+    int32_t *order = nullptr;
+    int rc;
+    if (rerank_order_pays(idx, n, d_s) &&
+        ((rc = s.get(&order, (size_t)B)) ||
+         (rc = launch_query_order(idx, ckeys, B, nprobe, order, st))))
+      return rc;
+    if ((rc = s.get(&qk, n)) || (profiling() && (rc = s.get(&np, 1)))) return rc;
+    if (np) ADN_CUDA(cudaMemsetAsync(np, 0, sizeof(int64_t), st));
+    {
+      StageTimer t(ST_RR_PAIRS, st);
+      if ((rc = launch_rerank_query(cand, kr, B, order, qs, ldq, d_s, idx, mscale, 16, qk, st,
+                                    np)))
+        return rc;
+    }
+    if (np) profile_count(PC_RERANK_PAIRS, np, st);
+    profile_count_host(PC_SHORTLIST_SLOTS, n);
+    StageTimer t(ST_RR_FINAL, st);
+    return launch_final_topk(qk, kr, B, k, out_ids, out_dist, st, dense);
+  }
   int32_t *ppos, *order, *mstart, *cursor;
   int2 *cpair;
   int64_t *npairs;
@@ -349,14 +369,8 @@ int launch_rerank_lists(const int64_t *cand, int kr, int64_t B, const float *qs,
       ADN_LAUNCH("rerank_chunks_kernel");
     }
   }
-  {
-    StageTimer t(ST_RR_FINAL, st);
-    const size_t fs = (size_t)4 * kr * 8;
-    ADN_CUDA(ensure_smem((const void *)final_topk_kernel, (size_t)(fs)));
-    final_topk_kernel<<<(unsigned)((B + 3) / 4), 128, fs, st>>>(keys, kr, B, k, out_ids, out_dist);
-    ADN_LAUNCH("final_topk_kernel");
-  }
-  return ADANNS_OK;
+  StageTimer t(ST_RR_FINAL, st);
+  return launch_final_topk(keys, kr, B, k, out_ids, out_dist, st, dense);
 }
 
 }  // namespace adn
