@@ -293,10 +293,17 @@ int search_ivfopq_select(const adanns_index *idx, const float *queries, int64_t 
     const int32_t *only = cert ? cnt + p0 : nullptr;
     {
       StageTimer t(ST_INVERT, st);
+      ProbePlan plan;
+      plan.zero = work;
+      plan.nzero = 1;
+      plan.list_off = idx->list_off;
+      plan.qbase = qbase;
+      plan.pbase = pbase;
       if ((rc = launch_invert_probes(ck, np, nprobe, nlist, qa, lcnt, lbeg, lfill, tbeg, pair_q,
-                                     pair_out, tl, tb, tc, ntiles, probes, st)))
+                                     pair_out, tl, tb, tc, ntiles, probes, st, &plan)))
         return rc;
-      if ((rc = launch_cand_segments(ck, np, nprobe, idx->list_off, qtot, qbase, pbase, st)))
+      if (!plan.planned &&
+          (rc = launch_cand_segments(ck, np, nprobe, idx->list_off, qtot, qbase, pbase, st)))
         return rc;
     }
     {
@@ -332,8 +339,8 @@ int search_ivfopq_select(const adanns_index *idx, const float *queries, int64_t 
                                     dcp, qs, dsp, st)))
         return rc;
     }
-    // work counters: cluster mapping, tensor-core scan, lookup scans
-    ADN_CUDA(cudaMemsetAsync(counter, 0, 4 * sizeof(int), st));
+    // work counters: cluster mapping, tensor-core scan, lookup scans (each cleared
+    // before its scan)
     {
       StageTimer t(ST_COARSE, st);
       if ((rc = run_coarse(idx, qc, dcp, nb, d_c, nprobe, ckeys, counter, st))) return rc;
@@ -352,10 +359,17 @@ int search_ivfopq_select(const adanns_index *idx, const float *queries, int64_t 
     } else {
       {
         StageTimer t(ST_INVERT, st);
+        ProbePlan plan;
+        plan.zero = counter + 1;
+        plan.nzero = 1;
+        plan.list_off = idx->list_off;
+        plan.qbase = qbase;
+        plan.pbase = pbase;
         if ((rc = launch_invert_probes(ckeys, nb, nprobe, nlist, QT, lcnt, lbeg, lfill, tbeg,
-                                       pair_q, pair_out, tl, tb, tc, ntiles, probes, st)))
+                                       pair_q, pair_out, tl, tb, tc, ntiles, probes, st, &plan)))
           return rc;
-        if ((rc = launch_cand_segments(ckeys, nb, nprobe, idx->list_off, qtot, qbase, pbase, st)))
+        if (!plan.planned && (rc = launch_cand_segments(ckeys, nb, nprobe, idx->list_off, qtot,
+                                                        qbase, pbase, st)))
           return rc;
       }
       {

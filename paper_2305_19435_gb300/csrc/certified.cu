@@ -414,7 +414,6 @@ int search_f32_certified(const adanns_index *idx, const float *queries, int64_t 
   ADN_CUDA(ensure_smem((const void *)rescore_kernel, rsm));
   for (int64_t b0 = 0; b0 < B; b0 += Bc) {
     const int64_t nb = std::min(Bc, B - b0);
-    const unsigned gq = (unsigned)((nb + 255) / 256);
     int64_t *oi = out_ids + b0 * k;
     float *od = out_dist + b0 * k;
     {
@@ -431,11 +430,16 @@ int search_f32_certified(const adanns_index *idx, const float *queries, int64_t 
     }
     {
       StageTimer t(ST_INVERT, st);
+      ProbePlan plan;
+      plan.list_off = idx->list_off;
+      plan.qbase = qbase;
+      plan.pbase = pbase;
       if ((rc = launch_invert_probes(ckeys, nb, nprobe, nlist, QT, lcnt, lbeg, lfill, tbeg, pair_q,
                                      pair_out, tl, tb, tc, ntiles,
-                                     out_probes ? out_probes + b0 * nprobe : nullptr, st)))
+                                     out_probes ? out_probes + b0 * nprobe : nullptr, st, &plan)))
         return rc;
-      if ((rc = launch_cand_segments(ckeys, nb, nprobe, idx->list_off, qtot, qbase, pbase, st)))
+      if (!plan.planned && (rc = launch_cand_segments(ckeys, nb, nprobe, idx->list_off, qtot,
+                                                      qbase, pbase, st)))
         return rc;
     }
     {

@@ -183,7 +183,75 @@ __global__ void __launch_bounds__(CM_THREADS) coarse_topk_kernel(
   }
 }
 
+// Small batches: one CTA per query over the prefix-major centroid table, a
+// centroid per thread with the same sums, a running top-k per warp in registers
+// and the warps' lists merged in a tree.  One launch instead of the tensor-core
+// path's four (1,024 lists at d_c 32: one query 36 us against 11, 256 queries 43
+// against 14, 1,024 queries 43 against 28; 64 lists, 200 queries 21 against 5 by
+// the register top-k kernel), with 1,024 threads while there are fewer queries
+// than SMs.
+template <int NT>
+__global__ void __launch_bounds__(NT) coarse_small_kernel(
+    const float *__restrict__ cpm, int nlist, int d_c, const float *__restrict__ qc, int ldq, int k,
+    uint64_t *__restrict__ out) {
+  __shared__ __align__(16) float s_q[2048];
+  __shared__ uint64_t s_k[NT / 32][32];
+  const int64_t q = blockIdx.x;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int j = threadIdx.x; j < d_c; j += NT) s_q[j] = qc[q * ldq + j];
+  __syncthreads();
+  const int64_t bs = (int64_t)16 * nlist;
+  uint64_t best = KEY_MAX;
+  for (int c0 = warp * 32; c0 < nlist; c0 += NT) {
+    const int c = c0 + lane;
+    float acc = 0.f;
+    const float *x = cpm + (int64_t)min(c, nlist - 1) * 16;
+#pragma unroll 4
+    for (int j = 0; j < d_c; j += 8) {  // d_c is a multiple of 8
+      const float *xb = x + (j >> 4) * bs + (j & 15);
+      const float4 a = __ldg((const float4 *)xb), b = __ldg((const float4 *)(xb + 4));
+      const float4 u = *(const float4 *)&s_q[j], v = *(const float4 *)&s_q[j + 4];
+      float d;
+      d = fmaf(-1.f, a.x, u.x); acc = fmaf(d, d, acc);
+      d = fmaf(-1.f, a.y, u.y); acc = fmaf(d, d, acc);
+      d = fmaf(-1.f, a.z, u.z); acc = fmaf(d, d, acc);
+      d = fmaf(-1.f, a.w, u.w); acc = fmaf(d, d, acc);
+      d = fmaf(-1.f, b.x, v.x); acc = fmaf(d, d, acc);
+      d = fmaf(-1.f, b.y, v.y); acc = fmaf(d, d, acc);
+      d = fmaf(-1.f, b.z, v.z); acc = fmaf(d, d, acc);
+      d = fmaf(-1.f, b.w, v.w); acc = fmaf(d, d, acc);
+    }
+    topk_insert(best, c < nlist ? pack_key(acc, (uint32_t)c) : KEY_MAX, k);
+  }
+#pragma unroll
+  for (int h = NT / 64; h > 0; h >>= 1) {
+    if (warp >= h && warp < 2 * h) s_k[warp][lane] = lane < k ? best : KEY_MAX;
+    __syncthreads();
+    if (warp < h && (warp + h) * 32 < nlist) topk_insert(best, s_k[warp + h][lane], k);
+  }
+  if (warp == 0 && lane < k) out[q * k + lane] = best;
+}
+
 }  // namespace
+
+// Up to 5e7 query-centroid coordinates (1,536 queries over 1,024 lists at d_c
+// 32), where it meets the tensor-core path.  Returns 1 (nothing launched) for
+// other shapes.
+static int launch_coarse_small(const adanns_index *idx, const float *qc, int ldq, int64_t B,
+                               int d_c, int k, uint64_t *out, cudaStream_t st) {
+  if (k > CM_MAXK || idx->nlist < k || d_c > 2048 || (d_c & 7) != 0 ||
+      (double)B * idx->nlist * d_c > 5e7)
+    return 1;
+  if (B == 0) return ADANNS_OK;
+  if (B <= num_sms() && idx->nlist > CM_THREADS)
+    coarse_small_kernel<1024><<<(unsigned)B, 1024, 0, st>>>(idx->cent_pm, idx->nlist, d_c, qc, ldq,
+                                                            k, out);
+  else
+    coarse_small_kernel<CM_THREADS><<<(unsigned)B, CM_THREADS, 0, st>>>(idx->cent_pm, idx->nlist,
+                                                                        d_c, qc, ldq, k, out);
+  ADN_LAUNCH("coarse_small_kernel");
+  return ADANNS_OK;
+}
 
 // Returns 1 (nothing launched) when the shape is outside the fast path.
 int launch_coarse(const float *cent, int ldc, int nlist, int d_c, const float *qc, int ldq,
@@ -609,10 +677,12 @@ int launch_coarse_tc(const adanns_index *idx, const float *qc, int ldq, int64_t 
 
 int run_coarse(const adanns_index *idx, const float *qc, int ldq, int64_t B, int d_c, int k,
                uint64_t *out, int *counter, cudaStream_t st) {
-  int rc = launch_coarse_tc(idx, qc, ldq, B, d_c, k, out, st);
+  int rc = launch_coarse_small(idx, qc, ldq, B, d_c, k, out, st);
+  if (rc == 1) rc = launch_coarse_tc(idx, qc, ldq, B, d_c, k, out, st);
   if (rc == 1) rc = launch_coarse(idx->centroids, idx->d_c, idx->nlist, d_c, qc, ldq, B, k, out, st);
   if (rc == 1) {
     // the general scan over the prefix-major centroid table (one list)
+    ADN_CUDA(cudaMemsetAsync(counter, 0, sizeof(int), st));
     ScanArgs c{};
     c.xpm = idx->cent_pm;
     c.d_pad = idx->dc_pad;  // stored centroid width; d_c <= built d_c (IVF-D)

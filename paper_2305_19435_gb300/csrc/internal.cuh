@@ -120,19 +120,24 @@ int set_option(int opt, int64_t value);
 int64_t max_probe_members(const adanns_index *idx, int nprobe);
 
 // Stream-ordered scratch allocation from that pool on the call's stream.
+// Arrays of up to SLAB_MAX bytes are cut from slabs of SLAB bytes: a search
+// asks for some 25 arrays, and an allocation and a release by the pool cost the
+// host about a microsecond each, more than a small batch's kernels take.
 struct Scratch {
+  static constexpr size_t SLAB = 512 << 10, SLAB_MAX = 128 << 10;
   cudaStream_t st;
   void *ptrs[64];
   int n = 0;
+  char *slab = nullptr;
+  size_t left = 0;
   explicit Scratch(cudaStream_t s) : st(s) {}
+  Scratch(const Scratch &) = delete;
+  Scratch &operator=(const Scratch &) = delete;
   ~Scratch() {
     for (int i = 0; i < n; ++i) cudaFreeAsync(ptrs[i], st);
   }
-  template <class T>
-  int get(T **out, size_t count) {
+  int alloc(void **out, size_t bytes) {
     void *p = nullptr;
-    size_t bytes = count * sizeof(T);
-    if (bytes == 0) bytes = 16;
     cudaMemPool_t pool = scratch_pool();
     cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, bytes, pool, st)
                          : cudaMallocAsync(&p, bytes, st);
@@ -142,6 +147,27 @@ struct Scratch {
       return fail(ADANNS_ERR_OOM, "scratch allocation of " + std::to_string(bytes) + " bytes failed");
     }
     ptrs[n++] = p;
+    *out = p;
+    return ADANNS_OK;
+  }
+  template <class T>
+  int get(T **out, size_t count) {
+    const size_t bytes = (count * sizeof(T) + 255) & ~(size_t)255;  // the pool's alignment
+    void *p = nullptr;
+    int rc;
+    if (bytes > SLAB_MAX) {
+      if ((rc = alloc(&p, bytes))) return rc;
+    } else {
+      const size_t need = bytes ? bytes : 256;
+      if (left < need) {
+        if ((rc = alloc(&p, SLAB))) return rc;
+        slab = (char *)p;
+        left = SLAB;
+      }
+      p = slab;
+      slab += need;
+      left -= need;
+    }
     *out = (T *)p;
     return ADANNS_OK;
   }
@@ -197,18 +223,38 @@ int launch_prep_queries(const float *q, int64_t B, int ld, int dims_a, int dims_
                         const int32_t *dims_b_q = nullptr, const int32_t *rows = nullptr);
 int launch_keys_to_result(const uint64_t *keys, int64_t rows, int k, int64_t *ids, int32_t *ids32,
                           float *dist, cudaStream_t st);
+// What else is derived from a batch's probe keys along with its (list, query
+// tile) work: the work counters to clear, the candidate segments (as
+// launch_cand_segments gives them) and the streaming scan's work units.  With
+// few pairs one kernel does all of it (planned is then set); otherwise the
+// inversion clears the counters and the caller derives the rest.
+struct ProbePlan {
+  int *zero = nullptr;  // nzero work counters
+  int nzero = 0;
+  const int64_t *list_off = nullptr;  // segments: qbase [B], pbase [pairs] (or null)
+  int64_t *qbase = nullptr, *pbase = nullptr;
+  // units of unit_members members x unit_queries queries of a tile (or null):
+  // the first unit of each tile, the number of units, and optionally every
+  // unit (list, first pair, pairs, first member)
+  int unit_members = 0, unit_queries = 0;
+  int64_t *uoff = nullptr, *nunits = nullptr;
+  int4 *unit = nullptr;
+  bool planned = false;
+};
+bool probe_plan_small(int64_t pairs, int nlist);  // whether one kernel does it all
 int launch_invert_probes(const uint64_t *ckeys, int64_t B, int nprobe, int nlist, int qt,
                          int32_t *lcnt, int32_t *lbeg, int32_t *lfill, int32_t *tbeg,
                          int32_t *pair_q, int32_t *pair_out, int32_t *tile_list,
                          int32_t *tile_beg, int32_t *tile_cnt, int *ntiles, int32_t *probes_out,
-                         cudaStream_t st);
+                         cudaStream_t st, ProbePlan *plan = nullptr);
 // The same over probe slots [s0, s0 + ns) of each query only (pair_out still
 // holds the pair index q * nprobe + slot; probes_out gets those slots' lists).
 int launch_invert_probe_slots(const uint64_t *ckeys, int64_t B, int nprobe, int s0, int ns,
                               int nlist, int qt, int32_t *lcnt, int32_t *lbeg, int32_t *lfill,
                               int32_t *tbeg, int32_t *pair_q, int32_t *pair_out,
                               int32_t *tile_list, int32_t *tile_beg, int32_t *tile_cnt,
-                              int *ntiles, int32_t *probes_out, cudaStream_t st);
+                              int *ntiles, int32_t *probes_out, cudaStream_t st,
+                              ProbePlan *plan = nullptr);
 // Per-query budgets in the merge (all null: none): ckeys / nsplit mark the runs
 // of masked probe slots, kq the per-query k, orow each query's output row.
 // only: merge (and write) just the queries with only[q] < 0.
@@ -309,8 +355,8 @@ int launch_coarse(const float *cent, int ldc, int nlist, int d_c, const float *q
 // k > 32 with more than 16,384 lists.
 int launch_coarse_tc(const adanns_index *idx, const float *qc, int ldq, int64_t B, int d_c, int k,
                      uint64_t *out, cudaStream_t st);
-// Both, in order of preference, then the general scan over the prefix-major
-// centroid table (counter: the scan's work counter, zeroed by the caller).
+// The small-batch kernel, both of these, in order of preference, then the
+// general scan over the prefix-major centroid table (counter: its work counter).
 int run_coarse(const adanns_index *idx, const float *qc, int ldq, int64_t B, int d_c, int k,
                uint64_t *out, int *counter, cudaStream_t st);
 constexpr int64_t CT_SLICE_MIN = 4096;  // fewest points per tensor-core assignment slice
@@ -447,6 +493,12 @@ int launch_adc_dist(const uint8_t *codes, const int64_t *list_off, int M, const 
 int launch_select32(const uint32_t *cand, const uint64_t *ckeys, int nprobe, const int64_t *qbase,
                     const int64_t *list_off, const int32_t *list_ids, int64_t B, int kk,
                     uint64_t *out, cudaStream_t st, const int32_t *only = nullptr);
+// The same, sorted and written as results: rows of k ids and distances, from
+// the query's kq-th entry on (kq null: none) (-1, +inf)
+int launch_select32_results(const uint32_t *cand, const uint64_t *ckeys, int nprobe,
+                            const int64_t *qbase, const int64_t *list_off, const int32_t *list_ids,
+                            int64_t B, int k, const int32_t *kq, int64_t *out_ids, float *out_dist,
+                            cudaStream_t st);
 // IVF-OPQ through the certified tensor-core filter (certified_adc.cu): rows of
 // decoded codes for the scan, and the exact ADC scores of the shortlist.
 // Squared norms of every decoded code row y2 [N] and their maximum.

@@ -507,7 +507,7 @@ int search_mixed(const adanns_index *idx, const float *queries, int64_t B, int d
     m.rcnt = thr ? rcnt : nullptr;
     m.tau = thr;
     m.err = err;
-    m.tile_counter = counter + 1 + set;  // zeroed with the cluster-mapping counter
+    m.tile_counter = counter + 1 + set;  // cleared by the probe inversion
     m.fp8 = fp8;
     m.few = (double)B * nprobe <= 24.0 * nlist ? 1 : 0;
     return narrow ? launch_mma_narrow(qtile + t0 * nkb * qt * 128, ntile_cap * nkb * qt,
@@ -526,7 +526,6 @@ int search_mixed(const adanns_index *idx, const float *queries, int64_t B, int d
                                                                  qn2, qsc, qrho);
       ADN_LAUNCH("prep_lowp_kernel");
     }
-    ADN_CUDA(cudaMemsetAsync(counter, 0, 3 * sizeof(int), st));
     {
       StageTimer t(ST_COARSE, st);
       if ((rc = run_coarse(idx, qc, dcp, nb, d_c, nprobe, ckeys, counter, st))) return rc;
@@ -538,8 +537,17 @@ int search_mixed(const adanns_index *idx, const float *queries, int64_t B, int d
       // tile set 0: every slot (unfiltered) or slot 0 (filtered); tile set 1:
       // slots 1.. (filtered); pairs of set 1 follow those of set 0
       const int ns0 = filt ? 1 : nprobe;
+      ProbePlan plan;
+      plan.zero = counter + 1;
+      plan.nzero = 2;
+      if (!filt) {
+        plan.list_off = idx->list_off;
+        plan.qbase = qbase;
+        plan.pbase = pbase;
+      }
       if ((rc = launch_invert_probe_slots(ckeys, nb, nprobe, 0, ns0, nlist, qt, lcnt, lbeg, lfill,
-                                          tbeg, pair_q, pair_out, tl, tb, tc, ntiles, probes, st)))
+                                          tbeg, pair_q, pair_out, tl, tb, tc, ntiles, probes, st,
+                                          &plan)))
         return rc;
       if ((rc = launch_gather_qtiles(qlow, nkb, tiles_a, tb, tc, ntiles, pair_q, qt, qtile, st)))
         return rc;
@@ -554,7 +562,8 @@ int search_mixed(const adanns_index *idx, const float *queries, int64_t B, int d
                                        pair_q + o1, qt, qtile + tiles_a * nkb * qt * 128, st)))
           return rc;
       }
-      if ((rc = launch_cand_segments(ckeys, nb, nprobe, idx->list_off, qtot, qbase, pbase, st)))
+      if ((filt || !plan.planned) &&
+          (rc = launch_cand_segments(ckeys, nb, nprobe, idx->list_off, qtot, qbase, pbase, st)))
         return rc;
     }
     {

@@ -465,22 +465,201 @@ __global__ void probe_tiles_kernel(const int32_t *__restrict__ lcnt,
   }
 }
 
+// The whole plan of a small batch in one CTA: pairs per list counted in shared
+// memory, one scan over the lists for the first pair, tile and streaming unit
+// of each, pairs placed, tiles and units written, and one scan over the pairs'
+// padded list sizes for the candidate segments.  The chain of five to ten
+// kernels and two clears it stands for is 2 to 9 us of launch and latency each
+// (one query, 16 of 1,024 lists: 43 us in all against 11; 1,024 pairs 50 against
+// 31); above PP_MAXN pairs their grids are the faster ones (16,336 pairs: 63
+// against 92).
+constexpr int PP_THREADS = 1024;
+constexpr int PP_MAXN = 8192, PP_MAXL = 4096, PP_EACH = PP_MAXN / PP_THREADS;
+
+// inclusive scan of v over the block (64-bit sums); s_w: 32 shared values
+__device__ __forceinline__ uint64_t block_scan64(uint64_t v, uint64_t *s_w) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
+  }
+  __syncthreads();  // s_w may still be read from a scan before
+  if (lane == 31) s_w[warp] = v;
+  __syncthreads();
+  if (warp == 0) {
+    uint64_t w = s_w[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint64_t y = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += y;
+    }
+    s_w[lane] = w;
+  }
+  __syncthreads();
+  return v + (warp ? s_w[warp - 1] : 0ull);
+}
+
+__global__ void __launch_bounds__(PP_THREADS) probe_plan_kernel(
+    const uint64_t *__restrict__ ckeys, int n, int nprobe, int s0, int ns, int nlist, int qt,
+    int32_t *__restrict__ lcnt, int32_t *__restrict__ pair_q, int32_t *__restrict__ pair_out,
+    int32_t *__restrict__ tile_list, int32_t *__restrict__ tile_beg,
+    int32_t *__restrict__ tile_cnt, int *__restrict__ ntiles, int32_t *__restrict__ probes_out,
+    ProbePlan p) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  int64_t *s_u = (int64_t *)smem;          // [nlist] first unit
+  int *s_cnt = (int *)(s_u + nlist);       // [nlist] pairs
+  int *s_pos = s_cnt + nlist;              // [nlist] next pair
+  int *s_pad = s_pos + nlist;              // [nlist] padded size
+  int *s_tb = s_pad + nlist;               // [nlist + 1] first tile
+  __shared__ int s_l[PP_MAXN];             // every pair's list
+  __shared__ uint64_t s_w[32];
+  const int tid = threadIdx.x;
+  if (tid < p.nzero) p.zero[tid] = 0;
+  int lst[PP_EACH];  // the lists of pairs tid, tid + PP_THREADS, ..., all loads in flight
+#pragma unroll
+  for (int u = 0; u < PP_EACH; ++u) {
+    const int i = tid + u * PP_THREADS;
+    lst[u] = i < n ? probe_list(ckeys[slot_pair(i, nprobe, s0, ns)]) : -1;
+  }
+  for (int l = tid; l < nlist; l += PP_THREADS) {
+    s_cnt[l] = 0;
+    s_pad[l] = p.list_off ? (int)((p.list_off[l + 1] - p.list_off[l] + 7) & ~7ll) : 0;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < PP_EACH; ++u) {
+    const int i = tid + u * PP_THREADS;
+    if (i >= n) break;
+    s_l[i] = lst[u];
+    if (probes_out) probes_out[slot_pair(i, nprobe, s0, ns)] = lst[u];
+    if (lst[u] >= 0) atomicAdd(&s_cnt[lst[u]], 1);
+  }
+  __syncthreads();
+  // a thread scans `per` consecutive lists: pairs and tiles in one word, units
+  const int per = (nlist + PP_THREADS - 1) / PP_THREADS;
+  const int l0 = min(nlist, tid * per), l1 = min(nlist, l0 + per);
+  auto units_of = [&](int l) -> int64_t {
+    const int c = s_cnt[l];
+    if (c == 0 || !p.uoff) return 0;
+    const int full = c / qt, rest = c - full * qt, uq = p.unit_queries;
+    return (int64_t)((s_pad[l] + p.unit_members - 1) / p.unit_members) *
+           (full * ((qt + uq - 1) / uq) + (rest + uq - 1) / uq);
+  };
+  uint64_t ct = 0;
+  int64_t us = 0;
+  for (int l = l0; l < l1; ++l) {
+    const int c = s_cnt[l];
+    ct += ((uint64_t)(uint32_t)c << 32) | (uint32_t)((c + qt - 1) / qt);
+    us += units_of(l);
+  }
+  const uint64_t cti = block_scan64(ct, s_w);
+  const int64_t usi = p.uoff ? (int64_t)block_scan64((uint64_t)us, s_w) : 0;
+  {
+    uint64_t run = cti - ct;
+    int64_t u = usi - us;
+    for (int l = l0; l < l1; ++l) {
+      const int c = s_cnt[l];
+      lcnt[l] = c;
+      s_pos[l] = (int)(run >> 32);
+      s_tb[l] = (int)(uint32_t)run;
+      s_u[l] = u;
+      run += ((uint64_t)(uint32_t)c << 32) | (uint32_t)((c + qt - 1) / qt);
+      u += units_of(l);
+    }
+  }
+  if (tid == PP_THREADS - 1) {
+    s_tb[nlist] = (int)(uint32_t)cti;
+    *ntiles = (int)(uint32_t)cti;
+    if (p.uoff) *p.nunits = usi;
+  }
+  __syncthreads();
+  // tiles and their units: a tile's list is the last one whose first tile is at
+  // or before it (lists without pairs have no tile).  A thread per tile, or a
+  // warp while there are few (their units are then written together).
+  const int nt = s_tb[nlist], grp = nt < 64 ? 32 : 1, lane = tid & (grp - 1);
+  for (int t = tid / grp; t < nt; t += PP_THREADS / grp) {
+    int lo = 0, hi = nlist - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (s_tb[mid] <= t) lo = mid; else hi = mid - 1;
+    }
+    const int k = t - s_tb[lo], c = s_cnt[lo], beg = s_pos[lo] + k * qt, cnt = min(qt, c - k * qt);
+    if (lane == 0) {
+      tile_list[t] = lo;
+      tile_beg[t] = beg;
+      tile_cnt[t] = cnt;
+    }
+    if (p.uoff) {
+      const int uq = p.unit_queries, um = p.unit_members, nch = (s_pad[lo] + um - 1) / um;
+      const int64_t u0 = s_u[lo] + (int64_t)k * nch * ((qt + uq - 1) / uq);
+      if (lane == 0) p.uoff[t] = u0;
+      if (p.unit) {
+        const int ng = (cnt + uq - 1) / uq;
+        for (int u = lane; u < nch * ng; u += grp) {
+          const int ch = u / ng, g = u - ch * ng;
+          p.unit[u0 + u] = make_int4(lo, beg + g * uq, min(uq, cnt - g * uq), ch * um);
+        }
+      }
+    }
+  }
+  __syncthreads();  // s_pos becomes the pairs' cursor
+#pragma unroll
+  for (int u = 0; u < PP_EACH; ++u) {
+    if (lst[u] < 0) continue;  // past the end, or a masked slot: no pair
+    const int64_t e = slot_pair(tid + u * PP_THREADS, nprobe, s0, ns);
+    const int pos = atomicAdd(&s_pos[lst[u]], 1);
+    pair_q[pos] = (int32_t)(e / nprobe);
+    pair_out[pos] = (int32_t)e;
+  }
+  if (p.pbase) {  // candidate segments: pairs laid end to end in (query, slot) order
+    const int pp = (n + PP_THREADS - 1) / PP_THREADS, i0 = min(n, tid * pp), i1 = min(n, i0 + pp);
+    int64_t sum = 0;
+    for (int i = i0; i < i1; ++i) sum += s_l[i] >= 0 ? s_pad[s_l[i]] : 0;
+    int64_t run = (int64_t)block_scan64((uint64_t)sum, s_w) - sum;
+    for (int i = i0; i < i1; ++i) {
+      p.pbase[i] = run;
+      if (i % nprobe == 0) p.qbase[i / nprobe] = run;
+      run += s_l[i] >= 0 ? s_pad[s_l[i]] : 0;
+    }
+  }
+}
+
+bool probe_plan_small(int64_t pairs, int nlist) {
+  return pairs >= 1 && pairs <= PP_MAXN && nlist <= PP_MAXL;
+}
+
 int launch_invert_probes(const uint64_t *ckeys, int64_t B, int nprobe, int nlist, int qt,
                          int32_t *lcnt, int32_t *lbeg, int32_t *lfill, int32_t *tbeg,
                          int32_t *pair_q, int32_t *pair_out, int32_t *tile_list,
                          int32_t *tile_beg, int32_t *tile_cnt, int *ntiles, int32_t *probes_out,
-                         cudaStream_t st) {
+                         cudaStream_t st, ProbePlan *plan) {
   return launch_invert_probe_slots(ckeys, B, nprobe, 0, nprobe, nlist, qt, lcnt, lbeg, lfill, tbeg,
                                    pair_q, pair_out, tile_list, tile_beg, tile_cnt, ntiles,
-                                   probes_out, st);
+                                   probes_out, st, plan);
 }
 
 int launch_invert_probe_slots(const uint64_t *ckeys, int64_t B, int nprobe, int s0, int ns,
                               int nlist, int qt, int32_t *lcnt, int32_t *lbeg, int32_t *lfill,
                               int32_t *tbeg, int32_t *pair_q, int32_t *pair_out,
                               int32_t *tile_list, int32_t *tile_beg, int32_t *tile_cnt,
-                              int *ntiles, int32_t *probes_out, cudaStream_t st) {
+                              int *ntiles, int32_t *probes_out, cudaStream_t st,
+                              ProbePlan *plan) {
   const int64_t n = B * ns;
+  if (probe_plan_small(n, nlist)) {
+    ProbePlan p = plan ? *plan : ProbePlan{};
+    if (p.pbase && ns != nprobe) return fail(ADANNS_ERR_ARG, "segments need every probe slot");
+    const size_t sm = (size_t)nlist * 24 + 16;
+    ADN_CUDA(ensure_smem((const void *)probe_plan_kernel, sm));
+    probe_plan_kernel<<<1, PP_THREADS, sm, st>>>(ckeys, (int)n, nprobe, s0, ns, nlist, qt, lcnt,
+                                                 pair_q, pair_out, tile_list, tile_beg, tile_cnt,
+                                                 ntiles, probes_out, p);
+    ADN_LAUNCH("probe_plan_kernel");
+    if (plan) plan->planned = true;
+    return ADANNS_OK;
+  }
+  if (plan && plan->nzero)
+    ADN_CUDA(cudaMemsetAsync(plan->zero, 0, sizeof(int) * plan->nzero, st));
   ADN_CUDA(cudaMemsetAsync(lcnt, 0, sizeof(int32_t) * nlist, st));
   ADN_CUDA(cudaMemsetAsync(lfill, 0, sizeof(int32_t) * nlist, st));
   const unsigned g = (unsigned)((std::max<int64_t>(n, 1) + 255) / 256);

@@ -51,6 +51,7 @@ struct StreamArgs {
   const int *ntiles_dev;
   const int64_t *uoff;  // first work unit of each tile (exclusive scan of its units)
   const int64_t *nunits;
+  const int4 *unit;     // dist_f32_few_kernel: the units themselves
   const int32_t *pair_q, *pair_out;
   const int64_t *pbase;  // candidate segment start of each (query, probe) pair
   uint32_t *cand;
@@ -280,6 +281,102 @@ __global__ void __launch_bounds__(SF_THREADS, 4) dist_f32_kernel(StreamArgs a) {
   }
 }
 
+// Small batches, whose members in flight would not fill the GPU one 64-byte
+// block ahead (80 CTAs of one query over 16 lists): units of 64 members and
+// SFF_PF blocks of a row in flight per thread, from the plan's unit table (no
+// search for the tile), the unit's query rows staged in shared memory beside
+// the first blocks.  The sums are those above.  One query, 16 lists of
+// about 1,250 at d_s 512: 59 us with its units' two kernels before, 18 here.
+constexpr int SFF_THREADS = 64, SFF_PF = 6;
+
+template <bool VAR>
+__global__ void __launch_bounds__(SFF_THREADS) dist_f32_few_kernel(StreamArgs a) {
+  extern __shared__ __align__(16) float s_q[];  // [SF_QG][dims]
+  const int64_t nunits = *a.nunits;
+  for (int64_t item = blockIdx.x; item < nunits; item += gridDim.x) {
+    const int4 un = a.unit[item];  // (list, first pair, pairs, first member)
+    const int cnt = un.z, m = un.w + threadIdx.x, nq4 = a.dims >> 2;
+    const float *sp[SF_QG];
+    int64_t pb[SF_QG];
+    int ds[SF_QG], dmax = VAR ? 0 : a.dims;
+    __syncthreads();  // the previous unit's queries are no longer read
+#pragma unroll
+    for (int j = 0; j < SF_QG; ++j) {
+      const int pr = un.y + min(j, cnt - 1), q = a.pair_q[pr];
+      if (j < cnt) {
+        const float4 *src = (const float4 *)(a.qn + (int64_t)q * a.ldq);
+        for (int t = threadIdx.x; t < nq4; t += SFF_THREADS)
+          cp_async16(s_q + 4 * (j * nq4 + t), src + t);
+      }
+      pb[j] = a.pbase[a.pair_out[pr]];
+      ds[j] = VAR ? a.qds[q] : a.dims;
+      sp[j] = VAR ? (a.invn ? a.invn + (int64_t)a.qgi[q] * a.N : nullptr) : a.mscale;
+      if (VAR) dmax = max(dmax, ds[j]);
+    }
+    cp_async_commit();
+    const int64_t moff = a.list_off[un.x];
+    const int nl = (int)(a.list_off[un.x + 1] - moff), npad = (nl + 7) & ~7;
+    const int nblk = (dmax + 15) >> 4;
+    const float *xr = a.xpm + moff * (int64_t)a.d_pad + (int64_t)m * 16;
+    const int64_t bstride = (int64_t)16 * nl;
+    float4 x[SFF_PF][4];
+#pragma unroll
+    for (int b = 0; b < SFF_PF; ++b)
+      if (m < nl && b < nblk) {
+#pragma unroll
+        for (int s = 0; s < 4; ++s) x[b][s] = ldg4(xr + b * bstride + 4 * s);
+      }
+    float sc[SF_QG], acc[SF_QG];
+#pragma unroll
+    for (int j = 0; j < SF_QG; ++j) {
+      sc[j] = m < nl && sp[j] ? __ldg(sp[j] + moff + m) : 1.f;
+      acc[j] = 0.f;
+    }
+    cp_async_wait<0>();
+    __syncthreads();  // the queries are staged
+    if (m < nl) {
+      for (int b0 = 0; b0 < nblk; b0 += SFF_PF) {
+#pragma unroll
+        for (int b = 0; b < SFF_PF; ++b) {
+          if (b0 + b >= nblk) break;
+          const int off = 16 * (b0 + b);
+#pragma unroll
+          for (int j = 0; j < SF_QG; ++j) {
+            if (j >= cnt) break;
+            const int nd4 = (ds[j] - off) >> 2;
+            const float4 *qb = (const float4 *)s_q + j * nq4 + (off >> 2);
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+              if (s >= nd4) break;
+              const float4 q = qb[s];
+              float t;
+              t = fmaf(-sc[j], x[b][s].x, q.x);
+              acc[j] = fmaf(t, t, acc[j]);
+              t = fmaf(-sc[j], x[b][s].y, q.y);
+              acc[j] = fmaf(t, t, acc[j]);
+              t = fmaf(-sc[j], x[b][s].z, q.z);
+              acc[j] = fmaf(t, t, acc[j]);
+              t = fmaf(-sc[j], x[b][s].w, q.w);
+              acc[j] = fmaf(t, t, acc[j]);
+            }
+          }
+          if (b0 + b + SFF_PF < nblk) {
+#pragma unroll
+            for (int s = 0; s < 4; ++s) x[b][s] = ldg4(xr + (b0 + b + SFF_PF) * bstride + 4 * s);
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < SF_QG; ++j)
+        if (j < cnt) a.cand[pb[j] + m] = __float_as_uint(acc[j]);
+    } else if (m < npad) {
+#pragma unroll
+      for (int j = 0; j < SF_QG; ++j)
+        if (j < cnt) a.cand[pb[j] + m] = 0xFFFFFFFFu;
+    }
+  }
+}
+
 }  // namespace
 
 // Few queries per probed list: prefer the streaming scan (ADANNS_OPT_FP32_STREAM = 0
@@ -301,9 +398,17 @@ int search_f32_stream(const adanns_index *idx, const float *queries, int64_t B, 
       seg_q * 4 + (int64_t)(dcp + dsp) * 4 + (int64_t)k * 8 + (int64_t)nprobe * 40 + 16;
   const int64_t Bc = std::max<int64_t>(1, std::min<int64_t>(B, scratch_budget() / per_q));
   const int64_t max_tiles = (Bc * nprobe + SF_QT - 1) / SF_QT + nlist;
+  // few members in all: small units (the whole batch is then one slice)
+  // (a unit per 64 members of each probed list and group of queries at most)
+  const int64_t max_units =
+      B * nprobe * (((int64_t)idx->max_list + 7 + SFF_THREADS) / SFF_THREADS);
+  const bool few = Bc >= B && probe_plan_small(B * nprobe, nlist) && max_units <= 1 << 20 &&
+                   (double)B * nprobe * idx->N / nlist <= (double)num_sms() * 1024;
+  const int um = few ? SFF_THREADS : SF_THREADS;
   Scratch s(st);
   float *qc, *qs;
-  uint64_t *ckeys, *keys;
+  uint64_t *ckeys;
+  int4 *unit = nullptr;
   uint32_t *cand;
   int64_t *qtot, *qbase, *pbase, *units, *uoff, *nunits;
   int32_t *lcnt, *lbeg, *lfill, *tbeg, *pair_q, *pair_out, *tl, *tb, *tc;
@@ -311,14 +416,15 @@ int search_f32_stream(const adanns_index *idx, const float *queries, int64_t B, 
   int rc;
   if ((rc = s.get(&qc, (size_t)Bc * dcp)) || (rc = s.get(&qs, (size_t)Bc * dsp)) ||
       (rc = s.get(&ckeys, (size_t)Bc * nprobe)) || (rc = s.get(&cand, (size_t)(Bc * seg_q))) ||
-      (rc = s.get(&keys, (size_t)Bc * k)) || (rc = s.get(&qtot, (size_t)Bc)) ||
+      (rc = s.get(&qtot, (size_t)Bc)) ||
       (rc = s.get(&qbase, (size_t)Bc)) || (rc = s.get(&pbase, (size_t)Bc * nprobe)) ||
       (rc = s.get(&lcnt, nlist)) || (rc = s.get(&lbeg, nlist)) || (rc = s.get(&lfill, nlist)) ||
       (rc = s.get(&tbeg, nlist)) || (rc = s.get(&pair_q, (size_t)Bc * nprobe)) ||
       (rc = s.get(&pair_out, (size_t)Bc * nprobe)) || (rc = s.get(&tl, max_tiles)) ||
       (rc = s.get(&tb, max_tiles)) || (rc = s.get(&tc, max_tiles)) || (rc = s.get(&ntiles, 1)) ||
       (rc = s.get(&counter, 2)) || (rc = s.get(&units, max_tiles)) ||
-      (rc = s.get(&uoff, max_tiles)) || (rc = s.get(&nunits, 1)))
+      (rc = s.get(&uoff, max_tiles)) || (rc = s.get(&nunits, 1)) ||
+      (few && (rc = s.get(&unit, (size_t)max_units))))
     return rc;
   const float *mscale = idx->metric == ADANNS_METRIC_L2_PREFIXNORM
                             ? idx->invn + (int64_t)gran_index(d_s) * idx->N
@@ -332,27 +438,40 @@ int search_f32_stream(const adanns_index *idx, const float *queries, int64_t B, 
                                     dcp, qs, dsp, st, bq.ds)))
         return rc;
     }
-    ADN_CUDA(cudaMemsetAsync(counter, 0, 2 * sizeof(int), st));
     {
       StageTimer t(ST_COARSE, st);
       if ((rc = run_coarse(idx, qc, dcp, nb, d_c, nprobe, ckeys, counter, st))) return rc;
       if ((rc = launch_mask_probes(ckeys, nb, nprobe, bq.np, st))) return rc;
     }
+    ProbePlan plan;
     {
       StageTimer t(ST_INVERT, st);
+      plan.zero = counter + 1;
+      plan.nzero = 1;
+      plan.list_off = idx->list_off;
+      plan.qbase = qbase;
+      plan.pbase = pbase;
+      plan.unit_members = um;
+      plan.unit_queries = SF_QG;
+      plan.uoff = uoff;
+      plan.nunits = nunits;
+      plan.unit = unit;
       if ((rc = launch_invert_probes(ckeys, nb, nprobe, nlist, SF_QT, lcnt, lbeg, lfill, tbeg,
                                      pair_q, pair_out, tl, tb, tc, ntiles,
-                                     out_probes ? out_probes + b0 * nprobe : nullptr, st)))
+                                     out_probes ? out_probes + b0 * nprobe : nullptr, st, &plan)))
         return rc;
-      if ((rc = launch_cand_segments(ckeys, nb, nprobe, idx->list_off, qtot, qbase, pbase, st)))
+      if (!plan.planned && (rc = launch_cand_segments(ckeys, nb, nprobe, idx->list_off, qtot,
+                                                      qbase, pbase, st)))
         return rc;
     }
     {
       StageTimer t(ST_SCAN, st);
-      stream_units_kernel<<<(unsigned)((max_tiles + 255) / 256), 256, 0, st>>>(
-          tl, tc, ntiles, idx->list_off, max_tiles, units);
-      ADN_LAUNCH("stream_units_kernel");
-      if ((rc = launch_scan64(units, max_tiles, uoff, nunits, st))) return rc;
+      if (!plan.planned) {
+        stream_units_kernel<<<(unsigned)((max_tiles + 255) / 256), 256, 0, st>>>(
+            tl, tc, ntiles, idx->list_off, max_tiles, units);
+        ADN_LAUNCH("stream_units_kernel");
+        if ((rc = launch_scan64(units, max_tiles, uoff, nunits, st))) return rc;
+      }
       StreamArgs a{};
       a.xpm = idx->xpm;
       a.d_pad = idx->d_pad;
@@ -367,6 +486,7 @@ int search_f32_stream(const adanns_index *idx, const float *queries, int64_t B, 
       a.ntiles_dev = ntiles;
       a.uoff = uoff;
       a.nunits = nunits;
+      a.unit = unit;
       a.pair_q = pair_q;
       a.pair_out = pair_out;
       a.pbase = pbase;
@@ -376,25 +496,34 @@ int search_f32_stream(const adanns_index *idx, const float *queries, int64_t B, 
       a.qgi = bq.gi;
       a.invn = idx->metric == ADANNS_METRIC_L2_PREFIXNORM ? idx->invn : nullptr;
       a.N = idx->N;
-      auto kern = bq.ds ? dist_f32_var_kernel : dist_f32_kernel;
-      int per_sm = 1;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SF_THREADS, 0) !=
-              cudaSuccess ||
-          per_sm < 1) {
-        cudaGetLastError();
-        per_sm = 1;
+      if (few) {
+        // about as many CTAs as units if no query shared a list
+        const int64_t est = nb * nprobe * (idx->N / nlist / SFF_THREADS + 1);
+        const unsigned grid =
+            (unsigned)std::min<int64_t>(std::min(max_units, est), (int64_t)num_sms() * 16);
+        const size_t sm = (size_t)SF_QG * d_s * 4;
+        auto kern = bq.ds ? dist_f32_few_kernel<true> : dist_f32_few_kernel<false>;
+        ADN_CUDA(ensure_smem((const void *)kern, sm));
+        kern<<<grid, SFF_THREADS, sm, st>>>(a);
+        ADN_LAUNCH("dist_f32_few_kernel");
+      } else {
+        auto kern = bq.ds ? dist_f32_var_kernel : dist_f32_kernel;
+        int per_sm = 1;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SF_THREADS, 0) !=
+                cudaSuccess ||
+            per_sm < 1) {
+          cudaGetLastError();
+          per_sm = 1;
+        }
+        kern<<<num_sms() * per_sm, SF_THREADS, 0, st>>>(a);
+        ADN_LAUNCH(bq.ds ? "dist_f32_var_kernel" : "dist_f32_kernel");
       }
-      kern<<<num_sms() * per_sm, SF_THREADS, 0, st>>>(a);
-      ADN_LAUNCH(bq.ds ? "dist_f32_var_kernel" : "dist_f32_kernel");
     }
     {
       StageTimer t(ST_MERGE, st);
-      if ((rc = launch_select32(cand, ckeys, nprobe, qbase, idx->list_off, idx->list_ids, nb, k,
-                                keys, st)))
+      if ((rc = launch_select32_results(cand, ckeys, nprobe, qbase, idx->list_off, idx->list_ids,
+                                        nb, k, bq.k, out_ids + b0 * k, out_dist + b0 * k, st)))
         return rc;
-      if ((rc = launch_final_topk(keys, k, nb, k, out_ids + b0 * k, out_dist + b0 * k, st)))
-        return rc;
-      if ((rc = launch_pad_rows(out_ids + b0 * k, out_dist + b0 * k, nb, k, bq.k, st))) return rc;
     }
   }
   return ADANNS_OK;
