@@ -51,22 +51,6 @@ __device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
 __device__ __forceinline__ uint64_t umin64(uint64_t a, uint64_t b) { return a < b ? a : b; }
 __device__ __forceinline__ uint64_t umax64(uint64_t a, uint64_t b) { return a < b ? b : a; }
 
-// ascending bitonic sort of one key per lane across the warp (shuffles only)
-__device__ __forceinline__ uint64_t warp_sort32(uint64_t v) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int size = 2; size <= 32; size <<= 1) {
-#pragma unroll
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      const uint64_t o = __shfl_xor_sync(0xffffffffu, v, stride);
-      const bool up = (lane & size) == 0;        // direction of this lane's sequence
-      const bool lower = (lane & stride) == 0;   // this lane holds the smaller position
-      v = (lower == up) ? umin64(o, v) : umax64(o, v);
-    }
-  }
-  return v;
-}
-
 // lst: the 32 smallest keys so far, ascending across the lanes.  Adds the
 // warp's candidate keys c (one per lane) that beat the k-th entry.
 __device__ __forceinline__ void topk_insert(uint64_t &lst, uint64_t c, int k) {
@@ -78,7 +62,7 @@ __device__ __forceinline__ void topk_insert(uint64_t &lst, uint64_t c, int k) {
   if (__popc(m) > 4) {
     // sort the survivors, reverse them, keep the lane-wise minimum (the 32
     // smallest of both, as a bitonic sequence) and clean it to ascending order
-    uint64_t s = warp_sort32(take ? c : KEY_MAX);
+    uint64_t s = warp_sort_lane(take ? c : KEY_MAX);
     s = __shfl_sync(0xffffffffu, s, 31 - lane);
     uint64_t v = umin64(lst, s);
 #pragma unroll

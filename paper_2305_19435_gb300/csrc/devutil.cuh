@@ -220,6 +220,22 @@ __device__ __forceinline__ void warp_sort(uint64_t *a, int n) {
   }
 }
 
+// ascending bitonic sort of one key per lane across the warp (shuffles only)
+__device__ __forceinline__ uint64_t warp_sort_lane(uint64_t v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int size = 2; size <= 32; size <<= 1) {
+#pragma unroll
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      const uint64_t o = __shfl_xor_sync(0xffffffffu, v, stride);
+      const bool up = (lane & size) == 0;        // direction of this lane's sequence
+      const bool lower = (lane & stride) == 0;   // this lane holds the smaller position
+      v = (lower == up) == (o < v) ? o : v;  // the smaller where lower == up, else the larger
+    }
+  }
+  return v;
+}
+
 // Ascending bitonic sort of 32 J keys held J per lane (lane l holds positions
 // J l .. J l + J - 1): strides below J compare within a lane, larger ones across
 // lanes by shuffles; the direction of each compare-exchange is that of the
