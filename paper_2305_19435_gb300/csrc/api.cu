@@ -146,7 +146,8 @@ int nearest_centroid(const float *cent, int nc, int dim, int metric, const float
     shell.cent_pm = const_cast<float *>(cent_pm);
     shell.cent_off = const_cast<int64_t *>(cent_off);
     shell.dev_err = err;
-    int rc = build_centroid_lowp(&shell, st);
+    Scratch table(st);
+    int rc = scratch_centroid_lowp(table, &shell, st);
     if (rc == ADANNS_OK) {
       // slices keep the 2-byte keys of (point, centroid) pairs near 1 GiB
       const int64_t rows = std::max<int64_t>(CT_SLICE_MIN, (1ll << 29) / ((nc + 7) & ~7));
@@ -154,10 +155,6 @@ int nearest_centroid(const float *cent, int nc, int dim, int metric, const float
         rc = launch_coarse_tc(&shell, pts + i0 * ldq, ldq, std::min(rows, n - i0), dim, 1,
                               keys + i0, st);
     }
-    cudaStreamSynchronize(st);  // the table copies are released below
-    cudaFree(shell.cent_low);
-    cudaFree(shell.cent_sc);
-    cudaFree(shell.cent_n2);
     if (rc != 1) return rc;  // 1: the shape does not fit the tensor-core path
   }
   return top1_sweep(pts, n, ldq, cent_pm, cent_off, nc, dim, keys, counter, st);

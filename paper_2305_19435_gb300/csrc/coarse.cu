@@ -326,44 +326,54 @@ __global__ void centroid_lowp_kernel(const float *__restrict__ cent, int d_c, in
   if (lane == 0) atomicMax((int *)maxnorm, __float_as_int(sqrtf(xpre)));
 }
 
-// query rows P_dc(q) (FP32, zero beyond d_c) -> BF16 tensor-core tiles
-// [tile][kb][128 rows][64], the squared norm, the scale and the residual norm
-__global__ void coarse_prep_kernel(const float *__restrict__ qc, int ldq, int64_t B, int d_c,
-                                   int nkb, int64_t rows, __nv_bfloat16 *__restrict__ tiles,
-                                   float *__restrict__ qn2, float *__restrict__ qsc,
-                                   float *__restrict__ qrho) {
-  const int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (q >= rows) return;
-  const int64_t t = q / CT_BM, r = q - t * CT_BM;
-  const bool valid = q < B;
-  const float *src = qc + q * ldq;
+// query rows P_dc(q) (FP32, d_c a multiple of 8 up to 64, zero beyond) -> BF16
+// tensor-core tiles [tile][128 rows][64], the squared norm, the scale and the
+// residual norm.  Eight lanes per query, eight consecutive coordinates each
+// (262,144 queries at d_c 32: 70 us with a warp per query, 15 here).
+__global__ void __launch_bounds__(256) coarse_prep_kernel(
+    const float *__restrict__ qc, int ldq, int64_t B, int d_c, int64_t rows,
+    __nv_bfloat16 *__restrict__ tiles, float *__restrict__ qn2, float *__restrict__ qsc,
+    float *__restrict__ qrho) {
+  const int64_t q = (int64_t)blockIdx.x * 32 + (threadIdx.x >> 3);
+  const int g = threadIdx.x & 7;
+  if (q >= rows) return;  // rows is a multiple of 128: whole groups of lanes
+  float v[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) v[u] = 0.f;
+  if (q < B && 8 * g < d_c) {
+    const float4 *src = (const float4 *)(qc + q * ldq + 8 * g);
+    const float4 a = __ldg(src), b = __ldg(src + 1);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  }
   float s2 = 0.f, mx = 0.f;
-  if (valid)
-    for (int j = lane; j < d_c; j += 32) {
-      const float v = src[j];
-      s2 = fmaf(v, v, s2);
-      mx = fmaxf(mx, fabsf(v));
-    }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  for (int u = 0; u < 8; ++u) {
+    s2 = fmaf(v[u], v[u], s2);
+    mx = fmaxf(mx, fabsf(v[u]));
   }
-  const float s = mx > 0.f ? mx : 1.f;
+  const unsigned grp = 0xFFu << (threadIdx.x & 24);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+    s2 += __shfl_xor_sync(grp, s2, o);
+    mx = fmaxf(mx, __shfl_xor_sync(grp, mx, o));
+  }
+  const float s = mx > 0.f ? mx : 1.f, inv = 1.f / s;
   float r2 = 0.f;
-  for (int j = lane; j < nkb * 64; j += 32) {
-    const float v = (valid && j < d_c) ? src[j] / s : 0.f;
-    const __nv_bfloat16 b = __float2bfloat16_rn(v);
-    tiles[((t * nkb + (j >> 6)) * CT_BM + r) * 64 + (j & 63)] = b;
-    if (valid && j < d_c) {
-      const float e = fmaf(-s, __bfloat162float(b), src[j]);
-      r2 = fmaf(e, e, r2);
-    }
-  }
+  uint32_t w[4];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
-  if (valid && lane == 0) {
+  for (int u = 0; u < 8; u += 2) {
+    const __nv_bfloat162 h =
+        __halves2bfloat162(__float2bfloat16_rn(v[u] * inv), __float2bfloat16_rn(v[u + 1] * inv));
+    w[u >> 1] = *(const uint32_t *)&h;
+    const float e0 = fmaf(-s, __low2float(h), v[u]), e1 = fmaf(-s, __high2float(h), v[u + 1]);
+    r2 = fmaf(e0, e0, r2);
+    r2 = fmaf(e1, e1, r2);
+  }
+  *(uint4 *)(tiles + q * 64 + 8 * g) = make_uint4(w[0], w[1], w[2], w[3]);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) r2 += __shfl_xor_sync(grp, r2, o);
+  if (q < B && g == 0) {
     qn2[q] = s2;
     qsc[q] = s;
     qrho[q] = sqrtf(r2);
@@ -392,6 +402,95 @@ __global__ void coarse_tiles_kernel(int64_t B, int ntiles, int64_t npad, int32_t
   }
 }
 
+// The largest residual of the centroids' BF16 copies at the mapping's prefix and
+// the largest centroid norm: known on the host (an index), or still on the
+// device (the assignment step's own table).
+struct CentBound {
+  float r, c;
+  const float *rd, *cd;  // or null
+  __device__ float rmax() const { return rd ? *rd * 1.001f : r; }
+  __device__ float cmax() const { return cd ? *cd * 1.001f : c; }
+};
+
+// |q - c|^2 of centroid c in the prefix-major table (16-byte loads; d_c a
+// multiple of 8, q 16-byte aligned): the FP32 kernels' sums
+__device__ __forceinline__ float centroid_dist(const float *__restrict__ cpm, int nlist, int c,
+                                               const float *q, int d_c) {
+  float acc = 0.f;
+#pragma unroll 8
+  for (int t = 0; t < d_c; t += 4) {
+    const float4 x =
+        __ldg((const float4 *)(cpm + (int64_t)(t >> 4) * 16 * nlist + (int64_t)c * 16 + (t & 15)));
+    const float4 p = *(const float4 *)(q + t);
+    float d;
+    d = fmaf(-1.f, x.x, p.x); acc = fmaf(d, d, acc);
+    d = fmaf(-1.f, x.y, p.y); acc = fmaf(d, d, acc);
+    d = fmaf(-1.f, x.z, p.z); acc = fmaf(d, d, acc);
+    d = fmaf(-1.f, x.w, p.w); acc = fmaf(d, d, acc);
+  }
+  return acc;
+}
+
+// k = 1 over at most 256 NV centroids (the assignment step): a warp holds its
+// query's key row in registers (NV 16-byte loads per lane, all in flight), takes
+// its minimum, and scores every centroid within the bound of it exactly, the
+// lanes' candidates side by side.  Bound by reading the keys (262,144 points,
+// 1,024 centroids, 0.54 GB: 321 us with coarse_pick_kernel, 157 here).
+template <int NV>
+__global__ void __launch_bounds__(256) coarse_nearest_kernel(
+    const uint16_t *__restrict__ keys, int64_t npad, int nlist, const float *__restrict__ qc,
+    int ldq, int d_c, const float *__restrict__ cpm, const float *__restrict__ qrho,
+    CentBound bound, float e_rest, int64_t B, uint64_t *__restrict__ out) {
+  const int64_t q = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (q >= B) return;
+  const uint4 *kq = (const uint4 *)(keys + q * npad);  // npad is a multiple of 8
+  const int nvec = (int)(npad >> 3);
+  uint4 v[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i)
+    v[i] = lane + 32 * i < nvec ? __ldg(kq + lane + 32 * i)
+                                : make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+  const float rq = qrho[q], rmax = bound.rmax(), cmax = bound.cmax();
+  // key e of word w of group i belongs to centroid 8 (lane + 32 i) + 2 w + e;
+  // the padding's keys are the largest
+  uint32_t mn = 0xFFFFu;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) mn = min(mn, min(w[j] & 0xFFFFu, w[j] >> 16));
+  }
+  mn = __reduce_min_sync(0xffffffffu, mn);
+  const uint32_t thr =
+      mn + (uint32_t)key_margin(2.f * (rmax + rq * cmax + rmax * rq) * (1.f + 1e-3f) + e_rest);
+  uint64_t best = KEY_MAX;
+#pragma unroll 1
+  for (int i = 0; i < NV; ++i) {
+    uint32_t in = 0;
+#pragma unroll
+    for (int t = 0; t < NV; ++t)
+      if (t == i) {
+        const uint32_t w[4] = {v[t].x, v[t].y, v[t].z, v[t].w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          in |= ((w[j] & 0xFFFFu) <= thr ? 1u : 0u) << (2 * j);
+          in |= ((w[j] >> 16) <= thr ? 1u : 0u) << (2 * j + 1);
+        }
+      }
+    while (in) {
+      const int c = 8 * (lane + 32 * i) + __ffs(in) - 1;
+      in &= in - 1;
+      if (c >= nlist) break;
+      const uint64_t key =
+          pack_key(centroid_dist(cpm, nlist, c, qc + q * ldq, d_c), (uint32_t)c);
+      best = key < best ? key : best;
+    }
+  }
+  best = warp_min_u64(best);
+  if (lane == 0) out[q] = best;
+}
+
 // One warp per query (k <= 32): the top byte of the k-th smallest key (one
 // radix pass over the key row) gives an upper bound of that key, the end of
 // its 256-key bucket, and the threshold above it; the centroids under the
@@ -404,9 +503,10 @@ constexpr int CP_CAND = 96;
 
 __global__ void __launch_bounds__(CP_WARPS * 32) coarse_pick_kernel(
     const uint16_t *__restrict__ keys, int64_t npad, int nlist, const float *__restrict__ qc,
-    int ldq, int d_c, const float *__restrict__ cent, int ldc, const float *__restrict__ qrho,
-    float rmax, float cmax, float e_rest, int64_t B, int k, uint64_t *__restrict__ out) {
-  __shared__ float s_q[CP_WARPS][CM_MAXD];
+    int ldq, int d_c, const float *__restrict__ cpm, const float *__restrict__ qrho,
+    CentBound bound, float e_rest, int64_t B, int k, uint64_t *__restrict__ out) {
+  __shared__ __align__(16) float s_q[CP_WARPS][CM_MAXD];
+  const float rmax = bound.rmax(), cmax = bound.cmax();
   __shared__ int s_hist[CP_WARPS][256];
   __shared__ int s_sh[CP_WARPS][2];
   __shared__ int s_cand[CP_WARPS][CP_CAND];
@@ -420,18 +520,11 @@ __global__ void __launch_bounds__(CP_WARPS * 32) coarse_pick_kernel(
                             nlist, k, [&](int i) -> uint32_t { return __ldg(kq + i) >> 8; },
                             s_hist[warp], s_sh[warp], below, neq)
                         << 8) | 0xFFu;
-  const double rq = (double)qrho[q];
-  const double E = 2.0 * (rmax + rq * cmax + rmax * rq) * (1.0 + 1e-3) + e_rest;
-  const uint32_t thr = kth + (uint32_t)ceil(2.0 * 16384.0 * (ldexp(1.0, -15) + E)) + 1u;
+  const float rq = qrho[q];
+  const uint32_t thr =
+      kth + (uint32_t)key_margin(2.f * (rmax + rq * cmax + rmax * rq) * (1.f + 1e-3f) + e_rest);
   auto score = [&](int c) -> uint64_t {
-    const float *x = cent + (int64_t)c * ldc;
-    float acc = 0.f;
-#pragma unroll 8
-    for (int t = 0; t < d_c; ++t) {
-      const float d = fmaf(-1.f, __ldg(x + t), s_q[warp][t]);
-      acc = fmaf(d, d, acc);
-    }
-    return pack_key(acc, (uint32_t)c);
+    return pack_key(centroid_dist(cpm, nlist, c, s_q[warp], d_c), (uint32_t)c);
   };
   // candidates under the threshold, in list order
   int nc = 0;
@@ -471,12 +564,13 @@ constexpr int CPB_MAXLIST = 16384;
 
 __global__ void __launch_bounds__(CPB_THREADS) coarse_pick_block_kernel(
     const uint16_t *__restrict__ keys, int64_t npad, int nlist, const float *__restrict__ qc,
-    int ldq, int d_c, const float *__restrict__ cent, int ldc, const float *__restrict__ qrho,
-    float rmax, float cmax, float e_rest, int k, uint64_t *__restrict__ out) {
+    int ldq, int d_c, const float *__restrict__ cpm, const float *__restrict__ qrho,
+    CentBound bound, float e_rest, int k, uint64_t *__restrict__ out) {
+  const float rmax = bound.rmax(), cmax = bound.cmax();
   extern __shared__ __align__(16) unsigned char smem[];
   uint32_t *cd = (uint32_t *)smem;          // [nlist] exact distance bits
   uint16_t *k16 = (uint16_t *)(cd + nlist);  // [nlist] tensor-core keys
-  __shared__ float s_q[CM_MAXD];
+  __shared__ __align__(16) float s_q[CM_MAXD];
   __shared__ int hist[256], sh[2], wsum[CPB_THREADS / 32];
   __shared__ int s_lt;
   __shared__ uint64_t s_out[CPB_MAXK];
@@ -490,19 +584,13 @@ __global__ void __launch_bounds__(CPB_THREADS) coarse_pick_block_kernel(
   int below, neq;
   const uint32_t kth = block_radix_kth<CPB_THREADS, 2>(
       nlist, k, [&](int i) -> uint32_t { return k16[i]; }, hist, sh, &below, &neq);
-  const double rq = (double)qrho[q];
-  const double E = 2.0 * (rmax + rq * cmax + rmax * rq) * (1.0 + 1e-3) + e_rest;
-  const uint32_t thr = kth + (uint32_t)ceil(2.0 * 16384.0 * (ldexp(1.0, -15) + E)) + 1u;
+  const float rq = qrho[q];
+  const uint32_t thr =
+      kth + (uint32_t)key_margin(2.f * (rmax + rq * cmax + rmax * rq) * (1.f + 1e-3f) + e_rest);
   for (int c = tid; c < nlist; c += CPB_THREADS) {
     uint32_t v = 0xFFFFFFFFu;
     if (k16[c] <= thr) {
-      const float *x = cent + (int64_t)c * ldc;
-      float acc = 0.f;
-      for (int t = 0; t < d_c; ++t) {
-        const float d = fmaf(-1.f, x[t], s_q[t]);
-        acc = fmaf(d, d, acc);
-      }
-      v = __float_as_uint(acc);
+      v = __float_as_uint(centroid_dist(cpm, nlist, c, s_q, d_c));
     }
     cd[c] = v;
   }
@@ -539,17 +627,29 @@ __global__ void __launch_bounds__(CPB_THREADS) coarse_pick_block_kernel(
 
 }  // namespace
 
-int build_centroid_lowp(adanns_index *x, cudaStream_t st) {
-  if (x->metric != ADANNS_METRIC_L2_PREFIXNORM || x->nlist < 256) return ADANNS_OK;
+// blocks, scales, norms and bounds of a centroid table (x: centroids, nlist, d_c)
+static int fill_centroid_lowp(const adanns_index *x, void *lowp, float *sc, float *n2,
+                              float *bound, cudaStream_t st) {
   const int nblk = (x->d_c + 63) / 64;
   int ng = 0;
   for (int g = 0; g < NGRAN; ++g)
     if (kGran[g] <= x->d_c) ng = g + 1;
+  ADN_CUDA(cudaMemsetAsync(bound, 0, sizeof(float) * (NGRAN + 1), st));
+  centroid_lowp_kernel<<<(unsigned)((x->nlist + 7) / 8), 256, 0, st>>>(
+      x->centroids, x->d_c, x->nlist, nblk, ng, (__nv_bfloat16 *)lowp, sc, n2, bound,
+      bound + NGRAN);
+  ADN_LAUNCH("centroid_lowp_kernel");
+  return ADANNS_OK;
+}
+
+int build_centroid_lowp(adanns_index *x, cudaStream_t st) {
+  if (x->metric != ADANNS_METRIC_L2_PREFIXNORM || x->nlist < 256) return ADANNS_OK;
+  const int nblk = (x->d_c + 63) / 64;
   void *lowp = nullptr;
   float *sc = nullptr, *n2 = nullptr, *tmp = nullptr;
   if (cudaMalloc(&lowp, (size_t)nblk * x->nlist * 64 * 2) != cudaSuccess ||
       cudaMalloc(&sc, sizeof(float) * x->nlist) != cudaSuccess ||
-      cudaMalloc(&n2, sizeof(float) * x->nlist * std::max(ng, 1)) != cudaSuccess ||
+      cudaMalloc(&n2, sizeof(float) * x->nlist * NGRAN) != cudaSuccess ||
       cudaMalloc(&tmp, sizeof(float) * (NGRAN + 1)) != cudaSuccess) {
     cudaGetLastError();
     cudaFree(lowp);
@@ -558,19 +658,19 @@ int build_centroid_lowp(adanns_index *x, cudaStream_t st) {
     cudaFree(tmp);
     return fail(ADANNS_ERR_OOM, "centroid low-precision copy allocation failed");
   }
-  ADN_CUDA(cudaMemsetAsync(tmp, 0, sizeof(float) * (NGRAN + 1), st));
-  centroid_lowp_kernel<<<(unsigned)((x->nlist + 7) / 8), 256, 0, st>>>(
-      x->centroids, x->d_c, x->nlist, nblk, ng, (__nv_bfloat16 *)lowp, sc, n2, tmp, tmp + NGRAN);
-  ADN_LAUNCH("centroid_lowp_kernel");
+  int rc = fill_centroid_lowp(x, lowp, sc, n2, tmp, st);
   float h[NGRAN + 1];
-  cudaError_t e = cudaMemcpyAsync(h, tmp, sizeof(h), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  cudaError_t e = cudaSuccess;
+  if (rc == ADANNS_OK) {
+    e = cudaMemcpyAsync(h, tmp, sizeof(h), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  }
   cudaFree(tmp);
-  if (e != cudaSuccess) {
+  if (rc != ADANNS_OK || e != cudaSuccess) {
     cudaFree(lowp);
     cudaFree(sc);
     cudaFree(n2);
-    return cuda_fail(e, "centroid low-precision copy");
+    return rc != ADANNS_OK ? rc : cuda_fail(e, "centroid low-precision copy");
   }
   x->cent_low = lowp;
   x->cent_low_blocks = nblk;
@@ -578,6 +678,24 @@ int build_centroid_lowp(adanns_index *x, cudaStream_t st) {
   x->cent_n2 = n2;
   for (int g = 0; g < NGRAN; ++g) x->cent_rmax[g] = h[g];
   x->cent_maxnorm = h[NGRAN];
+  return ADANNS_OK;
+}
+
+// The same in scratch for the duration of a call, its bounds left on the device.
+int scratch_centroid_lowp(Scratch &s, adanns_index *x, cudaStream_t st) {
+  const int nblk = (x->d_c + 63) / 64;
+  __nv_bfloat16 *lowp;
+  float *sc, *n2, *bound;
+  int rc;
+  if ((rc = s.get(&lowp, (size_t)nblk * x->nlist * 64)) || (rc = s.get(&sc, x->nlist)) ||
+      (rc = s.get(&n2, (size_t)x->nlist * NGRAN)) || (rc = s.get(&bound, NGRAN + 1)) ||
+      (rc = fill_centroid_lowp(x, lowp, sc, n2, bound, st)))
+    return rc;
+  x->cent_low = lowp;
+  x->cent_low_blocks = nblk;
+  x->cent_sc = sc;
+  x->cent_n2 = n2;
+  x->cent_bound = bound;
   return ADANNS_OK;
 }
 
@@ -616,8 +734,8 @@ int launch_coarse_tc(const adanns_index *idx, const float *qc, int ldq, int64_t 
   coarse_tiles_kernel<<<(unsigned)((nfill + 255) / 256), 256, 0, st>>>(
       B, ntiles, npad, tl, tb, tc, pair_out, pbase, ntiles_dev, counter);
   ADN_LAUNCH("coarse_tiles_kernel");
-  coarse_prep_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(qc, ldq, B, d_c, nkb, rows, tiles,
-                                                                 qn2, qsc, qrho);
+  coarse_prep_kernel<<<(unsigned)(rows / 32), 256, 0, st>>>(qc, ldq, B, d_c, rows, tiles, qn2, qsc,
+                                                            qrho);
   ADN_LAUNCH("coarse_prep_kernel");
   MmaScanArgs m{};
   m.tile_list = tl;
@@ -643,17 +761,32 @@ int launch_coarse_tc(const adanns_index *idx, const float *qc, int ldq, int64_t 
     return rc;
   const float e_rest = (float)(2.0 * nkb * 64 * std::ldexp(1.0, -22) +
                                8.0 * (d_c + 2) * std::ldexp(1.0, -24) + 1e-4);
-  if (k <= CM_MAXK) {
+  CentBound bound{};
+  if (idx->cent_bound) {
+    bound.rd = idx->cent_bound + gi;
+    bound.cd = idx->cent_bound + NGRAN;
+  } else {
+    bound.r = idx->cent_rmax[gi] * 1.001f;
+    bound.c = idx->cent_maxnorm * 1.001f;
+  }
+  if (k == 1 && nlist <= 4096) {
+    auto kern = nlist <= 256    ? coarse_nearest_kernel<1>
+                : nlist <= 512  ? coarse_nearest_kernel<2>
+                : nlist <= 1024 ? coarse_nearest_kernel<4>
+                : nlist <= 2048 ? coarse_nearest_kernel<8>
+                                : coarse_nearest_kernel<16>;
+    kern<<<(unsigned)((B + 7) / 8), 256, 0, st>>>(keys, npad, nlist, qc, ldq, d_c, idx->cent_pm,
+                                                  qrho, bound, e_rest, B, out);
+    ADN_LAUNCH("coarse_nearest_kernel");
+  } else if (k <= CM_MAXK) {
     coarse_pick_kernel<<<(unsigned)((B + CP_WARPS - 1) / CP_WARPS), CP_WARPS * 32, 0, st>>>(
-        keys, npad, nlist, qc, ldq, d_c, idx->centroids, idx->d_c, qrho,
-        idx->cent_rmax[gi] * 1.001f, idx->cent_maxnorm * 1.001f, e_rest, B, k, out);
+        keys, npad, nlist, qc, ldq, d_c, idx->cent_pm, qrho, bound, e_rest, B, k, out);
     ADN_LAUNCH("coarse_pick_kernel");
   } else {
     const size_t sm = (size_t)nlist * 6;
     ADN_CUDA(ensure_smem((const void *)coarse_pick_block_kernel, sm));
     coarse_pick_block_kernel<<<(unsigned)B, CPB_THREADS, sm, st>>>(
-        keys, npad, nlist, qc, ldq, d_c, idx->centroids, idx->d_c, qrho,
-        idx->cent_rmax[gi] * 1.001f, idx->cent_maxnorm * 1.001f, e_rest, k, out);
+        keys, npad, nlist, qc, ldq, d_c, idx->cent_pm, qrho, bound, e_rest, k, out);
     ADN_LAUNCH("coarse_pick_block_kernel");
   }
   return ADANNS_OK;

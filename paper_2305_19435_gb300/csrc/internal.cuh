@@ -60,6 +60,15 @@ __host__ __device__ inline uint64_t pack_key(float d, uint32_t id) {
 #endif
 }
 
+// How far apart two 16-bit keys (round(2^14 d), +-2^-15) can be while their exact
+// distances still order the other way round, when every approximate distance is
+// within E of the exact one: 2 * 2^14 * (2^-15 + E), rounded up past the FP32
+// rounding of this expression.  (In FP32: a warp's handful of FP64 operations
+// is a hundred cycles of an SM here, 110 us over 262,144 points.)
+__device__ __forceinline__ int key_margin(float E) {
+  return (int)fminf(ceilf((1.f + 32768.f * E) * 1.00001f), 1048575.f) + 1;
+}
+
 // MR granularities (Sec. 3: nested sizes 8 .. 2048)
 constexpr int NGRAN = 14;
 extern const int kGran[NGRAN];
@@ -361,6 +370,7 @@ int run_coarse(const adanns_index *idx, const float *qc, int ldq, int64_t B, int
                uint64_t *out, int *counter, cudaStream_t st);
 constexpr int64_t CT_SLICE_MIN = 4096;  // fewest points per tensor-core assignment slice
 int build_centroid_lowp(adanns_index *x, cudaStream_t st);
+int scratch_centroid_lowp(Scratch &s, adanns_index *x, cudaStream_t st);
 // Candidate segments of a batch: per query, the probed lists' sizes rounded
 // up to 8, laid end to end (qtot: per-query total, qbase: its start, pbase:
 // start of each (query, probe) segment).
@@ -554,6 +564,7 @@ struct adanns_index {
   float *cent_n2 = nullptr;
   float cent_rmax[adn::NGRAN] = {};
   float cent_maxnorm = 0.f;
+  const float *cent_bound = nullptr;  // or both on the device [NGRAN + 1] (a call's own table)
   float *cent_pm = nullptr;     // centroids prefix-major, one list of nlist members
   int64_t *cent_off = nullptr;  // {0, nlist}
   int64_t *list_off = nullptr;  // nlist + 1

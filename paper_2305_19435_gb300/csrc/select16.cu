@@ -207,10 +207,8 @@ __global__ void __launch_bounds__(SW_WARPS * 32, 6) select16_kernel(
   if (q >= B) return;
   int prune_delta = 0;
   if (prune) {
-    const double rq = (double)qrho[q];
-    const double E = 2.0 * (rmax + rq + rmax * rq) * (1.0 + 1e-3) + e_rest;
-    prune_delta = (int)ceil(2.0 * 16384.0 * (ldexp(1.0, -15) + E)) + 1;
-    if (prune_delta > (1 << 20)) prune_delta = 1 << 20;
+    const float rq = qrho[q];
+    prune_delta = key_margin(2.f * (rmax + rq + rmax * rq) * (1.f + 1e-3f) + e_rest);
   }
   int total, ptotal;
   warp_lists(s, ckeys + q * nprobe, nprobe, list_off, total, ptotal);
@@ -348,8 +346,7 @@ __global__ void __launch_bounds__(SW_WARPS * 32, 6) certify16_kernel(
   SwState &s = ((SwState *)smem)[warp];
   const int64_t q = (int64_t)blockIdx.x * SW_WARPS + warp;
   if (q >= B) return;
-  const int delta =
-      (int)fmin(ceil(2.0 * 16384.0 * (ldexp(1.0, -15) + (double)qerr[q])) + 1.0, 1048576.0);
+  const int delta = key_margin(qerr[q]);
   int total, ptotal;
   warp_lists(s, ckeys + q * nprobe, nprobe, list_off, total, ptotal);
   int64_t *o = out + q * kk;
@@ -592,10 +589,8 @@ __global__ void __launch_bounds__(SW_WARPS * 32, 3) select_surv_kernel(
   if (q >= B) return;
   int prune_delta = 0;
   if (prune) {
-    const double rq = (double)qrho[q];
-    const double E = 2.0 * (rmax + rq + rmax * rq) * (1.0 + 1e-3) + e_rest;
-    prune_delta = (int)ceil(2.0 * 16384.0 * (ldexp(1.0, -15) + E)) + 1;
-    if (prune_delta > (1 << 20)) prune_delta = 1 << 20;
+    const float rq = qrho[q];
+    prune_delta = key_margin(2.f * (rmax + rq + rmax * rq) * (1.f + 1e-3f) + e_rest);
   }
   // probed lists: ids, sizes, padded candidate starts, survivor counts
   int ln[4], pl[4], sc[4], tot = 0, ptot = 0, stot = 0;
