@@ -22,7 +22,12 @@
 // that more loads are in flight, and 16-column staging to make room for them;
 // FP8 (twice the MMA rate, the drain is the limit) keeps three stages and
 // 64-column staging, whose stores are fewer and wider, except where few
-// queries share a list (the loads are the limit there: four stages).  Every mbarrier wait is
+// queries share a list (the loads are the limit there: four stages); short
+// 16-bit prefixes, whose drain is the limit as well, take FP8's configuration.
+// The drain works on two columns per FP32 instruction, rounds to the key by
+// adding 2^23 and joins two keys by one byte permutation, keeps each lane's row
+// segments in registers, and arrives at the barriers once per warp (scan of
+// 50,000 queries x 16 lists at d_s 512: 1.50 -> 1.46 ms).  Every mbarrier wait is
 // bounded: on timeout the kernel records an error, stops issuing work, lets
 // in-flight copies land and frees TMEM.
 #include <cuda.h>
@@ -70,6 +75,13 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// one arrival for a whole warp, once all its lanes are here (a barrier that
+// counts every lane of 16 warps takes 512 updates one after the other)
+__device__ __forceinline__ void mbar_arrive_warp(uint64_t *bar) {
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+}
+
 __device__ __forceinline__ uint64_t global_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -98,6 +110,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64
     if (ok) return true;
   }
   return false;
+}
+
+// the same by a whole warp: one answer for all its lanes, so that a wait that
+// runs out for some of them cannot leave the others at a warp barrier
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, uint64_t limit_ns) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit_ns));
 }
 
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, uint64_t *bar,
@@ -229,12 +247,12 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&tfull[s], 1);
-      mbar_init(&tempty[s], EPI_THREADS);
-      mbar_init(&sfull[s], EPI_THREADS);
+      mbar_init(&tempty[s], EPI_WARPS);
+      mbar_init(&sfull[s], EPI_WARPS);
     }
     for (int s = 0; s < TQD; ++s) {
       mbar_init(&qfull[s], 1);
-      mbar_init(&qempty[s], 1 + EPI_THREADS);
+      mbar_init(&qempty[s], 1 + EPI_WARPS);
     }
     abort_s = 0;
     for (int i = 0; i < 2 * BM; ++i) s_rc[i / BM][i % BM] = 0;
@@ -378,13 +396,13 @@ __global__ void __launch_bounds__(THREADS, 1)
     // the count to rcnt and clears its slot for the item after that
     int ib = 0;
     for (;;) {
-      if (!mbar_wait(&qfull[qs], qph, a.wait_ns)) {
+      if (!mbar_wait_warp(&qfull[qs], qph, a.wait_ns)) {
         atomicExch(&abort_s, 1);
         atomicCAS(a.err, 0, 8);
         break;
       }
       const int t = qids[qs];
-      mbar_arrive(&qempty[qs]);
+      mbar_arrive_warp(&qempty[qs]);
       if (++qs == TQD) { qs = 0; qph ^= 1; }
       if (t < 0) break;
       const int tile = t / nsplit, list = a.tile_list[tile];
@@ -409,10 +427,18 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       const int cbuf = ib & 1;
       bool stop = false;
+      // the key segments of the rows this lane stores (-1: no such query), the
+      // same for every member tile: NI rows of a staging tile, LPR lanes each
+      constexpr int CPR = SC / 8, LPR = CPR, RPI = 32 / LPR, NI = 32 / RPI;
+      long long rbase[NI];
+#pragma unroll
+      for (int i = 0; i < NI; ++i)
+        rbase[i] = __shfl_sync(0xffffffffu, valid ? (long long)base : -1ll, i * RPI + lane / LPR);
       // the row's terms in key units: key = round(clamp(d) * 2^14) with
       // d * 2^14 = (2^14 s_q) (-2 s_x nu_x) (q~ . x~) + 2^14 (|q|^2 + |x|^2);
       // scaling by 2^14 is exact, so the keys are those of the unscaled form
       const float qsk = 16384.f * qs, q2k = 16384.f * q2;
+      const uint64_t qsk2 = pack2(qsk, qsk), q2k2 = pack2(q2k, q2k);
       // per-member terms of member tile mt (thread et < BN holds member et of
       // the tile), loaded one tile ahead so the loads overlap the drain
       auto load_terms = [&](int mt) -> float2 {
@@ -428,7 +454,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       };
       float2 terms = load_terms(mr.x);
       for (int mt = mr.x; mt < mr.y; ++mt) {
-        if (!mbar_wait(&tfull[acc], aphase, a.wait_ns)) {
+        if (!mbar_wait_warp(&tfull[acc], aphase, a.wait_ns)) {
           atomicExch(&abort_s, 1);
           atomicCAS(a.err, 0, 4);
           stop = true;
@@ -442,8 +468,8 @@ __global__ void __launch_bounds__(THREADS, 1)
             s_ca[acc][et] = terms.y;
           }
           // hand-off through an mbarrier: a bounded wait, unlike bar.sync
-          mbar_arrive(&sfull[acc]);
-          if (!mbar_wait(&sfull[acc], aphase, a.wait_ns)) {
+          mbar_arrive_warp(&sfull[acc]);
+          if (!mbar_wait_warp(&sfull[acc], aphase, a.wait_ns)) {
             atomicExch(&abort_s, 1);
             atomicCAS(a.err, 0, 5);
             stop = true;
@@ -467,7 +493,6 @@ __global__ void __launch_bounds__(THREADS, 1)
           // with its row's tau (two keys per word) and writes only the
           // survivors, as records, after one shared-memory atomic on the row's
           // count
-          constexpr int CPR = SC / 8, LPR = CPR, RPI = 32 / LPR;
           uint4 *stg = (uint4 *)(sStage + (size_t)(warp - 2) * stg_bytes(SC));
           auto swz = [](int row, int ch) -> int {
             return CPR == 8 ? (ch ^ (row & 7)) : (ch ^ ((row >> 2) & 1));
@@ -480,23 +505,30 @@ __global__ void __launch_bounds__(THREADS, 1)
             uint32_t packed[16];
 #pragma unroll
             for (int j = 0; j < 32; j += 4) {
-              // the four columns' member terms in one 16-byte read each
-              const float4 cb = *(const float4 *)&s_cb[acc][c_lo + c0 + j];
-              const float4 ca = *(const float4 *)&s_ca[acc][c_lo + c0 + j];
-              const float cbv[4] = {cb.x, cb.y, cb.z, cb.w}, cav[4] = {ca.x, ca.y, ca.z, ca.w};
-              uint32_t kk[4];
+              // the four columns' member terms in one 16-byte read each, two
+              // columns per FP32 instruction (each half rounds as the scalar one)
+              const ulonglong2 cb = *(const ulonglong2 *)&s_cb[acc][c_lo + c0 + j];
+              const ulonglong2 ca = *(const ulonglong2 *)&s_ca[acc][c_lo + c0 + j];
+              const uint64_t cbv[2] = {cb.x, cb.y}, cav[2] = {ca.x, ca.y};
 #pragma unroll
-              for (int u = 0; u < 4; ++u) {
+              for (int u = 0; u < 2; ++u) {
                 // approximate squared distance as a 16-bit fixed-point key:
                 // round(d * 2^14), d clamped to [0, 3.9999]; members past the
-                // list end get the largest key.  The lower clamp is the
-                // conversion's saturation.
-                const float dk = fminf(fmaf(qsk * cbv[u], __uint_as_float(r[j + u]), q2k + cav[u]),
-                                       3.9999f * 16384.f);
-                asm("cvt.rni.sat.u32.f32 %0, %1;" : "=r"(kk[u]) : "f"(dk));
+                // list end get the largest key.  Adding 2^23 rounds to the
+                // nearest integer (ties to even) and leaves it in the low bits,
+                // where one byte permutation joins the two keys; a conversion
+                // instruction per key has a quarter of that rate.
+                const uint64_t dot =
+                    pack2(__uint_as_float(r[j + 2 * u]), __uint_as_float(r[j + 2 * u + 1]));
+                const float2 d = unpack2(fma2(mul2(qsk2, cbv[u]), dot, add2(q2k2, cav[u])));
+                const uint64_t t = add2(
+                    pack2(fmaxf(fminf(d.x, 3.9999f * 16384.f), 0.f),
+                          fmaxf(fminf(d.y, 3.9999f * 16384.f), 0.f)),
+                    pack2(8388608.f, 8388608.f));
+                const float2 k = unpack2(t);
+                packed[(j >> 1) + u] =
+                    __byte_perm(__float_as_uint(k.x), __float_as_uint(k.y), 0x5410);
               }
-              packed[j >> 1] = kk[0] | (kk[1] << 16);
-              packed[(j >> 1) + 1] = kk[2] | (kk[3] << 16);
             }
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
@@ -508,16 +540,15 @@ __global__ void __launch_bounds__(THREADS, 1)
                 // LPR lanes per row: one instruction stores RPI rows x SC * 2 bytes
                 const int m0 = mt * BN + c_lo + col + 8 - SC;
 #pragma unroll
-                for (int i = 0; i < 32 / RPI; ++i) {
+                for (int i = 0; i < NI; ++i) {
                   const int rr = i * RPI + lane / LPR;
-                  const long long b = __shfl_sync(0xffffffffu, (long long)base, rr);
-                  const int ok = __shfl_sync(0xffffffffu, valid ? 1 : 0, rr);
-                  const uint32_t tr = __shfl_sync(0xffffffffu, tau, rr);
+                  const long long b = rbase[i];
                   const uint4 v = stg[rr * CPR + swz(rr, chl)];
                   const int mb = m0 + 8 * chl;
+                  const uint32_t tr = filt ? __shfl_sync(0xffffffffu, tau, rr) : 0u;
                   if (!filt) {
-                    if (ok && mb < npad) *(uint4 *)(a.cand + b + mb) = v;
-                  } else if (ok && mb < nl) {
+                    if (b >= 0 && mb < npad) *(uint4 *)(a.cand + b + mb) = v;
+                  } else if (b >= 0 && mb < nl) {
                     uint32_t msk = keys_le8(v, tr);
                     if (mb + 8 > nl) msk &= (1u << (nl - mb)) - 1u;  // members past the list end
                     if (msk) {
@@ -541,7 +572,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
         }
         tc_fence_before();
-        mbar_arrive(&tempty[acc]);
+        mbar_arrive_warp(&tempty[acc]);
         if (++acc == 2) { acc = 0; aphase ^= 1; }
       }
       if (stop) break;
@@ -551,7 +582,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         fl_buf = cbuf;
         ++ib;
       }
-      if (ld_abort(&abort_s)) break;
+      if (__any_sync(0xffffffffu, ld_abort(&abort_s))) break;
     }
   }
 
@@ -608,11 +639,11 @@ __global__ void __launch_bounds__(N_THREADS, 1)
     }
     for (int s = 0; s < NACC; ++s) {
       mbar_init(&tfull[s], 1);
-      mbar_init(&tempty[s], 128);
+      mbar_init(&tempty[s], 4);
     }
     for (int s = 0; s < TQD; ++s) {
       mbar_init(&qfull[s], 1);
-      mbar_init(&qempty[s], 1 + 128);
+      mbar_init(&qempty[s], 1 + 4);
     }
     abort_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -726,12 +757,12 @@ __global__ void __launch_bounds__(N_THREADS, 1)
     int acc = 0, qs = 0;
     uint32_t aphase = 0, qph = 0;
     for (;;) {
-      if (!mbar_wait(&qfull[qs], qph, a.wait_ns)) {
+      if (!mbar_wait_warp(&qfull[qs], qph, a.wait_ns)) {
         give_up(14);
         break;
       }
       const int t = qids[qs];
-      mbar_arrive(&qempty[qs]);
+      mbar_arrive_warp(&qempty[qs]);
       if (++qs == TQD) { qs = 0; qph ^= 1; }
       if (t < 0) break;
       const int list = a.tile_list[t];
@@ -759,7 +790,7 @@ __global__ void __launch_bounds__(N_THREADS, 1)
           cb = -2.f * c;
           cak = 16384.f * (a.x2 ? __ldg(a.x2 + off + m) : (c > 0.f ? 1.f : 0.f));
         }
-        if (!mbar_wait(&tfull[acc], aphase, a.wait_ns)) {
+        if (!mbar_wait_warp(&tfull[acc], aphase, a.wait_ns)) {
           give_up(15);
           stop = true;
           break;
@@ -782,10 +813,10 @@ __global__ void __launch_bounds__(N_THREADS, 1)
           }
         }
         tc_fence_before();
-        mbar_arrive(&tempty[acc]);
+        mbar_arrive_warp(&tempty[acc]);
         if (++acc == NACC) { acc = 0; aphase ^= 1; }
       }
-      if (stop || ld_abort(&abort_s)) break;
+      if (stop || __any_sync(0xffffffffu, ld_abort(&abort_s))) break;
     }
   }
   __syncthreads();
@@ -876,6 +907,11 @@ int mma_scan_nsplit(const adanns_index *idx, int64_t pairs) {
 
 // stage count and staging width per element type (see the kernel's notes)
 constexpr int NS_BF16 = 4, SC_BF16 = 16, NS_FP8 = 3, SC_FP8 = 64;
+// 16-bit operands of at most this many K-blocks take FP8's configuration too:
+// their drain is the limit (scan stage, narrow against wide staging: 2 K-blocks,
+// one list of 1.28 M x 1,000 queries 1.09 against 0.81 ms; 6 K-blocks, 5.25 M rows
+// x 8,000 queries 2.29 against 1.96; 8 K-blocks 1.457 against 1.482)
+constexpr int NKB_DRAIN = 6;
 size_t mma_scan_smem(int ns, int sc) {
   return (size_t)ns * STAGE_BYTES + (size_t)EPI_WARPS * stg_bytes(sc) + 1024;
 }
@@ -890,7 +926,7 @@ int launch_mma_scan(const void *qtiles, int64_t qrows, const void *xlow, int64_t
   MmaScanArgs b = a;
   b.wait_ns = (uint64_t)option(ADANNS_OPT_WAIT_LIMIT_NS);
   b.skip_fill = (int)take_option(ADANNS_OPT_TEST_SKIP_LOAD, -1);
-  if (a.fp8 && !a.few) {
+  if ((a.fp8 && !a.few) || (!a.fp8 && a.nkb <= NKB_DRAIN)) {
     const size_t smem = mma_scan_smem(NS_FP8, SC_FP8);
     ADN_CUDA(ensure_smem((const void *)mma_scan_kernel<NS_FP8, SC_FP8>, smem));
     mma_scan_kernel<NS_FP8, SC_FP8><<<num_sms(), THREADS, smem, st>>>(tA, tB, b);
