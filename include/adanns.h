@@ -79,9 +79,9 @@ int64_t adanns_launch_count(void);
  * after that.  A change applies to calls issued after it; a search plan keeps
  * what it captured.
  *   ADANNS_OPT_FP32_STREAM    1 (default): FP32 search by the streaming scan
- *                             where few queries share a probed list, through
- *                             the certified tensor-core filter where several
- *                             do; 0: tiled scan always
+ *                             unless very many queries share a probed list,
+ *                             through the certified tensor-core filter where it
+ *                             pays; 0: tiled scan always
  *   ADANNS_OPT_ADC_SELECT     1 (default): IVF-OPQ distance-then-select stage
  *                             for nprobe <= 256; 0: running top-k per list
  *   ADANNS_OPT_COARSE_TC      1 (default): tensor-core cluster mapping where it
@@ -296,10 +296,11 @@ int adanns_kmeans_update(const float *points, int64_t n, int ld, int dim, int me
  *            probed with P_dc(q) against the first d_c coordinates of each
  *            centroid, taken as stored (not renormalised).
  *   storage  ADANNS_STORE_F32: the exact FP32 scan (rerank_k must be 0).
- *            With few queries per probed list (B * nprobe / nlist <= 16,
- *            nprobe <= 256) the lists are streamed once per 16-query tile
+ *            Unless very many queries share a probed list (nprobe <= 256;
+ *            beyond 16 per list also by d_s, k and the scratch at hand) the
+ *            lists are streamed once per group of 8 queries
  *            and the distances selected per query afterwards (4 bytes per
- *            probed member of scratch).  Where more share one (prefix-
+ *            probed member of scratch).  Where several share one (prefix-
  *            normalised metric, k <= 256, nprobe <= 128, and a batch large
  *            enough to pay for it), FP16 tensor-core products of the probed
  *            lists first shortlist every member within a rounding-error bound

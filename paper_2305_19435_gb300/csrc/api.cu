@@ -619,13 +619,6 @@ int search_f32_tiled(const adanns_index *idx, const float *queries, int64_t B, i
   return ADANNS_OK;
 }
 
-int64_t stream_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,
-                             int k) {
-  const int64_t per_q = max_probe_members(idx, nprobe) * 4 + (int64_t)(pad16(d_c) + pad16(d_s)) * 4 +
-                        (int64_t)k * 8 + (int64_t)nprobe * 40 + 16;
-  const int64_t Bc = std::max<int64_t>(1, std::min<int64_t>(B, scratch_budget() / per_q));
-  return Bc * per_q + (int64_t)idx->nlist * 64 + (16ll << 20);
-}
 }  // namespace adn
 
 extern "C" {
@@ -645,7 +638,7 @@ int64_t adanns_search_scratch_bytes(const adanns_index *idx, int64_t B, int d_c,
   }
   if (f32_certified(idx, B, d_s, nprobe, k))
     return certified_scratch_bytes(idx, B, d_c, d_s, nprobe, k);
-  if (fp32_stream_enabled((double)B * nprobe / idx->nlist, nprobe, k, d_s))
+  if (fp32_stream_enabled(idx, B, B * nprobe, d_c, d_s, nprobe, k))
     return stream_scratch_bytes(idx, B, d_c, d_s, nprobe, k);
   int tq, qt, nsplit;
   fp32_scan_shape(idx, B, d_s, nprobe, k, &tq, &qt, &nsplit);
@@ -740,7 +733,7 @@ int adanns_search_ivf(const adanns_index *idx, const float *queries, int64_t B, 
   if (f32_certified(idx, B, d_s, nprobe, k))
     return search_f32_certified(idx, queries, B, d_c, d_s, nprobe, k, out_ids, out_dist,
                                 out_probes, st);
-  if (fp32_stream_enabled((double)B * nprobe / idx->nlist, nprobe, k, d_s))
+  if (fp32_stream_enabled(idx, B, B * nprobe, d_c, d_s, nprobe, k))
     return search_f32_stream(idx, queries, B, d_c, d_s, nprobe, k, out_ids, out_dist, out_probes,
                              st);
   return search_f32_tiled(idx, queries, B, d_c, d_s, nprobe, k, out_ids, out_dist, out_probes,
@@ -798,7 +791,7 @@ int adanns_search_ivf_budgets(const adanns_index *idx, const float *queries, int
   if (B == 0) return ADANNS_OK;
   // FP32 with many queries per probed list: the tiled scan, one launch
   // sequence per distinct d_s over that group of queries (rows in place)
-  const bool tiled = !lowp && !fp32_stream_enabled((double)np_sum / idx->nlist, np_max);
+  const bool tiled = !lowp && !fp32_stream_enabled(idx, B, np_sum, d_c, ds_max, np_max, k_max, true);
   std::vector<std::pair<int64_t, int64_t>> grp;  // [begin, end) of each d_s group in the order
   if (tiled) {
     std::vector<int32_t> perm((size_t)B);

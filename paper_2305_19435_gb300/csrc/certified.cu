@@ -337,19 +337,19 @@ Shape shape_of(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,
 }  // namespace
 
 // Where the filter pays.  It costs a pass over the probed lists (4 bytes read,
-// 2 written per coordinate), a dozen more launches and the re-score; it saves
-// the FFMA scan.  Above 16 queries per probed list (where the tiled scan is
-// the alternative) it was ahead at every measured size down to 20,000 rows x 64
-// (193 against 172 us at 17 queries per list; 16.2 against 2.1 ms at 1.28 M
-// rows x 512, 128 per list); smaller products are left to the tiled scan.  Up
-// to 16, in units of a coordinate (about a picosecond): the streaming scan
-// spends 0.32 per (query, member), the filter 1.25 per member and 0.5 per
-// re-scored coordinate, and 2e8 covers its extra launches (100,000 x 512: equal
-// at 15 queries per list; 400,000 x 512: 712 against 710 us at 8; 1.28 M x 64:
-// equal at 8 to 12; 1.28 M x 512: 1.79 against 1.08 ms at 8).  k and the probes
-// must fit the shortlist's buffers, and the FP16 rows may take half of the
-// call's scratch budget.  Turning the streaming scan off asks for the tiled
-// scan everywhere.
+// 2 written per coordinate), a dozen more launches and the re-score.  Against
+// the streaming scan, in picoseconds: that spends 0.112 more per (query, member,
+// coordinate), the filter 1.01 per member coordinate, 1 per re-scored coordinate
+// and 57 us of launches.  Streaming against filter, k 10: 1.28 M rows x 512, 8 /
+// 12 / 16 queries per list 845 / 1197 / 1504 against 967 / 1046 / 1058 us;
+// 400,000 x 64 at 20 / 32 / 64 171 / 269 / 445 against 208 / 269 / 315; 60,000 x 64
+// equal at 128.  Above 100 queries per list the line is lower, where the tiled
+// scan (the alternative for long prefixes) comes out even: 20,000 rows x 64 193
+// against 172 us at 17; the streaming scan would save at most 50 us there (10,000 x
+// 64 at 128: 76 against 124), and such batches stay on one path.  k and the probes must
+// fit the shortlist's buffers, and the FP16 rows may take half of the call's
+// scratch budget.  Turning the streaming scan off asks for the tiled scan
+// everywhere.
 bool f32_certified(const adanns_index *idx, int64_t B, int d_s, int nprobe, int k) {
   if (idx->metric != ADANNS_METRIC_L2_PREFIXNORM || k > CE_MAX_K || nprobe > 128) return false;
   if (!option(ADANNS_OPT_FP32_STREAM) || scan_choice_forced()) return false;
@@ -357,8 +357,8 @@ bool f32_certified(const adanns_index *idx, int64_t B, int d_s, int nprobe, int 
   if (idx->N * nkb > INT32_MAX - 256) return false;  // 32-bit row coordinates of the copies
   if (idx->N * (nkb * 128 + 4) > scratch_budget() / 2) return false;
   const double qpl = (double)B * nprobe / idx->nlist, nd = (double)idx->N * d_s;
-  if (qpl > 16.0) return nd * qpl > 2e7;
-  return nd * (0.32 * qpl - 1.25) - 0.5 * B * k * d_s > 2e8;
+  if (qpl > 100.0 && nd * qpl > 2e7) return true;
+  return nd * (0.112 * qpl - 1.01) - (double)B * k * d_s > 5.7e7;
 }
 
 int64_t certified_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,

@@ -3,14 +3,16 @@
 // member row is used by a handful of queries and the scan is a stream of the
 // probed lists' d_s prefixes.
 //
-// Work unit = (probe tile, chunk of 256 members, group of up to 4 of the
+// Work unit = (probe tile, chunk of 128 members, group of up to 8 of the
 // tile's queries): units cost about the same whatever the list's popularity,
 // and are enumerated by an exclusive scan of each tile's unit count.  One
 // thread per member: the member's 16-coordinate prefix blocks are read with
 // 16-byte loads straight into registers (a warp covers 32 consecutive
 // members, 2 KB contiguous per block in the prefix-major layout), the next
-// block in flight while one is used, and the distances to the group's
-// queries accumulate in registers; no barrier inside the stream.  The
+// two blocks in flight, and the distances to the group's queries accumulate
+// in registers; no barrier inside the stream.  The group's rows are staged in
+// shared memory: a query operand is then one broadcast read a few tens of
+// cycles away, also while the member stream evicts whatever L1 holds.  The
 // arithmetic is the FP32 scan's (t = q_j - s_x x_j, acc += t * t over j
 // ascending), so the distances are bit-identical to it; each one is written
 // as FP32 bits into the query's candidate segment, and select32_kernel then
@@ -21,7 +23,16 @@
 // streams its member rows up to the largest d_s of its queries while each
 // query stops accumulating at its own d_s (with its own per-member scale at
 // that prefix), and the selection keeps the batch's largest k, of which a
-// query's own k results are the prefix.
+// query's own k results are the prefix.  A tile's queries are grouped by
+// descending d_s: the queries still active in a block are a prefix of the group,
+// and the second group of a full tile streams short prefixes only.
+//
+// Bound by the broadcast reads and the latency of the member stream (six CTAs of
+// 128 threads per SM; 256 x 3 and 64 x 12 were 10% and 5% slower, groups of 4 and
+// 16 18% and 10%).  Measured on 1,281,167 x 2048 (1,024 lists), 1,021 queries with
+// d_s 64 to 512, 1 to 16 probes: 1.33 ms with groups of 4 in arrival order and
+// operands from L1, 0.61 ms here (4.3 TB/s of the rows); one d_s for all, 300,000 x
+// 1024 (300 lists), 300 queries x 8 lists at 256: 220 -> 147 us.
 #include <algorithm>
 
 #include "devutil.cuh"
@@ -30,9 +41,12 @@
 namespace adn {
 namespace {
 
-constexpr int SF_THREADS = 256;  // one chunk of members per work unit
+constexpr int SF_THREADS = 128;  // one chunk of members per work unit
+constexpr int SF_CTAS = 6;       // resident per SM
 constexpr int SF_QT = 16;        // queries per probe tile
-constexpr int SF_QG = 4;         // queries per work unit
+constexpr int SF_QG = 8;         // queries per work unit, as far as
+constexpr int SF_SMEM = 32768;   // their staged rows fit (six CTAs: 192 KB)
+constexpr int SFF_QG = 4;        // the same in dist_f32_few_kernel
 
 struct StreamArgs {
   const float *xpm;  // prefix-major FP32 lists
@@ -47,6 +61,7 @@ struct StreamArgs {
   const int32_t *qds, *qgi;
   const float *invn;
   int64_t N;
+  int qg;  // queries per unit
   const int32_t *tile_list, *tile_beg, *tile_cnt;
   const int *ntiles_dev;
   const int64_t *uoff;  // first work unit of each tile (exclusive scan of its units)
@@ -63,81 +78,63 @@ __device__ __forceinline__ float4 ldg4(const float *p) { return __ldg((const flo
 // units of a tile: member chunks x query groups (0 past the tile count)
 __global__ void stream_units_kernel(const int32_t *__restrict__ tl, const int32_t *__restrict__ tc,
                                     const int *__restrict__ ntiles, const int64_t *__restrict__ list_off,
-                                    int64_t max_tiles, int64_t *__restrict__ units) {
+                                    int64_t max_tiles, int um, int qg, int64_t *__restrict__ units) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= max_tiles) return;
   int64_t u = 0;
   if (t < *ntiles) {
     const int l = tl[t];
     const int64_t npad = (list_off[l + 1] - list_off[l] + 7) & ~7ll;
-    u = ((npad + SF_THREADS - 1) / SF_THREADS) * ((tc[t] + SF_QG - 1) / SF_QG);
+    u = ((npad + um - 1) / um) * ((tc[t] + qg - 1) / qg);
   }
   units[t] = u;
 }
 
-// acc[j] += sum over the block's coordinates (nd4 groups of 4) of (q - s x)^2
+// One block of one query: nd4 groups of 4 coordinates of a row in shared memory.
 template <bool FULL>
-__device__ __forceinline__ void block_step(float (&acc)[SF_QG], const float4 (&x)[4], float sc,
-                                           const float *const *qrow, int cnt, int off, int nd4) {
+__device__ __forceinline__ void row_step(float &acc, const float4 (&x)[4], float sc,
+                                         const float4 *qb, int nd4) {
 #pragma unroll
-  for (int j = 0; j < SF_QG; ++j) {
-    if (j >= cnt) break;
-    const float *qb = qrow[j] + off;
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      if (!FULL && s >= nd4) break;
-      const float4 q = ldg4(qb + 4 * s);
-      float t;
-      t = fmaf(-sc, x[s].x, q.x);
-      acc[j] = fmaf(t, t, acc[j]);
-      t = fmaf(-sc, x[s].y, q.y);
-      acc[j] = fmaf(t, t, acc[j]);
-      t = fmaf(-sc, x[s].z, q.z);
-      acc[j] = fmaf(t, t, acc[j]);
-      t = fmaf(-sc, x[s].w, q.w);
-      acc[j] = fmaf(t, t, acc[j]);
-    }
+  for (int s = 0; s < 4; ++s) {
+    if (!FULL && s >= nd4) break;
+    const float4 q = qb[s];
+    float t;
+    t = fmaf(-sc, x[s].x, q.x);
+    acc = fmaf(t, t, acc);
+    t = fmaf(-sc, x[s].y, q.y);
+    acc = fmaf(t, t, acc);
+    t = fmaf(-sc, x[s].z, q.z);
+    acc = fmaf(t, t, acc);
+    t = fmaf(-sc, x[s].w, q.w);
+    acc = fmaf(t, t, acc);
   }
 }
 
-// The same for a group whose queries stop at their own prefixes: query j
-// takes the block's coordinates below ds[j] (multiples of 4), scaled by its
-// own sc[j].
-__device__ __forceinline__ void block_step_var(float (&acc)[SF_QG], const float4 (&x)[4],
-                                               const float (&sc)[SF_QG],
-                                               const float *const *qrow, const int (&ds)[SF_QG],
-                                               int cnt, int off) {
-#pragma unroll
-  for (int j = 0; j < SF_QG; ++j) {
-    if (j >= cnt) break;
-    const int nd4 = min(4, (ds[j] - off) >> 2);
-    const float *qb = qrow[j] + off;
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      if (s >= nd4) break;
-      const float4 q = ldg4(qb + 4 * s);
-      float t;
-      t = fmaf(-sc[j], x[s].x, q.x);
-      acc[j] = fmaf(t, t, acc[j]);
-      t = fmaf(-sc[j], x[s].y, q.y);
-      acc[j] = fmaf(t, t, acc[j]);
-      t = fmaf(-sc[j], x[s].z, q.z);
-      acc[j] = fmaf(t, t, acc[j]);
-      t = fmaf(-sc[j], x[s].w, q.w);
-      acc[j] = fmaf(t, t, acc[j]);
-    }
+// The last tile whose first unit is <= item, found by a warp 32 tiles at a time.
+__device__ __forceinline__ int unit_tile(const int64_t *__restrict__ uoff, int ntiles,
+                                         int64_t item) {
+  int lo = 0, n = ntiles;  // it lies in [lo, lo + n)
+  while (n > 1) {
+    const int step = (n + 31) >> 5, i = lo + (int)(threadIdx.x & 31) * step;
+    const unsigned le = __ballot_sync(0xffffffffu, i < lo + n && uoff[i] <= item);
+    const int at = 31 - __clz(le);  // uoff[lo] <= item: lane 0 always votes
+    n = min(step, n - at * step);
+    lo += at * step;
   }
+  return lo;
 }
 
-// Per-query prefixes: units as in dist_f32_kernel; a unit's member rows are
-// streamed to the largest d_s of its queries.
-__global__ void __launch_bounds__(SF_THREADS, 4) dist_f32_var_kernel(StreamArgs a) {
+// VAR: every query its own d_s (see the file's header).
+template <bool VAR>
+__global__ void __launch_bounds__(SF_THREADS, SF_CTAS) dist_f32_kernel(StreamArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
-  __shared__ const float *s_qp[SF_QG];
+  __shared__ const float *s_qp[SF_QG];  // the unit's query rows
   __shared__ const float *s_sp[SF_QG];  // each query's per-member scales (or null)
   __shared__ int64_t s_pb[SF_QG];
   __shared__ int s_ds[SF_QG];
-  const int tid = threadIdx.x;
+  float4 *s_q = (float4 *)smem;  // [qg][a.dims / 4]
+  const int nq4 = a.dims >> 2, qg = a.qg, tid = threadIdx.x;
   const int64_t nunits = *a.nunits;
   const int ntiles = *a.ntiles_dev;
   for (;;) {
@@ -145,59 +142,91 @@ __global__ void __launch_bounds__(SF_THREADS, 4) dist_f32_var_kernel(StreamArgs 
     __syncthreads();
     const int64_t item = s_item;
     if (item >= nunits) break;
-    int lo = 0, hi = ntiles - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (a.uoff[mid] <= item) lo = mid; else hi = mid - 1;
-    }
-    const int tile = lo;
+    const int tile = unit_tile(a.uoff, ntiles, item);
     const int list = a.tile_list[tile], beg = a.tile_beg[tile], tcnt = a.tile_cnt[tile];
-    const int ngrp = (tcnt + SF_QG - 1) / SF_QG;
+    const int ngrp = (tcnt + qg - 1) / qg;
     const int u = (int)(item - a.uoff[tile]);
     const int chunk = u / ngrp, g = u - chunk * ngrp;
-    const int q0 = g * SF_QG, cnt = min(SF_QG, tcnt - q0);
-    if (tid < cnt) {
-      const int q = a.pair_q[beg + q0 + tid];
-      s_qp[tid] = a.qn + (int64_t)q * a.ldq;
-      s_pb[tid] = a.pbase[a.pair_out[beg + q0 + tid]];
-      s_ds[tid] = a.qds[q];
-      s_sp[tid] = a.invn ? a.invn + (int64_t)a.qgi[q] * a.N : nullptr;
+    const int q0 = g * qg, cnt = min(qg, tcnt - q0);
+    if (tid < 32) {  // rank of each of the tile's pairs by descending d_s
+      const int q = tid < tcnt ? a.pair_q[beg + tid] : 0;
+      const int ds = tid >= tcnt ? -1 : VAR ? a.qds[q] : a.dims;
+      int r = VAR ? 0 : tid;
+      if (VAR) {
+#pragma unroll
+        for (int i = 0; i < SF_QT; ++i) {
+          const int o = __shfl_sync(0xffffffffu, ds, i);
+          r += o > ds || (o == ds && i < tid);
+        }
+      }
+      const int j = r - q0;
+      if (tid < tcnt && j >= 0 && j < cnt) {
+        s_qp[j] = a.qn + (int64_t)q * a.ldq;
+        s_pb[j] = a.pbase[a.pair_out[beg + tid]];
+        if (VAR) {
+          s_ds[j] = ds;
+          s_sp[j] = a.invn ? a.invn + (int64_t)a.qgi[q] * a.N : nullptr;
+        }
+      }
     }
     __syncthreads();
+    for (int j = tid >> 5; j < cnt; j += SF_THREADS / 32) {
+      const int n4 = (VAR ? s_ds[j] : a.dims) >> 2;
+      for (int t = tid & 31; t < n4; t += 32) cp_async16(s_q + j * nq4 + t, s_qp[j] + 4 * t);
+    }
+    cp_async_commit();
     const int64_t moff = a.list_off[list];
     const int nl = (int)(a.list_off[list + 1] - moff), npad = (nl + 7) & ~7;
     const int m = chunk * SF_THREADS + tid;
-    if (m < nl) {
-      int ds[SF_QG], dmax = 0;
-      float sc[SF_QG];
+    const bool live = m < nl;
+    const int nblk = ((VAR ? s_ds[0] : a.dims) + 15) >> 4;
+    const float *xr = a.xpm + moff * (int64_t)a.d_pad + (int64_t)m * 16;
+    const int64_t bstride = (int64_t)16 * nl;
+    float4 x[2][4];
+    float sc[VAR ? SF_QG : 1], acc[SF_QG];
+    if (!VAR) sc[0] = live && a.mscale ? __ldg(a.mscale + moff + m) : 1.f;
 #pragma unroll
-      for (int j = 0; j < SF_QG; ++j) {
-        ds[j] = j < cnt ? s_ds[j] : 0;
-        sc[j] = j < cnt && s_sp[j] ? __ldg(s_sp[j] + moff + m) : 1.f;
-        dmax = max(dmax, ds[j]);
+    for (int b = 0; b < 2; ++b)
+      if (live && b < nblk) {
+#pragma unroll
+        for (int s = 0; s < 4; ++s) x[b][s] = ldg4(xr + b * bstride + 4 * s);
       }
-      const int nblk = (dmax + 15) >> 4;
-      const float *xr = a.xpm + moff * (int64_t)a.d_pad + (int64_t)m * 16;
-      const int64_t bstride = (int64_t)16 * nl;
-      const float *const *qrow = s_qp;
-      float acc[SF_QG];
 #pragma unroll
-      for (int j = 0; j < SF_QG; ++j) acc[j] = 0.f;
-      float4 xa[4], xb[4];
+    for (int j = 0; j < SF_QG; ++j) {
+      if (VAR) sc[j] = live && j < cnt && s_sp[j] ? __ldg(s_sp[j] + moff + m) : 1.f;
+      acc[j] = 0.f;
+    }
+    cp_async_wait<0>();
+    __syncthreads();  // the queries are staged
+    if (live) {
+      int na = cnt;  // queries that reach the current block
+      for (int b0 = 0; b0 < nblk; b0 += 2) {
 #pragma unroll
-      for (int s = 0; s < 4; ++s) xa[s] = ldg4(xr + 4 * s);
-      int b = 0;
-      for (; b + 2 <= nblk; b += 2) {
+        for (int b = 0; b < 2; ++b) {
+          if (b0 + b >= nblk) break;
+          const int off = 16 * (b0 + b);
+          if (VAR)
+            while (s_ds[na - 1] <= off) --na;  // the first one does
+          const float4 *qb = s_q + (off >> 2);
+          if ((VAR ? s_ds[na - 1] : a.dims) >= off + 16) {
 #pragma unroll
-        for (int s = 0; s < 4; ++s) xb[s] = ldg4(xr + (b + 1) * bstride + 4 * s);
-        block_step_var(acc, xa, sc, qrow, ds, cnt, 16 * b);
-        if (b + 2 < nblk) {
+            for (int j = 0; j < SF_QG; ++j) {
+              if (j >= na) break;
+              row_step<true>(acc[j], x[b], sc[VAR ? j : 0], qb + j * nq4, 4);
+            }
+          } else {
 #pragma unroll
-          for (int s = 0; s < 4; ++s) xa[s] = ldg4(xr + (b + 2) * bstride + 4 * s);
+            for (int j = 0; j < SF_QG; ++j) {
+              if (j >= na) break;
+              row_step<false>(acc[j], x[b], sc[VAR ? j : 0], qb + j * nq4, ((VAR ? s_ds[j] : a.dims) - off) >> 2);
+            }
+          }
+          if (b0 + b + 2 < nblk) {
+#pragma unroll
+            for (int s = 0; s < 4; ++s) x[b][s] = ldg4(xr + (b0 + b + 2) * bstride + 4 * s);
+          }
         }
-        block_step_var(acc, xb, sc, qrow, ds, cnt, 16 * (b + 1));
       }
-      if (b < nblk) block_step_var(acc, xa, sc, qrow, ds, cnt, 16 * b);
 #pragma unroll
       for (int j = 0; j < SF_QG; ++j)
         if (j < cnt) a.cand[s_pb[j] + m] = __float_as_uint(acc[j]);
@@ -205,79 +234,6 @@ __global__ void __launch_bounds__(SF_THREADS, 4) dist_f32_var_kernel(StreamArgs 
       for (int j = 0; j < cnt; ++j) a.cand[s_pb[j] + m] = 0xFFFFFFFFu;
     }
     __syncthreads();
-  }
-}
-
-__global__ void __launch_bounds__(SF_THREADS, 4) dist_f32_kernel(StreamArgs a) {
-  __shared__ int s_item;
-  __shared__ const float *s_qp[SF_QG];  // the unit's query rows
-  __shared__ int64_t s_pb[SF_QG];
-  const int tid = threadIdx.x;
-  const int64_t nunits = *a.nunits;
-  const int ntiles = *a.ntiles_dev;
-  const int nblk = (a.dims + 15) >> 4;
-  for (;;) {
-    if (tid == 0) s_item = atomicAdd(a.counter, 1);
-    __syncthreads();
-    const int64_t item = s_item;
-    if (item >= nunits) break;
-    // the tile holding this unit: the last tile whose first unit is <= item
-    int lo = 0, hi = ntiles - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (a.uoff[mid] <= item) lo = mid; else hi = mid - 1;
-    }
-    const int tile = lo;
-    const int list = a.tile_list[tile], beg = a.tile_beg[tile], tcnt = a.tile_cnt[tile];
-    const int ngrp = (tcnt + SF_QG - 1) / SF_QG;
-    const int u = (int)(item - a.uoff[tile]);
-    const int chunk = u / ngrp, g = u - chunk * ngrp;
-    const int q0 = g * SF_QG, cnt = min(SF_QG, tcnt - q0);
-    if (tid < cnt) {
-      s_qp[tid] = a.qn + (int64_t)a.pair_q[beg + q0 + tid] * a.ldq;
-      s_pb[tid] = a.pbase[a.pair_out[beg + q0 + tid]];
-    }
-    __syncthreads();
-    const int64_t moff = a.list_off[list];
-    const int nl = (int)(a.list_off[list + 1] - moff), npad = (nl + 7) & ~7;
-    const int m = chunk * SF_THREADS + tid;
-    if (m < nl) {
-      const float sc = a.mscale ? __ldg(a.mscale + moff + m) : 1.f;
-      const float *xr = a.xpm + moff * (int64_t)a.d_pad + (int64_t)m * 16;
-      const int64_t bstride = (int64_t)16 * nl;
-      const float *const *qrow = s_qp;
-      float acc[SF_QG];
-#pragma unroll
-      for (int j = 0; j < SF_QG; ++j) acc[j] = 0.f;
-      float4 xa[4], xb[4];
-#pragma unroll
-      for (int s = 0; s < 4; ++s) xa[s] = ldg4(xr + 4 * s);
-      int b = 0;
-      // two blocks per trip: the next block loads while this one is used
-      for (; b + 2 <= nblk; b += 2) {
-#pragma unroll
-        for (int s = 0; s < 4; ++s) xb[s] = ldg4(xr + (b + 1) * bstride + 4 * s);
-        block_step<true>(acc, xa, sc, qrow, cnt, 16 * b, 4);
-        if (b + 2 < nblk) {
-#pragma unroll
-          for (int s = 0; s < 4; ++s) xa[s] = ldg4(xr + (b + 2) * bstride + 4 * s);
-        }
-        const int nd4b = min(4, (a.dims - 16 * (b + 1)) >> 2);
-        if (nd4b == 4) block_step<true>(acc, xb, sc, qrow, cnt, 16 * (b + 1), 4);
-        else block_step<false>(acc, xb, sc, qrow, cnt, 16 * (b + 1), nd4b);
-      }
-      if (b < nblk) {  // odd block count: the last block is in xa
-        const int nd4 = min(4, (a.dims - 16 * b) >> 2);
-        if (nd4 == 4) block_step<true>(acc, xa, sc, qrow, cnt, 16 * b, 4);
-        else block_step<false>(acc, xa, sc, qrow, cnt, 16 * b, nd4);
-      }
-#pragma unroll
-      for (int j = 0; j < SF_QG; ++j)
-        if (j < cnt) a.cand[s_pb[j] + m] = __float_as_uint(acc[j]);
-    } else if (m < npad) {  // the segment's padding
-      for (int j = 0; j < cnt; ++j) a.cand[s_pb[j] + m] = 0xFFFFFFFFu;
-    }
-    __syncthreads();  // s_qp / s_pb are rewritten by the next unit
   }
 }
 
@@ -291,17 +247,17 @@ constexpr int SFF_THREADS = 64, SFF_PF = 6;
 
 template <bool VAR>
 __global__ void __launch_bounds__(SFF_THREADS) dist_f32_few_kernel(StreamArgs a) {
-  extern __shared__ __align__(16) float s_q[];  // [SF_QG][dims]
+  extern __shared__ __align__(16) float s_q[];  // [SFF_QG][dims]
   const int64_t nunits = *a.nunits;
   for (int64_t item = blockIdx.x; item < nunits; item += gridDim.x) {
     const int4 un = a.unit[item];  // (list, first pair, pairs, first member)
     const int cnt = un.z, m = un.w + threadIdx.x, nq4 = a.dims >> 2;
-    const float *sp[SF_QG];
-    int64_t pb[SF_QG];
-    int ds[SF_QG], dmax = VAR ? 0 : a.dims;
+    const float *sp[SFF_QG];
+    int64_t pb[SFF_QG];
+    int ds[SFF_QG], dmax = VAR ? 0 : a.dims;
     __syncthreads();  // the previous unit's queries are no longer read
 #pragma unroll
-    for (int j = 0; j < SF_QG; ++j) {
+    for (int j = 0; j < SFF_QG; ++j) {
       const int pr = un.y + min(j, cnt - 1), q = a.pair_q[pr];
       if (j < cnt) {
         const float4 *src = (const float4 *)(a.qn + (int64_t)q * a.ldq);
@@ -326,9 +282,9 @@ __global__ void __launch_bounds__(SFF_THREADS) dist_f32_few_kernel(StreamArgs a)
 #pragma unroll
         for (int s = 0; s < 4; ++s) x[b][s] = ldg4(xr + b * bstride + 4 * s);
       }
-    float sc[SF_QG], acc[SF_QG];
+    float sc[SFF_QG], acc[SFF_QG];
 #pragma unroll
-    for (int j = 0; j < SF_QG; ++j) {
+    for (int j = 0; j < SFF_QG; ++j) {
       sc[j] = m < nl && sp[j] ? __ldg(sp[j] + moff + m) : 1.f;
       acc[j] = 0.f;
     }
@@ -341,7 +297,7 @@ __global__ void __launch_bounds__(SFF_THREADS) dist_f32_few_kernel(StreamArgs a)
           if (b0 + b >= nblk) break;
           const int off = 16 * (b0 + b);
 #pragma unroll
-          for (int j = 0; j < SF_QG; ++j) {
+          for (int j = 0; j < SFF_QG; ++j) {
             if (j >= cnt) break;
             const int nd4 = (ds[j] - off) >> 2;
             const float4 *qb = (const float4 *)s_q + j * nq4 + (off >> 2);
@@ -367,11 +323,11 @@ __global__ void __launch_bounds__(SFF_THREADS) dist_f32_few_kernel(StreamArgs a)
         }
       }
 #pragma unroll
-      for (int j = 0; j < SF_QG; ++j)
+      for (int j = 0; j < SFF_QG; ++j)
         if (j < cnt) a.cand[pb[j] + m] = __float_as_uint(acc[j]);
     } else if (m < npad) {
 #pragma unroll
-      for (int j = 0; j < SF_QG; ++j)
+      for (int j = 0; j < SFF_QG; ++j)
         if (j < cnt) a.cand[pb[j] + m] = 0xFFFFFFFFu;
     }
   }
@@ -379,13 +335,38 @@ __global__ void __launch_bounds__(SFF_THREADS) dist_f32_few_kernel(StreamArgs a)
 
 }  // namespace
 
-// Few queries per probed list: prefer the streaming scan (ADANNS_OPT_FP32_STREAM = 0
-// keeps the shared-memory tiled scan everywhere)
-bool fp32_stream_enabled(double queries_per_list, int nprobe, int k, int d_s) {
+static int64_t stream_per_query(const adanns_index *idx, int d_c, int d_s, int nprobe, int k) {
+  return max_probe_members(idx, nprobe) * 4 + (int64_t)(pad16(d_c) + pad16(d_s)) * 4 +
+         (int64_t)k * 8 + (int64_t)nprobe * 40 + 16;
+}
+
+int64_t stream_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,
+                             int k) {
+  const int64_t per_q = stream_per_query(idx, d_c, d_s, nprobe, k);
+  const int64_t Bc = std::max<int64_t>(1, std::min<int64_t>(B, scratch_budget() / per_q));
+  return Bc * per_q + (int64_t)idx->nlist * 64 + (16ll << 20);
+}
+
+// Where the streaming scan is taken (ADANNS_OPT_FP32_STREAM = 0 keeps the
+// shared-memory tiled scan everywhere).  Up to 16 queries per probed list it
+// always is.  Above, per (query, member) in picoseconds, it spends 6 + 0.122 per
+// coordinate (0.166 beyond 1,024, where fewer staged rows fit) and the tiled scan
+// 9 + 0.27 k + 0.104 per coordinate, more while its tiles are not full: tiled
+// against streaming, 400,000 rows in 400 lists, 500 queries per list, k 10: d_s 64
+// 3.65 / 2.85 ms, 512 12.9 / 13.8, 1024 23.5 / 26.3; k 100: 8.4 / 3.0, 17.6 / 13.9,
+// 28.0 / 26.5; 100,000 x 2048, k 10, 32 and 64 queries per list: 1.39 / 1.19 and
+// 2.05 / 2.23.  The distances must fit the scratch at once, or in slices of at
+// least 64 queries per list, which still share their rows.
+bool fp32_stream_enabled(const adanns_index *idx, int64_t B, int64_t pairs, int d_c, int d_s,
+                         int nprobe, int k, bool budgets) {
   if (!option(ADANNS_OPT_FP32_STREAM) || nprobe > 256) return false;
-  const int t = k > 0 ? tuned_scan_tq(k, d_s, queries_per_list) : 0;
+  const double qpl = (double)pairs / idx->nlist;
+  const int t = budgets ? 0 : tuned_scan_tq(k, d_s, qpl);
   if (t != 0) return t == TUNE_STREAM;
-  return queries_per_list <= 16.0;
+  if (qpl <= 16.0) return true;
+  if (qpl * d_s > 65536.0 && k < (d_s <= 1024 ? (d_s - 256) / 14 : d_s / 4)) return false;
+  const int64_t fit = scratch_budget() / stream_per_query(idx, d_c, d_s, nprobe, k);
+  return fit >= B || (double)fit * pairs / B >= 64.0 * idx->nlist;
 }
 
 int search_f32_stream(const adanns_index *idx, const float *queries, int64_t B, int d_c, int d_s,
@@ -394,8 +375,7 @@ int search_f32_stream(const adanns_index *idx, const float *queries, int64_t B, 
   const int nlist = idx->nlist;
   const int dcp = pad16(d_c), dsp = pad16(d_s);
   const int64_t seg_q = max_probe_members(idx, nprobe);
-  const int64_t per_q =
-      seg_q * 4 + (int64_t)(dcp + dsp) * 4 + (int64_t)k * 8 + (int64_t)nprobe * 40 + 16;
+  const int64_t per_q = stream_per_query(idx, d_c, d_s, nprobe, k);
   const int64_t Bc = std::max<int64_t>(1, std::min<int64_t>(B, scratch_budget() / per_q));
   const int64_t max_tiles = (Bc * nprobe + SF_QT - 1) / SF_QT + nlist;
   // few members in all: small units (the whole batch is then one slice)
@@ -404,7 +384,9 @@ int search_f32_stream(const adanns_index *idx, const float *queries, int64_t B, 
       B * nprobe * (((int64_t)idx->max_list + 7 + SFF_THREADS) / SFF_THREADS);
   const bool few = Bc >= B && probe_plan_small(B * nprobe, nlist) && max_units <= 1 << 20 &&
                    (double)B * nprobe * idx->N / nlist <= (double)num_sms() * 1024;
+  const bool var = qb && qb->ds;
   const int um = few ? SFF_THREADS : SF_THREADS;
+  const int qg = few ? SFF_QG : std::max(1, std::min(SF_QG, SF_SMEM / (d_s * 4)));
   Scratch s(st);
   float *qc, *qs;
   uint64_t *ckeys;
@@ -452,7 +434,7 @@ int search_f32_stream(const adanns_index *idx, const float *queries, int64_t B, 
       plan.qbase = qbase;
       plan.pbase = pbase;
       plan.unit_members = um;
-      plan.unit_queries = SF_QG;
+      plan.unit_queries = qg;
       plan.uoff = uoff;
       plan.nunits = nunits;
       plan.unit = unit;
@@ -468,7 +450,7 @@ int search_f32_stream(const adanns_index *idx, const float *queries, int64_t B, 
       StageTimer t(ST_SCAN, st);
       if (!plan.planned) {
         stream_units_kernel<<<(unsigned)((max_tiles + 255) / 256), 256, 0, st>>>(
-            tl, tc, ntiles, idx->list_off, max_tiles, units);
+            tl, tc, ntiles, idx->list_off, max_tiles, um, qg, units);
         ADN_LAUNCH("stream_units_kernel");
         if ((rc = launch_scan64(units, max_tiles, uoff, nunits, st))) return rc;
       }
@@ -496,27 +478,30 @@ int search_f32_stream(const adanns_index *idx, const float *queries, int64_t B, 
       a.qgi = bq.gi;
       a.invn = idx->metric == ADANNS_METRIC_L2_PREFIXNORM ? idx->invn : nullptr;
       a.N = idx->N;
+      a.qg = qg;
       if (few) {
         // about as many CTAs as units if no query shared a list
         const int64_t est = nb * nprobe * (idx->N / nlist / SFF_THREADS + 1);
         const unsigned grid =
             (unsigned)std::min<int64_t>(std::min(max_units, est), (int64_t)num_sms() * 16);
-        const size_t sm = (size_t)SF_QG * d_s * 4;
+        const size_t sm = (size_t)SFF_QG * d_s * 4;
         auto kern = bq.ds ? dist_f32_few_kernel<true> : dist_f32_few_kernel<false>;
         ADN_CUDA(ensure_smem((const void *)kern, sm));
         kern<<<grid, SFF_THREADS, sm, st>>>(a);
         ADN_LAUNCH("dist_f32_few_kernel");
       } else {
-        auto kern = bq.ds ? dist_f32_var_kernel : dist_f32_kernel;
+        auto kern = var ? dist_f32_kernel<true> : dist_f32_kernel<false>;
+        const size_t sm = (size_t)qg * d_s * 4;
+        ADN_CUDA(ensure_smem((const void *)kern, sm));
         int per_sm = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SF_THREADS, 0) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, um, sm) !=
                 cudaSuccess ||
             per_sm < 1) {
           cudaGetLastError();
           per_sm = 1;
         }
-        kern<<<num_sms() * per_sm, SF_THREADS, 0, st>>>(a);
-        ADN_LAUNCH(bq.ds ? "dist_f32_var_kernel" : "dist_f32_kernel");
+        kern<<<num_sms() * per_sm, um, sm, st>>>(a);
+        ADN_LAUNCH("dist_f32_kernel");
       }
     }
     {
