@@ -12,9 +12,9 @@
 // are left to it.
 //
 // Measured: 8,000 queries, 32 of 1,024 lists, 5.25 M rows, 32-byte codes of 384
-// coordinates, rerank 400: 24.2 -> 8.5 ms (ADC stage and selection 22.0 -> 5.6:
-// decode 1.3, tensor cores 2.2, shortlist 1.1 of 494 members per query, exact
-// scores 0.8); one list of 1.28 M 16-byte codes, 1,000 queries: 10.9 -> 2.1 ms.
+// coordinates, rerank 400: 24.2 -> 7.0 ms (ADC stage and selection 22.0 -> 5.2:
+// decode 1.05, tensor cores 1.96, shortlist 1.2 of 494 members per query, exact
+// scores 0.8); one list of 1.28 M 16-byte codes, 1,000 queries: 10.9 -> 1.9 ms.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -28,7 +28,8 @@ namespace {
 
 constexpr float AC_Y2MAX = 4.f;  // largest squared norm of a decoded row
 constexpr int AC_MAX_M = 96;     // lookup table of one query in shared memory
-constexpr int AC_CHUNKS = 32;    // 64-member chunks per decode CTA
+constexpr int AC_CTAS = 6;       // decode CTAs per SM (their tables: 192 KB)
+constexpr int AC_WAVES = 2;
 
 // c2[m][c] = |C_m[c]|^2
 __global__ void codeword_norms_kernel(const float *__restrict__ C, int n, int dsub,
@@ -59,13 +60,18 @@ __global__ void code_norms_kernel(const uint8_t *__restrict__ codes, const float
 // coordinates), in the scan's layout [(off nkb + kb n_l + m)][64].  The block's
 // slice of the codebook is staged in shared memory as [16 groups of 4
 // coordinates][256 codes] (32 KB), so that a member's row is 16 eight-byte
-// lookups; eight lanes write a row's 128 bytes.  VEC4: the groups do not cross
+// lookups; eight lanes write a row's 128 bytes.  The chunk after the next and the
+// next one's codes are on their way meanwhile (a CTA has only 8 KB of a chunk to
+// write per chain of dependent reads), and a CTA takes as many chunks as make two
+// waves of CTAs, since staging the table costs as much as a few dozen of them:
+// 5.25 M rows x 384 1.38 -> 1.05 ms (two thirds of the measured copy bandwidth);
+// four waves 1.05, one or two of 1.28 M x 128 0.12, four 0.16.  VEC4: the groups do not cross
 // sub-vectors (d_s / M a multiple of 4), else each coordinate looks up its own
 // code.
 template <bool VEC4>
 __global__ void __launch_bounds__(256) decode_f16_kernel(
     const uint8_t *__restrict__ codes, int M, int dsub, const float *__restrict__ C,
-    const int4 *__restrict__ cmap, int nchunk, const int32_t *__restrict__ lcnt, int nkb,
+    const int4 *__restrict__ cmap, int nchunk, int per, const int32_t *__restrict__ lcnt, int nkb,
     uint4 *__restrict__ out) {
   __shared__ __align__(16) __half tab[16 * 256 * 4];
   const int kb = blockIdx.y, d_s = M * dsub;
@@ -83,25 +89,49 @@ __global__ void __launch_bounds__(256) decode_f16_kernel(
   int ms[8];  // their sub-vectors
 #pragma unroll
   for (int u = 0; u < 8; ++u) ms[u] = j0 + u < d_s ? (j0 + u) / dsub : -1;
-  const int ch0 = blockIdx.x * AC_CHUNKS, ch1 = min(nchunk, ch0 + AC_CHUNKS);
+  const int ch0 = blockIdx.x * per, ch1 = min(nchunk, ch0 + per);
+  // a chunk (list, first member, list offset, list size); size 0: nothing to write
+  auto head = [&](int ch) {
+    int4 cl = make_int4(0, 0, 0, 0);
+    if (ch < ch1) {
+      cl = cmap[ch];
+      if (lcnt && lcnt[cl.x] == 0) cl.w = 0;
+    }
+    return cl;
+  };
+  // this lane's codes of the chunk's two members
+  constexpr int NC = VEC4 ? 2 : 8;
+  auto fetch = [&](const int4 &cl, uint32_t(&r)[2][NC]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int m = cl.y + 32 * h + (threadIdx.x >> 3);
+      const uint8_t *cp = codes + ((int64_t)cl.z + m) * M;
+#pragma unroll
+      for (int u = 0; u < NC; ++u) {
+        const int sv = ms[VEC4 ? 4 * u : u];
+        r[h][u] = m < cl.w && sv >= 0 ? cp[sv] : 0u;
+      }
+    }
+  };
+  int4 cl = head(ch0), nx = head(ch0 + 1);
+  uint32_t cd[2][NC], cn[2][NC];
+  fetch(cl, cd);
   for (int ch = ch0; ch < ch1; ++ch) {
-    const int4 cl = cmap[ch];  // (list, first member, list offset, list size)
-    if (lcnt && lcnt[cl.x] == 0) continue;
-    const int64_t off = cl.z;
+    const int4 n2 = head(ch + 2);
+    fetch(nx, cn);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int m = cl.y + 32 * h + (threadIdx.x >> 3);
       if (m >= cl.w) continue;
-      const uint8_t *cp = codes + (off + m) * M;
       uint4 r = make_uint4(0u, 0u, 0u, 0u);
       if (VEC4) {
         if (ms[0] >= 0) {
-          const uint2 a = *(const uint2 *)(tab + 2 * c8 * 1024 + cp[ms[0]] * 4);
+          const uint2 a = *(const uint2 *)(tab + 2 * c8 * 1024 + cd[h][0] * 4);
           r.x = a.x;
           r.y = a.y;
         }
         if (ms[4] >= 0) {
-          const uint2 a = *(const uint2 *)(tab + (2 * c8 + 1) * 1024 + cp[ms[4]] * 4);
+          const uint2 a = *(const uint2 *)(tab + (2 * c8 + 1) * 1024 + cd[h][1] * 4);
           r.z = a.x;
           r.w = a.y;
         }
@@ -109,14 +139,20 @@ __global__ void __launch_bounds__(256) decode_f16_kernel(
         unsigned short hv[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-          hv[u] = ms[u] >= 0 ? __half_as_ushort(tab[(2 * c8 + (u >> 2)) * 1024 + cp[ms[u]] * 4 +
-                                                    (u & 3)])
+          hv[u] = ms[u] >= 0 ? __half_as_ushort(tab[(2 * c8 + (u >> 2)) * 1024 +
+                                                    cd[h][VEC4 ? 0 : u] * 4 + (u & 3)])
                              : (unsigned short)0;
         r = make_uint4(hv[0] | (uint32_t)hv[1] << 16, hv[2] | (uint32_t)hv[3] << 16,
                        hv[4] | (uint32_t)hv[5] << 16, hv[6] | (uint32_t)hv[7] << 16);
       }
-      out[(off * nkb + (int64_t)kb * cl.w + m) * 8 + c8] = r;
+      out[((int64_t)cl.z * nkb + (int64_t)kb * cl.w + m) * 8 + c8] = r;
     }
+    cl = nx;
+    nx = n2;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int u = 0; u < NC; ++u) cd[h][u] = cn[h][u];
   }
 }
 
@@ -237,9 +273,11 @@ int launch_decode_f16(const adanns_index *idx, const int32_t *lcnt, int nkb, voi
                       cudaStream_t st) {
   const int M = idx->opq_M, dsub = idx->opq_ds / M, nch = idx->rr_chunks[0];
   if (nch <= 0) return ADANNS_OK;
-  const dim3 grid((nch + AC_CHUNKS - 1) / AC_CHUNKS, nkb);
+  const int64_t ctas = (int64_t)num_sms() * AC_CTAS * AC_WAVES;
+  const int per = (int)std::max<int64_t>(16, ((int64_t)nch * nkb + ctas - 1) / ctas);
+  const dim3 grid((nch + per - 1) / per, nkb);
   auto kern = dsub % 4 == 0 ? decode_f16_kernel<true> : decode_f16_kernel<false>;
-  kern<<<grid, 256, 0, st>>>(idx->codes, M, dsub, idx->opq_C, idx->rr_cmap[0], nch, lcnt, nkb,
+  kern<<<grid, 256, 0, st>>>(idx->codes, M, dsub, idx->opq_C, idx->rr_cmap[0], nch, per, lcnt, nkb,
                              (uint4 *)rows);
   ADN_LAUNCH("decode_f16_kernel");
   return ADANNS_OK;
