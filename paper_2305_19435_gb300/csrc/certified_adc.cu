@@ -14,7 +14,7 @@
 // Measured: 8,000 queries, 32 of 1,024 lists, 5.25 M rows, 32-byte codes of 384
 // coordinates, rerank 400: 24.2 -> 7.0 ms (ADC stage and selection 22.0 -> 5.2:
 // decode 1.05, tensor cores 1.96, shortlist 1.2 of 494 members per query, exact
-// scores 0.8); one list of 1.28 M 16-byte codes, 1,000 queries: 10.9 -> 1.9 ms.
+// scores 0.8); one list of 1.28 M 16-byte codes, 1,000 queries: 10.9 -> 1.7 ms.
 #include <cuda_fp16.h>
 
 #include <algorithm>

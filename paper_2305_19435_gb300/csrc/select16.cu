@@ -26,6 +26,7 @@ namespace {
 constexpr int SW_WARPS = 4;
 constexpr int SW_SAMPLE = 2048;
 constexpr int SW_BUF = 1024;
+constexpr int64_t CERT_FEW = 8;  // queries per SM: certify16_kernel's line between its variants
 constexpr int SW_TIE = 128;
 constexpr int SW_MAXP = 128;
 constexpr int SW_PF = 12;
@@ -336,7 +337,12 @@ __global__ void __launch_bounds__(SW_WARPS * 32, 6) select16_kernel(
 // k-th smallest of a part is at least that of the whole), so the pass never
 // needs a second one unless the sampled T was too low.  More than kk
 // candidates, or more than the buffer holds within the bound: cnt[q] = -1.
-__global__ void __launch_bounds__(SW_WARPS * 32, 6) certify16_kernel(
+// HB: 16-byte loads per lane and half of the pipeline.  Up to CERT_FEW queries
+// per SM the warps are too few to cover the reads' latency with 6 (six CTAs per
+// SM fit): 1,000 queries of 1.28 M keys 848 us with 6, 634 with 10, 665 with 16,
+// 787 with 24; 1,000 of 31,000 89 and 82; no difference at 2,000.
+template <int HB, int CTAS>
+__global__ void __launch_bounds__(SW_WARPS * 32, CTAS) certify16_kernel(
     const uint16_t *__restrict__ cand, const uint64_t *__restrict__ ckeys, int nprobe,
     const int64_t *__restrict__ qbase, const int64_t *__restrict__ list_off, int kk, int k,
     const float *__restrict__ qerr, int64_t B, int64_t *__restrict__ out,
@@ -390,7 +396,6 @@ __global__ void __launch_bounds__(SW_WARPS * 32, 6) certify16_kernel(
             warp_kth16(ns, r + 1, [&](int i) -> uint32_t { return s.u.samp[i]; }, s, b_, n_) + 1u);
     __syncwarp();  // the sample's space becomes the buffer
   }
-  constexpr int HB = SW_PF / 2;
   auto load = [&](uint4(&v)[HB], int cb) {
 #pragma unroll
     for (int f = 0; f < HB; ++f) {
@@ -748,8 +753,9 @@ int launch_certify16(const uint16_t *cand, const uint64_t *ckeys, int nprobe, co
     return fail(ADANNS_ERR_ARG, "certify16: shape outside its buffers");
   if (B <= 0) return ADANNS_OK;
   const size_t sm = sizeof(SwState) * SW_WARPS;
-  ADN_CUDA(ensure_smem((const void *)certify16_kernel, sm));
-  certify16_kernel<<<(unsigned)((B + SW_WARPS - 1) / SW_WARPS), SW_WARPS * 32, sm, st>>>(
+  auto kern = B <= CERT_FEW * num_sms() ? certify16_kernel<10, 3> : certify16_kernel<SW_PF / 2, 6>;
+  ADN_CUDA(ensure_smem((const void *)kern, sm));
+  kern<<<(unsigned)((B + SW_WARPS - 1) / SW_WARPS), SW_WARPS * 32, sm, st>>>(
       cand, ckeys, nprobe, qbase, list_off, kk, k, qerr, B, out, cnt, stats);
   ADN_LAUNCH("certify16_kernel");
   return ADANNS_OK;
