@@ -20,9 +20,9 @@
 // on those queries alone.
 //
 // Measured (1,281,167 x 2048, 50,000 queries, d_s 512, 16 of 1,024 lists,
-// k 100): 83.4 ms by the tiled scan (36% of the FFMA peak), 5.62 ms here: FP16
-// rows 0.75, tensor-core scan 1.44, shortlist 0.95, re-score of the 118 members
-// per query left by the bound 1.85, the rest 0.6.
+// k 100): 83.4 ms by the tiled scan (36% of the FFMA peak), 5.25 ms here: FP16
+// rows 0.58, tensor-core scan 1.45, shortlist 1.0, re-score of the 118 members
+// per query left by the bound 1.7, the rest 0.5.
 //
 // The bound.  With u = 2^-11 (FP16 rounding; entries of a unit vector below
 // 2^-14 lose at most 2^-25 each), p = P(q), y = P(x) of norm at most 1.005:
