@@ -791,7 +791,10 @@ int adanns_search_ivf_budgets(const adanns_index *idx, const float *queries, int
   if (B == 0) return ADANNS_OK;
   // FP32 with many queries per probed list: the tiled scan, one launch
   // sequence per distinct d_s over that group of queries (rows in place)
-  const bool tiled = !lowp && !fp32_stream_enabled(idx, B, np_sum, d_c, ds_max, np_max, k_max, true);
+  int64_t ds_sum = 0;
+  for (int64_t i = 0; i < B; ++i) ds_sum += d_s[i];
+  const bool tiled = !lowp && !fp32_stream_enabled(idx, B, np_sum, d_c, ds_max, np_max, k_max,
+                                                   (int)(ds_sum / B));
   std::vector<std::pair<int64_t, int64_t>> grp;  // [begin, end) of each d_s group in the order
   if (tiled) {
     std::vector<int32_t> perm((size_t)B);

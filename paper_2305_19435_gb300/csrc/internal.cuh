@@ -383,9 +383,10 @@ int launch_cand_segments(const uint64_t *ckeys, int64_t B, int nprobe, const int
 int launch_scan_i32(const int32_t *v, int64_t n, int32_t *out, cudaStream_t st);
 int launch_scan64(const int64_t *in, int64_t n, int64_t *out, int64_t *total, cudaStream_t st);
 // the streaming FP32 scan for this batch shape (the autotuned choice when the
-// bucket is tuned, else few queries per probed list); pairs: (query, list) pairs
+// bucket is tuned, else by a rule); pairs: (query, list) pairs; mean_ds: of a batch
+// with a d_s per query (d_s the largest), else 0
 bool fp32_stream_enabled(const adanns_index *idx, int64_t B, int64_t pairs, int d_c, int d_s,
-                         int nprobe, int k, bool budgets = false);
+                         int nprobe, int k, int mean_ds = 0);
 // scratch bytes of search_f32_stream for these arguments (host arithmetic)
 int64_t stream_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,
                              int k);
