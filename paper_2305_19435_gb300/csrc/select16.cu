@@ -440,6 +440,7 @@ __global__ void __launch_bounds__(SW_WARPS * 32, CTAS) certify16_kernel(
       const uint32_t kv = i < n ? s.u.b.key[i] : 0xFFFFFFFFu;
       const uint32_t ix = i < n ? s.u.b.idx[i] : 0u;
       const unsigned b = __ballot_sync(0xffffffffu, kv < T);
+      __syncwarp();  // every lane has read its entry before any is overwritten
       if (kv < T) {
         const int d = w + __popc(b & lanemask_lt());
         s.u.b.key[d] = (uint16_t)kv;
@@ -468,8 +469,8 @@ __global__ void __launch_bounds__(SW_WARPS * 32, CTAS) certify16_kernel(
       for (int f = 0; f < HB; ++f) collect(v[f], cb + f * 32 + lane);
       __syncwarp();
       int m = s.n;
+      __syncwarp();  // every lane has read the count before the next keys add to it
       if (m > SW_BUF) {  // again, 64 keys at a time, tightening in between
-        __syncwarp();
         if (lane == 0) s.n = n;
         __syncwarp();
         m = n;
