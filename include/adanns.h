@@ -122,6 +122,11 @@ int64_t adanns_launch_count(void);
  *                             path runs (nothing happens when item 0 has fewer
  *                             loads).  That call's results are invalid.  Never
  *                             needed outside tests.
+ *   ADANNS_OPT_TEST_SCRATCH_LIMIT  test hook, -1 (default).  n >= 0: the
+ *                             library's scratch allocations fail, as if the
+ *                             device had no more memory, where they would bring
+ *                             the scratch of all calls in progress above n
+ *                             bytes.
  * adanns_set_option returns ADANNS_ERR_ARG for an unknown option or a value
  * out of range (the option keeps its value).
  */
@@ -134,7 +139,8 @@ int64_t adanns_launch_count(void);
 #define ADANNS_OPT_TEST_SKIP_LOAD 6
 #define ADANNS_OPT_SCAN_FILTER 7
 #define ADANNS_OPT_NARROW_SCAN 8
-#define ADANNS_OPT_COUNT 9
+#define ADANNS_OPT_TEST_SCRATCH_LIMIT 9
+#define ADANNS_OPT_COUNT 10
 int adanns_set_option(int option, int64_t value);
 int adanns_get_option(int option, int64_t *value);
 
@@ -307,7 +313,9 @@ int adanns_kmeans_update(const float *points, int64_t n, int ld, int dim, int me
  *            of the query's k-th nearest (scratch: 2 d_s bytes per database
  *            row, at most half of ADANNS_OPT_SCRATCH_BYTES), and the scan's own
  *            FP32 arithmetic re-scores those.  ADANNS_FP32_STREAM=0 keeps the
- *            shared-memory tiled scan.  All give the same result, bit for bit.
+ *            shared-memory tiled scan.  All give the same result, bit for bit,
+ *            and a batch whose scratch cannot be had for one of the first two
+ *            takes the next (the tiled scan's slices hold 2 GiB at most).
  *            ADANNS_STORE_BF16 / ADANNS_STORE_FP8E4M3 (tier built into the
  *            index, metric ADANNS_METRIC_L2_PREFIXNORM, nprobe <= 128): the
  *            probed lists are scanned on the tensor cores with FP32

@@ -120,6 +120,7 @@ OPT_WAIT_LIMIT_NS = 5
 OPT_TEST_SKIP_LOAD = 6
 OPT_SCAN_FILTER = 7
 OPT_NARROW_SCAN = 8
+OPT_TEST_SCRATCH_LIMIT = 9
 
 
 def set_option(opt: int, value: int):

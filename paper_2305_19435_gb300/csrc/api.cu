@@ -619,6 +619,30 @@ int search_f32_tiled(const adanns_index *idx, const float *queries, int64_t B, i
   return ADANNS_OK;
 }
 
+// A route that cannot get its scratch leaves the batch to the next one: the
+// filter and the streaming scan size their slices by the scratch budget, the
+// tiled scan holds 2 GiB at most.  (A variant that the autotuner is timing is
+// not replaced.)
+int search_f32(const adanns_index *idx, const float *queries, int64_t B, int d_c, int d_s,
+               int nprobe, int k, int64_t *out_ids, float *out_dist, int32_t *out_probes,
+               cudaStream_t st, int first, int *took) {
+  for (int r = first;; ++r) {
+    if (r == F32_FILTER && !f32_certified(idx, B, d_s, nprobe, k)) continue;
+    if (r == F32_STREAM && !fp32_stream_enabled(idx, B, B * nprobe, d_c, d_s, nprobe, k)) continue;
+    if (took) *took = r;
+    const int rc = r == F32_FILTER
+                       ? search_f32_certified(idx, queries, B, d_c, d_s, nprobe, k, out_ids,
+                                              out_dist, out_probes, st)
+                   : r == F32_STREAM
+                       ? search_f32_stream(idx, queries, B, d_c, d_s, nprobe, k, out_ids, out_dist,
+                                           out_probes, st)
+                       : search_f32_tiled(idx, queries, B, d_c, d_s, nprobe, k, out_ids, out_dist,
+                                          out_probes, st);
+    if (rc != ADANNS_ERR_OOM || r >= F32_TILED || scan_choice_forced()) return rc;
+    release_scratch(st);
+  }
+}
+
 }  // namespace adn
 
 extern "C" {
@@ -729,15 +753,8 @@ int adanns_search_ivf(const adanns_index *idx, const float *queries, int64_t B, 
   if (storage != ADANNS_STORE_F32) return fail(ADANNS_ERR_ARG, "unknown storage tier");
   if (rerank_k != 0) return fail(ADANNS_ERR_ARG, "rerank_k must be 0 for the FP32 scan");
   if (B == 0) return ADANNS_OK;
-  cudaStream_t st = S(cuda_stream);
-  if (f32_certified(idx, B, d_s, nprobe, k))
-    return search_f32_certified(idx, queries, B, d_c, d_s, nprobe, k, out_ids, out_dist,
-                                out_probes, st);
-  if (fp32_stream_enabled(idx, B, B * nprobe, d_c, d_s, nprobe, k))
-    return search_f32_stream(idx, queries, B, d_c, d_s, nprobe, k, out_ids, out_dist, out_probes,
-                             st);
-  return search_f32_tiled(idx, queries, B, d_c, d_s, nprobe, k, out_ids, out_dist, out_probes,
-                          st);
+  return search_f32(idx, queries, B, d_c, d_s, nprobe, k, out_ids, out_dist, out_probes,
+                    S(cuda_stream));
 }
 
 int adanns_search_ivf_budgets(const adanns_index *idx, const float *queries, int64_t B, int d_c,
@@ -789,14 +806,15 @@ int adanns_search_ivf_budgets(const adanns_index *idx, const float *queries, int
     return fail(ADANNS_ERR_ARG, "rerank_k must be 0 for the FP32 scan");
   }
   if (B == 0) return ADANNS_OK;
-  // FP32 with many queries per probed list: the tiled scan, one launch
-  // sequence per distinct d_s over that group of queries (rows in place)
+  // FP32 with many queries per probed list, or without the streaming scan's
+  // scratch: the tiled scan, one launch sequence per distinct d_s over that
+  // group of queries (rows in place)
   int64_t ds_sum = 0;
   for (int64_t i = 0; i < B; ++i) ds_sum += d_s[i];
   const bool tiled = !lowp && !fp32_stream_enabled(idx, B, np_sum, d_c, ds_max, np_max, k_max,
                                                    (int)(ds_sum / B));
   std::vector<std::pair<int64_t, int64_t>> grp;  // [begin, end) of each d_s group in the order
-  if (tiled) {
+  auto group = [&] {
     std::vector<int32_t> perm((size_t)B);
     for (int64_t i = 0; i < B; ++i) perm[(size_t)i] = (int32_t)i;
     std::stable_sort(perm.begin(), perm.end(),
@@ -809,7 +827,8 @@ int adanns_search_ivf_budgets(const adanns_index *idx, const float *queries, int
       if (i == 0 || d_s[r] != d_s[perm[(size_t)i - 1]]) grp.push_back({i, i + 1});
       else grp.back().second = i + 1;
     }
-  }
+  };
+  if (tiled) group();
   cudaStream_t st = S(cuda_stream);
   Scratch s(st);
   int32_t *dq;
@@ -826,24 +845,28 @@ int adanns_search_ivf_budgets(const adanns_index *idx, const float *queries, int
     return search_mixed(idx, queries, B, d_c, ds_max, np_max, k_max, which, rerank_k, out_ids,
                         out_dist, nullptr, st, &qb);
   }
-  if (tiled) {
-    for (const auto &g : grp) {
-      const int32_t *perm = dq + 4 * B + g.first;
-      int gnp = 0;
-      for (int64_t i = g.first; i < g.second; ++i)
-        gnp = std::max(gnp, (int)h[(size_t)(5 * B + i)]);
-      QueryBudgets gb;
-      gb.np = dq + 5 * B + g.first;
-      gb.k = dq + 6 * B + g.first;
-      if ((rc = search_f32_tiled(idx, queries, g.second - g.first, d_c,
-                                 d_s[h[(size_t)(4 * B + g.first)]], gnp, k_max, out_ids, out_dist,
-                                 nullptr, st, &gb, perm)))
-        return rc;
-    }
-    return ADANNS_OK;
-  }
-  return search_f32_stream(idx, queries, B, d_c, ds_max, np_max, k_max, out_ids, out_dist, nullptr,
+  if (!tiled) {
+    rc = search_f32_stream(idx, queries, B, d_c, ds_max, np_max, k_max, out_ids, out_dist, nullptr,
                            st, &qb);
+    if (rc != ADANNS_ERR_OOM) return rc;
+    release_scratch(st);
+    group();
+    ADN_CUDA(cudaMemcpyAsync(dq, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+  }
+  for (const auto &g : grp) {
+    const int32_t *perm = dq + 4 * B + g.first;
+    int gnp = 0;
+    for (int64_t i = g.first; i < g.second; ++i)
+      gnp = std::max(gnp, (int)h[(size_t)(5 * B + i)]);
+    QueryBudgets gb;
+    gb.np = dq + 5 * B + g.first;
+    gb.k = dq + 6 * B + g.first;
+    if ((rc = search_f32_tiled(idx, queries, g.second - g.first, d_c,
+                               d_s[h[(size_t)(4 * B + g.first)]], gnp, k_max, out_ids, out_dist,
+                               nullptr, st, &gb, perm)))
+      return rc;
+  }
+  return ADANNS_OK;
 }
 
 }  // extern "C"

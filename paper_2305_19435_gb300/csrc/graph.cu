@@ -45,21 +45,45 @@ int adanns_plan_create(const adanns_index *idx, const float *queries, int64_t B,
     destroy(p);
     return cuda_fail(e, "plan stream");
   }
-  e = cudaStreamBeginCapture(p->cap, cudaStreamCaptureModeRelaxed);
+  // a graph's scratch is its own, on top of the pool's: an FP32 route whose graph
+  // cannot have it leaves the plan to the next
+  int first = F32_FILTER;
+  for (;;) {
+    e = cudaStreamBeginCapture(p->cap, cudaStreamCaptureModeRelaxed);
+    if (e != cudaSuccess) {
+      destroy(p);
+      return cuda_fail(e, "begin capture");
+    }
+    int took = F32_TILED;
+    rc = storage == ADANNS_STORE_F32 && B > 0
+             ? search_f32(idx, queries, B, d_c, d_s, nprobe, k, out_ids, out_dist, nullptr, p->cap,
+                          first, &took)
+             : adanns_search_ivf(idx, queries, B, d_c, d_s, nprobe, k, storage, rerank_k, out_ids,
+                                 out_dist, nullptr, p->cap);
+    e = cudaStreamEndCapture(p->cap, &p->graph);
+    if (rc) {
+      destroy(p);
+      return rc;
+    }
+    if (e != cudaSuccess) {
+      destroy(p);
+      return cuda_fail(e, "end capture");
+    }
+    e = cudaGraphInstantiate(&p->exec, p->graph, 0);
+    // (its memory is mapped by the upload, otherwise by the first launch)
+    if (e == cudaSuccess && took < F32_TILED && (e = cudaGraphUpload(p->exec, p->cap)) == cudaSuccess)
+      e = cudaStreamSynchronize(p->cap);
+    if (e != cudaErrorMemoryAllocation || took >= F32_TILED) break;
+    cudaGetLastError();
+    if (p->exec) cudaGraphExecDestroy(p->exec);
+    cudaGraphDestroy(p->graph);
+    p->exec = nullptr;
+    p->graph = nullptr;
+    first = took + 1;
+  }
   if (e != cudaSuccess) {
     destroy(p);
-    return cuda_fail(e, "begin capture");
-  }
-  rc = adanns_search_ivf(idx, queries, B, d_c, d_s, nprobe, k, storage, rerank_k, out_ids,
-                         out_dist, nullptr, p->cap);
-  e = cudaStreamEndCapture(p->cap, &p->graph);
-  if (rc) {
-    destroy(p);
-    return rc;
-  }
-  if (e != cudaSuccess) {
-    destroy(p);
-    return cuda_fail(e, "end capture");
+    return cuda_fail(e, "instantiate");
   }
   size_t nn = 0;
   if (cudaGraphGetNodes(p->graph, nullptr, &nn) == cudaSuccess && nn > 0) {
@@ -71,11 +95,6 @@ int adanns_plan_create(const adanns_index *idx, const float *queries, int64_t B,
       }
   }
   cudaGetLastError();
-  e = cudaGraphInstantiate(&p->exec, p->graph, 0);
-  if (e != cudaSuccess) {
-    destroy(p);
-    return cuda_fail(e, "instantiate");
-  }
   *out = p;
   return ADANNS_OK;
 }

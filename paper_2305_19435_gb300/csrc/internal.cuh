@@ -128,6 +128,9 @@ int64_t take_option(int opt, int64_t reset);
 int set_option(int opt, int64_t value);
 int64_t max_probe_members(const adanns_index *idx, int nprobe);
 
+extern std::atomic<int64_t> g_scratch_held;  // bytes held by all calls in progress
+void release_scratch(cudaStream_t st);       // after an allocation failed
+
 // Stream-ordered scratch allocation from that pool on the call's stream.
 // Arrays of up to SLAB_MAX bytes are cut from slabs of SLAB bytes: a search
 // asks for some 25 arrays, and an allocation and a release by the pool cost the
@@ -137,6 +140,7 @@ struct Scratch {
   cudaStream_t st;
   void *ptrs[64];
   int n = 0;
+  int64_t held = 0;
   char *slab = nullptr;
   size_t left = 0;
   explicit Scratch(cudaStream_t s) : st(s) {}
@@ -144,18 +148,25 @@ struct Scratch {
   Scratch &operator=(const Scratch &) = delete;
   ~Scratch() {
     for (int i = 0; i < n; ++i) cudaFreeAsync(ptrs[i], st);
+    g_scratch_held.fetch_sub(held, std::memory_order_relaxed);
   }
   int alloc(void **out, size_t bytes) {
     void *p = nullptr;
+    const int64_t lim = option(ADANNS_OPT_TEST_SCRATCH_LIMIT);
     cudaMemPool_t pool = scratch_pool();
-    cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, bytes, pool, st)
-                         : cudaMallocAsync(&p, bytes, st);
+    const cudaError_t e =
+        lim >= 0 && g_scratch_held.load(std::memory_order_relaxed) + (int64_t)bytes > lim
+            ? cudaErrorMemoryAllocation
+        : pool ? cudaMallocFromPoolAsync(&p, bytes, pool, st)
+               : cudaMallocAsync(&p, bytes, st);
     if (e != cudaSuccess || n >= 64) {
       cudaGetLastError();
       if (p) cudaFreeAsync(p, st);
       return fail(ADANNS_ERR_OOM, "scratch allocation of " + std::to_string(bytes) + " bytes failed");
     }
     ptrs[n++] = p;
+    held += (int64_t)bytes;
+    g_scratch_held.fetch_add((int64_t)bytes, std::memory_order_relaxed);
     *out = p;
     return ADANNS_OK;
   }
@@ -419,6 +430,13 @@ int run_tiled_scan(const adanns_index *idx, const TiledScan &t, const float *qs,
                    int64_t nb, int d_s, int nprobe, int k, const uint64_t *ckeys, int *counter,
                    int32_t *probes_out, int64_t *out_ids, float *out_dist, const MergeMask &mm,
                    cudaStream_t st);
+// An FP32 batch by the first of these routes, from `first` on, that its shape
+// takes and whose scratch can be had; *took (or null): which.  All give the
+// same result.
+enum F32Route { F32_FILTER, F32_STREAM, F32_TILED };
+int search_f32(const adanns_index *idx, const float *queries, int64_t B, int d_c, int d_s,
+               int nprobe, int k, int64_t *out_ids, float *out_dist, int32_t *out_probes,
+               cudaStream_t st, int first = F32_FILTER, int *took = nullptr);
 // The FP32 search through a certified tensor-core filter (certified.cu): same
 // results as the tiled and streaming scans, bit for bit.  The first says
 // whether a batch of this shape takes it.

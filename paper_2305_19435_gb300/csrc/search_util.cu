@@ -60,6 +60,19 @@ cudaMemPool_t scratch_pool() {
   return pools[dev];
 }
 
+std::atomic<int64_t> g_scratch_held{0};
+
+// After a call could not get its scratch: hand back what the pool grew by
+// meanwhile, so that the process does not keep memory that no call uses.
+void release_scratch(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaMemPool_t pool = scratch_pool();
+  if (pool && cudaStreamIsCapturing(st, &cap) == cudaSuccess &&
+      cap == cudaStreamCaptureStatusNone && cudaStreamSynchronize(st) == cudaSuccess)
+    cudaMemPoolTrimTo(pool, 0);
+  cudaGetLastError();
+}
+
 // the largest candidate segment one query can have: the n_p longest lists,
 // each padded to 8 members
 int64_t max_probe_members(const adanns_index *idx, int nprobe) {
@@ -100,6 +113,7 @@ void init_options() {
     g_opt[ADANNS_OPT_TEST_SKIP_LOAD] = -1;
     g_opt[ADANNS_OPT_SCAN_FILTER] = 0;
     g_opt[ADANNS_OPT_NARROW_SCAN] = 1;
+    g_opt[ADANNS_OPT_TEST_SCRATCH_LIMIT] = -1;
   });
 }
 }  // namespace
@@ -137,6 +151,9 @@ int set_option(int o, int64_t v) {
       break;
     case ADANNS_OPT_TEST_SKIP_LOAD:
       if (v < -1 || v > INT32_MAX) return fail(ADANNS_ERR_ARG, "bad skip index");
+      break;
+    case ADANNS_OPT_TEST_SCRATCH_LIMIT:
+      if (v < -1) return fail(ADANNS_ERR_ARG, "bad scratch limit");
       break;
   }
   g_opt[o].store(v);
