@@ -229,18 +229,17 @@ int encode_lists(adanns_index *x, const float *db, cudaStream_t st) {
 // (no rerank) or the exact FP32 rerank of the k'.
 // qb (or null): per-query nprobe and k, at most the call's nprobe and k (rows
 // of k entries, a query's own k results first, then padding)
-int search_ivfopq_select(const adanns_index *idx, const float *queries, int64_t B, int d_c,
-                         int nprobe, int k, int kr, bool rerank, int64_t *out_ids, float *out_dist,
-                         int32_t *out_probes, cudaStream_t st, const QueryBudgets *qb = nullptr) {
+// cert (many queries per probed list): 16-bit keys from the tensor cores, the
+// exact scores for the certified shortlist only, the lookup scan (in `parts`
+// parts of the batch, in the keys' space) for the queries left over
+int run_ivfopq_select(const adanns_index *idx, const float *queries, int64_t B, int d_c,
+                      int nprobe, int k, int kr, bool rerank, int64_t *out_ids, float *out_dist,
+                      int32_t *out_probes, cudaStream_t st, const QueryBudgets *qb, bool cert) {
   const int d_s = idx->opq_ds, M = idx->opq_M, dsub = d_s / M;
   const int nlist = idx->nlist;
   const int dcp = pad16(d_c), dsp = pad16(d_s);
   const int qa = adc_dist_query_tile(M);
   const int64_t seg_q = max_probe_members(idx, nprobe);
-  // many queries per probed list: 16-bit keys from the tensor cores, the exact
-  // scores for the certified shortlist only, the lookup scan (in `parts` parts
-  // of the batch, in the keys' space) for the queries left over
-  const bool cert = adc_certified(idx, B, nprobe, kr);
   const int nkb = (d_s + 63) / 64, QT = 128, kk = CERT_MAX_KK;
   const int64_t budget = scratch_budget() - (cert ? idx->N * nkb * 128ll : 0);
   auto per_q_of = [&](int cand_bytes) -> int64_t {
@@ -447,6 +446,20 @@ int search_ivfopq_select(const adanns_index *idx, const float *queries, int64_t 
       return rc;
   }
   return ADANNS_OK;
+}
+
+// The filter's copy of the decoded rows comes on top of the lookup scan's
+// scratch: where it cannot be had, the lookup scan alone.
+int search_ivfopq_select(const adanns_index *idx, const float *queries, int64_t B, int d_c,
+                         int nprobe, int k, int kr, bool rerank, int64_t *out_ids, float *out_dist,
+                         int32_t *out_probes, cudaStream_t st, const QueryBudgets *qb = nullptr) {
+  const bool cert = adc_certified(idx, B, nprobe, kr);
+  int rc = run_ivfopq_select(idx, queries, B, d_c, nprobe, k, kr, rerank, out_ids, out_dist,
+                             out_probes, st, qb, cert);
+  if (rc != ADANNS_ERR_OOM || !cert) return rc;
+  release_scratch(st);
+  return run_ivfopq_select(idx, queries, B, d_c, nprobe, k, kr, rerank, out_ids, out_dist,
+                           out_probes, st, qb, false);
 }
 
 }  // namespace

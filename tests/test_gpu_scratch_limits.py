@@ -69,3 +69,26 @@ def test_fp32_falls_back(P, data, metric, B):
     same(P.search_ivf(g, q, 16, 128, 4, 10), want1[:2])
     g.status()
     g.free()
+
+
+def test_ivfopq_falls_back(P, data):
+    """The filter's FP16 rows (5 MB) on top of the lookup scan's scratch."""
+    db, q = torch.from_numpy(data["db"]).cuda(), torch.from_numpy(data["queries"][:3000]).cuda()
+    g = P.flat_index(db)
+    R = torch.eye(128, device="cuda")
+    z = torch.nn.functional.normalize(db[:256], dim=1)
+    C = z.view(256, 16, 8).transpose(0, 1).contiguous()
+    P.set_opq(g, 128, 16, R, C, P.opq_encode(db, 128, 16, R, C))
+    for kw in ({}, {"rerank_k": 40}):
+        f = lambda: P.search_ivfopq(g, q, 8, 1, 10, return_probes=True, **kw)
+        want, stages = profiled(P, f)
+        assert "mma" in stages
+        # MiB: scores 229, tables 47, the rest under 8; the filter 31 more
+        with P.option(P.OPT_TEST_SCRATCH_LIMIT, 296 << 20):
+            got, stages = profiled(P, f)
+        assert "mma" not in stages and "adc" in stages
+        same(got, want)
+    want = P.search_ivfopq_budgets(g, q, 8, [1] * 3000, [10] * 3000)
+    with P.option(P.OPT_TEST_SCRATCH_LIMIT, 296 << 20):
+        same(P.search_ivfopq_budgets(g, q, 8, [1] * 3000, [10] * 3000), want)
+    g.free()
