@@ -123,9 +123,10 @@ int64_t adanns_launch_count(void);
  *                             loads).  That call's results are invalid.  Never
  *                             needed outside tests.
  *   ADANNS_OPT_TEST_SCRATCH_LIMIT  test hook, -1 (default).  n >= 0: the
- *                             library's scratch allocations fail, as if the
- *                             device had no more memory, where they would bring
- *                             the scratch of all calls in progress above n
+ *                             library's scratch allocations, and those of the
+ *                             tables that an index can do without, fail as if
+ *                             the device had no more memory, where they would
+ *                             bring the scratch of all calls in progress above n
  *                             bytes.
  * adanns_set_option returns ADANNS_ERR_ARG for an unknown option or a value
  * out of range (the option keeps its value).

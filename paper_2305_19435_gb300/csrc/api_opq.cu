@@ -169,14 +169,23 @@ int finish_residual(adanns_index *x, cudaStream_t st) {
 }
 
 // squared norms of the decoded rows, for the tensor-core filter (plain codes
-// of the prefix-normalised metric); synchronises
+// of the prefix-normalised metric); synchronises.  Where there is no memory for
+// them the index has none, and its searches take the lookup scan.
 int finish_code_norms(adanns_index *x, cudaStream_t st) {
   if (x->metric != ADANNS_METRIC_L2_PREFIXNORM) return ADANNS_OK;
-  if (cudaMalloc(&x->opq_y2, sizeof(float) * x->N) != cudaSuccess) {
+  const size_t bytes = sizeof(float) * x->N;
+  int rc = ADANNS_ERR_OOM;
+  if (scratch_refused(bytes) || cudaMalloc(&x->opq_y2, bytes) != cudaSuccess) {
     cudaGetLastError();
-    return fail(ADANNS_ERR_OOM, "OPQ allocation failed");
+    x->opq_y2 = nullptr;
+  } else {
+    rc = launch_code_norms(x, x->opq_y2, &x->opq_y2max, st);
   }
-  return launch_code_norms(x, x->opq_y2, &x->opq_y2max, st);
+  if (rc != ADANNS_ERR_OOM) return rc;
+  cudaFree(x->opq_y2);
+  x->opq_y2 = nullptr;
+  x->opq_y2max = INFINITY;
+  return ADANNS_OK;
 }
 
 int alloc_opq(adanns_index *x, int d_s, int M) {

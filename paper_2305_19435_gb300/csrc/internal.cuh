@@ -130,6 +130,10 @@ int64_t max_probe_members(const adanns_index *idx, int nprobe);
 
 extern std::atomic<int64_t> g_scratch_held;  // bytes held by all calls in progress
 void release_scratch(cudaStream_t st);       // after an allocation failed
+inline bool scratch_refused(size_t bytes) {  // by ADANNS_OPT_TEST_SCRATCH_LIMIT
+  const int64_t lim = option(ADANNS_OPT_TEST_SCRATCH_LIMIT);
+  return lim >= 0 && g_scratch_held.load(std::memory_order_relaxed) + (int64_t)bytes > lim;
+}
 
 // Stream-ordered scratch allocation from that pool on the call's stream.
 // Arrays of up to SLAB_MAX bytes are cut from slabs of SLAB bytes: a search
@@ -152,13 +156,10 @@ struct Scratch {
   }
   int alloc(void **out, size_t bytes) {
     void *p = nullptr;
-    const int64_t lim = option(ADANNS_OPT_TEST_SCRATCH_LIMIT);
     cudaMemPool_t pool = scratch_pool();
-    const cudaError_t e =
-        lim >= 0 && g_scratch_held.load(std::memory_order_relaxed) + (int64_t)bytes > lim
-            ? cudaErrorMemoryAllocation
-        : pool ? cudaMallocFromPoolAsync(&p, bytes, pool, st)
-               : cudaMallocAsync(&p, bytes, st);
+    const cudaError_t e = scratch_refused(bytes) ? cudaErrorMemoryAllocation
+                          : pool                 ? cudaMallocFromPoolAsync(&p, bytes, pool, st)
+                                                 : cudaMallocAsync(&p, bytes, st);
     if (e != cudaSuccess || n >= 64) {
       cudaGetLastError();
       if (p) cudaFreeAsync(p, st);

@@ -92,3 +92,26 @@ def test_ivfopq_falls_back(P, data):
     with P.option(P.OPT_TEST_SCRATCH_LIMIT, 296 << 20):
         same(P.search_ivfopq_budgets(g, q, 8, [1] * 3000, [10] * 3000), want)
     g.free()
+
+
+def test_codes_load_without_their_norms(P, data):
+    """The code rows' norms are only for the filter: codes load without them,
+    and the lookup scan answers."""
+    db, q = torch.from_numpy(data["db"]).cuda(), torch.from_numpy(data["queries"][:3000]).cuda()
+    g = P.flat_index(db)
+    R = torch.eye(128, device="cuda")
+    z = torch.nn.functional.normalize(db[:256], dim=1)
+    C = z.view(256, 16, 8).transpose(0, 1).contiguous()
+    codes = P.opq_encode(db, 128, 16, R, C)
+    f = lambda: P.search_ivfopq(g, q, 8, 1, 10, return_probes=True)
+    P.set_opq(g, 128, 16, R, C, codes)
+    want, stages = profiled(P, f)
+    assert "mma" in stages
+    with P.option(P.OPT_TEST_SCRATCH_LIMIT, 0):
+        P.set_opq(g, 128, 16, R, C, codes)
+    got, stages = profiled(P, f)
+    assert "mma" not in stages and "adc" in stages
+    same(got, want)
+    P.set_opq(g, 128, 16, R, C, codes)
+    assert "mma" in profiled(P, f)[1]
+    g.free()
