@@ -656,17 +656,24 @@ static int build_opq_impl(adanns_index *idx, const float *db, int d_s, int M, in
   return ADANNS_OK;
 }
 
-int adanns_index_set_opq(adanns_index *idx, int d_s, int M, const float *R,
-                         const float *codebooks, const uint8_t *codes_by_id, void *cuda_stream) {
+// rotation, codebooks and codes of an index (its code norms or residual tables follow)
+static int set_codes(adanns_index *idx, int d_s, int M, const float *R, const float *codebooks,
+                     const uint8_t *codes_by_id, cudaStream_t st) {
   if (!idx || !R || !codebooks || !codes_by_id) return fail(ADANNS_ERR_ARG, "NULL argument");
   int rc;
   if ((rc = check_opq_shape(d_s, M, idx->d))) return rc;
-  cudaStream_t st = S(cuda_stream);
   if ((rc = alloc_opq(idx, d_s, M))) return rc;
   ADN_CUDA(cudaMemcpyAsync(idx->opq_R, R, sizeof(float) * d_s * d_s, cudaMemcpyDeviceToDevice, st));
   ADN_CUDA(cudaMemcpyAsync(idx->opq_C, codebooks, sizeof(float) * M * 256 * (d_s / M),
                            cudaMemcpyDeviceToDevice, st));
-  if ((rc = launch_permute_codes(codes_by_id, idx->list_ids, idx->N, M, idx->codes, st)) ||
+  return launch_permute_codes(codes_by_id, idx->list_ids, idx->N, M, idx->codes, st);
+}
+
+int adanns_index_set_opq(adanns_index *idx, int d_s, int M, const float *R,
+                         const float *codebooks, const uint8_t *codes_by_id, void *cuda_stream) {
+  cudaStream_t st = S(cuda_stream);
+  int rc;
+  if ((rc = set_codes(idx, d_s, M, R, codebooks, codes_by_id, st)) ||
       (rc = finish_code_norms(idx, st)))
     return rc;
   ADN_CUDA(cudaStreamSynchronize(st));
@@ -677,10 +684,13 @@ int adanns_index_set_opq_residual(adanns_index *idx, int d_s, int M, const float
                                   const float *codebooks, const uint8_t *codes_by_id,
                                   const float *list_centres, void *cuda_stream) {
   if (!list_centres) return fail(ADANNS_ERR_ARG, "NULL argument");
-  int rc;
-  if ((rc = adanns_index_set_opq(idx, d_s, M, R, codebooks, codes_by_id, cuda_stream))) return rc;
   cudaStream_t st = S(cuda_stream);
-  if ((rc = alloc_residual(idx, d_s, M))) return rc;
+  int rc;
+  if ((rc = set_codes(idx, d_s, M, R, codebooks, codes_by_id, st))) return rc;
+  if ((rc = alloc_residual(idx, d_s, M))) {
+    cudaStreamSynchronize(st);  // the caller's arrays are no longer read
+    return rc;
+  }
   ADN_CUDA(cudaMemcpyAsync(idx->opq_lcent, list_centres, sizeof(float) * idx->nlist * d_s,
                            cudaMemcpyDeviceToDevice, st));
   if ((rc = finish_residual(idx, st))) return rc;

@@ -115,3 +115,32 @@ def test_codes_load_without_their_norms(P, data):
     P.set_opq(g, 128, 16, R, C, codes)
     assert "mma" in profiled(P, f)[1]
     g.free()
+
+
+def test_residual_codes_hold_no_norms(P):
+    """Residual codes are never searched by the filter: loading them takes the
+    codes (N M bytes) and the list tables, not 4 bytes per row of code norms."""
+    N = 4_000_000
+    db = torch.randn(N, 8, device="cuda")
+    g = P.flat_index(db)
+    R, C = torch.eye(8, device="cuda"), torch.randn(1, 256, 8, device="cuda")
+    codes = torch.zeros(N, 1, dtype=torch.uint8, device="cuda")
+    centres = torch.zeros(1, 8, device="cuda")
+
+    def held(load):  # by a second load: the pool and the kernels' modules are there
+        load()
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        g2 = P.flat_index(db)
+        torch.cuda.synchronize()
+        bare = before - torch.cuda.mem_get_info()[0]
+        load(g2)
+        torch.cuda.synchronize()
+        used = before - torch.cuda.mem_get_info()[0] - bare
+        g2.free()
+        return used
+
+    plain = held(lambda x=g: P.set_opq(x, 8, 1, R, C, codes))
+    residual = held(lambda x=g: P.set_opq_residual(x, 8, 1, R, C, codes, centres))
+    assert plain - residual >= 4 * N - (8 << 20)  # 16 MB; 2 MB pages of the small tables
+    g.free()
