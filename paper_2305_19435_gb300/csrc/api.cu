@@ -619,6 +619,28 @@ int search_f32_tiled(const adanns_index *idx, const float *queries, int64_t B, i
   return ADANNS_OK;
 }
 
+// Fitted to 952 calls by each route (3,000 to 1.28 M rows in 1 to 1,024 lists, 8 to
+// 2,048 coordinates, 1 to 32 probes, k 1 to 256, 5 to 2,000 queries per list); nine
+// of ten are within a fifth of it.  Per call: the launches; per member and its
+// coordinates: the conversion to FP16, or a first read; per (query, member): key and
+// shortlist, or distance and selection; per query and probe: the CTAs of the
+// selection and the re-score.  The filter re-scores about 1.3 k members per query, and
+// all of them where the probed lists fit its shortlist.
+double f32_cost(F32Route route, const adanns_index *idx, int64_t B, int64_t pairs, int d_s,
+                int k) {
+  const double N = (double)idx->N, q = (double)B, p = (double)pairs, d = d_s;
+  const double mem = p / q * N / idx->nlist, P = q * mem;  // members per query, in all
+  if (route == F32_FILTER) {
+    const double rescored = mem <= shortlist_cap(k) ? mem : 1.3 * k;
+    return 1.03e8 + N * (160 + 1.22 * d) + 1.05 * P + q * (20500 + 0.455 * rescored * d) + 910 * p;
+  }
+  if (route == F32_STREAM)
+    return 4.2e7 + 0.67 * N * d + P * (4.7 + 0.113 * d) + q * (9150 + 43.0 * k) + 1460 * p;
+  // (and no less than one CTA over a range of a list)
+  return 5.1e7 + std::max(3.5 * N * d + P * (1.02 + 0.101 * d) + 3300 * q + 1150 * p,
+                          3000 * d * std::min(256.0, N / idx->nlist));
+}
+
 // A route that cannot get its scratch leaves the batch to the next one: the
 // filter and the streaming scan size their slices by the scratch budget, the
 // tiled scan holds 2 GiB at most.  (A variant that the autotuner is timing is

@@ -310,9 +310,6 @@ int launch_mask_answered(uint64_t *ckeys, int64_t B, int nprobe, const int32_t *
 
 namespace {
 
-// shortlist slots: room for the k nearest and as many more near the k-th
-int shortlist_cap(int k) { return std::min(CERT_MAX_KK, std::max(4 * k, 256)); }
-
 struct Shape {
   int nkb, kk;
   int64_t seg;        // largest candidate segment of a query
@@ -336,29 +333,33 @@ Shape shape_of(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,
 
 }  // namespace
 
-// Where the filter pays.  It costs a pass over the probed lists (4 bytes read,
-// 2 written per coordinate), a dozen more launches and the re-score.  Against
-// the streaming scan, in picoseconds: that spends 0.112 more per (query, member,
-// coordinate), the filter 1.01 per member coordinate, 1 per re-scored coordinate
-// and 57 us of launches.  Streaming against filter, k 10: 1.28 M rows x 512, 8 /
-// 12 / 16 queries per list 845 / 1197 / 1504 against 967 / 1046 / 1058 us;
-// 400,000 x 64 at 20 / 32 / 64 171 / 269 / 445 against 208 / 269 / 315; 60,000 x 64
-// equal at 128.  Above 100 queries per list the line is lower, where the tiled
-// scan (the alternative for long prefixes) comes out even: 20,000 rows x 64 193
-// against 172 us at 17; the streaming scan would save at most 50 us there (10,000 x
-// 64 at 128: 76 against 124), and such batches stay on one path.  k and the probes must
-// fit the shortlist's buffers, and the FP16 rows may take half of the call's
-// scratch budget.  Turning the streaming scan off asks for the tiled scan
-// everywhere.
+// Where the filter pays: where its estimated time is the smallest (f32_cost).
+// Measured, filter / streaming / tiled in us: 1.28 M rows x 512, 16 of 1,024 lists, k
+// 10, 8 queries per list 967 / 845 / -, 16: 1058 / 1504 / -; 10,000 x 64 in 64 lists, 2
+// probed, k 1, 256 queries per list 276 / - / 115; 20,000 x 64 in 64 lists, 2 probed,
+// k 256 (every member of the lists is re-scored), 600 per list 1948 / - / 991.
+// Below F32_SMALL rows all routes are bound by launches; there the filter stays
+// above 100 queries per list while it is within 80 us of the others (65 at k 1), so
+// that its small sizes keep being run.  k and the probes must fit the shortlist's buffers,
+// and the FP16 rows may take half of the call's scratch budget.  Turning the
+// streaming scan off asks for the tiled scan everywhere.
+constexpr int64_t F32_SMALL = 8192;
+
 bool f32_certified(const adanns_index *idx, int64_t B, int d_s, int nprobe, int k) {
   if (idx->metric != ADANNS_METRIC_L2_PREFIXNORM || k > CE_MAX_K || nprobe > 128) return false;
   if (!option(ADANNS_OPT_FP32_STREAM) || scan_choice_forced()) return false;
   const int64_t nkb = (d_s + 63) / 64;
   if (idx->N * nkb > INT32_MAX - 256) return false;  // 32-bit row coordinates of the copies
   if (idx->N * (nkb * 128 + 4) > scratch_budget() / 2) return false;
-  const double qpl = (double)B * nprobe / idx->nlist, nd = (double)idx->N * d_s;
-  if (qpl > 100.0 && nd * qpl > 2e7) return true;
-  return nd * (0.112 * qpl - 1.01) - (double)B * k * d_s > 5.7e7;
+  const int64_t pairs = B * nprobe;
+  double other = f32_cost(F32_STREAM, idx, B, pairs, d_s, k);
+  if (k == 1 && pairs > 16ll * idx->nlist)
+    other = std::min(other, f32_cost(F32_TILED, idx, B, pairs, d_s, k));
+  const double qpl = (double)pairs / idx->nlist;
+  if (idx->N < F32_SMALL && qpl > 100.0 && (double)idx->N * d_s * qpl > 2e7 &&
+      nprobe * idx->N > shortlist_cap(k) * (int64_t)idx->nlist)
+    other += k == 1 ? 6.5e7 : 8e7;
+  return f32_cost(F32_FILTER, idx, B, pairs, d_s, k) < other;
 }
 
 int64_t certified_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,

@@ -435,6 +435,9 @@ int run_tiled_scan(const adanns_index *idx, const TiledScan &t, const float *qs,
 // takes and whose scratch can be had; *took (or null): which.  All give the
 // same result.
 enum F32Route { F32_FILTER, F32_STREAM, F32_TILED };
+// Estimated picoseconds of a batch of B queries and `pairs` (query, list) pairs
+// (F32_TILED: at k = 1 only, where it keeps no buffer)
+double f32_cost(F32Route route, const adanns_index *idx, int64_t B, int64_t pairs, int d_s, int k);
 int search_f32(const adanns_index *idx, const float *queries, int64_t B, int d_c, int d_s,
                int nprobe, int k, int64_t *out_ids, float *out_dist, int32_t *out_probes,
                cudaStream_t st, int first = F32_FILTER, int *took = nullptr);
@@ -481,6 +484,9 @@ int launch_select16(const uint16_t *cand, const uint64_t *ckeys, int nprobe, con
 // CERT_MAX_KK.  stats (NULL, or 2 zeroed device counters): candidates listed,
 // queries with -1.
 constexpr int CERT_MAX_K = 512, CERT_MAX_KK = 1024;
+// shortlist slots of the FP32 filter: room for the k nearest and as many more near
+// the k-th
+inline int shortlist_cap(int k) { return k > 256 ? CERT_MAX_KK : k > 64 ? 4 * k : 256; }
 int launch_certify16(const uint16_t *cand, const uint64_t *ckeys, int nprobe, const int64_t *qbase,
                      const int64_t *list_off, int kk, int k, const float *qerr, int64_t B,
                      int64_t *out, int32_t *cnt, unsigned long long *stats, cudaStream_t st);

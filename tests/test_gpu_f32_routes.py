@@ -1,0 +1,46 @@
+"""Which route an FP32 batch takes: the certified filter only where it is estimated
+to be the fastest.  The results are the tiled scan's, bit for bit, on each."""
+import numpy as np
+import pytest
+
+import synthdata
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    import paper_2305_19435_gb300 as P
+    P.build()
+    assert torch.cuda.is_available()
+    return P
+
+
+@pytest.fixture(scope="module")
+def index(P):
+    data = synthdata.small(20000, 8192, 512, 64, 41)
+    g = P.build_ivf(torch.from_numpy(data["db"]).cuda(), 16, 64, 4, 20000, 3)
+    yield g, torch.from_numpy(data["queries"]).cuda()
+    g.free()
+
+
+# 256 queries per list: few members per query beside its own cost (k 1 and 10, two
+# probes), all of them re-scored (k 256, two probes); enough of them (k 100, eight
+# probes); 64 per list at a long and a short prefix
+@pytest.mark.parametrize("d_s,nprobe,k,B,filtered", [
+    (64, 2, 1, 8192, False), (16, 2, 10, 8192, False), (64, 2, 256, 8192, False),
+    (512, 8, 100, 2048, True), (512, 8, 1, 2048, True), (512, 8, 10, 1024, True),
+    (16, 8, 1, 512, False)])
+def test_route(P, index, d_s, nprobe, k, B, filtered):
+    g, q = index
+    q = q[:B]
+    P.profile_enable(True)
+    a = [t.cpu().numpy() for t in P.search_ivf(g, q, 16, d_s, nprobe, k)]
+    stages = P.profile_read()
+    P.profile_enable(False)
+    assert ("mma" in stages) == filtered
+    with P.option(P.OPT_FP32_STREAM, 0):
+        b = [t.cpu().numpy() for t in P.search_ivf(g, q, 16, d_s, nprobe, k)]
+    np.testing.assert_array_equal(a[0], b[0])
+    np.testing.assert_array_equal(a[1].view(np.int32), b[1].view(np.int32))
