@@ -355,7 +355,11 @@ int64_t stream_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_
 // against streaming, 400,000 rows in 400 lists, 500 queries per list, k 10: d_s 64
 // 3.65 / 2.85 ms, 512 12.9 / 13.8, 1024 23.5 / 26.3; k 100: 8.4 / 3.0, 17.6 / 13.9,
 // 28.0 / 26.5; 100,000 x 2048, k 10, 32 and 64 queries per list: 1.39 / 1.19 and
-// 2.05 / 2.23.  A batch with a d_s per query goes by their mean (6,000 queries with
+// 2.05 / 2.23.  At k = 1, where the tiled scan keeps no buffer and the selection's CTA
+// per query is most of the call, by their estimated times (f32_cost): 200,000 rows in
+// 256 lists, d_s 16, 2 probes, 90 queries per list 197 / 323 us; 640,000 in 700, d_s 64, 1
+// probe, 47 per list 529 / 759; 60,000 in 60, d_s 64, 4 probes, 68 per list 109 / 100.
+// A batch with a d_s per query goes by their mean (6,000 queries with
 // d_s 64 to 2048, 20,000 rows in 16 lists, k 100: 9.98 / 9.25; 2,000 with 64 to 512, 1
 // M rows, k 10: 2.45 / 1.08).  The distances must fit the scratch at once, or in slices of at
 // least 64 queries per list, which still share their rows.
@@ -367,7 +371,12 @@ bool fp32_stream_enabled(const adanns_index *idx, int64_t B, int64_t pairs, int 
   if (t != 0) return t == TUNE_STREAM;
   if (qpl <= 16.0) return true;
   const int ds = mean_ds ? mean_ds : d_s;
-  if (qpl * ds > 65536.0 && k < (ds <= 1024 ? (ds - 256) / 14 : ds / 4)) return false;
+  if (k == 1 && !mean_ds) {
+    if (f32_cost(F32_TILED, idx, B, pairs, d_s, k) < f32_cost(F32_STREAM, idx, B, pairs, d_s, k))
+      return false;
+  } else if (qpl * ds > 65536.0 && k < (ds <= 1024 ? (ds - 256) / 14 : ds / 4)) {
+    return false;
+  }
   const int64_t fit = scratch_budget() / stream_per_query(idx, d_c, d_s, nprobe, k);
   return fit >= B || (double)fit * pairs / B >= 64.0 * idx->nlist;
 }

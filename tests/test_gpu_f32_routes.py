@@ -44,3 +44,22 @@ def test_route(P, index, d_s, nprobe, k, B, filtered):
         b = [t.cpu().numpy() for t in P.search_ivf(g, q, 16, d_s, nprobe, k)]
     np.testing.assert_array_equal(a[0], b[0])
     np.testing.assert_array_equal(a[1].view(np.int32), b[1].view(np.int32))
+
+
+# the raw metric (no filter): at k 1 the tiled scan where the selection's CTA per
+# query would be most of the call, told by the scratch of the route
+@pytest.mark.parametrize("d_s,nprobe,k,B,tiled", [
+    (16, 2, 1, 2880, True), (64, 1, 1, 8192, True), (16, 2, 2, 2880, False),
+    (64, 2, 1, 320, False), (16, 2, 1, 500, False)])
+def test_stream_or_tiled(P, d_s, nprobe, k, B, tiled):
+    data = synthdata.small(20000, 8192, 64, 64, 43)
+    g = P.build_ivf(torch.from_numpy(data["db"]).cuda(), 16, 64, 4, 20000, 3, metric=P.METRIC_L2)
+    q = torch.from_numpy(data["queries"][:B]).cuda()
+    with P.option(P.OPT_FP32_STREAM, 0):
+        b = [t.cpu().numpy() for t in P.search_ivf(g, q, 16, d_s, nprobe, k)]
+        need = P.scratch_bytes(g, B, 16, d_s, nprobe, k)
+    assert (P.scratch_bytes(g, B, 16, d_s, nprobe, k) == need) == tiled
+    a = [t.cpu().numpy() for t in P.search_ivf(g, q, 16, d_s, nprobe, k)]
+    np.testing.assert_array_equal(a[0], b[0])
+    np.testing.assert_array_equal(a[1].view(np.int32), b[1].view(np.int32))
+    g.free()
