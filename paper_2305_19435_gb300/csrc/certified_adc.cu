@@ -255,6 +255,13 @@ int launch_code_norms(const adanns_index *x, float *y2, float *y2max_host, cudaS
 // against 1.15 at 128; 400,000 rows in 200 lists, M 32: 0.59 against 0.61 ms at
 // 32 queries per list, 0.96 against 0.66 at 64); far above it the gap is 3- to
 // 12-fold.
+// With few queries per list and short rows the tiles of 128 queries are mostly
+// empty, and what this line leaves out decides: the filter's cost per member and
+// per query, and the lookup scan's tables and codes per tile of its own.  There
+// the filter also has to be a tenth ahead by the estimates of both (fitted to 608
+// calls): without it, lookups against filter in us, 3 M rows in 1,500 lists, (64,
+// 32), 49 probes, 163 queries 557 / 841; 1 M in 1,000, (64, 8), 37, 808 486 / 639; (128,
+// 16), 15, 1,397 482 / 550.
 bool adc_certified(const adanns_index *idx, int64_t B, int nprobe, int kr) {
   const int M = idx->opq_M, d_s = idx->opq_ds;
   if (idx->metric != ADANNS_METRIC_L2_PREFIXNORM || idx->opq_S || !idx->opq_y2) return false;
@@ -263,10 +270,18 @@ bool adc_certified(const adanns_index *idx, int64_t B, int nprobe, int kr) {
   const int64_t nkb = (d_s + 63) / 64;
   if (idx->N * nkb > INT32_MAX - 256 || idx->N * nkb * 128 > scratch_budget() / 2) return false;
   const double N = (double)idx->N, per = N / idx->nlist, qpl = (double)B * nprobe / idx->nlist;
-  return N * qpl * (2.0 + 0.42 * M + 900.0 * M / per) -
-             N * d_s * (0.8 + 0.0022 * std::max(qpl, 128.0)) - B * (4e4 + 200.0 * d_s) -
-             500.0 * nprobe * per >
-         2e8;
+  if (N * qpl * (2.0 + 0.42 * M + 900.0 * M / per) -
+          N * d_s * (0.8 + 0.0022 * std::max(qpl, 128.0)) - B * (4e4 + 200.0 * d_s) -
+          500.0 * nprobe * per <=
+      2e8)
+    return false;
+  if (qpl >= 48.0 || d_s > 192) return true;
+  const double pairs = (double)B * nprobe, tiles = std::max(1.0, qpl / adc_dist_query_tile(M));
+  const double filter = 1.83e8 + N * (73.0 + 2.38 * d_s) + 1.89 * N * qpl +
+                        B * (14000.0 + 1260.0 * M) + 635.0 * pairs;
+  const double lookup = 1.06e8 + N * (6.3 * qpl + 1.68 * M * tiles) + B * (25500.0 + 1320.0 * M) +
+                        357.0 * M * pairs;
+  return filter < 0.9 * lookup;
 }
 
 int launch_decode_f16(const adanns_index *idx, const int32_t *lcnt, int nkb, void *rows,
