@@ -51,18 +51,21 @@ __global__ void pq_assign_kernel(const float *__restrict__ z, int64_t n, int ldz
 // negated in pairs, [c / 2][t][c % 2], so that one 16-byte broadcast read gives
 // two coordinates of two codewords and every add / multiply-add instruction
 // works on both (z - C = z + (-C), the same rounding); distances are compared
-// in codeword order.  A CTA takes PQA_THREADS * PQA_P points and PQA_MG
-// sub-vectors, whose codes leave together.  Bound by the FP32 pipe (an
-// add and a multiply-add per coordinate and codeword): 262,144 points, 32
-// sub-vectors of 12 in 1.66 ms, 84% of its rate (four points per thread: 1.70).
+// in codeword order.  A CTA takes PQA_THREADS * PQA_P points and mg sub-vectors:
+// PQA_MG, whose codes leave together, or fewer while there are not enough points for
+// a CTA per SM (encoding 507 points, 8 sub-vectors of 8: 65 us by the kernel above, 98
+// with 2 CTAs that take 8 in turn, 41 with 16 that take one).  Bound by the FP32 pipe
+// (an add and a multiply-add per coordinate and codeword): 262,144 points, 32
+// sub-vectors of 12 in 1.66 ms, 84% of the rate of those instructions (four points
+// per thread: 1.70).
 constexpr int PQA_THREADS = 128, PQA_P = 2, PQA_MG = 8;
 
 template <int DS>
 __global__ void __launch_bounds__(PQA_THREADS) pq_assign_regs_kernel(
-    const float *__restrict__ z, int64_t n, int ldz, int M, const float *__restrict__ C,
+    const float *__restrict__ z, int64_t n, int ldz, int M, int mg, const float *__restrict__ C,
     uint8_t *__restrict__ codes, float *__restrict__ mind) {
   extern __shared__ __align__(16) float Cs[];  // [128][DS][2]
-  const int m0 = blockIdx.y * PQA_MG, nm = min(PQA_MG, M - m0);
+  const int m0 = blockIdx.y * mg, nm = min(mg, M - m0);
   const int64_t i0 = (int64_t)blockIdx.x * (PQA_THREADS * PQA_P) + threadIdx.x;
   uint32_t cw[PQA_P][PQA_MG / 4];
 #pragma unroll
@@ -150,8 +153,11 @@ int launch_pq_assign(const float *z, int64_t n, int ldz, int M, int dsub, const 
     const size_t sm = (size_t)256 * dsub * 4;
     ADN_CUDA(ensure_smem((const void *)kern, sm));
     const int per = PQA_THREADS * PQA_P;
-    const dim3 grid((unsigned)((n + per - 1) / per), (M + PQA_MG - 1) / PQA_MG);
-    kern<<<grid, PQA_THREADS, sm, st>>>(z, n, ldz, M, C, codes, mind);
+    const int64_t gx = (n + per - 1) / per;
+    int mg = PQA_MG;
+    while (mg > 1 && gx * ((M + mg - 1) / mg) < num_sms()) mg >>= 1;
+    const dim3 grid((unsigned)gx, (M + mg - 1) / mg);
+    kern<<<grid, PQA_THREADS, sm, st>>>(z, n, ldz, M, mg, C, codes, mind);
     ADN_LAUNCH("pq_assign_regs_kernel");
     return ADANNS_OK;
   };
