@@ -238,6 +238,11 @@ int adanns_index_status(const adanns_index *idx, void *cuda_stream);
 int64_t adanns_search_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s,
                                     int nprobe, int k, int storage, int rerank_k);
 
+/* The most scratch that the library's calls have held at one time since the
+ * library was loaded or since the last call with reset != 0 (host-side; all
+ * threads and devices together). */
+int64_t adanns_scratch_high(int reset);
+
 /* Release an index (NULL is ignored).  Waits for the device to finish using it. */
 void adanns_index_free(adanns_index *idx);
 

@@ -362,6 +362,12 @@ int adanns_version(void) { return 100; }
 
 int64_t adanns_launch_count(void) { return (int64_t)g_launches.load(); }
 
+int64_t adanns_scratch_high(int reset) {
+  const int64_t v = g_scratch_high.load();
+  if (reset) g_scratch_high.store(g_scratch_held.load());
+  return v;
+}
+
 int adanns_set_option(int option, int64_t value) { return set_option(option, value); }
 
 int adanns_get_option(int option, int64_t *value) {
@@ -567,6 +573,24 @@ int run_tiled_scan(const adanns_index *idx, const TiledScan &t, const float *qs,
   return launch_merge(t.pkeys, nb, nprobe * t.nsplit, k, out_ids, out_dist, st, mm);
 }
 
+// slices of the batch whose per-(query, probe) partial results stay ~2 GiB
+static int64_t tiled_slice(const TiledScan &ts, int64_t B, int d_c, int d_s, int nprobe, int k,
+                           int64_t *per_q) {
+  *per_q = (int64_t)nprobe * ts.nsplit * k * 8 + (int64_t)(pad16(d_c) + pad16(d_s)) * 4 +
+           (int64_t)nprobe * 24;
+  return std::max<int64_t>(1, std::min<int64_t>(B, (2ll << 30) / *per_q));
+}
+
+int64_t tiled_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,
+                            int k) {
+  TiledScan ts{};
+  tiled_scan_shape(idx, B, d_s, nprobe, k, &ts);
+  int64_t per_q;
+  const int64_t Bc = tiled_slice(ts, B, d_c, d_s, nprobe, k, &per_q);
+  return Bc * (per_q + coarse_scratch_per_query(idx, d_c)) + (int64_t)idx->nlist * 64 +
+         Scratch::SLACK;
+}
+
 int search_f32_tiled(const adanns_index *idx, const float *queries, int64_t B, int d_c, int d_s,
                      int nprobe, int k, int64_t *out_ids, float *out_dist, int32_t *out_probes,
                      cudaStream_t st, const QueryBudgets *qb, const int32_t *rows) {
@@ -574,10 +598,8 @@ int search_f32_tiled(const adanns_index *idx, const float *queries, int64_t B, i
   const int dcp = pad16(d_c), dsp = pad16(d_s);
   TiledScan ts{};
   tiled_scan_shape(idx, B, d_s, nprobe, k, &ts);
-  // slice the batch so that the per-(query, probe) partial results stay ~2 GiB
-  const int64_t per_q =
-      (int64_t)nprobe * ts.nsplit * k * 8 + (int64_t)(dcp + dsp) * 4 + nprobe * 24;
-  const int64_t Bc = std::max<int64_t>(1, std::min<int64_t>(B, (2ll << 30) / per_q));
+  int64_t per_q;
+  const int64_t Bc = tiled_slice(ts, B, d_c, d_s, nprobe, k, &per_q);
   Scratch s(st);
   float *qc, *qs;
   uint64_t *ckeys;
@@ -671,27 +693,14 @@ extern "C" {
 int64_t adanns_search_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s,
                                     int nprobe, int k, int storage, int rerank_k) {
   if (!idx || B < 0 || nprobe < 1 || k < 1) return -1;
-  const int dcp = pad16(d_c), dsp = pad16(d_s);
-  if (storage == ADANNS_STORE_BF16 || storage == ADANNS_STORE_FP8E4M3) {
-    const int epb = storage == ADANNS_STORE_FP8E4M3 ? 128 : 64;
-    const int64_t nkb = (d_s + epb - 1) / epb;
-    const int64_t kk = rerank_k > k ? rerank_k : k;
-    const int64_t seg_q = (int64_t)nprobe * (((int64_t)idx->max_list + 7) & ~7ll);
-    const int64_t per_q = seg_q * 2 + (int64_t)nprobe * (nkb * 128 * 128 / 128 + 32) +
-                          (int64_t)(dcp + dsp) * 4 + nkb * 128 + kk * 8 + 64 + kk * 40;
-    const int64_t Bc = std::max<int64_t>(1, std::min<int64_t>(B, scratch_budget() / per_q));
-    return Bc * per_q + (int64_t)idx->nlist * 64 + (64ll << 20);
-  }
+  if (storage == ADANNS_STORE_BF16 || storage == ADANNS_STORE_FP8E4M3)
+    return mixed_scratch_bytes(idx, B, d_c, d_s, nprobe, storage == ADANNS_STORE_FP8E4M3,
+                               rerank_k > k ? rerank_k : k);
   if (f32_certified(idx, B, d_s, nprobe, k))
     return certified_scratch_bytes(idx, B, d_c, d_s, nprobe, k);
   if (fp32_stream_enabled(idx, B, B * nprobe, d_c, d_s, nprobe, k))
     return stream_scratch_bytes(idx, B, d_c, d_s, nprobe, k);
-  int tq, qt, nsplit;
-  fp32_scan_shape(idx, B, d_s, nprobe, k, &tq, &qt, &nsplit);
-  const int64_t per_q =
-      (int64_t)nprobe * nsplit * k * 8 + (int64_t)(dcp + dsp) * 4 + nprobe * 24;
-  const int64_t Bc = std::max<int64_t>(1, std::min<int64_t>(B, (2ll << 30) / per_q));
-  return Bc * per_q + (int64_t)idx->nlist * 64 + (16ll << 20);
+  return tiled_scratch_bytes(idx, B, d_c, d_s, nprobe, k);
 }
 
 void adanns_index_free(adanns_index *idx) {

@@ -312,22 +312,29 @@ namespace {
 
 struct Shape {
   int nkb, kk;
-  int64_t seg;        // largest candidate segment of a query
-  int64_t row_bytes;  // the FP16 copy and the members' |x|^2
-  int64_t per_q;      // scratch per query of a slice
+  int64_t seg;    // largest candidate segment of a query
+  int64_t fixed;  // scratch whatever the slice: rows, one part-filled tile per list
+  int64_t per_q;  // and per query of a slice
+  int64_t Bc;     // queries per slice
   TiledScan ts;
 };
+
+// the FP16 copy with the members' |x|^2, and each list's part-filled query tile
+int64_t filter_fixed_bytes(const adanns_index *idx, int64_t nkb) {
+  return idx->N * (nkb * 128 + 4) + 256 + idx->nlist * (nkb * 128 * 128 + 96);
+}
 
 Shape shape_of(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe, int k) {
   Shape h{};
   h.nkb = (d_s + 63) / 64;
   h.kk = shortlist_cap(k);
-  h.row_bytes = idx->N * ((int64_t)h.nkb * 128 + 4) + 256;
+  h.fixed = filter_fixed_bytes(idx, h.nkb);
   tiled_scan_shape(idx, B, d_s, nprobe, k, &h.ts);
   h.seg = max_probe_members(idx, nprobe);
   h.per_q = h.seg * 2 + (int64_t)nprobe * ((int64_t)h.nkb * 128 + 60) +
             (int64_t)(pad16(d_c) + pad16(d_s)) * 4 + (int64_t)h.nkb * 128 + (int64_t)h.kk * 8 + 64 +
-            (int64_t)nprobe * h.ts.nsplit * k * 8;
+            (int64_t)nprobe * h.ts.nsplit * k * 8 + coarse_scratch_per_query(idx, d_c);
+  h.Bc = std::max<int64_t>(1, std::min<int64_t>(B, (scratch_budget() - h.fixed) / h.per_q));
   return h;
 }
 
@@ -341,7 +348,7 @@ Shape shape_of(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,
 // Below F32_SMALL rows all routes are bound by launches; there the filter stays
 // above 100 queries per list while it is within 80 us of the others (65 at k 1), so
 // that its small sizes keep being run.  k and the probes must fit the shortlist's buffers,
-// and the FP16 rows may take half of the call's scratch budget.  Turning the
+// and the FP16 rows with the tiles' padding may take half of the call's scratch budget.  Turning the
 // streaming scan off asks for the tiled scan everywhere.
 constexpr int64_t F32_SMALL = 8192;
 
@@ -350,7 +357,7 @@ bool f32_certified(const adanns_index *idx, int64_t B, int d_s, int nprobe, int 
   if (!option(ADANNS_OPT_FP32_STREAM) || scan_choice_forced()) return false;
   const int64_t nkb = (d_s + 63) / 64;
   if (idx->N * nkb > INT32_MAX - 256) return false;  // 32-bit row coordinates of the copies
-  if (idx->N * (nkb * 128 + 4) > scratch_budget() / 2) return false;
+  if (filter_fixed_bytes(idx, nkb) > scratch_budget() / 2) return false;
   const int64_t pairs = B * nprobe;
   double other = f32_cost(F32_STREAM, idx, B, pairs, d_s, k);
   if (k == 1 && pairs > 16ll * idx->nlist)
@@ -365,10 +372,7 @@ bool f32_certified(const adanns_index *idx, int64_t B, int d_s, int nprobe, int 
 int64_t certified_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,
                                 int k) {
   const Shape h = shape_of(idx, B, d_c, d_s, nprobe, k);
-  const int64_t Bc = std::max<int64_t>(
-      1, std::min<int64_t>(B, (scratch_budget() - h.row_bytes) / h.per_q));
-  return h.row_bytes + Bc * h.per_q + (int64_t)idx->nlist * (h.nkb * 128ll * 128 + 96) +
-         (64ll << 20);
+  return h.fixed + h.Bc * h.per_q + Scratch::SLACK;
 }
 
 int search_f32_certified(const adanns_index *idx, const float *queries, int64_t B, int d_c,
@@ -377,8 +381,7 @@ int search_f32_certified(const adanns_index *idx, const float *queries, int64_t 
   const int nlist = idx->nlist, dcp = pad16(d_c), dsp = pad16(d_s), QT = 128;
   Shape h = shape_of(idx, B, d_c, d_s, nprobe, k);
   const int nkb = h.nkb, kk = h.kk;
-  const int64_t Bc = std::max<int64_t>(
-      1, std::min<int64_t>(B, (scratch_budget() - h.row_bytes) / h.per_q));
+  const int64_t Bc = h.Bc;
   const int64_t max_tiles = (Bc * nprobe + QT - 1) / QT + nlist;
   const bool ordered = Bc >= 4096 && nlist > 1;  // fewer queries: their rows fit in L2 anyway
   Scratch s(st);

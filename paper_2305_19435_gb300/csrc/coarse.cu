@@ -702,6 +702,10 @@ int scratch_centroid_lowp(Scratch &s, adanns_index *x, cudaStream_t st) {
 int launch_mma_scan(const void *qtiles, int64_t qrows, const void *xlow, int64_t xrows,
                     const MmaScanArgs &a, cudaStream_t st);
 
+int64_t coarse_scratch_per_query(const adanns_index *idx, int d_c) {
+  return ((idx->nlist + 7) & ~7) * 2ll + (d_c + 63) / 64 * 128 + 32;
+}
+
 int launch_coarse_tc(const adanns_index *idx, const float *qc, int ldq, int64_t B, int d_c, int k,
                      uint64_t *out, cudaStream_t st) {
   // small tables stay on the FP32 kernels (they are cheap there, and the

@@ -129,6 +129,7 @@ int set_option(int opt, int64_t value);
 int64_t max_probe_members(const adanns_index *idx, int nprobe);
 
 extern std::atomic<int64_t> g_scratch_held;  // bytes held by all calls in progress
+extern std::atomic<int64_t> g_scratch_high;  // their maximum (adanns_scratch_high)
 void release_scratch(cudaStream_t st);       // after an allocation failed
 inline bool scratch_refused(size_t bytes) {  // by ADANNS_OPT_TEST_SCRATCH_LIMIT
   const int64_t lim = option(ADANNS_OPT_TEST_SCRATCH_LIMIT);
@@ -141,6 +142,9 @@ inline bool scratch_refused(size_t bytes) {  // by ADANNS_OPT_TEST_SCRATCH_LIMIT
 // host about a microsecond each, more than a small batch's kernels take.
 struct Scratch {
   static constexpr size_t SLAB = 512 << 10, SLAB_MAX = 128 << 10;
+  // at most this much is held beyond a call's large arrays: its slabs (some 50 small
+  // arrays) and the roundings of its steps
+  static constexpr int64_t SLACK = 16 << 20;
   cudaStream_t st;
   void *ptrs[64];
   int n = 0;
@@ -167,7 +171,11 @@ struct Scratch {
     }
     ptrs[n++] = p;
     held += (int64_t)bytes;
-    g_scratch_held.fetch_add((int64_t)bytes, std::memory_order_relaxed);
+    const int64_t now =
+        g_scratch_held.fetch_add((int64_t)bytes, std::memory_order_relaxed) + (int64_t)bytes;
+    int64_t high = g_scratch_high.load(std::memory_order_relaxed);
+    while (now > high && !g_scratch_high.compare_exchange_weak(high, now, std::memory_order_relaxed)) {
+    }
     *out = p;
     return ADANNS_OK;
   }
@@ -380,6 +388,8 @@ int launch_coarse_tc(const adanns_index *idx, const float *qc, int ldq, int64_t 
 // general scan over the prefix-major centroid table (counter: its work counter).
 int run_coarse(const adanns_index *idx, const float *qc, int ldq, int64_t B, int d_c, int k,
                uint64_t *out, int *counter, cudaStream_t st);
+// the most scratch of the cluster mapping (launch_coarse_tc's) per query
+int64_t coarse_scratch_per_query(const adanns_index *idx, int d_c);
 constexpr int64_t CT_SLICE_MIN = 4096;  // fewest points per tensor-core assignment slice
 int build_centroid_lowp(adanns_index *x, cudaStream_t st);
 int scratch_centroid_lowp(Scratch &s, adanns_index *x, cudaStream_t st);
@@ -399,7 +409,13 @@ int launch_scan64(const int64_t *in, int64_t n, int64_t *out, int64_t *total, cu
 // with a d_s per query (d_s the largest), else 0
 bool fp32_stream_enabled(const adanns_index *idx, int64_t B, int64_t pairs, int d_c, int d_s,
                          int nprobe, int k, int mean_ds = 0);
-// scratch bytes of search_f32_stream for these arguments (host arithmetic)
+// upper bounds of the scratch that the tiers' searches hold, nested steps included
+// (host arithmetic); which: 0 BF16, 1 FP8
+int64_t mixed_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,
+                            int which, int kk);
+int64_t tiled_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,
+                            int k);
+int64_t rerank_scratch_bytes(const adanns_index *idx, int64_t B, int kr, int d_s);
 int64_t stream_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,
                              int k);
 // The tiled FP32 scan (many queries per probed list).  qb (or null): per-query

@@ -408,15 +408,23 @@ static bool scan_filter_enabled(const adanns_index *idx) {
   return option(ADANNS_OPT_SCAN_FILTER) != 0 && idx->max_list <= 65536;
 }
 
-int search_mixed(const adanns_index *idx, const float *queries, int64_t B, int d_c, int d_s,
-                 int nprobe, int k, int which, int kk, int64_t *out_ids, float *out_dist,
-                 int32_t *out_probes, cudaStream_t st, const QueryBudgets *qb) {
-  const int fp8 = which == 1;
-  const int epb = fp8 ? 128 : 64;
-  const int nkb = (d_s + epb - 1) / epb;
+namespace {
+struct MixedShape {
+  int nkb, qt;          // K-blocks, queries per tile
+  bool filt, narrow;    // filtered scan; tiles of 128 members x MMA_NARROW_QT queries
+  int64_t seg_q;        // candidate keys per query
+  int64_t stride0;      // filtered: the keys of each query's nearest list, one segment per query
+  int64_t per_q, Bc;    // scratch per query of a slice, queries per slice
+  int64_t tiles_a, tiles_b;
+};
+
+MixedShape mixed_shape(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe, int which,
+                       int kk) {
+  const int epb = which == 1 ? 128 : 64;
   const int nlist = idx->nlist;
-  const int dcp = pad16(d_c), dsp = pad16(d_s);
-  const bool filt = scan_filter_enabled(idx);
+  MixedShape h{};
+  h.nkb = (d_s + epb - 1) / epb;
+  h.filt = scan_filter_enabled(idx);
   // few queries per probed list: tiles of 128 members x 32 queries, where they
   // were measured faster than the wide tiles (16 K-blocks or more: d_s >= 1024
   // for BF16, 2048 for FP8), or at any d_s when the option asks for them
@@ -425,23 +433,45 @@ int search_mixed(const adanns_index *idx, const float *queries, int64_t B, int d
   const int64_t nopt = option(ADANNS_OPT_NARROW_SCAN);
   const double qpl = (double)B * nprobe / nlist;
   const int tuned = nopt == 1 ? tuned_lowp_qt(which, d_s, qpl) : 0;
-  const bool narrow = !filt && nopt != 0 &&
-                      (tuned ? tuned == MMA_NARROW_QT
-                             : qpl <= 24.0 && (nopt == 2 || nkb >= 16));
-  const int qt = narrow ? MMA_NARROW_QT : 128;
-  const int64_t seg_q = (int64_t)nprobe * (((int64_t)idx->max_list + 7) & ~7ll);
-  // filtered: the keys of each query's nearest list, one segment per query
-  const int64_t stride0 = ((int64_t)idx->max_list + 7) & ~7ll;
-  const int64_t per_q = (filt ? seg_q * 4 + stride0 * 2 : seg_q * 2) +
-                        (int64_t)nprobe * ((int64_t)nkb * 128 + 36) +
-                        (int64_t)(dcp + dsp) * 4 + (int64_t)nkb * 128 + (int64_t)kk * 8 + 64;
+  h.narrow = !h.filt && nopt != 0 &&
+             (tuned ? tuned == MMA_NARROW_QT : qpl <= 24.0 && (nopt == 2 || h.nkb >= 16));
+  h.qt = h.narrow ? MMA_NARROW_QT : 128;
+  h.seg_q = (int64_t)nprobe * (((int64_t)idx->max_list + 7) & ~7ll);
+  h.stride0 = ((int64_t)idx->max_list + 7) & ~7ll;
+  h.per_q = (h.filt ? h.seg_q * 4 + h.stride0 * 2 : h.seg_q * 2) +
+            (int64_t)nprobe * ((int64_t)h.nkb * 128 + 36) + (int64_t)(pad16(d_c) + pad16(d_s)) * 4 +
+            (int64_t)h.nkb * 128 + (int64_t)kk * 8 + 64;
   // slices bounded by a scratch budget (the candidate keys dominate it)
-  const int64_t Bc = std::max<int64_t>(1, std::min<int64_t>(B, scratch_budget() / per_q));
+  h.Bc = std::max<int64_t>(1, std::min<int64_t>(B, scratch_budget() / h.per_q));
   // work-item tiles: the filtered scan's two passes (slot 0; slots 1..) each
   // get their own, the unfiltered scan one set over every slot
-  const int64_t tiles_a = filt ? (Bc + qt - 1) / qt + nlist : (Bc * nprobe + qt - 1) / qt + nlist;
-  const int64_t tiles_b = filt && nprobe > 1 ? (Bc * (nprobe - 1) + qt - 1) / qt + nlist : 0;
-  const int64_t max_tiles = tiles_a + tiles_b;
+  h.tiles_a = ((h.filt ? h.Bc : h.Bc * nprobe) + h.qt - 1) / h.qt + nlist;
+  h.tiles_b = h.filt && nprobe > 1 ? (h.Bc * (nprobe - 1) + h.qt - 1) / h.qt + nlist : 0;
+  return h;
+}
+}  // namespace
+
+int64_t mixed_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,
+                            int which, int kk) {
+  const MixedShape h = mixed_shape(idx, B, d_c, d_s, nprobe, which, kk);
+  const int64_t sets = h.tiles_b ? 2 : 1;  // a part-filled tile per list and set
+  return h.Bc * (h.per_q + coarse_scratch_per_query(idx, d_c)) +
+         idx->nlist * (sets * h.nkb * h.qt * 128 + 96) + rerank_scratch_bytes(idx, h.Bc, kk, d_s) +
+         Scratch::SLACK;
+}
+
+int search_mixed(const adanns_index *idx, const float *queries, int64_t B, int d_c, int d_s,
+                 int nprobe, int k, int which, int kk, int64_t *out_ids, float *out_dist,
+                 int32_t *out_probes, cudaStream_t st, const QueryBudgets *qb) {
+  const int fp8 = which == 1;
+  const int epb = fp8 ? 128 : 64;
+  const int nlist = idx->nlist;
+  const int dcp = pad16(d_c), dsp = pad16(d_s);
+  const MixedShape h = mixed_shape(idx, B, d_c, d_s, nprobe, which, kk);
+  const int nkb = h.nkb, qt = h.qt;
+  const bool filt = h.filt, narrow = h.narrow;
+  const int64_t seg_q = h.seg_q, stride0 = h.stride0, Bc = h.Bc;
+  const int64_t tiles_a = h.tiles_a, tiles_b = h.tiles_b, max_tiles = tiles_a + tiles_b;
   const bool prune = shortlist_prune_enabled();
   const float rmax = idx->lowp_rmax[which][gran_index(d_s)] * 1.001f;
   const float e_rest = shortlist_e_rest(d_s, nkb * epb);

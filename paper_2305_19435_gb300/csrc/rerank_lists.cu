@@ -276,6 +276,13 @@ static bool rerank_by_query(int64_t slots, int64_t N, int d_s) {
   return slots <= (d_s >= 512 ? 7 : 2) * N;
 }
 
+int64_t rerank_scratch_bytes(const adanns_index *idx, int64_t B, int kr, int d_s) {
+  const int64_t n = B * kr;
+  if (rerank_by_query(n, idx->N, d_s)) return n * 8 + B * 4 + idx->nlist * 4;
+  return n * 16 + (idx->N + 1) * 8 +
+         idx->rr_chunks[rerank_chunk_index(rerank_chunk_members(d_s))] * (int64_t)sizeof(int2);
+}
+
 int launch_rerank_lists(const int64_t *cand, int kr, int64_t B, const uint64_t *ckeys, int nprobe,
                         const float *qs, int ldq, int d_s, const adanns_index *idx,
                         const float *mscale, int k, bool dense, int64_t *out_ids,

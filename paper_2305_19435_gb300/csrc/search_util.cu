@@ -60,7 +60,7 @@ cudaMemPool_t scratch_pool() {
   return pools[dev];
 }
 
-std::atomic<int64_t> g_scratch_held{0};
+std::atomic<int64_t> g_scratch_held{0}, g_scratch_high{0};
 
 // After a call could not get its scratch: hand back what the pool grew by
 // meanwhile, so that the process does not keep memory that no call uses.

@@ -199,12 +199,13 @@ bool adanns_server::launch_one(Lane &L) {
     if (b.method == ADANNS_METHOD_IVFOPQ)
       bytes = rows * (int64_t)(b.nprobe * 64 + b.k * 12 + idx->d * 4) + (64ll << 20);
     else if (mixed && b.storage == ADANNS_STORE_F32)
-      bytes = stream_scratch_bytes(idx, rows, b.d_c, b.d_s, b.nprobe, b.k);
+      bytes = std::max(stream_scratch_bytes(idx, rows, b.d_c, b.d_s, b.nprobe, b.k),
+                       tiled_scratch_bytes(idx, rows, b.d_c, b.d_s, b.nprobe, b.k));
     else
       bytes = adanns_search_scratch_bytes(idx, rows, b.d_c, b.d_s, b.nprobe, b.k, b.storage,
                                           b.rerank_k);
     if (bytes < 0) bytes = 0;
-    bytes += rows * (int64_t)(idx->d * 4 + b.k * 12 + (mixed ? 16 : 0));
+    bytes += rows * (int64_t)(idx->d * 4 + b.k * 12 + (mixed ? 28 : 0));
     const bool any_busy = std::any_of(lanes.begin(), lanes.end(),
                                       [](const std::unique_ptr<Lane> &x) { return x->busy; });
     if (any_busy && inflight + bytes > mem_budget) return false;  // wait for memory

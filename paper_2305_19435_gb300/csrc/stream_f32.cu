@@ -340,11 +340,21 @@ static int64_t stream_per_query(const adanns_index *idx, int d_c, int d_s, int n
          (int64_t)k * 8 + (int64_t)nprobe * 40 + 16;
 }
 
+// few members in all: small units from a table (the whole batch is then one slice),
+// a unit per 64 members of each probed list and group of queries at most; 0: not so
+static int64_t few_units(const adanns_index *idx, int64_t B, int64_t Bc, int nprobe) {
+  const int64_t n = B * nprobe * (((int64_t)idx->max_list + 7 + SFF_THREADS) / SFF_THREADS);
+  const bool few = Bc >= B && probe_plan_small(B * nprobe, idx->nlist) && n <= 1 << 20 &&
+                   (double)B * nprobe * idx->N / idx->nlist <= (double)num_sms() * 1024;
+  return few ? n : 0;
+}
+
 int64_t stream_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,
                              int k) {
   const int64_t per_q = stream_per_query(idx, d_c, d_s, nprobe, k);
   const int64_t Bc = std::max<int64_t>(1, std::min<int64_t>(B, scratch_budget() / per_q));
-  return Bc * per_q + (int64_t)idx->nlist * 64 + (16ll << 20);
+  return Bc * (per_q + coarse_scratch_per_query(idx, d_c)) + (int64_t)idx->nlist * 64 +
+         16 * few_units(idx, B, Bc, nprobe) + Scratch::SLACK;
 }
 
 // Where the streaming scan is taken (ADANNS_OPT_FP32_STREAM = 0 keeps the
@@ -390,12 +400,8 @@ int search_f32_stream(const adanns_index *idx, const float *queries, int64_t B, 
   const int64_t per_q = stream_per_query(idx, d_c, d_s, nprobe, k);
   const int64_t Bc = std::max<int64_t>(1, std::min<int64_t>(B, scratch_budget() / per_q));
   const int64_t max_tiles = (Bc * nprobe + SF_QT - 1) / SF_QT + nlist;
-  // few members in all: small units (the whole batch is then one slice)
-  // (a unit per 64 members of each probed list and group of queries at most)
-  const int64_t max_units =
-      B * nprobe * (((int64_t)idx->max_list + 7 + SFF_THREADS) / SFF_THREADS);
-  const bool few = Bc >= B && probe_plan_small(B * nprobe, nlist) && max_units <= 1 << 20 &&
-                   (double)B * nprobe * idx->N / nlist <= (double)num_sms() * 1024;
+  const int64_t max_units = few_units(idx, B, Bc, nprobe);
+  const bool few = max_units > 0;
   const bool var = qb && qb->ds;
   const int um = few ? SFF_THREADS : SF_THREADS;
   const int qg = few ? SFF_QG : std::max(1, std::min(SF_QG, SF_SMEM / (d_s * 4)));
