@@ -238,6 +238,10 @@ int adanns_index_status(const adanns_index *idx, void *cuda_stream);
 int64_t adanns_search_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int d_s,
                                     int nprobe, int k, int storage, int rerank_k);
 
+/* The same for adanns_search_ivfopq on the index's OPQ data (-1 without any). */
+int64_t adanns_ivfopq_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int nprobe, int k,
+                                    int rerank_k);
+
 /* The most scratch that the library's calls have held at one time since the
  * library was loaded or since the last call with reset != 0 (host-side; all
  * threads and devices together). */
@@ -683,7 +687,8 @@ void adanns_graph_free(adanns_graph *g);
  * budget.  The worker keeps requests in arrival order; whenever one of its
  * nstreams CUDA streams is free it packs the oldest pending request with later
  * ones of the same index and budget into one batch of at most max_batch rows,
- * admits the batch if its scratch estimate (adanns_search_scratch_bytes plus
+ * admits the batch if its scratch estimate (adanns_search_scratch_bytes or
+ * adanns_ivfopq_scratch_bytes, plus
  * the batch's rows and results) fits mem_budget bytes next to the batches in
  * flight (a batch is always admitted when nothing is in flight), and runs it
  * on that stream: pinned staging, host-to-device copy, the search,

@@ -74,6 +74,8 @@ def lib():
         L.adanns_index_status.argtypes = [P, P]
         L.adanns_search_scratch_bytes.argtypes = [P, i64, i32, i32, i32, i32, i32, i32]
         L.adanns_search_scratch_bytes.restype = i64
+        L.adanns_ivfopq_scratch_bytes.argtypes = [P, i64, i32, i32, i32, i32]
+        L.adanns_ivfopq_scratch_bytes.restype = i64
         L.adanns_scratch_high.argtypes = [i32]
         L.adanns_scratch_high.restype = i64
         L.adanns_autotune_search.argtypes = [P, P, i64, i32, i32, i32, i32, P, P, P, P, P]
@@ -426,6 +428,12 @@ def scratch_bytes(index: Index, B: int, d_c: int, d_s: int, nprobe: int, k: int,
     """Upper bound of the device scratch a search with these arguments holds."""
     return int(lib().adanns_search_scratch_bytes(index.handle, B, d_c, d_s, nprobe, k, storage,
                                                  rerank_k))
+
+
+def ivfopq_scratch_bytes(index: Index, B: int, d_c: int, nprobe: int, k: int,
+                         rerank_k: int = 0) -> int:
+    """The same bound for search_ivfopq on the index's OPQ data."""
+    return int(lib().adanns_ivfopq_scratch_bytes(index.handle, B, d_c, nprobe, k, rerank_k))
 
 
 def scratch_high(reset: bool = False) -> int:

@@ -231,6 +231,45 @@ int encode_lists(adanns_index *x, const float *db, cudaStream_t st) {
   return ADANNS_OK;
 }
 
+// slices and scratch of run_ivfopq_select
+struct SelectShape {
+  int nkb;        // K-blocks of the filter's rows
+  int parts;      // lookup scans per slice
+  int64_t seg_q;  // largest candidate segment of a query
+  int64_t fixed;  // scratch whatever the slice
+  int64_t per_q;  // and per query of a slice
+  int64_t Bc, Bp;  // queries per slice and per lookup scan
+};
+
+SelectShape select_shape(const adanns_index *idx, int64_t B, int d_c, int nprobe, int kr,
+                         bool rerank, bool cert) {
+  const int d_s = idx->opq_ds, M = idx->opq_M;
+  SelectShape h{};
+  h.nkb = (d_s + 63) / 64;
+  h.seg_q = max_probe_members(idx, nprobe);
+  h.fixed = cert ? adc_filter_fixed_bytes(idx) : 0;
+  const int64_t budget = scratch_budget() - h.fixed;
+  auto per_q_of = [&](int cand_bytes) -> int64_t {
+    return h.seg_q * cand_bytes + (int64_t)(pad16(d_c) + pad16(d_s) + d_s) * 4 + (int64_t)M * 1024 +
+           (int64_t)kr * (rerank ? 24 : 16) + (int64_t)nprobe * 40 + 20 +
+           coarse_scratch_per_query(idx, d_c) +
+           (cert ? (int64_t)nprobe * h.nkb * 128 + h.nkb * 128 + CERT_MAX_KK * 8 + 12 : 0);
+  };
+  h.parts = cert && budget / per_q_of(4) < B ? 2 : 1;
+  h.per_q = per_q_of(h.parts == 2 ? 2 : 4);
+  h.Bc = std::max<int64_t>(1, std::min<int64_t>(B, budget / h.per_q));
+  h.Bp = (h.Bc + h.parts - 1) / h.parts;
+  return h;
+}
+
+int64_t select_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int nprobe, int kr,
+                             bool rerank, bool cert) {
+  const SelectShape h = select_shape(idx, B, d_c, nprobe, kr, rerank, cert);
+  // with two lookup scans per slice the last query's scores may not halve
+  return h.fixed + h.Bc * h.per_q + (h.parts == 2 ? h.seg_q * 4 : 0) + (int64_t)idx->nlist * 64 +
+         Scratch::SLACK;
+}
+
 // AdANNS-IVFOPQ search with the distance-then-select ADC stage (Sec. 4.3):
 // per chunk of queries, prep -> cluster mapping -> (list, query tile) work
 // items -> LUTs -> every probed member's ADC distance into the query's
@@ -248,18 +287,9 @@ int run_ivfopq_select(const adanns_index *idx, const float *queries, int64_t B, 
   const int nlist = idx->nlist;
   const int dcp = pad16(d_c), dsp = pad16(d_s);
   const int qa = adc_dist_query_tile(M);
-  const int64_t seg_q = max_probe_members(idx, nprobe);
-  const int nkb = (d_s + 63) / 64, QT = 128, kk = CERT_MAX_KK;
-  const int64_t budget = scratch_budget() - (cert ? idx->N * nkb * 128ll : 0);
-  auto per_q_of = [&](int cand_bytes) -> int64_t {
-    return seg_q * cand_bytes + (int64_t)(dcp + dsp + d_s) * 4 + (int64_t)M * 1024 +
-           (int64_t)kr * 16 + (int64_t)nprobe * 40 + 16 +
-           (cert ? (int64_t)nprobe * nkb * 128 + nkb * 128 + kk * 8 + 12 : 0);
-  };
-  const int parts = cert && budget / per_q_of(4) < B ? 2 : 1;
-  const int64_t Bc =
-      std::max<int64_t>(1, std::min<int64_t>(B, budget / per_q_of(parts == 2 ? 2 : 4)));
-  const int64_t Bp = (Bc + parts - 1) / parts;  // queries per lookup scan
+  const SelectShape h = select_shape(idx, B, d_c, nprobe, kr, rerank, cert);
+  const int nkb = h.nkb, parts = h.parts, QT = 128, kk = CERT_MAX_KK;
+  const int64_t seg_q = h.seg_q, Bc = h.Bc, Bp = h.Bp;
   const int64_t max_tiles = (Bc * nprobe + qa - 1) / qa + nlist;
   const int64_t mma_tiles = (Bc * nprobe + QT - 1) / QT + nlist;
   Scratch s(st);
@@ -455,6 +485,15 @@ int run_ivfopq_select(const adanns_index *idx, const float *queries, int64_t B, 
       return rc;
   }
   return ADANNS_OK;
+}
+
+// slices of the running top-k search: partial results of ~2 GiB
+int64_t topk_slice(const adanns_index *idx, int64_t B, int d_c, int nprobe, int kr,
+                   int64_t *per_q) {
+  const int d_s = idx->opq_ds;
+  *per_q = (int64_t)nprobe * kr * 8 + (int64_t)(pad16(d_c) + pad16(d_s) + d_s) * 4 +
+           (int64_t)idx->opq_M * 1024 + (int64_t)kr * 12 + (int64_t)nprobe * 24;
+  return std::max<int64_t>(1, std::min<int64_t>(B, (2ll << 30) / *per_q));
 }
 
 // The filter's copy of the decoded rows comes on top of the lookup scan's
@@ -730,6 +769,21 @@ int adanns_index_get_opq(const adanns_index *idx, float *R, float *codebooks,
   return ADANNS_OK;
 }
 
+int64_t adanns_ivfopq_scratch_bytes(const adanns_index *idx, int64_t B, int d_c, int nprobe, int k,
+                                    int rerank_k) {
+  if (!idx || !idx->codes || B < 0 || nprobe < 1 || nprobe > idx->nlist || k < 1 || d_c < 1 ||
+      (rerank_k != 0 && rerank_k < k))
+    return -1;
+  const int kr = rerank_k > 0 ? rerank_k : k;
+  if (adc_select_enabled(nprobe) || idx->opq_S)
+    return select_scratch_bytes(idx, B, d_c, nprobe, kr, rerank_k > 0,
+                                adc_certified(idx, B, nprobe, kr));
+  int64_t per_q;
+  const int64_t Bc = topk_slice(idx, B, d_c, nprobe, kr, &per_q);
+  return Bc * (per_q + (int64_t)nprobe * 12 + coarse_scratch_per_query(idx, d_c) + kr * 8) +
+         (int64_t)idx->nlist * 64 + Scratch::SLACK;
+}
+
 int adanns_search_ivfopq(const adanns_index *idx, const float *queries, int64_t B, int d_c,
                          int nprobe, int k, int rerank_k, int64_t *out_ids, float *out_dist,
                          int32_t *out_probes, void *cuda_stream) {
@@ -756,9 +810,8 @@ int adanns_search_ivfopq(const adanns_index *idx, const float *queries, int64_t 
     return search_ivfopq_select(idx, queries, B, d_c, nprobe, k, kr, rerank_k > 0, out_ids,
                                 out_dist, out_probes, st);
   const int qa = adc_query_tile(M, kr);
-  const int64_t per_q = (int64_t)nprobe * kr * 8 + (int64_t)(dcp + dsp + d_s) * 4 +
-                        (int64_t)M * 1024 + (int64_t)kr * 12 + nprobe * 24;
-  const int64_t Bc = std::max<int64_t>(1, std::min<int64_t>(B, (2ll << 30) / per_q));
+  int64_t per_q;
+  const int64_t Bc = topk_slice(idx, B, d_c, nprobe, kr, &per_q);
   const int64_t max_tiles = (Bc * nprobe + qa - 1) / qa + nlist;
   Scratch s(st);
   float *qc, *qs, *z, *lut, *cdist;

@@ -244,6 +244,12 @@ int launch_code_norms(const adanns_index *x, float *y2, float *y2max_host, cudaS
   return ADANNS_OK;
 }
 
+// the FP16 rows and each list's part-filled query tile
+int64_t adc_filter_fixed_bytes(const adanns_index *idx) {
+  const int64_t nkb = (idx->opq_ds + 63) / 64;
+  return idx->N * nkb * 128 + idx->nlist * nkb * 128 * 128;
+}
+
 // Where the filter pays.  In picoseconds, fitted to both sides measured on
 // 50,000 to 3 M rows, one list to 1,024, (d_s, M) from (64, 8) to (768, 64):
 // the lookup scan spends 2 + 0.42 M + 900 M / (members per list) per (query,
@@ -268,7 +274,8 @@ bool adc_certified(const adanns_index *idx, int64_t B, int nprobe, int kr) {
   if (!(idx->opq_y2max <= AC_Y2MAX) || kr > CERT_MAX_K || nprobe > 128 || M > AC_MAX_M)
     return false;
   const int64_t nkb = (d_s + 63) / 64;
-  if (idx->N * nkb > INT32_MAX - 256 || idx->N * nkb * 128 > scratch_budget() / 2) return false;
+  if (idx->N * nkb > INT32_MAX - 256 || adc_filter_fixed_bytes(idx) > scratch_budget() / 2)
+    return false;
   const double N = (double)idx->N, per = N / idx->nlist, qpl = (double)B * nprobe / idx->nlist;
   if (N * qpl * (2.0 + 0.42 * M + 900.0 * M / per) -
           N * d_s * (0.8 + 0.0022 * std::max(qpl, 128.0)) - B * (4e4 + 200.0 * d_s) -

@@ -557,6 +557,7 @@ int launch_select32_results(const uint32_t *cand, const uint64_t *ckeys, int npr
 // Squared norms of every decoded code row y2 [N] and their maximum.
 int launch_code_norms(const adanns_index *x, float *y2, float *y2max_host, cudaStream_t st);
 bool adc_certified(const adanns_index *idx, int64_t B, int nprobe, int kr);
+int64_t adc_filter_fixed_bytes(const adanns_index *idx);
 int launch_decode_f16(const adanns_index *idx, const int32_t *lcnt, int nkb, void *rows,
                       cudaStream_t st);
 // per query with cnt[q] >= 0: the kr smallest (ADC score, id) keys of its cnt[q]

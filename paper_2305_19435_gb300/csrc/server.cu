@@ -197,7 +197,7 @@ bool adanns_server::launch_one(Lane &L) {
       b.k = std::max(b.k, r->b.k);
     }
     if (b.method == ADANNS_METHOD_IVFOPQ)
-      bytes = rows * (int64_t)(b.nprobe * 64 + b.k * 12 + idx->d * 4) + (64ll << 20);
+      bytes = adanns_ivfopq_scratch_bytes(idx, rows, b.d_c, b.nprobe, b.k, b.rerank_k);
     else if (mixed && b.storage == ADANNS_STORE_F32)
       bytes = std::max(stream_scratch_bytes(idx, rows, b.d_c, b.d_s, b.nprobe, b.k),
                        tiled_scratch_bytes(idx, rows, b.d_c, b.d_s, b.nprobe, b.k));

@@ -77,8 +77,9 @@ class GpuExecutor:
 
     def scratch_bytes(self, index_key, budget: Budget, n: int) -> int:
         idx = self.indexes[index_key]
-        if budget.method == 1:   # IVF-OPQ: per-member scores of the probed lists dominate
-            return n * (budget.nprobe * 64 + budget.k * 12 + idx.d * 4) + (64 << 20)
+        if budget.method == 1:   # IVF-OPQ
+            return self.P.ivfopq_scratch_bytes(idx, n, budget.d_c, budget.nprobe, budget.k,
+                                               budget.rerank_k)
         return self.P.scratch_bytes(idx, n, budget.d_c, budget.d_s, budget.nprobe, budget.k,
                                     budget.storage, budget.rerank_k)
 

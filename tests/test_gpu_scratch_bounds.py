@@ -68,3 +68,34 @@ def test_low_precision_and_padding(P):
             assert 0 < n <= P.scratch_bytes(g, 8000, 16, 2048, 8, 100)
             assert n <= budget + (16 << 20) or budget < 800 << 20
     g.free()
+
+
+def test_ivfopq(P):
+    """The lookup scan, the filter (whose FP16 rows count, at more than one part of the
+    batch too) and the running top-k scan; both servers admit by the same bound."""
+    from paper_2305_19435_gb300.serving import Budget, GpuExecutor
+    g, q = make(P, 60000, 128, 256)
+    R, C = torch.eye(128, device="cuda"), 0.05 * torch.randn(32, 256, 4, device="cuda")
+    codes = torch.randint(0, 256, (60000, 32), device="cuda", dtype=torch.uint8)
+    assert P.ivfopq_scratch_bytes(g, 10, 16, 4, 10) == -1  # no codes yet
+    P.set_opq(g, 128, 32, R, C, codes)
+    ex = GpuExecutor({0: g}, 1)
+    for B, npb, k, rr, filtered in [(8000, 16, 10, 0, True), (8000, 16, 100, 400, True),
+                                    (200, 16, 10, 40, False), (1, 4, 10, 0, False),
+                                    (8000, 1, 100, 1000, False), (300, 256, 10, 100, False)]:
+        for budget in (12 << 30, 400 << 20):
+            with P.option(P.OPT_SCRATCH_BYTES, budget):
+                bound = P.ivfopq_scratch_bytes(g, B, 16, npb, k, rr)
+                P.profile_enable(True)
+                n = held(P, lambda: P.search_ivfopq(g, q[:B], 16, npb, k, rerank_k=rr))
+                assert ("mma" in P.profile_read()) == filtered
+                P.profile_enable(False)
+                assert 0 < n <= bound, (B, npb, k, rr)
+                assert ex.scratch_bytes(0, Budget(16, 128, npb, k, 0, rr, 1), B) == bound
+                assert not filtered or bound >= 60000 * 2 * 128
+                assert n <= budget + (16 << 20) or B == 8000 and not filtered
+    with P.option(P.OPT_ADC_SELECT, 0):
+        for B, npb, k, rr in [(8000, 16, 10, 0), (3000, 16, 100, 400), (1, 300 - 44, 10, 10)]:
+            n = held(P, lambda: P.search_ivfopq(g, q[:B], 16, npb, k, rerank_k=rr))
+            assert 0 < n <= P.ivfopq_scratch_bytes(g, B, 16, npb, k, rr), (B, npb, k, rr)
+    g.free()
