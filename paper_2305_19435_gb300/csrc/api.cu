@@ -211,7 +211,8 @@ int make_index(const float *db, int64_t N, int d, const float *centroids, int nl
   x->nlist = nlist;
   x->metric = metric;
   x->storage = storage;
-  int rc;
+  Scratch s(st);
+  int rc, *unsure = nullptr;
   x->ng = 0;
   for (int g = 0; g < NGRAN; ++g)
     if (kGran[g] <= d) x->ng = g + 1;
@@ -222,7 +223,7 @@ int make_index(const float *db, int64_t N, int d, const float *centroids, int nl
       (rc = dmalloc(&x->xpm, (size_t)N * x->d_pad)) ||
       (rc = dmalloc(&x->invn, (size_t)std::max(x->ng, 1) * N)) ||
       (rc = dmalloc(&x->assign, (size_t)N)) || (rc = dmalloc(&x->pos_of_id, (size_t)N)) ||
-      (rc = dmalloc(&x->dev_err, 1))) {
+      (rc = dmalloc(&x->dev_err, 1)) || (rc = s.get(&unsure, 1))) {
     free_index(x);
     return rc;
   }
@@ -231,7 +232,8 @@ int make_index(const float *db, int64_t N, int d, const float *centroids, int nl
     free_index(x);
     return code;
   };
-  if (cudaMemsetAsync(x->dev_err, 0, sizeof(int), st) != cudaSuccess)
+  if (cudaMemsetAsync(x->dev_err, 0, sizeof(int), st) != cudaSuccess ||
+      cudaMemsetAsync(unsure, 0, sizeof(int), st) != cudaSuccess)
     return bail(cuda_fail(cudaGetLastError(), "clear status"));
   if (cudaMemcpyAsync(x->centroids, centroids, sizeof(float) * nlist * d_c,
                       cudaMemcpyDeviceToDevice, st) != cudaSuccess)
@@ -242,7 +244,7 @@ int make_index(const float *db, int64_t N, int d, const float *centroids, int nl
   if ((rc = launch_prefix_major(db, d, d, x->d_pad, x->list_off, x->list_ids, assign, N, x->xpm,
                                 st)))
     return bail(rc);
-  if ((rc = launch_inv_norms(db, d, d, x->list_ids, N, metric, x->invn, x->ng, st)))
+  if ((rc = launch_inv_norms(db, d, d, x->list_ids, N, metric, x->invn, x->ng, unsure, st)))
     return bail(rc);
   if (cudaMemcpyAsync(x->assign, assign, sizeof(int32_t) * N, cudaMemcpyDeviceToDevice, st) !=
       cudaSuccess)
@@ -252,7 +254,8 @@ int make_index(const float *db, int64_t N, int d, const float *centroids, int nl
   if ((storage & ADANNS_STORE_FP8E4M3) && (rc = build_lowp(x, db, 1, st))) return bail(rc);
   x->h_list_off = new int64_t[nlist + 1];
   if (cudaMemcpyAsync(x->h_list_off, x->list_off, sizeof(int64_t) * (nlist + 1),
-                      cudaMemcpyDeviceToHost, st) != cudaSuccess)
+                      cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaMemcpyAsync(&x->unsure, unsure, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
     return bail(cuda_fail(cudaGetLastError(), "copy list offsets"));
   cudaError_t e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return bail(cuda_fail(e, "index build"));

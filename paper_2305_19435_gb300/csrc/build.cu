@@ -426,9 +426,12 @@ int launch_positions(const int32_t *list_ids, int64_t N, int32_t *pos, cudaStrea
 }
 
 // invn[g][p] = 1 / ||x[list_ids[p]][0:G[g]]|| (0 for a zero prefix; 1 for raw L2)
+// unsure (or null): bit g is set when a row's squared norm at granularity g is NaN,
+// infinite or so small that its squares lost digits (its scaled prefix is then not
+// of norm 1)
 __global__ void inv_norms_kernel(const float *__restrict__ x, int ld, int d,
                                  const int32_t *__restrict__ list_ids, int64_t N, int metric,
-                                 float *__restrict__ invn, int ng) {
+                                 float *__restrict__ invn, int ng, int *__restrict__ unsure) {
   const int64_t p = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (p >= N) return;
@@ -443,15 +446,16 @@ __global__ void inv_norms_kernel(const float *__restrict__ x, int ld, int d,
       float v = 1.f;
       if (metric == ADANNS_METRIC_L2_PREFIXNORM) v = s > 0.f ? 1.f / sqrtf(s) : 0.f;
       invn[(int64_t)g * N + p] = v;
+      if (unsure && s != 0.f && !(s >= 1e-30f && s <= 1e38f)) atomicOr(unsure, 1 << g);
     }
   }
 }
 
 int launch_inv_norms(const float *x, int ld, int d, const int32_t *list_ids, int64_t N, int metric,
-                     float *invn, int ng, cudaStream_t st) {
+                     float *invn, int ng, int *unsure, cudaStream_t st) {
   if (N <= 0) return ADANNS_OK;
   inv_norms_kernel<<<(unsigned)((N + 7) / 8), 256, 0, st>>>(x, ld, d, list_ids, N, metric, invn,
-                                                           ng);
+                                                           ng, unsure);
   ADN_LAUNCH("inv_norms_kernel");
   return ADANNS_OK;
 }

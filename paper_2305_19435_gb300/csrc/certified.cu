@@ -29,8 +29,10 @@
 // |p.y - p~.y~| <= |p||r_y| + |r_p||y| + |r_p||r_y|, |r_y| <= 1.005 u + d 2^-25
 // (member side, a constant), |p| and |r_p| measured per query; the FP32 accumulation
 // and re-score terms are those of the mixed-precision pruning (e_rest).
-// Prefixes whose computed norm is off (sums of squares in the denormal range)
-// make the whole call take the tiled scan through the same mechanism.
+// An index that holds a row whose prefix has no usable norm (NaN, infinite, sums of
+// squares in the denormal range; known when it is formed) has its batches at that d_s
+// answered by the direct scans; where the filter runs all the same, such a row in a
+// probed list leaves every query to the tiled scan.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -347,7 +349,8 @@ Shape shape_of(const adanns_index *idx, int64_t B, int d_c, int d_s, int nprobe,
 // k 256 (every member of the lists is re-scored), 600 per list 1948 / - / 991.
 // Below F32_SMALL rows all routes are bound by launches; there the filter stays
 // above 100 queries per list while it is within 80 us of the others (65 at k 1), so
-// that its small sizes keep being run.  k and the probes must fit the shortlist's buffers,
+// that its small sizes keep being run.  A row without a usable norm would leave every
+// query to the tiled scan: the direct scans from the start.  k and the probes must fit the shortlist's buffers,
 // and the FP16 rows with the tiles' padding may take half of the call's scratch budget.  Turning the
 // streaming scan off asks for the tiled scan everywhere.
 constexpr int64_t F32_SMALL = 8192;
@@ -363,6 +366,7 @@ bool f32_certified(const adanns_index *idx, int64_t B, int d_s, int nprobe, int 
   if (k == 1 && pairs > 16ll * idx->nlist)
     other = std::min(other, f32_cost(F32_TILED, idx, B, pairs, d_s, k));
   const double qpl = (double)pairs / idx->nlist;
+  if (idx->N >= F32_SMALL && (idx->unsure >> gran_index(d_s) & 1)) return false;
   if (idx->N < F32_SMALL && qpl > 100.0 && (double)idx->N * d_s * qpl > 2e7 &&
       nprobe * idx->N > shortlist_cap(k) * (int64_t)idx->nlist)
     other += k == 1 ? 6.5e7 : 8e7;

@@ -305,7 +305,7 @@ int launch_prefix_major(const float *x, int ld, int d, int d_pad, const int64_t 
                         const int32_t *list_ids, const int32_t *assign, int64_t N, float *xpm,
                         cudaStream_t st);
 int launch_inv_norms(const float *x, int ld, int d, const int32_t *list_ids, int64_t N,
-                     int metric, float *invn /* [ng][N] */, int ng, cudaStream_t st);
+                     int metric, float *invn /* [ng][N] */, int ng, int *unsure, cudaStream_t st);
 int launch_kmeans_update(const float *t, int64_t n, int ld, int dim, const int32_t *assign,
                          int nc, double *sums, int32_t *counts, float *cent, cudaStream_t st);
 int launch_sum_keys(const uint64_t *keys, int64_t n, double *out, cudaStream_t st);
@@ -615,6 +615,7 @@ struct adanns_index {
   int32_t *list_ids = nullptr;  // N
   float *xpm = nullptr;         // prefix-major FP32 vectors
   float *invn = nullptr;        // [ng][N] inverse prefix norms in list order
+  int unsure = 0;               // bit g: a row's prefix at granularity g has no usable norm
   int ng = 0;
   int32_t *assign = nullptr;    // list of each id (N)
   int32_t *pos_of_id = nullptr; // list-order position of each id (N)

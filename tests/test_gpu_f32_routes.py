@@ -63,3 +63,28 @@ def test_stream_or_tiled(P, d_s, nprobe, k, B, tiled):
     np.testing.assert_array_equal(a[0], b[0])
     np.testing.assert_array_equal(a[1].view(np.int32), b[1].view(np.int32))
     g.free()
+
+
+# NaN, infinity, a squared norm that underflows and one that overflows, at the last
+# coordinate: only the prefixes that reach it are kept from the filter
+@pytest.mark.parametrize("value", [np.nan, -np.inf, 1e-21, 3e19])
+def test_rows_without_a_norm(P, value):
+    data = synthdata.small(20000, 2048, 256, 64, 45)
+    db = data["db"].copy()
+    if value == 1e-21:
+        db[777] = 0
+    db[777, 255] = value
+    g = P.index_create(torch.from_numpy(db).cuda(), torch.from_numpy(data["means"][:16, :16].copy()).cuda(),
+                       torch.arange(20000, dtype=torch.int32, device="cuda") % 16)
+    q = torch.from_numpy(data["queries"]).cuda()
+    for d_s in (128, 256):
+        P.profile_enable(True)
+        a = [t.cpu().numpy() for t in P.search_ivf(g, q, 16, d_s, 8, 20)]
+        stages = P.profile_read()
+        P.profile_enable(False)
+        assert ("mma" in stages) == (d_s == 128)
+        with P.option(P.OPT_FP32_STREAM, 0):
+            b = [t.cpu().numpy() for t in P.search_ivf(g, q, 16, d_s, 8, 20)]
+        np.testing.assert_array_equal(a[0], b[0])
+        np.testing.assert_array_equal(a[1].view(np.int32), b[1].view(np.int32))
+    g.free()
