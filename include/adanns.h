@@ -576,7 +576,9 @@ int adanns_tune_clear(void);
  * adanns_plan_create runs adanns_search_ivf once with the given arguments on
  * cuda_stream (validating them, setting kernel attributes, growing the
  * scratch pool; synchronises), then captures the same call on a private
- * stream into a CUDA graph.  The plan is bound to the given device buffers:
+ * stream into a CUDA graph (an FP32 search whose graph cannot have its memory
+ * by the next of adanns_search_ivf's routes, which needs less).  The plan is
+ * bound to the given device buffers:
  * each adanns_plan_launch re-runs the whole search (cluster mapping, probe
  * inversion, list scan, selection, rerank, merge) on the current contents of
  * `queries`, writing out_ids / out_dist, with one graph launch on

@@ -54,18 +54,19 @@ __global__ void pq_assign_kernel(const float *__restrict__ z, int64_t n, int ldz
 // in codeword order.  A CTA takes PQA_THREADS * PQA_P points and mg sub-vectors:
 // PQA_MG, whose codes leave together, or fewer while there are not enough points for
 // a CTA per SM (encoding 507 points, 8 sub-vectors of 8: 65 us by the kernel above, 98
-// with 2 CTAs that take 8 in turn, 41 with 16 that take one).  Bound by the FP32 pipe
+// with 2 CTAs that take 8 in turn, 41 with 16 that take one); FEW, a kernel of its
+// own, since a variable group costs the full one up to 1.6%.  Bound by the FP32 pipe
 // (an add and a multiply-add per coordinate and codeword): 262,144 points, 32
 // sub-vectors of 12 in 1.66 ms, 84% of the rate of those instructions (four points
 // per thread: 1.70).
 constexpr int PQA_THREADS = 128, PQA_P = 2, PQA_MG = 8;
 
-template <int DS>
+template <int DS, bool FEW>
 __global__ void __launch_bounds__(PQA_THREADS) pq_assign_regs_kernel(
     const float *__restrict__ z, int64_t n, int ldz, int M, int mg, const float *__restrict__ C,
     uint8_t *__restrict__ codes, float *__restrict__ mind) {
   extern __shared__ __align__(16) float Cs[];  // [128][DS][2]
-  const int m0 = blockIdx.y * mg, nm = min(mg, M - m0);
+  const int per = FEW ? mg : PQA_MG, m0 = blockIdx.y * per, nm = min(per, M - m0);
   const int64_t i0 = (int64_t)blockIdx.x * (PQA_THREADS * PQA_P) + threadIdx.x;
   uint32_t cw[PQA_P][PQA_MG / 4];
 #pragma unroll
@@ -149,13 +150,14 @@ int launch_pq_assign(const float *z, int64_t n, int ldz, int M, int dsub, const 
                      uint8_t *codes, float *mind, cudaStream_t st) {
   if (n <= 0) return ADANNS_OK;
   // the register kernel for the sub-vector sizes it is built for
-  auto regs = [&](auto kern) -> int {
+  auto regs = [&](auto many, auto few) -> int {
     const size_t sm = (size_t)256 * dsub * 4;
-    ADN_CUDA(ensure_smem((const void *)kern, sm));
     const int per = PQA_THREADS * PQA_P;
     const int64_t gx = (n + per - 1) / per;
     int mg = PQA_MG;
     while (mg > 1 && gx * ((M + mg - 1) / mg) < num_sms()) mg >>= 1;
+    auto kern = mg < PQA_MG ? few : many;
+    ADN_CUDA(ensure_smem((const void *)kern, sm));
     const dim3 grid((unsigned)gx, (M + mg - 1) / mg);
     kern<<<grid, PQA_THREADS, sm, st>>>(z, n, ldz, M, mg, C, codes, mind);
     ADN_LAUNCH("pq_assign_regs_kernel");
@@ -163,12 +165,12 @@ int launch_pq_assign(const float *z, int64_t n, int ldz, int M, int dsub, const 
   };
   if ((ldz & 3) == 0 && ((uintptr_t)z & 15) == 0) {
     switch (dsub) {
-      case 4: return regs(pq_assign_regs_kernel<4>);
-      case 8: return regs(pq_assign_regs_kernel<8>);
-      case 12: return regs(pq_assign_regs_kernel<12>);
-      case 16: return regs(pq_assign_regs_kernel<16>);
-      case 24: return regs(pq_assign_regs_kernel<24>);
-      case 32: return regs(pq_assign_regs_kernel<32>);
+      case 4: return regs(pq_assign_regs_kernel<4, false>, pq_assign_regs_kernel<4, true>);
+      case 8: return regs(pq_assign_regs_kernel<8, false>, pq_assign_regs_kernel<8, true>);
+      case 12: return regs(pq_assign_regs_kernel<12, false>, pq_assign_regs_kernel<12, true>);
+      case 16: return regs(pq_assign_regs_kernel<16, false>, pq_assign_regs_kernel<16, true>);
+      case 24: return regs(pq_assign_regs_kernel<24, false>, pq_assign_regs_kernel<24, true>);
+      case 32: return regs(pq_assign_regs_kernel<32, false>, pq_assign_regs_kernel<32, true>);
       default: break;
     }
   }
