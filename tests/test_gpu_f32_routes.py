@@ -88,3 +88,27 @@ def test_rows_without_a_norm(P, value):
         np.testing.assert_array_equal(a[0], b[0])
         np.testing.assert_array_equal(a[1].view(np.int32), b[1].view(np.int32))
     g.free()
+
+
+# an index small enough to keep the filter: the row's lists leave their queries, and
+# with them all others, to the tiled scan
+@pytest.mark.parametrize("value", [np.nan, np.inf, -3e19, 1e-21])
+def test_rows_without_a_norm_in_the_filter(P, value):
+    data = synthdata.small(6000, 333, 64, 24, 46)
+    db, q = data["db"].copy(), data["queries"].copy()
+    db[11], db[77, 3], q[5] = 0, value, 0
+    db[11, 0] = value
+    g = P.index_create(torch.from_numpy(db).cuda(), torch.from_numpy(data["means"][:24, :16].copy()).cuda(),
+                       torch.arange(6000, dtype=torch.int32, device="cuda") % 24)
+    q = torch.from_numpy(q).cuda()
+    P.profile_enable(True)
+    a = [t.cpu().numpy() for t in P.search_ivf(g, q, 16, 64, 24, 100)]
+    stages = P.profile_read()
+    P.profile_enable(False)
+    assert "mma" in stages
+    with P.option(P.OPT_FP32_STREAM, 0):
+        b = [t.cpu().numpy() for t in P.search_ivf(g, q, 16, 64, 24, 100)]
+    g.status()
+    np.testing.assert_array_equal(a[0], b[0])
+    np.testing.assert_array_equal(a[1].view(np.int32), b[1].view(np.int32))
+    g.free()
