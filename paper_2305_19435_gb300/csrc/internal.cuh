@@ -532,6 +532,11 @@ int launch_rerank_query(const int64_t *cand, int kr, int64_t B, const int32_t *o
                         const float *qs, int ldq, int d_s, const adanns_index *idx,
                         const float *mscale, int lanes, uint64_t *keys, cudaStream_t st,
                         int64_t *npairs = nullptr);  // zeroed counter of re-scored pairs
+// the same of short shortlists, with the k best as results (1: longer ones)
+int launch_rerank_few(const int64_t *cand, int kr, int64_t B, const int32_t *order, const float *qs,
+                      int ldq, int d_s, const adanns_index *idx, const float *mscale, int lanes,
+                      int k, int64_t *out_ids, float *out_dist, cudaStream_t st,
+                      int64_t *npairs = nullptr);
 int adc_dist_query_tile(int M);
 // res_S / res_w / res_w2 / z (NULL for plain codes): residual terms and the
 // queries' rotated vectors [B][d_s]; the score of a member of list l is then

@@ -474,9 +474,11 @@ int launch_rerank(const int64_t *cand, int kr, int64_t B, const int32_t *order, 
                   int ldq, int d_s, const adanns_index *idx, const float *mscale, int k,
                   int64_t *out_ids, float *out_dist, cudaStream_t st) {
   if (B <= 0) return ADANNS_OK;
+  int rc = launch_rerank_few(cand, kr, B, order, qs, ldq, d_s, idx, mscale, 8, k, out_ids, out_dist,
+                             st);
+  if (rc != 1) return rc;
   Scratch s(st);
   uint64_t *keys;
-  int rc;
   if ((rc = s.get(&keys, (size_t)B * kr)) ||
       (rc = launch_rerank_query(cand, kr, B, order, qs, ldq, d_s, idx, mscale, 8, keys, st)))
     return rc;

@@ -293,7 +293,7 @@ int launch_rerank_lists(const int64_t *cand, int kr, int64_t B, const uint64_t *
   const int64_t N = idx->N;
   Scratch s(st);
   if (rerank_by_query(n, N, d_s)) {
-    uint64_t *qk;
+    uint64_t *qk = nullptr;
     int64_t *np = nullptr;
     int32_t *order = nullptr;
     int rc;
@@ -301,16 +301,19 @@ int launch_rerank_lists(const int64_t *cand, int kr, int64_t B, const uint64_t *
         ((rc = s.get(&order, (size_t)B)) ||
          (rc = launch_query_order(idx, ckeys, B, nprobe, order, st))))
       return rc;
-    if ((rc = s.get(&qk, n)) || (profiling() && (rc = s.get(&np, 1)))) return rc;
+    if (profiling() && (rc = s.get(&np, 1))) return rc;
     if (np) ADN_CUDA(cudaMemsetAsync(np, 0, sizeof(int64_t), st));
     {
       StageTimer t(ST_RR_PAIRS, st);
-      if ((rc = launch_rerank_query(cand, kr, B, order, qs, ldq, d_s, idx, mscale, 16, qk, st,
-                                    np)))
-        return rc;
+      rc = launch_rerank_few(cand, kr, B, order, qs, ldq, d_s, idx, mscale, 16, k, out_ids,
+                             out_dist, st, np);
+      if (rc == 1 && (rc = s.get(&qk, n)) == ADANNS_OK)
+        rc = launch_rerank_query(cand, kr, B, order, qs, ldq, d_s, idx, mscale, 16, qk, st, np);
+      if (rc) return rc;
     }
     if (np) profile_count(PC_RERANK_PAIRS, np, st);
     profile_count_host(PC_SHORTLIST_SLOTS, n);
+    if (!qk) return ADANNS_OK;
     StageTimer t(ST_RR_FINAL, st);
     return launch_final_topk(qk, kr, B, k, out_ids, out_dist, st, dense);
   }

@@ -20,14 +20,47 @@ namespace {
 
 constexpr int RQ_THREADS = 128;
 
-// GL lanes per candidate: lane s takes the 16-byte groups s, s + GL, ... of the
-// row in ascending order, and the lanes' sums are added by shuffles (distances
-// GL / 2 .. 1 for 16 lanes, 1 .. GL / 2 for 8): the sums of the member-major
-// rerank (16) and of the IVF-OPQ rerank (8), bit for bit.  Up to eight groups
-// per lane are requested before the first is used: a row's four consecutive
-// lanes read 64 contiguous bytes.  IDS: cand holds database ids, else (list <<
-// 32 | member); -1 is padding.  A CTA takes `per` slots of its query, 128 at a
-// time: their addresses are looked up by one thread each, empty slots dropped.
+// |q - nu x|^2 of one row by GL lanes (this one is lane s): lane s takes the 16-byte
+// groups s, s + GL, ... of the row in ascending order, up to eight of them requested
+// before the first is used, and the lanes' sums are added by shuffles (distances
+// GL / 2 .. 1 for 16 lanes, 1 .. GL / 2 for 8)
+template <int GL>
+__device__ __forceinline__ float row_dist(const float *x0, int nl, float nu, const float *sq, int s,
+                                          int nseg, unsigned gmask) {
+  const int64_t bs = (int64_t)16 * nl;  // floats between a row's blocks
+  const float *row = x0 + (s >> 2) * bs + (s & 3) * 4;
+  float acc = 0.f;
+  for (int e0 = s; e0 < nseg; e0 += 8 * GL, row += 2 * GL * bs) {
+    float4 x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (e0 + GL * u < nseg) x[u] = __ldg((const float4 *)(row + u * (GL / 4) * bs));
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (e0 + GL * u >= nseg) break;
+      const float4 p = *(const float4 *)(sq + 4 * (e0 + GL * u));
+      float d;
+      d = fmaf(-nu, x[u].x, p.x); acc = fmaf(d, d, acc);
+      d = fmaf(-nu, x[u].y, p.y); acc = fmaf(d, d, acc);
+      d = fmaf(-nu, x[u].z, p.z); acc = fmaf(d, d, acc);
+      d = fmaf(-nu, x[u].w, p.w); acc = fmaf(d, d, acc);
+    }
+  }
+  if (GL == 16) {
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(gmask, acc, o);
+  } else {
+#pragma unroll
+    for (int o = 1; o < GL; o <<= 1) acc += __shfl_xor_sync(gmask, acc, o);
+  }
+  return acc;
+}
+
+// GL lanes per candidate (row_dist): the sums of the member-major rerank (16) and
+// of the IVF-OPQ rerank (8), bit for bit.  A row's four consecutive lanes read 64
+// contiguous bytes.  IDS: cand holds database ids, else (list << 32 | member); -1
+// is padding.  A CTA takes `per` slots of its query, 128 at a time: their addresses
+// are looked up by one thread each, empty slots dropped.
 template <int GL, bool IDS>
 __global__ void __launch_bounds__(RQ_THREADS, 7) rerank_query_kernel(
     const int64_t *__restrict__ cand, int kr, int per, const int32_t *__restrict__ order,
@@ -72,36 +105,89 @@ __global__ void __launch_bounds__(RQ_THREADS, 7) rerank_query_kernel(
     const int n = s_n;
     if (npairs && tid == 0) atomicAdd(npairs, (unsigned long long)n);
     for (int t = grp; t < n; t += RQ_THREADS / GL) {
-      const int64_t bs = (int64_t)16 * s_nl[t];  // floats between a row's blocks
-      const float *row = xpm + s_base[t] + (s >> 2) * bs + (s & 3) * 4;
-      const float nu = s_nu[t];
-      float acc = 0.f;
-      for (int e0 = s; e0 < nseg; e0 += 8 * GL, row += 2 * GL * bs) {
-        float4 x[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (e0 + GL * u < nseg) x[u] = __ldg((const float4 *)(row + u * (GL / 4) * bs));
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          if (e0 + GL * u >= nseg) break;
-          const float4 p = *(const float4 *)(sq + 4 * (e0 + GL * u));
-          float d;
-          d = fmaf(-nu, x[u].x, p.x); acc = fmaf(d, d, acc);
-          d = fmaf(-nu, x[u].y, p.y); acc = fmaf(d, d, acc);
-          d = fmaf(-nu, x[u].z, p.z); acc = fmaf(d, d, acc);
-          d = fmaf(-nu, x[u].w, p.w); acc = fmaf(d, d, acc);
-        }
-      }
-      if (GL == 16) {
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(gmask, acc, o);
-      } else {
-#pragma unroll
-        for (int o = 1; o < GL; o <<= 1) acc += __shfl_xor_sync(gmask, acc, o);
-      }
+      const float acc = row_dist<GL>(xpm + s_base[t], s_nl[t], s_nu[t], sq, s, nseg, gmask);
       if (s == 0) keys[q * kr + s_slot[t]] = pack_key(acc, s_id[t]);
     }
     __syncthreads();  // the slots' data are rewritten
+  }
+}
+
+// Short shortlists: a CTA takes nq whole queries, at most 128 slots in all, and a warp
+// sorts a query's distances in registers and writes its results, so that the slots'
+// dependent lookups (list, offset, scale, id) and the barriers are paid once for nq
+// queries and no second kernel reads the keys.  With a CTA per query and a kernel for
+// the sort these cost more than the rows: rerank stage of 12,000 queries x 4 slots at
+// d_s 64 (IVF-OPQ) 93 us, 26 here; x 64 slots 116 and 76; 50,000 x 4 at d_s 1,024 (FP8)
+// 446 and 340.
+template <int GL, bool IDS, int J>  // up to 32 J slots per query
+__global__ void __launch_bounds__(RQ_THREADS, 7) rerank_few_kernel(
+    const int64_t *__restrict__ cand, int kr, int nq, int64_t B, const int32_t *__restrict__ order,
+    const float *__restrict__ qs, int ldq, int d_s, const float *__restrict__ xpm, int d_pad,
+    const int64_t *__restrict__ list_off, const int32_t *__restrict__ list_ids,
+    const int32_t *__restrict__ assign, const int32_t *__restrict__ pos,
+    const float *__restrict__ mscale, int k, int64_t *__restrict__ out_ids,
+    float *__restrict__ out_dist, unsigned long long *__restrict__ npairs) {
+  extern __shared__ __align__(16) float sq[];  // [nq][d_s] the query rows
+  __shared__ int64_t s_base[RQ_THREADS];       // float offset of the member's first block
+  __shared__ int s_nl[RQ_THREADS], s_slot[RQ_THREADS], s_n;
+  __shared__ int64_t s_qid[RQ_THREADS];
+  __shared__ float s_nu[RQ_THREADS];
+  __shared__ uint32_t s_id[RQ_THREADS];
+  __shared__ uint64_t s_key[RQ_THREADS];
+  const int64_t q0 = (int64_t)blockIdx.x * nq;
+  const int tid = threadIdx.x, n_q = (int)min((int64_t)nq, B - q0);
+  const int nseg = d_s >> 2;  // 16-byte groups (d_s is a multiple of 8)
+  if (tid < n_q) s_qid[tid] = order ? order[q0 + tid] : q0 + tid;
+  if (tid == 0) s_n = 0;
+  __syncthreads();
+  for (int e = tid; e < n_q * nseg; e += RQ_THREADS) {
+    const int ql = e / nseg;
+    cp_async16((float4 *)sq + e, (const float4 *)(qs + s_qid[ql] * ldq) + (e - ql * nseg));
+  }
+  cp_async_commit();
+  if (tid < n_q * kr) {
+    const int ql = tid / kr;
+    const int64_t v = cand[s_qid[ql] * kr + (tid - ql * kr)];
+    s_key[tid] = KEY_MAX;
+    if (v >= 0) {
+      const int l = IDS ? assign[v] : (int)(v >> 32);
+      const int64_t off = list_off[l], p = IDS ? (int64_t)pos[v] : off + (v & 0xffffffffll);
+      const int t = atomicAdd(&s_n, 1);
+      s_base[t] = off * d_pad + (p - off) * 16;
+      s_nl[t] = (int)(list_off[l + 1] - off);
+      s_nu[t] = mscale ? mscale[p] : 1.f;
+      s_id[t] = IDS ? (uint32_t)v : (uint32_t)list_ids[p];
+      s_slot[t] = tid;
+    }
+  }
+  cp_async_wait<0>();
+  __syncthreads();
+  const int n = s_n;
+  if (npairs && tid == 0) atomicAdd(npairs, (unsigned long long)n);
+  const int s = tid & (GL - 1);
+  const unsigned gmask = (GL == 16 ? 0xFFFFu : 0xFFu) << (threadIdx.x & 31 & ~(GL - 1));
+  for (int t = tid / GL; t < n; t += RQ_THREADS / GL) {
+    const float acc = row_dist<GL>(xpm + s_base[t], s_nl[t], s_nu[t], sq + s_slot[t] / kr * d_s, s,
+                                   nseg, gmask);
+    if (s == 0) s_key[s_slot[t]] = pack_key(acc, s_id[t]);
+  }
+  __syncthreads();
+  const int lane = tid & 31;
+  for (int ql = tid >> 5; ql < n_q; ql += RQ_THREADS / 32) {
+    uint64_t key[J];  // positions J lane ..
+#pragma unroll
+    for (int j = 0; j < J; ++j)
+      key[j] = J * lane + j < kr ? s_key[ql * kr + J * lane + j] : KEY_MAX;
+    if (J == 1) key[0] = warp_sort_lane(key[0]);
+    else warp_sort_lanes<J>(key);
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      if (J * lane + j >= k) continue;
+      const int64_t o = s_qid[ql] * k + J * lane + j;
+      out_ids[o] = key[j] == KEY_MAX ? -1 : (int64_t)(uint32_t)(key[j] & 0xffffffffu);
+      out_dist[o] = key[j] == KEY_MAX ? __int_as_float(0x7f800000)
+                                      : __uint_as_float((uint32_t)(key[j] >> 32));
+    }
   }
 }
 
@@ -114,6 +200,28 @@ __global__ void __launch_bounds__(RQ_THREADS, 7) rerank_query_kernel(
 // 2.0).
 bool rerank_order_pays(const adanns_index *idx, int64_t slots, int d_s) {
   return idx->nlist > 1 && (double)slots * d_s * 4 > 1e9;
+}
+
+// Rerank and results of short shortlists in one launch; returns 1 (nothing launched)
+// for longer ones: above 32 slots, above 64 of rows of at most 128 coordinates (whose
+// reads cost less than what is saved).  As many queries per CTA as leave the GPU two waves of CTAs, their
+// rows 24 KB at most.
+int launch_rerank_few(const int64_t *cand, int kr, int64_t B, const int32_t *order, const float *qs,
+                      int ldq, int d_s, const adanns_index *idx, const float *mscale, int lanes,
+                      int k, int64_t *out_ids, float *out_dist, cudaStream_t st, int64_t *npairs) {
+  if (kr > 64 || (kr > 32 && d_s > 128)) return 1;
+  if (B <= 0) return ADANNS_OK;
+  const int64_t fill = B / ((int64_t)num_sms() * 14);
+  const int nq = (int)std::max<int64_t>(
+      1, std::min<int64_t>(fill, std::min(RQ_THREADS / kr, 24576 / (d_s * 4))));
+  const unsigned grid = (unsigned)((B + nq - 1) / nq);
+  auto kern = lanes == 16 ? (kr > 32 ? rerank_few_kernel<16, false, 2> : rerank_few_kernel<16, false, 1>)
+                          : (kr > 32 ? rerank_few_kernel<8, true, 2> : rerank_few_kernel<8, true, 1>);
+  kern<<<grid, RQ_THREADS, (size_t)nq * d_s * 4, st>>>(
+      cand, kr, nq, B, order, qs, ldq, d_s, idx->xpm, idx->d_pad, idx->list_off, idx->list_ids,
+      idx->assign, idx->pos_of_id, mscale, k, out_ids, out_dist, (unsigned long long *)npairs);
+  ADN_LAUNCH("rerank_few_kernel");
+  return ADANNS_OK;
 }
 
 // lanes: 16 (the low-precision tiers' rerank) or 8 (IVF-OPQ's, cand = ids)
