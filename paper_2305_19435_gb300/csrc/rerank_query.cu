@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(RQ_THREADS, 7) rerank_query_kernel(
 // queries and no second kernel reads the keys.  With a CTA per query and a kernel for
 // the sort these cost more than the rows: rerank stage of 12,000 queries x 4 slots at
 // d_s 64 (IVF-OPQ) 93 us, 26 here; x 64 slots 116 and 76; 50,000 x 4 at d_s 1,024 (FP8)
-// 446 and 340.
+// 446 and 215.
 template <int GL, bool IDS, int J>  // up to 32 J slots per query
 __global__ void __launch_bounds__(RQ_THREADS, 7) rerank_few_kernel(
     const int64_t *__restrict__ cand, int kr, int nq, int64_t B, const int32_t *__restrict__ order,
@@ -204,16 +204,19 @@ bool rerank_order_pays(const adanns_index *idx, int64_t slots, int d_s) {
 
 // Rerank and results of short shortlists in one launch; returns 1 (nothing launched)
 // for longer ones: above 32 slots, above 64 of rows of at most 128 coordinates (whose
-// reads cost less than what is saved).  As many queries per CTA as leave the GPU two waves of CTAs, their
-// rows 24 KB at most.
+// reads cost less than what is saved).  As many queries per CTA as leave the GPU two
+// waves of CTAs, but 64 KB of member rows at most: more queries in flight at a time
+// share less of their rows in L2 (150,000 x 2,048, 16,400 queries x 32 slots: rerank
+// stage 1,230 us with three queries per CTA, 379 with one).
 int launch_rerank_few(const int64_t *cand, int kr, int64_t B, const int32_t *order, const float *qs,
                       int ldq, int d_s, const adanns_index *idx, const float *mscale, int lanes,
                       int k, int64_t *out_ids, float *out_dist, cudaStream_t st, int64_t *npairs) {
   if (kr > 64 || (kr > 32 && d_s > 128)) return 1;
   if (B <= 0) return ADANNS_OK;
   const int64_t fill = B / ((int64_t)num_sms() * 14);
-  const int nq = (int)std::max<int64_t>(
-      1, std::min<int64_t>(fill, std::min(RQ_THREADS / kr, 24576 / (d_s * 4))));
+  // (their query rows 24 KB at most)
+  const int cap = std::min({RQ_THREADS / kr, 65536 / (kr * d_s * 4), 24576 / (d_s * 4)});
+  const int nq = (int)std::max<int64_t>(1, std::min<int64_t>(fill, cap));
   const unsigned grid = (unsigned)((B + nq - 1) / nq);
   auto kern = lanes == 16 ? (kr > 32 ? rerank_few_kernel<16, false, 2> : rerank_few_kernel<16, false, 1>)
                           : (kr > 32 ? rerank_few_kernel<8, true, 2> : rerank_few_kernel<8, true, 1>);
